@@ -72,19 +72,31 @@ struct OzTile {
   static_assert(STAGE_BYTES % 1024 == 0, "stages stay 1024-byte aligned");
 };
 
-// Digit planes are stored K-blocked: element (s, r, k) of an operand with R rows lives at
-//   s*plane + (k / BK) * (Rpad * BK) + r * BK + (k % BK),   Rpad = R rounded up to ROWPAD,
-// so that every pipeline stage of every tile is one contiguous block per plane.  A tile box that
-// reaches past Rpad reads the next K block's rows (finite digits) or, at the end of a plane, the
-// TMA's zero fill: those rows only feed output rows or columns beyond M or N, which are never
-// stored.
+// Digit planes are stored K-blocked: the 16 values of K block k / BK of row r of plane s lie at
+//   s*plane + (k / BK) * (Rpad * BK) + r * BK,   Rpad = R rounded up to ROWPAD,
+// so that every pipeline stage of every tile is one contiguous block per plane, and the two
+// 8-value halves of such a 32-byte row are swapped when bit 2 of r is set.  That is the image the
+// MMA's 32-byte-swizzle operand has in shared memory (16-byte chunk index ^= address bit 7), so a
+// stage is a plain copy: the tensor maps see rows of 256 elements (16 stored rows, 512 bytes) and
+// do not swizzle.  The TMA unit works through a box row by row, about 1.4 clocks per row however
+// short it is: loads of 32-byte rows with the swizzle done by the TMA took 1810 clocks per 42 KB
+// stage on every SM, as long as the MMAs, and 512-byte rows take 760 (18 TB/s over the chip).  Row
+// coordinates of a box are therefore multiples of ROWGRAN (OzParams::row_skip).
+// A tile box that reaches past Rpad reads the next K block's rows (finite digits) or, at the end
+// of a plane, the TMA's zero fill: those rows only feed output rows or columns beyond M or N,
+// which are never stored.
 constexpr long ROWPAD = 384;
+constexpr int ROWGRAN = 16;      // stored rows per 512-byte row of the tensor maps
 
 struct Planes {
   __nv_bfloat16* p;
   long R, Rpad, K, nkb, plane;   // rows, padded rows, K, K blocks, elements per plane
   __host__ __device__ __forceinline__ long idx(int s, long r, long k) const {
-    return s * plane + (k / BK) * (Rpad * BK) + r * BK + (k % BK);
+    return s * plane + (k / BK) * (Rpad * BK) + swz(r, (int)(k % BK));
+  }
+  // Position of value c (0..15) of row r inside a K block: the 8-value halves swap with bit 2 of r.
+  static __host__ __device__ __forceinline__ long swz(long r, int c) {
+    return r * BK + (c ^ ((int)(r & 4) << 1));
   }
 };
 
@@ -110,13 +122,15 @@ static inline Planes make_planes(void* p, long R, long K) {
 // L T + I (I + 1) / 2 + J, each as 8 K blocks of 128 rows x 16 (the Planes layout with 128 rows
 // and 8 X T K blocks).  The half transform reads a tile as it is stored for the rows of block I
 // and MN-major (transposed) for the rows of block J.  The r = n - n1 ragged rows mu >= n1 of each
-// b^L are stored whole (rows (L, mu - n1), K = nu); they are read as they are for their own rows
-// and MN-major for the columns nu >= n1 of the full blocks.  One exponent per L (max |b^L| <
-// 2^e(L)), so that a stored element has the same scale for both rows that use it.
+// b^L are stored whole (rows (L, mu - n1), K = nu; when there are full blocks each L's rows are
+// padded with zero rows to rp, a multiple of ROWGRAN, so that every L starts at a box coordinate);
+// they are read as they are for their own rows and MN-major for the columns nu >= n1 of the full
+// blocks.  One exponent per L (max |b^L| < 2^e(L)), so that a stored element has the same scale for
+// both rows that use it.
 struct BPacked {
-  int n, X, nb1, T, r, n1;
+  int n, X, nb1, T, r, rp, n1;
   Planes tiles;       // R = Rpad = 128, nkb = 8 X T
-  Planes rag;         // rows (L, j), j < r, of all X r; K = n
+  Planes rag;         // rows (L, j), j < rp, of all X rp; K = n
   int* exp;           // [X]
   unsigned long long* mx;   // [X] max |b^L| as ordered bit patterns (set-up scratch)
 };
@@ -130,6 +144,7 @@ static inline BPacked bpacked_geometry(int n, int X) {
   b.T = b.nb1 * (b.nb1 + 1) / 2;
   b.n1 = 128 * b.nb1;
   b.r = n - b.n1;
+  b.rp = b.nb1 > 0 ? (b.r + ROWGRAN - 1) / ROWGRAN * ROWGRAN : b.r;
   return b;
 }
 static inline size_t bpacked_tile_bytes(const BPacked& b) {
@@ -139,7 +154,8 @@ static inline size_t bpacked_tile_bytes(const BPacked& b) {
 struct OzParams {
   int M, N;                // output rows / columns
   int a_rpad, b_rpad;      // padded rows of the A / B plane layouts
-  int a_row0, b_row0;      // first row of A / B used (row offset inside the layouts)
+  int a_row0, b_row0;      // first row of A / B used: multiples of ROWGRAN (box coordinates)
+  int row_skip;            // rows between a_row0 and the product's first row (computed, not stored)
   int kb_total;            // K blocks of BK
   int kb_per_split;
   int ksplit;
@@ -160,9 +176,10 @@ struct OzParams {
   // from the stored tile (J, R) MN-major (R < J < pk_nb1), or from the ragged rows nu >= n1 of
   // b^L MN-major (tensor maps tmA, tmA2 and tmA3)
   int a_pack;
-  int pk_nb1, pk_T, pk_r;  // full row blocks per L, stored tiles per L, ragged rows per L
+  int pk_nb1, pk_T, pk_rp; // full row blocks per L, stored tiles per L, stored ragged rows per L
   int pk_L0;               // first auxiliary index of the chunk
   int ht_rows, ht_mu0;     // mode 1: rows of the product per L, and mu of its first row
+  int ht_live;             // mode 1: rows per L that are stored (the others are padding)
   int ea_perL;             // the row exponents are per auxiliary index: ea[L], not ea[row]
   int* status;
 };
@@ -403,7 +420,7 @@ k_ozaki(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtenso
         const long Lg = (long)p.pk_L0 + Lr;
         pk_row = (Lg * p.pk_T + pk_R * (pk_R + 1) / 2) * 8;
         pk_col = Lg * p.pk_T + pk_R;
-        pk_rag = Lg * p.pk_r - 8L * p.pk_nb1 * BK;
+        pk_rag = Lg * p.pk_rp - 8L * p.pk_nb1 * BK;
       }
       for (int i = 0; i < cur.nkb; ++i, ++gs) {
         const int st = (int)(gs % NSTAGE);
@@ -418,20 +435,21 @@ k_ozaki(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtenso
         if (PACK && p.a_pack) {   // K block kb = 8 J + kk lies in column block J of b^L
           const int J = kb >> 3;
           if (J <= pk_R)           // stored lower tile (R, J): rows mu, K = nu
-            sm100::tma_load_3d(sa, cur.ma, &full[st], 0, (int)((pk_row + kb) * BM), 0);
+            sm100::tma_load_3d(sa, cur.ma, &full[st], 0, (int)((pk_row + kb) * (BM / ROWGRAN)), 0);
           else if (J < p.pk_nb1)   // stored tile (J, R) read MN-major: its rows are this K
-            sm100::tma_load_4d(sa, cur.ma2, &full[st], 0, (kb & 7) * BK,
+            sm100::tma_load_4d(sa, cur.ma2, &full[st], 0, kb & 7,
                                (int)((pk_col + J * (J + 1) / 2) * 8), 0);
           else                     // ragged rows nu >= n1 of b^L, MN-major
-            sm100::tma_load_4d(sa, cur.ma3, &full[st], 0, (int)(pk_rag + (long)kb * BK),
+            sm100::tma_load_4d(sa, cur.ma3, &full[st], 0, (int)((pk_rag + (long)kb * BK) / ROWGRAN),
                                pk_R * (BM / BK), 0);
         } else if (p.a_mn) {   // rows of the stored planes are this product's K, their K blocks its M
-          sm100::tma_load_4d(sa, cur.ma, &full[st], 0, p.a_row0 + kb * BK, cur.m0 / BK, 0);
+          sm100::tma_load_4d(sa, cur.ma, &full[st], 0, p.a_row0 / ROWGRAN + kb, cur.m0 / BK, 0);
         } else {
-          sm100::tma_load_3d(sa, cur.ma, &full[st], 0, kb * p.a_rpad + p.a_row0 + cur.m0, 0);
+          sm100::tma_load_3d(sa, cur.ma, &full[st], 0,
+                             (int)(((long)kb * p.a_rpad + p.a_row0 + cur.m0) / ROWGRAN), 0);
         }
         sm100::tma_load_3d(sa + A_BYTES, cur.mb, &full[st], 0,
-                           kb * p.b_rpad + p.b_row0 + cur.n0, 0);
+                           (int)(((long)kb * p.b_rpad + p.b_row0 + cur.n0) / ROWGRAN), 0);
       }
     }
     // never leave the CTA with a bulk copy still writing its shared memory
@@ -683,17 +701,20 @@ k_ozaki(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtenso
       }
       if (!ok) break;
       // FP64 results (overlaps the next tile's MMAs)
-      const int row = m0 + lq * 32 + lane;
+      const int row = m0 + lq * 32 + lane - p.row_skip;
+      bool live = row >= 0 && row < p.M;
       long L = 0, mu = 0;
       int ea;
       if constexpr (PACK) {
         if (p.mode == 1) {   // row (L, mu) of the Ht layout
           L = row / p.ht_rows;
-          mu = p.ht_mu0 + (row - L * p.ht_rows);
+          const int j = (int)(row - L * p.ht_rows);
+          mu = p.ht_mu0 + j;
+          live = live && j < p.ht_live;
         }
-        ea = (p.ea && row < p.M) ? p.ea[p.ea_perL ? L : row] : 0;
+        ea = (p.ea && live) ? p.ea[p.ea_perL ? L : row] : 0;
       } else {
-        ea = (p.ea && row < p.M) ? p.ea[row] : 0;
+        ea = (p.ea && live) ? p.ea[row] : 0;
         if (p.mode == 1) {
           L = row / p.ht_n;
           mu = row - L * p.ht_n;
@@ -706,7 +727,7 @@ k_ozaki(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtenso
 #pragma unroll
           for (int e = 0; e < 8; ++e) {
             const int col = n0 + (cg + 4 * b) * 8 + e;
-            if (row < p.M && col < p.N) {
+            if (live && col < p.N) {
               const int E = ea + p.eb[col] - 14 - 8 * (NEXACT - 1) - p.sh;
               const double v = make_double((long long)acc[b * 8 + e], E);
               if (p.mode == 0)
@@ -942,15 +963,16 @@ k_bpacked_tiles(const double* __restrict__ Bp, long npair, int T, const int* __r
   const long hi = mu > nu ? mu : nu, lo = mu > nu ? nu : mu;
   __nv_bfloat16 d[NDIG];
   digits_of(Bp[L * npair + hi * (hi + 1) / 2 + lo], ex[L], d);
-  const long o = (tt * 8 + kk) * (128L * BK) + row * BK + c;
+  const long o = (tt * 8 + kk) * (128L * BK) + Planes::swz(row, c);
 #pragma unroll
   for (int s = 0; s < NDIG; ++s) P.p[s * P.plane + o] = d[s];
 }
 
-// Pass 3: the ragged rows mu = n1 + j (rows (L, j) of all X r, then zero padding rows), every
-// K block of the layout (zero digits for nu >= n), in the K-blocked storage order.
+// Pass 3: the ragged rows mu = n1 + j (rows (L, j), j < rp, of all X rp, zeros for j >= r; then
+// zero padding rows), every K block of the layout (zero digits for nu >= n), in the K-blocked
+// storage order.
 __global__ void __launch_bounds__(256)
-k_bpacked_ragged(const double* __restrict__ Bp, long npair, int n, int n1, int r,
+k_bpacked_ragged(const double* __restrict__ Bp, long npair, int n, int n1, int r, int rp,
                  const int* __restrict__ ex, Planes P, long live_rows) {
   const long kend = P.nkb * BK;
   const long i = blockIdx.x * (long)blockDim.x + threadIdx.x;
@@ -960,9 +982,9 @@ k_bpacked_ragged(const double* __restrict__ Bp, long npair, int n, int n1, int r
   double x = 0.0;
   int e = 0;
   if (row < live_rows) {
-    const long L = row / r, mu = n1 + (row - L * r);
+    const long L = row / rp, j = row - L * rp, mu = n1 + j;
     e = ex[L];
-    if (k < n) {
+    if (k < n && j < r) {
       const long hi = mu > k ? mu : k, lo = mu > k ? k : mu;
       x = Bp[L * npair + hi * (hi + 1) / 2 + lo];
     }
@@ -1120,39 +1142,46 @@ static EncodeTiledFn encode_fn() {
   return fn;
 }
 
-// 3D map over K-blocked digit planes: dims {BK, nkb*Rpad, NDIG}, box {BK, box_rows, NDIG},
-// 32-byte swizzle.  Each box is box_rows * 32 contiguous bytes per plane.
+// 3D map over K-blocked digit planes: dims {256, nkb*Rpad/16, NDIG} (rows of 16 stored rows), box
+// {256, box_rows/16, NDIG}: box_rows * 32 contiguous bytes per plane, copied as they are.
 static las_status make_plane_map(CUtensorMap* m, const Planes& P, int box_rows) {
   EncodeTiledFn fn = encode_fn();
   if (!fn) return LAS_ERR_CUDA;
-  const long rows = P.nkb * P.Rpad;
-  if (((uintptr_t)P.p & 15) || rows <= 0 || rows > 0x7FFFFFFFL) return LAS_ERR_INTERNAL;
-  cuuint64_t dims[3] = {(cuuint64_t)BK, (cuuint64_t)rows, (cuuint64_t)NDIG};
-  cuuint64_t strides[2] = {(cuuint64_t)BK * 2, (cuuint64_t)P.plane * 2};
-  cuuint32_t box[3] = {(cuuint32_t)BK, (cuuint32_t)box_rows, (cuuint32_t)NDIG};
+  const long rows = P.nkb * P.Rpad / ROWGRAN;
+  if (((uintptr_t)P.p & 15) || P.Rpad % ROWGRAN || box_rows % ROWGRAN || rows <= 0 ||
+      rows > 0x7FFFFFFFL / ROWGRAN)
+    return LAS_ERR_INTERNAL;
+  cuuint64_t dims[3] = {(cuuint64_t)ROWGRAN * BK, (cuuint64_t)rows, (cuuint64_t)NDIG};
+  cuuint64_t strides[2] = {(cuuint64_t)ROWGRAN * BK * 2, (cuuint64_t)P.plane * 2};
+  cuuint32_t box[3] = {(cuuint32_t)(ROWGRAN * BK), (cuuint32_t)(box_rows / ROWGRAN),
+                       (cuuint32_t)NDIG};
   cuuint32_t es[3] = {1, 1, 1};
   CUresult r = fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, (void*)P.p, dims, strides, box, es,
-                  CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_32B,
+                  CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
                   CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   return r == CUDA_SUCCESS ? LAS_OK : LAS_ERR_INTERNAL;
 }
 
 // 4D map for reading planes MN-major (as the A operand of a product whose K runs along the
-// stored rows): dims {BK, Rpad, nkb, NDIG}; a box is 16 stored rows (16 values of K) of BM / BK
-// consecutive K blocks of the stored layout (BM values of M), every plane: BM * 32 bytes per
-// plane, as in the K-major case.  Boxes past the last stored K block read the TMA's zero fill.
+// stored rows): dims {256, Rpad/16, nkb, NDIG}; a box is 16 stored rows (16 values of K, 512
+// bytes) of BM / BK consecutive K blocks of the stored layout (BM values of M), every plane:
+// BM * 32 bytes per plane, as in the K-major case.  Boxes past the last stored K block read the
+// TMA's zero fill.
 static las_status make_plane_map_mn(CUtensorMap* m, const Planes& P) {
   EncodeTiledFn fn = encode_fn();
   if (!fn) return LAS_ERR_CUDA;
-  if (((uintptr_t)P.p & 15) || P.Rpad <= 0 || P.Rpad > 0x7FFFFFFFL || P.nkb <= 0)
+  static_assert(ROWGRAN == BK, "a 512-byte row holds the 16 values of K of one stage");
+  if (((uintptr_t)P.p & 15) || P.Rpad <= 0 || P.Rpad % ROWGRAN || P.Rpad > 0x7FFFFFFFL ||
+      P.nkb <= 0)
     return LAS_ERR_INTERNAL;
-  cuuint64_t dims[4] = {(cuuint64_t)BK, (cuuint64_t)P.Rpad, (cuuint64_t)P.nkb, (cuuint64_t)NDIG};
-  cuuint64_t strides[3] = {(cuuint64_t)BK * 2, (cuuint64_t)P.Rpad * BK * 2,
+  cuuint64_t dims[4] = {(cuuint64_t)ROWGRAN * BK, (cuuint64_t)(P.Rpad / ROWGRAN),
+                        (cuuint64_t)P.nkb, (cuuint64_t)NDIG};
+  cuuint64_t strides[3] = {(cuuint64_t)ROWGRAN * BK * 2, (cuuint64_t)P.Rpad * BK * 2,
                            (cuuint64_t)P.plane * 2};
-  cuuint32_t box[4] = {(cuuint32_t)BK, (cuuint32_t)BK, (cuuint32_t)(BM / BK), (cuuint32_t)NDIG};
+  cuuint32_t box[4] = {(cuuint32_t)(ROWGRAN * BK), 1, (cuuint32_t)(BM / BK), (cuuint32_t)NDIG};
   cuuint32_t es[4] = {1, 1, 1, 1};
   CUresult r = fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, (void*)P.p, dims, strides, box, es,
-                  CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_32B,
+                  CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
                   CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   return r == CUDA_SUCCESS ? LAS_OK : LAS_ERR_INTERNAL;
 }
@@ -1357,6 +1386,11 @@ static las_status ozaki_setup(OzProblem& pr, const Planes& A, long a_row0, const
                          : (a_row0 + M <= A.Rpad && K <= A.nkb * BK);
   if (!a_ok || b_row0 + N > B.Rpad || K > B.nkb * BK || !valid_bn(bn) || (a_mn && lower))
     return LAS_ERR_INTERNAL;
+  // box coordinates are multiples of ROWGRAN rows: the product starts up to 15 rows early and
+  // drops what it computes there
+  const int skip = (int)(a_row0 % ROWGRAN);
+  if (b_row0 % ROWGRAN || (skip && (a_mn || lower)) || M + skip > 0x7FFFFFFFL)
+    return LAS_ERR_INTERNAL;
   las_status s = ozaki_prepare();
   if (s != LAS_OK) return s;
   memset(&pr, 0, sizeof(pr));
@@ -1368,7 +1402,8 @@ static las_status ozaki_setup(OzProblem& pr, const Planes& A, long a_row0, const
   p.N = (int)N;
   p.a_rpad = (int)A.Rpad;
   p.b_rpad = (int)B.Rpad;
-  p.a_row0 = (int)a_row0;
+  p.a_row0 = (int)(a_row0 - skip);
+  p.row_skip = skip;
   p.b_row0 = (int)b_row0;
   p.kb_total = (int)((K + BK - 1) / BK);
   if (p.kb_total < 1) p.kb_total = 1;
@@ -1384,10 +1419,10 @@ static las_status ozaki_setup(OzProblem& pr, const Planes& A, long a_row0, const
   p.zstride = zstride;
   p.ht_n = ht_n;
   p.ht_op = ht_op;
-  p.ht_rows = ht_n;
+  p.ht_rows = p.ht_live = ht_n;
   p.ht_mu0 = 0;
   p.lower = lower;
-  p.tiles_z = ozaki_tiles(M, N, lower, bn);
+  p.tiles_z = ozaki_tiles(M + skip, N, lower, bn);
   p.sh = tail_shift(p.kb_per_split);
   p.bn = bn;
   p.a_mn = a_mn;
@@ -1414,7 +1449,8 @@ static las_status bpacked_half(const BPacked& b, int l0, int nL, const Planes& X
                                const int* xexp, long N, double* out, int ht_op, int* status,
                                cudaStream_t st, int bn) {
   if (nL <= 0 || N <= 0) return LAS_OK;
-  if (l0 < 0 || l0 + nL > b.X || x_row0 + N > Xd.Rpad || b.n > Xd.nkb * BK || !valid_bn(bn))
+  if (l0 < 0 || l0 + nL > b.X || x_row0 + N > Xd.Rpad || x_row0 % ROWGRAN ||
+      b.n > Xd.nkb * BK || !valid_bn(bn))
     return LAS_ERR_INTERNAL;
   las_status rc = ozaki_prepare();
   if (rc != LAS_OK) return rc;
@@ -1442,7 +1478,7 @@ static las_status bpacked_half(const BPacked& b, int l0, int nL, const Planes& X
     p.mode = 1;
     p.ht_n = b.n;
     p.ht_op = ht_op;
-    p.ht_rows = b.n1;
+    p.ht_rows = p.ht_live = b.n1;
     p.ht_mu0 = 0;
     p.ea_perL = 1;
     p.tiles_z = ozaki_tiles(M, N, 0, bn);
@@ -1451,17 +1487,18 @@ static las_status bpacked_half(const BPacked& b, int l0, int nL, const Planes& X
     p.a_pack = 1;
     p.pk_nb1 = b.nb1;
     p.pk_T = b.T;
-    p.pk_r = b.r;
+    p.pk_rp = b.rp;
     p.pk_L0 = l0;
     p.status = status;
     if ((rc = ozaki_submit(pr, st)) != LAS_OK) return rc;
   }
   if (b.r > 0) {
     OzProblem pr;
-    rc = ozaki_setup(pr, b.rag, (long)l0 * b.r, b.exp + l0, (long)nL * b.r, Xd, x_row0, xexp, N,
-                     b.n, 1, 1, out, 0, 0, b.n, ht_op, status, 0, bn, 0);
+    rc = ozaki_setup(pr, b.rag, (long)l0 * b.rp, b.exp + l0, (long)nL * b.rp, Xd, x_row0, xexp,
+                     N, b.n, 1, 1, out, 0, 0, b.n, ht_op, status, 0, bn, 0);
     if (rc != LAS_OK) return rc;
-    pr.p.ht_rows = b.r;
+    pr.p.ht_rows = b.rp;
+    pr.p.ht_live = b.r;
     pr.p.ht_mu0 = b.n1;
     pr.p.ea_perL = 1;
     rc = ozaki_submit(pr, st);
@@ -1610,8 +1647,8 @@ las_status split_create(SplitState** out, int n, int X, int op, int Lc, const do
     q = nullptr;
   }
   if (bp.r > 0) {
-    A(&q, planes_bytes((long)X * bp.r, n));
-    bp.rag = make_planes(q, (long)X * bp.r, n);
+    A(&q, planes_bytes((long)X * bp.rp, n));
+    bp.rag = make_planes(q, (long)X * bp.rp, n);
     q = nullptr;
   }
   A((void**)&bp.exp, (size_t)X * 4);
@@ -1662,7 +1699,7 @@ las_status split_create(SplitState** out, int n, int X, int op, int Lc, const do
     if (bp.r > 0) {
       const long total = bp.rag.Rpad * bp.rag.nkb * BK;
       k_bpacked_ragged<<<(unsigned)((total + 255) / 256), 256, 0, st>>>(
-          Bp, npair, n, bp.n1, bp.r, bp.exp, bp.rag, (long)X * bp.r);
+          Bp, npair, n, bp.n1, bp.r, bp.rp, bp.exp, bp.rag, (long)X * bp.rp);
       las_count_launch();
     }
     cudaError_t e = cudaGetLastError();
