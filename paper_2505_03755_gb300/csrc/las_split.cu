@@ -42,7 +42,8 @@ constexpr int A_PLANE = BM * BK * 2;                 // 4096 B
 constexpr int A_BYTES = NDIG * A_PLANE;              // 24576
 constexpr int TMEM_COLS = 512;
 constexpr int EPI_WARPS = 16;    // epilogue warps: 4 column groups x 4 TMEM lane quarters
-constexpr int NTHREADS = 64 + 32 * EPI_WARPS;   // warp 0 TMA, warp 1 MMA, warps 2.. epilogue
+constexpr int EPI_WARP0 = 3;     // warp 0 TMA, warps 1 and 2 MMA, then the epilogue warps
+constexpr int NTHREADS = 32 * (EPI_WARP0 + EPI_WARPS);
 
 // Tile width bn (columns of the output per CTA tile, a product's parameter: 64 or 96) and the
 // stage layout, sized for the widest tile BN.  The exact weight groups q = 0..3 each own one
@@ -327,10 +328,15 @@ __device__ __forceinline__ void mma_exact(uint32_t tmem, uint32_t sa, uint32_t s
 }
 
 // Persistent CTAs (one per SM) walk the tiles (row tile, column tile, K split).  Roles:
-// warp 0 streams digit-plane stages with TMA, warp 1 issues tcgen05.mma, warps 2..17 drain the
-// TMEM accumulators.  Stage, chunk and tile counters run on across tiles so that the loads of the
-// next tile overlap the last MMAs of the current one, and its MMAs overlap the current tile's
-// conversion and stores.
+// warp 0 streams digit-plane stages with TMA, warp 1 issues the tcgen05.mma of the exact groups and
+// warp 2 those of the tail, warps 3.. drain the TMEM accumulators.  Stage, chunk and tile counters
+// run on across tiles so that the loads of the next tile overlap the last MMAs of the current one,
+// and its MMAs overlap the current tile's conversion and stores.
+// One thread issues an MMA about every 65 clocks (descriptors and all), so a single issuer's 17 MMAs
+// took as long at 64 columns as at 96: the issue, not the tensor pipe, set the stage time.  The
+// two issuers write disjoint accumulators and each wait only for what they overwrite: the exact
+// issuer for the drain of the previous chunk, the tail issuer for the read-out of the previous
+// tile's tail, so that tail products of up to NSTAGE stages run during a drain.
 // GROUPED: the launch walks the concatenated tiles of nprob products described in global
 // memory (probs); otherwise the one product of the kernel parameters.  FIXBN: the tile width of
 // every product of the launch as a compile-time constant (64 or 96), or 0 when products of both
@@ -356,9 +362,10 @@ k_ozaki(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtenso
   uint64_t* empty = bars + NSTAGE;    // [NSTAGE]
   uint64_t* accf = bars + 2 * NSTAGE;
   uint64_t* acce = bars + 2 * NSTAGE + 1;
-  uint64_t* drain = bars + 2 * NSTAGE + 2;
-  uint64_t* accT = bars + 2 * NSTAGE + 3;   // tail accumulators read out (once per tile)
-  uint32_t* tmem_slot = (uint32_t*)(bars + 2 * NSTAGE + 4);
+  uint64_t* drain = bars + 2 * NSTAGE + 2;  // [2] teardown of the two issuers
+  uint64_t* accT = bars + 2 * NSTAGE + 4;   // tail accumulator read out (once per tile)
+  uint64_t* tailf = bars + 2 * NSTAGE + 5;  // tail accumulator complete (once per tile)
+  uint32_t* tmem_slot = (uint32_t*)(bars + 2 * NSTAGE + 6);
   volatile int* abort_flag = (volatile int*)(tmem_slot + 1);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -368,12 +375,14 @@ k_ozaki(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtenso
   if (threadIdx.x == 0) {
     for (int s = 0; s < NSTAGE; ++s) {
       sm100::mbar_init(&full[s], 1);
-      sm100::mbar_init(&empty[s], 1);
+      sm100::mbar_init(&empty[s], 2);   // both issuers
     }
     sm100::mbar_init(accf, 1);
     sm100::mbar_init(acce, EPI_WARPS);
     sm100::mbar_init(accT, EPI_WARPS);
-    sm100::mbar_init(drain, 1);
+    sm100::mbar_init(&drain[0], 1);
+    sm100::mbar_init(&drain[1], 1);
+    sm100::mbar_init(tailf, 1);
     *abort_flag = 0;
     sm100::fence_mbar_init();
     if (!GROUPED) {
@@ -394,9 +403,77 @@ k_ozaki(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtenso
   sm100::tc_fence_after();
   const uint32_t tmem = *tmem_slot;
 
+  // ---------------- MMA issuers: the exact groups (warp 1) or the tail (warp 2) ----------------
+  auto issue = [&](auto exact_c) {
+    constexpr bool exact = decltype(exact_c)::value;
+    int st = 0;
+    uint32_t phase = 0;
+    uint32_t nstart = 0;   // accumulations started so far (exact: chunks; tail: tiles)
+    bool ok = true;
+    OzCursor<GROUPED> cur;
+    for (long t = blockIdx.x; t < ntiles && ok; t += gridDim.x) {
+      cur.seek(t, p1, &tmA, &tmB, &tmA2, &tmA3, probs, nprob);
+      const OzParams& p = *cur.P;
+      const int nkb = cur.nkb;
+      const int bn = FIXBN ? FIXBN : p.bn;
+      const bool amn_tile = p.a_mn != 0;
+      // packed-triangle A: K blocks of column blocks J > R (above the diagonal) are read MN-major
+      const bool pack = PACK && p.a_pack != 0;
+      const int kb_mn = pack ? 8 * ((cur.m0 / BM) % p.pk_nb1 + 1) : 0;
+      // Stages [i0, i1) of the tile with one A orientation (a compile-time constant where the
+      // launch fixes it); false when a wait ran out.
+      auto stages = [&](auto amn, int i0, int i1) -> bool {
+        for (int i = i0; i < i1; ++i) {
+          if (!sm100::mbar_wait(&full[st], phase, abort_flag, p.status, LAS_ERR_TIMEOUT))
+            return false;
+          const bool first = exact ? (i % CHUNK) == 0 : i == 0;
+          if (first) {   // the accumulators this stage starts must have been read out
+            if (nstart > 0 && !sm100::mbar_wait(exact ? acce : accT, (nstart - 1) & 1,
+                                                abort_flag, p.status, LAS_ERR_TIMEOUT))
+              return false;
+            ++nstart;
+          }
+          sm100::tc_fence_after();
+          const uint32_t sa = sm100::smem_u32(smem + st * T::STAGE_BYTES);
+          const uint32_t sb = sa + A_BYTES;
+          if constexpr (exact) {
+            if (bn == 64) mma_exact<64>(tmem, sa, sb, first, amn);
+            else mma_exact<96>(tmem, sa, sb, first, amn);
+          } else {
+            if (bn == 64) mma_tail<64>(tmem + T::TAIL_COL, sa, sb, first, amn);
+            else mma_tail<96>(tmem + T::TAIL_COL, sa, sb, first, amn);
+          }
+          sm100::mma_commit(&empty[st]);
+          if (exact && ((i % CHUNK) == CHUNK - 1 || i == nkb - 1)) sm100::mma_commit(accf);
+          if (++st == NSTAGE) {
+            st = 0;
+            phase ^= 1;
+          }
+        }
+        return true;
+      };
+      using K_MAJOR = std::integral_constant<bool, false>;
+      using MN_MAJOR = std::integral_constant<bool, true>;
+      if constexpr (PACK) {
+        // packed-triangle A: the K-major stages (up to the diagonal block), then the MN-major ones
+        const int isplit = pack ? min(nkb, max(0, kb_mn - cur.kb0)) : amn_tile ? 0 : nkb;
+        ok = stages(K_MAJOR(), 0, isplit) && stages(MN_MAJOR(), isplit, nkb);
+      } else if constexpr (AMN == 2) {
+        ok = stages(amn_tile, 0, nkb);
+      } else {
+        ok = stages(std::integral_constant<bool, AMN == 1>(), 0, nkb);
+      }
+      if (ok && !exact) sm100::mma_commit(tailf);
+    }
+    // make sure no MMA is still writing TMEM when the CTA tears down
+    sm100::mma_commit(&drain[exact]);
+    sm100::mbar_wait(&drain[exact], 0, abort_flag, status0, LAS_ERR_TIMEOUT);
+  };
+
   if (warp == 0 && lane == 0) {
     // ---------------- TMA producer ----------------
-    long gs = 0;
+    int st = 0, filled = 0;     // ring slot; slots filled so far (at most NSTAGE)
+    uint32_t phase = 0;         // completed rounds of the ring, modulo 2
     bool ok = true;
     OzCursor<GROUPED> cur;
     for (long t = blockIdx.x; t < ntiles && ok; t += gridDim.x) {
@@ -422,10 +499,9 @@ k_ozaki(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtenso
         pk_col = Lg * p.pk_T + pk_R;
         pk_rag = Lg * p.pk_rp - 8L * p.pk_nb1 * BK;
       }
-      for (int i = 0; i < cur.nkb; ++i, ++gs) {
-        const int st = (int)(gs % NSTAGE);
-        if (gs >= NSTAGE && !sm100::mbar_wait(&empty[st], (uint32_t)((gs / NSTAGE) - 1) & 1,
-                                              abort_flag, p.status, LAS_ERR_TIMEOUT)) {
+      for (int i = 0; i < cur.nkb; ++i) {
+        if (filled == NSTAGE && !sm100::mbar_wait(&empty[st], phase ^ 1, abort_flag, p.status,
+                                                  LAS_ERR_TIMEOUT)) {
           ok = false;
           break;
         }
@@ -450,188 +526,31 @@ k_ozaki(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtenso
         }
         sm100::tma_load_3d(sa + A_BYTES, cur.mb, &full[st], 0,
                            (int)(((long)kb * p.b_rpad + p.b_row0 + cur.n0) / ROWGRAN), 0);
+        if (filled < NSTAGE) ++filled;
+        if (++st == NSTAGE) {
+          st = 0;
+          phase ^= 1;
+        }
       }
     }
-    // never leave the CTA with a bulk copy still writing its shared memory
-    for (long g = (gs > NSTAGE ? gs - NSTAGE : 0); g < gs; ++g)
-      sm100::mbar_wait(&full[g % NSTAGE], (uint32_t)(g / NSTAGE) & 1, abort_flag, status0,
+    // never leave the CTA with a bulk copy still writing its shared memory: wait for the last
+    // copy into every slot (slots before st in this round of the ring, the others in the last one)
+    for (int k = 0; k < filled; ++k)
+      sm100::mbar_wait(&full[k], k < st ? phase : phase ^ 1, abort_flag, status0,
                        LAS_ERR_TIMEOUT);
   } else if (warp == 1 && lane == 0) {
-    // ---------------- MMA issuer ----------------
-    // Per stage the tail MMAs (groups 4 and 5) are issued at once; the exact-group MMAs of the
-    // first stages of a chunk may be deferred (their stages stay resident) until the epilogue
-    // has drained the previous chunk, so that the drain overlaps tensor work.
-    long gs = 0, gc = 0, tcount = 0;
-    bool ok = true, need_acce = false;
-    OzCursor<GROUPED> cur;
-    for (long t = blockIdx.x; t < ntiles && ok; t += gridDim.x) {
-      cur.seek(t, p1, &tmA, &tmB, &tmA2, &tmA3, probs, nprob);
-      const OzParams& p = *cur.P;
-      const int nkb = cur.nkb;
-      const int bn = FIXBN ? FIXBN : p.bn;
-      const bool amn_tile = p.a_mn != 0;
-      // packed-triangle A: K blocks of column blocks J > R (above the diagonal) are read MN-major
-      const bool pack = PACK && p.a_pack != 0;
-      const int kb_mn = pack ? 8 * ((cur.m0 / BM) % p.pk_nb1 + 1) : 0;
-      // the tail accumulators of the previous tile must have been read out
-      if (tcount > 0) {
-        if (!sm100::mbar_wait(accT, (uint32_t)(tcount - 1) & 1, abort_flag, p.status,
-                              LAS_ERR_TIMEOUT)) {
-          ok = false;
-          break;
-        }
-        sm100::tc_fence_after();
-      }
-      long pend0 = 0;     // first deferred stage (global index) and count
-      int npend = 0, pend_i0 = 0;
-      // One stage: wait for its data, issue its tail MMAs, then the exact-group MMAs of the
-      // deferred stages and its own unless they are deferred again (never at the end of a chunk
-      // or of a phase: flush).  amn is the stage's A orientation.  False when a wait ran out.
-      auto stage = [&](auto amn_c, int i, bool flush) -> bool {
-        constexpr bool amn = decltype(amn_c)::value;   // the orientation as a constant
-        const int st = (int)(gs % NSTAGE);
-        if (!sm100::mbar_wait(&full[st], (uint32_t)(gs / NSTAGE) & 1, abort_flag, p.status,
-                              LAS_ERR_TIMEOUT))
-          return false;
-        sm100::tc_fence_after();
-        {
-          const uint32_t sa = sm100::smem_u32(smem + st * T::STAGE_BYTES);
-          const uint32_t sb = sa + A_BYTES;
-          // tail: the 11 products of groups 4 and 5 into the one tail accumulator
-          if (bn == 64) mma_tail<64>(tmem + T::TAIL_COL, sa, sb, i == 0, amn);
-          else mma_tail<96>(tmem + T::TAIL_COL, sa, sb, i == 0, amn);
-        }
-        const bool last_in_chunk = (i % CHUNK) == CHUNK - 1 || i == nkb - 1;
-        if (need_acce) {
-          if (!last_in_chunk && !flush && npend < NSTAGE - 1 &&
-              !sm100::mbar_test_wait(acce, (uint32_t)(gc - 1) & 1)) {
-            if (npend == 0) {
-              pend0 = gs;
-              pend_i0 = i;
-            }
-            ++npend;
-            return true;   // defer this stage's exact-group MMAs
-          }
-          if (!sm100::mbar_wait(acce, (uint32_t)(gc - 1) & 1, abort_flag, p.status,
-                                LAS_ERR_TIMEOUT))
-            return false;
-          sm100::tc_fence_after();
-          need_acce = false;
-        }
-        if (npend == 0) {
-          pend0 = gs;
-          pend_i0 = i;
-        }
-        // exact groups q = 0..3 for the deferred stages and this one, in stage order: A_s
-        // against planes 0 .. 3-s; s = 0 spans all four groups and starts them at a chunk's
-        // first stage
-        for (int j = 0; j <= npend; ++j) {
-          const long g2 = pend0 + j;
-          const int i2 = pend_i0 + j;
-          const int st2 = (int)(g2 % NSTAGE);
-          const bool first_in_chunk = (i2 % CHUNK) == 0;
-          const uint32_t sa = sm100::smem_u32(smem + st2 * T::STAGE_BYTES);
-          const uint32_t sb = sa + A_BYTES;
-          if (bn == 64) mma_exact<64>(tmem, sa, sb, first_in_chunk, amn);
-          else mma_exact<96>(tmem, sa, sb, first_in_chunk, amn);
-          sm100::mma_commit(&empty[st2]);
-        }
-        npend = 0;
-        if (last_in_chunk) {
-          sm100::mma_commit(accf);
-          ++gc;
-          need_acce = true;   // the next chunk's exact MMAs wait for this chunk's drain
-        }
-        return true;
-      };
-      if constexpr (PACK) {
-        using K_MAJOR = std::integral_constant<bool, false>;
-        using MN_MAJOR = std::integral_constant<bool, true>;
-        if (pack) {
-          // packed-triangle A: the K-major stages (up to the diagonal block) and the MN-major
-          // ones as two loops, each of one orientation; the first leaves nothing deferred
-          const int isplit = min(nkb, max(0, kb_mn - cur.kb0));
-          for (int i = 0; i < isplit && ok; ++i, ++gs) ok = stage(K_MAJOR(), i, i == isplit - 1);
-          for (int i = isplit; i < nkb && ok; ++i, ++gs) ok = stage(MN_MAJOR(), i, false);
-        } else if (amn_tile) {
-          for (int i = 0; i < nkb && ok; ++i, ++gs) ok = stage(MN_MAJOR(), i, false);
-        } else {
-          for (int i = 0; i < nkb && ok; ++i, ++gs) ok = stage(K_MAJOR(), i, false);
-        }
-      } else {
-        // the same per stage as `stage`, written out: one orientation for the whole tile
-        const bool amn = AMN == 2 ? amn_tile : AMN == 1;
-        for (int i = 0; i < nkb; ++i, ++gs) {
-          const int st = (int)(gs % NSTAGE);
-          if (!sm100::mbar_wait(&full[st], (uint32_t)(gs / NSTAGE) & 1, abort_flag, p.status,
-                                LAS_ERR_TIMEOUT)) {
-            ok = false;
-            break;
-          }
-          sm100::tc_fence_after();
-          {
-            const uint32_t sa = sm100::smem_u32(smem + st * T::STAGE_BYTES);
-            const uint32_t sb = sa + A_BYTES;
-            if (bn == 64) mma_tail<64>(tmem + T::TAIL_COL, sa, sb, i == 0, amn);
-            else mma_tail<96>(tmem + T::TAIL_COL, sa, sb, i == 0, amn);
-          }
-          const bool last_in_chunk = (i % CHUNK) == CHUNK - 1 || i == nkb - 1;
-          if (need_acce) {
-            if (!last_in_chunk && npend < NSTAGE - 1 &&
-                !sm100::mbar_test_wait(acce, (uint32_t)(gc - 1) & 1)) {
-              if (npend == 0) {
-                pend0 = gs;
-                pend_i0 = i;
-              }
-              ++npend;
-              continue;   // defer this stage's exact-group MMAs
-            }
-            if (!sm100::mbar_wait(acce, (uint32_t)(gc - 1) & 1, abort_flag, p.status,
-                                  LAS_ERR_TIMEOUT)) {
-              ok = false;
-              break;
-            }
-            sm100::tc_fence_after();
-            need_acce = false;
-          }
-          if (npend == 0) {
-            pend0 = gs;
-            pend_i0 = i;
-          }
-          for (int j = 0; j <= npend; ++j) {
-            const long g2 = pend0 + j;
-            const int i2 = pend_i0 + j;
-            const int st2 = (int)(g2 % NSTAGE);
-            const bool first_in_chunk = (i2 % CHUNK) == 0;
-            const uint32_t sa = sm100::smem_u32(smem + st2 * T::STAGE_BYTES);
-            const uint32_t sb = sa + A_BYTES;
-            if (bn == 64) mma_exact<64>(tmem, sa, sb, first_in_chunk, amn);
-            else mma_exact<96>(tmem, sa, sb, first_in_chunk, amn);
-            sm100::mma_commit(&empty[st2]);
-          }
-          npend = 0;
-          if (last_in_chunk) {
-            sm100::mma_commit(accf);
-            ++gc;
-            need_acce = true;
-          }
-        }
-      }
-      if (!ok) break;
-      ++tcount;
-    }
-    // make sure no MMA is still writing TMEM when the CTA tears down
-    sm100::mma_commit(drain);
-    sm100::mbar_wait(drain, 0, abort_flag, status0, LAS_ERR_TIMEOUT);
-  } else if (warp >= 2) {
+    issue(std::true_type());    // exact groups
+  } else if (warp == 2 && lane == 0) {
+    issue(std::false_type());   // tail
+  } else if (warp >= EPI_WARP0) {
     // ---------------- epilogue (16 warps) ----------------
     const int lq = warp & 3;                 // TMEM lane quarter this warp may access
-    const int cg = (warp - 2) >> 2;          // column blocks cg, cg + 4, cg + 8, ... of 8
+    const int cg = (warp - EPI_WARP0) >> 2;          // column blocks cg, cg + 4, cg + 8, ... of 8
     const uint32_t tl = tmem + ((uint32_t)(lq * 32) << 16);
-    long gc = 0;
+    uint32_t gc = 0, tcount = 0;
     bool ok = true;
     OzCursor<GROUPED> cur;
-    for (long t = blockIdx.x; t < ntiles && ok; t += gridDim.x) {
+    for (long t = blockIdx.x; t < ntiles && ok; t += gridDim.x, ++tcount) {
       cur.seek(t, p1, &tmA, &tmB, &tmA2, &tmA3, probs, nprob);
       const OzParams& p = *cur.P;
       const int m0 = cur.m0, n0 = cur.n0, kb0 = cur.kb0, nkb = cur.nkb;
@@ -643,13 +562,14 @@ k_ozaki(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtenso
 #pragma unroll
       for (int j = 0; j < MAXB * 8; ++j) acc[j] = 0;
       for (int c = 0; c < nchunks; ++c, ++gc) {
-        if (!sm100::mbar_wait(accf, (uint32_t)gc & 1, abort_flag, p.status, LAS_ERR_TIMEOUT,
-                              256)) {
+        const bool fin = (c == nchunks - 1);
+        if (!sm100::mbar_wait(accf, gc & 1, abort_flag, p.status, LAS_ERR_TIMEOUT, 256) ||
+            (fin && !sm100::mbar_wait(tailf, tcount & 1, abort_flag, p.status, LAS_ERR_TIMEOUT,
+                                      64))) {
           ok = false;
           break;
         }
         sm100::tc_fence_after();
-        const bool fin = (c == nchunks - 1);
         int extra = 0;
         if (fin) {
           // tail first, so that the next tile's tail MMAs can start:
