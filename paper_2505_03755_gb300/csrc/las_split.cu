@@ -185,14 +185,30 @@ struct OzParams {
   int* status;
 };
 
-// W * 2^E rounded once to FP64 (round to nearest even): the hardware int64 -> FP64 conversion,
-// then an exponent-field shift (exact for normal results; the rare others go through ldexp).
+// W * 2^E (|W| < 2^63) rounded once to FP64 (round to nearest even), built from the integer: the
+// leading one moved to bit 62, half a unit of bit 10 added (ties to even), the exponent field
+// put in front.  Results outside the normal range (rare) go through ldexp.
+// The 64-bit conversions run on the FP64 path of this part, a few per clock and SM: with
+// __ll2double_rn here and __float2ll_rn in the tail, a 128 x 96 tile's conversions took about
+// 12000 clocks, half of them before the next tile could start.
 __device__ __forceinline__ double make_double(long long W, int E) {
-  const double v = __ll2double_rn(W);
-  const long long b = __double_as_longlong(v);
-  const int ex = (int)((b >> 52) & 0x7FF);
-  if (ex == 0 || ex + E <= 0 || ex + E >= 2047) return ldexp(v, E);
-  return __longlong_as_double(b + ((long long)E << 52));
+  const unsigned long long a = (unsigned long long)(W < 0 ? -W : W);
+  const int n = __clzll((long long)a);            // 1..63 for a != 0
+  unsigned long long m = a << (n - 1);
+  m += 511 + ((m >> 10) & 1);
+  const int ex = 1086 - n + E;                    // biased exponent: 63 - n + E + 1023
+  if (a == 0) return 0.0;
+  if (ex <= 0 || ex >= 2046) return ldexp(__ll2double_rn(W), E);
+  const unsigned long long b = ((unsigned long long)(ex - 1) << 52) + (m >> 10);
+  return __longlong_as_double((long long)(b | ((unsigned long long)W & (1ull << 63))));
+}
+
+// rint(f) as int64 for |f| < 2^46, without a 64-bit conversion: the part above 2^16 first, then
+// the exact rest (the first part is even, so ties round as in one step).
+__device__ __forceinline__ long long rint_ll(float f) {
+  const int hi = __float2int_rn(f * 0x1p-16f);
+  const int lo = __float2int_rn(fmaf((float)hi, -65536.0f, f));
+  return (long long)hi * 65536 + lo;
 }
 
 // Column tiles of row tile i that touch the lower triangle (column tile j with j*bn < (i+1)*BM).
@@ -574,23 +590,21 @@ k_ozaki(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtenso
         if (fin) {
           // tail first, so that the next tile's tail MMAs can start:
           // acc <- acc * 2^sh + rint(tail * 2^(24+sh))  (int64, modulo 2^64)
+          uint32_t r[MAXB][8];
 #pragma unroll
-          for (int b = 0; b < MAXB; ++b) {
-            if (b < nb) {
-              const uint32_t col = (uint32_t)((cg + 4 * b) * 8);
-              uint32_t r[8];
-              sm100::tmem_ld8(tl + T::TAIL_COL + col, r);
-              sm100::tmem_wait_ld();
-#pragma unroll
-              for (int e = 0; e < 8; ++e)
-                acc[b * 8 + e] =
-                    (acc[b * 8 + e] << p.sh) +
-                    (unsigned long long)__float2ll_rn(__uint_as_float(r[e]) * tscale);
-            }
-          }
+          for (int b = 0; b < MAXB; ++b)
+            if (b < nb) sm100::tmem_ld8(tl + T::TAIL_COL + (uint32_t)((cg + 4 * b) * 8), r[b]);
+          sm100::tmem_wait_ld();
           sm100::tc_fence_before();
           __syncwarp();
           if (lane == 0) sm100::mbar_arrive(accT);
+#pragma unroll
+          for (int b = 0; b < MAXB; ++b)
+            if (b < nb)
+#pragma unroll
+              for (int e = 0; e < 8; ++e)
+                acc[b * 8 + e] = (acc[b * 8 + e] << p.sh) +
+                                 (unsigned long long)rint_ll(__uint_as_float(r[b][e]) * tscale);
           extra = p.sh;
         }
         // exact groups: integers g_q (|g_q| <= 2^24) in units of 2^-8q, merged as
