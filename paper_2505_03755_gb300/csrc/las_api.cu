@@ -48,7 +48,8 @@ struct las_ctx {
   cudaStream_t stream;
   size_t ws_cap;
   int Lc;       // auxiliary chunk length
-  int ksplit;   // split of the projection GEMM
+  int ksplit;   // K splits that `part` holds for an n x op product (FP64 GEMMs)
+  int sms;      // SMs of the device
   // workspace (device)
   double* Cocc;   // [n][op]
   double* Ht;     // [Lc][op][n]
@@ -79,10 +80,10 @@ struct las_ctx {
   int fnmo, fma;
   FragSplit* fsplit;
   double *vJ, *vK;   // scratch of las_veff (allocated by its first call)
-  // scratch of las_orbital_hvp (allocated by its first call): dC = C X and G(C) [n][nmo]; the
-  // tangent chain's dC_occ, h dC_occ and projection [n][op], dH [Lc][op][n], X = H^T dC, dT and
+  // scratch of las_orbital_hvp (allocated by its first call): G(C) [n][nmo] and C^T G [nmo][op];
+  // the tangent chain's dC_occ, h dC_occ and projection [n][op], dH [Lc][op][n], X = H^T dC, dT and
   // the two W matrices of the tangent [Lc][op][op]
-  double *hdC, *hG, *tCocc, *thC, *tOut, *tHt, *tX, *tdT, *tdW, *tWd;
+  double *hM, *hG, *tCocc, *thC, *tOut, *tHt, *tX, *tdT, *tdW, *tWd;
   int* widx;          // [2*o + 2] columns of each weight sign and their counts (JK density)
   int wcount[2];      // host copy of those counts
   // timing: a ring of LAS_TIMING_RING evaluations x 6 stage marks, read without per-call syncs
@@ -126,7 +127,7 @@ static void free_all(las_ctx* x) {
     if (p) cudaFree(p);
   if (x->split) split_destroy(x->split);
   if (x->fsplit) frag_split_destroy(x->fsplit);
-  for (double* q : {x->fH, x->fT, x->fpart, x->vJ, x->vK, x->hdC, x->hG, x->tCocc, x->thC,
+  for (double* q : {x->fH, x->fT, x->fpart, x->vJ, x->vK, x->hM, x->hG, x->tCocc, x->thC,
                     x->tOut, x->tHt, x->tX, x->tdT, x->tdW, x->tWd})
     if (q) cudaFree(q);
   if (x->ev) {
@@ -207,6 +208,13 @@ extern "C" las_status las_create(las_ctx** out, const las_dims* d, const double*
   }
   x->Lc = Lc;
   x->ws_cap = cap;
+  {
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&x->sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+        x->sms <= 0)
+      x->sms = 152;
+  }
   {
     int tiles = ((x->n + 63) / 64) * ((x->op + 63) / 64);
     int ks = (4 * 152 + tiles - 1) / tiles;
@@ -381,6 +389,30 @@ static inline void stage_mark(las_ctx* x, int i) {
 // ------------------------------------------------------------------------------------------
 // Chain pieces
 // ------------------------------------------------------------------------------------------
+// out (+)= A B (M x N, row stride ld) in FP64, split over K through `part` where that fills the
+// SMs: one CTA's 64 x 80 x 400 block alone takes 450 us (400 orbitals: C^T G in 7 CTAs, 500 us;
+// split over 152 SMs, 50 us).
+template <class LA, class LB>
+static void gemm_f64_wide(las_ctx* x, int M, int N, int K, LA A, LB B, double* out, int ld,
+                          int accumulate) {
+  const long room = (long)x->ksplit * x->n * x->op, mn = (long)M * N;
+  const int cap = (int)std::max(1L, std::min(64L, mn > 0 ? room / mn : 1L));
+  const int ks = f64_balanced_ksplit(f64_tiles(M, N), K, cap, x->sms);
+  if (ks == 1) {
+    gemm_f64(M, N, K, 1, 1, A, B, StridedC{out, 0, ld, 1, 1.0, accumulate}, x->stream);
+    return;
+  }
+  gemm_f64(M, N, K, 1, ks, A, B, StridedC{x->part, mn, N, 1, 1.0, 0}, x->stream);
+  launch_reduce_partials(x->part, ks, mn, out, accumulate, x->stream, N, ld);
+}
+
+// Out (+)= sum_{b < nL} H_b^T W_b (n x op), H [nL][op][n], W [nL][op][op]
+static void project_f64(las_ctx* x, int nL, const double* H, const double* W, double* Out,
+                        int accumulate) {
+  gemm_f64_wide(x, x->n, x->op, nL * x->op, StridedA{H, 0, 1, x->n}, StridedA{W, 0, x->op, 1},
+                Out, x->op, accumulate);
+}
+
 // S1 + S2 on auxiliary rows [l0, l0+nL): Ht[b][p][mu] = (b^L C_occ)(mu,p), T[b] = C_occ^T H
 // H_L = b^L C_occ for the chunk's aux rows, over the first oc columns of C_occ (Ht layout
 // [nL][oc][n]); with want_T (only for oc = op) also T_L = C_occ^T H_L.
@@ -403,23 +435,17 @@ static las_status half_and_full(las_ctx* x, int l0, int nL, int want_T, int mark
   if (want_T) {
     StridedA Ah{x->Ht, (long)op * n, n, 1};
     StridedC Ct{x->T, (long)op * op, op, 1, 1.0, 0};
-    gemm_f64(op, op, n, nL, 1, Ah, Bm, Ct, x->stream);
+    gemm_f64<true>(op, op, n, nL, 1, Ah, Bm, Ct, x->stream);   // T_L is symmetric
   }
   return check_launch();
 }
 
 // Out (+)= sum_{b < nL} Ht_b^T W_b   (n x op), split over K = nL*op, partials reduced in order
 static las_status project(las_ctx* x, int nL, int accumulate) {
-  const int n = x->n, op = x->op;
   if (x->prec == LAS_SPLIT_BF16) {
     return split_project(x->split, nL, x->W, x->Out, accumulate, x->stream);
   }
-  int ks = std::max(1, std::min(x->ksplit, (nL * op) / 64));
-  StridedA A{x->Ht, 0, 1, n};
-  StridedA Bw{x->W, 0, op, 1};
-  StridedC Cp{x->part, (long)n * op, op, 1, 1.0, 0};
-  gemm_f64(n, op, nL * op, 1, ks, A, Bw, Cp, x->stream);
-  launch_reduce_partials(x->part, ks, (long)n * op, x->Out, accumulate, x->stream);
+  project_f64(x, nL, x->Ht, x->W, x->Out, accumulate);
   return check_launch();
 }
 
@@ -452,23 +478,15 @@ static las_status evaluate(las_ctx* x, const double* C, const double* h, const d
   if (x->prec == LAS_SPLIT_BF16) {  // one-electron pieces: hC = h C_occ, hmo = C_occ^T hC
     if ((st = split_one_electron(x->split, h, x->hC, x->hmo, x->stream)) != LAS_OK) return st;
   } else {
-    StridedA Ah{h, 0, n, 1};
-    StridedA Bc{x->Cocc, 0, op, 1};
-    StridedC Ch{x->hC, 0, op, 1, 1.0, 0};
-    gemm_f64(n, op, n, 1, 1, Ah, Bc, Ch, x->stream);
-    StridedA Act{x->Cocc, 0, 1, op};
-    StridedA Bh{x->hC, 0, op, 1};
-    StridedC Cm{x->hmo, 0, op, 1, 1.0, 0};
-    gemm_f64(op, op, n, 1, 1, Act, Bh, Cm, x->stream);
+    gemm_f64_wide(x, n, op, n, StridedA{h, 0, n, 1}, StridedA{x->Cocc, 0, op, 1}, x->hC, op, 0);
+    gemm_f64_wide(x, op, op, n, StridedA{x->Cocc, 0, 1, op}, StridedA{x->hC, 0, op, 1}, x->hmo,
+                  op, 0);
   }
   launch_energy_final(x->eps, x->X, x->hmo, op, dm1s, x->fi, E, x->stream);
   if (with_grad) {
     launch_assemble_grad(x->Out, x->hC, dm1s, x->fi, n, nmo, op, G, x->stream);
     if (gorb) {
-      StridedA Act{C, 0, 1, nmo};
-      StridedA Bg{G, 0, nmo, 1};
-      StridedC Cm{x->M, 0, op, 1, 1.0, 0};
-      gemm_f64(nmo, x->o, n, 1, 1, Act, Bg, Cm, x->stream);
+      gemm_f64_wide(x, nmo, x->o, n, StridedA{C, 0, 1, nmo}, StridedA{G, 0, nmo, 1}, x->M, op, 0);
       launch_antisym(x->M, nmo, x->o, op, gorb, x->stream);
     }
   }
@@ -535,15 +553,17 @@ static las_status jk_raw(las_ctx* x, int r, double* J, double* K) {
     } else if (K) {
       StridedA A{x->Ht, 0, 1, n};
       StridedA B{x->Ht, 0, n, 1};
-      int ks = std::max(1, std::min(x->ksplit, (nL * r) / 64));
-      // reuse `part` as [ks][n][n] only when it is large enough; otherwise accumulate directly
-      if ((size_t)ks * n * n <= (size_t)x->ksplit * n * op) {
+      // K is symmetric; split over (L, k) as far as `part` holds [ks][n][n]
+      const long mt = (n + 63) / 64, tiles = (f64_tiles(n, n) + mt) / 2;   // about half of them
+      const int cap = (int)std::min(64L, (long)x->ksplit * op / n);
+      const int ks = cap > 1 ? f64_balanced_ksplit((int)tiles, nL * r, cap, x->sms) : 1;
+      if (ks > 1) {
         StridedC Pk{x->part, (long)n * n, n, 1, 1.0, 0};
-        gemm_f64(n, n, nL * r, 1, ks, A, B, Pk, x->stream);
+        gemm_f64<true>(n, n, nL * r, 1, ks, A, B, Pk, x->stream);
         launch_reduce_partials(x->part, ks, (long)n * n, K, l0 > 0, x->stream);
       } else {
         StridedC Kd{K, 0, n, 1, 1.0, l0 > 0};
-        gemm_f64(n, n, nL * r, 1, 1, A, B, Kd, x->stream);
+        gemm_f64<true>(n, n, nL * r, 1, 1, A, B, Kd, x->stream);
       }
     }
     if ((st = check_launch()) != LAS_OK) return st;
@@ -686,10 +706,9 @@ extern "C" las_status las_veff(las_ctx* x, const double* Ca, const double* wa, i
 // of H, the operand each is projected against.  G(C) itself (for Dg) is one plain evaluation.
 static las_status tangent_grad(las_ctx* x, const double* h, const double* dm1s,
                                const double* dm2, double* dG) {
-  const int n = x->n, op = x->op, nmo = x->nmo;
+  const int n = x->n, op = x->op, nmo = x->nmo;   // x->tCocc holds dC_occ
   const bool split = x->prec == LAS_SPLIT_BF16;
   las_status st;
-  launch_pack_cocc(x->hdC, n, nmo, x->o, op, x->tCocc, x->stream);   // dC_occ
   if (split && (st = split_tangent_prepare(x->split, x->tCocc, x->stream, &x->bytes)) != LAS_OK)
     return st;
   if (split && (st = split_prepare_C(x->split, x->Cocc, x->stream)) != LAS_OK) return st;
@@ -707,7 +726,8 @@ static las_status tangent_grad(las_ctx* x, const double* h, const double* dm1s,
       gemm_f64(n, op, n, nL, 1, A, Bc, StridedC{x->Ht, (long)op * n, 1, n, 1.0, 0}, x->stream);
       gemm_f64(n, op, n, nL, 1, A, Bd, StridedC{x->tHt, (long)op * n, 1, n, 1.0, 0}, x->stream);
       StridedA Ah{x->Ht, (long)op * n, n, 1};
-      gemm_f64(op, op, n, nL, 1, Ah, Bc, StridedC{x->T, (long)op * op, op, 1, 1.0, 0}, x->stream);
+      gemm_f64<true>(op, op, n, nL, 1, Ah, Bc, StridedC{x->T, (long)op * op, op, 1, 1.0, 0},
+                     x->stream);
       gemm_f64(op, op, n, nL, 1, Ah, Bd, StridedC{x->tX, (long)op * op, op, 1, 1.0, 0},
                x->stream);
     }
@@ -726,16 +746,8 @@ static las_status tangent_grad(las_ctx* x, const double* h, const double* dm1s,
           (st = split_tangent_project(x->split, nL, 1, x->tWd, x->tOut, 1, x->stream)) != LAS_OK)
         return st;
     } else {
-      const int ks = std::max(1, std::min(x->ksplit, (nL * op) / 64));
-      const double* Hs[2] = {x->Ht, x->tHt};
-      const double* Ws[2] = {x->tdW, x->tWd};
-      for (int k = 0; k < 2; ++k) {
-        StridedA A{Hs[k], 0, 1, n};
-        StridedA Bw{Ws[k], 0, op, 1};
-        StridedC Cp{x->part, (long)n * op, op, 1, 1.0, 0};
-        gemm_f64(n, op, nL * op, 1, ks, A, Bw, Cp, x->stream);
-        launch_reduce_partials(x->part, ks, (long)n * op, x->tOut, l0 > 0 || k > 0, x->stream);
-      }
+      project_f64(x, nL, x->Ht, x->tdW, x->tOut, l0 > 0);
+      project_f64(x, nL, x->tHt, x->tWd, x->tOut, 1);
     }
     if ((st = check_launch()) != LAS_OK) return st;
   }
@@ -745,8 +757,7 @@ static las_status tangent_grad(las_ctx* x, const double* h, const double* dm1s,
         (st = split_tangent_one_electron(x->split, x->thC, x->stream)) != LAS_OK)
       return st;
   } else {
-    gemm_f64(n, op, n, 1, 1, StridedA{h, 0, n, 1}, StridedA{x->tCocc, 0, op, 1},
-             StridedC{x->thC, 0, op, 1, 1.0, 0}, x->stream);
+    gemm_f64_wide(x, n, op, n, StridedA{h, 0, n, 1}, StridedA{x->tCocc, 0, op, 1}, x->thC, op, 0);
   }
   launch_assemble_grad(x->tOut, x->thC, dm1s, x->fi, n, nmo, op, dG, x->stream);
   return check_launch();
@@ -757,36 +768,33 @@ extern "C" las_status las_orbital_hvp(las_ctx* x, const double* C, const double*
                                       double* dG, double* Dg) {
   if (!x || !C || !h || !X || !dG) return LAS_ERR_ARG;
   if (x->a > 0 && (!dm1s || !dm2)) return LAS_ERR_ARG;
-  const int n = x->n, nmo = x->nmo, op = x->op;
+  const int n = x->n, nmo = x->nmo, op = x->op, o = x->o;
   const long nC = (long)n * nmo;
   const size_t chunk = (size_t)x->Lc * op;
   las_status st = LAS_OK;
-  if (!x->hdC) {
+  if (!x->tWd) {   // the last of the buffers below: all are there once it is
     const struct { double** p; size_t cnt; } bufs[] = {
-        {&x->hdC, (size_t)nC}, {&x->hG, (size_t)nC}, {&x->tCocc, (size_t)n * op},
+        {&x->hM, (size_t)nmo * op}, {&x->hG, (size_t)nC}, {&x->tCocc, (size_t)n * op},
         {&x->thC, (size_t)n * op}, {&x->tOut, (size_t)n * op}, {&x->tHt, chunk * n},
         {&x->tX, chunk * op}, {&x->tdT, chunk * op}, {&x->tdW, chunk * op},
         {&x->tWd, chunk * op}};
     for (const auto& b : bufs)
-      if ((st = dalloc(x, (void**)b.p, sizeof(double) * b.cnt)) != LAS_OK) return st;
+      if (!*b.p && (st = dalloc(x, (void**)b.p, sizeof(double) * b.cnt)) != LAS_OK) return st;
   }
-  // dC = C X
-  gemm_f64(n, nmo, nmo, 1, 1, StridedA{C, 0, nmo, 1}, StridedA{X, 0, nmo, 1},
-           StridedC{x->hdC, 0, nmo, 1, 1.0, 0}, x->stream);
+  // dC_occ = C X_occ (only the occupied columns of C X are ever needed); zero padding columns
+  LAS_CUDA_TRY(cudaMemsetAsync(x->tCocc, 0, sizeof(double) * n * op, x->stream));
+  gemm_f64_wide(x, n, o, nmo, StridedA{C, 0, nmo, 1}, StridedA{X, 0, nmo, 1}, x->tCocc, op, 0);
   // G(C): C_occ, its digits and those of h stay in place for the tangent chain
   if ((st = evaluate(x, C, h, dm1s, dm2, x->dE, x->hG, nullptr)) != LAS_OK) return st;
   if ((st = tangent_grad(x, h, dm1s, dm2, dG)) != LAS_OK) return st;
   if (Dg) {
-    // Dg = (C X)^T G + C^T dG - transpose  (virtual columns of G and dG are zero)
-    StridedA Ad{x->hdC, 0, 1, nmo};
-    StridedA Bg{x->hG, 0, nmo, 1};
-    StridedC Cm{x->M, 0, x->op, 1, 1.0, 0};
-    gemm_f64(nmo, x->o, n, 1, 1, Ad, Bg, Cm, x->stream);
-    StridedA Acc{C, 0, 1, nmo};
-    StridedA Bdg{dG, 0, nmo, 1};
-    StridedC Cm2{x->M, 0, x->op, 1, 1.0, 1};
-    gemm_f64(nmo, x->o, n, 1, 1, Acc, Bdg, Cm2, x->stream);
-    launch_antisym(x->M, nmo, x->o, x->op, Dg, x->stream);
+    // Dg = (C X)^T G + C^T dG - transpose = X^T (C^T G) + C^T dG - transpose  (virtual columns
+    // of G and dG are zero)
+    const StridedA Ct{C, 0, 1, nmo};
+    gemm_f64_wide(x, nmo, o, n, Ct, StridedA{x->hG, 0, nmo, 1}, x->hM, op, 0);
+    gemm_f64_wide(x, nmo, o, nmo, StridedA{X, 0, 1, nmo}, StridedA{x->hM, 0, op, 1}, x->M, op, 0);
+    gemm_f64_wide(x, nmo, o, n, Ct, StridedA{dG, 0, nmo, 1}, x->M, op, 1);
+    launch_antisym(x->M, nmo, o, op, Dg, x->stream);
   }
   return check_launch();
 }

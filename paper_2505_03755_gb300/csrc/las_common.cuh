@@ -38,9 +38,8 @@ struct FragInfo {
 
 // ------------------------------------------------------------------------------------------
 // Generic FP64 GEMM on DMMA (mma.sync.m16n8k4.f64):  C[b](m,n) (+)= alpha * sum_k A[b](m,k) B[b](k,n)
-// Operands are read through small loader objects so that packed-symmetric B, transposed views
-// and batched/strided layouts share one kernel.  FP64 arithmetic on this part is slow enough
-// (about 3.5 flop/clk/SM) that element-wise staging through shared memory is never the bound.
+// (gemm_f64.cuh).  Operands are read through small loader objects so that packed-symmetric B,
+// transposed views and batched/strided layouts share one kernel.
 // ------------------------------------------------------------------------------------------
 struct StridedA {  // element (b, m, k) = p[b*sb + m*sm + k*sk]
   const double* p;
@@ -72,9 +71,6 @@ struct StridedC {  // C[b*sb + m*sm + n*sn] (=|+=) alpha * acc
   }
 };
 
-template <class LA, class LB, class SC>
-void gemm_f64(int M, int N, int K, int batch, int ksplit, LA a, LB b, SC c, cudaStream_t s);
-
 // Small helpers implemented in las_kernels.cu
 void launch_pack_cocc(const double* C, int n, int nmo, int o, int op, double* Cocc,
                       cudaStream_t s);
@@ -100,8 +96,10 @@ void launch_sign_split(const double* w, int r, int* idx_pos, int* idx_neg, int* 
                        cudaStream_t s);
 void launch_pack_weighted(const double* Cx, const double* w, const int* idx, int cnt,
                           double sign, int n, int r, int op, double* Cocc, cudaStream_t s);
+// out (+)= sum_k part[k*count ...] in order of k; with cols < ld the values are rows of `cols`
+// that land `ld` apart in out
 void launch_reduce_partials(const double* part, int nsplit, long count, double* out,
-                            int accumulate, cudaStream_t s);
+                            int accumulate, cudaStream_t s, int cols = 0, int ld = 0);
 void launch_assemble_grad(const double* Out, const double* hC, const double* dm1s,
                           const FragInfo& fi, int n, int nmo, int op, double* G,
                           cudaStream_t s);

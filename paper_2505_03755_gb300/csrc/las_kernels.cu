@@ -304,13 +304,16 @@ __global__ void k_scale(double* __restrict__ p, long count, double a) {
   if (i < count) p[i] *= a;
 }
 
+// Partials of rows of `cols` values, summed in order into rows `ld` apart.
 __global__ void k_reduce_partials(const double* __restrict__ part, int nsplit, long count,
-                                  double* __restrict__ out, int accumulate) {
+                                  double* __restrict__ out, int accumulate, int cols, int ld) {
   long i = blockIdx.x * (long)blockDim.x + threadIdx.x;
   if (i >= count) return;
-  double s = accumulate ? out[i] : 0.0;
+  const long o = cols == ld ? i : i / cols * ld + i % cols;
+  double s = accumulate ? out[o] : 0.0;
+#pragma unroll 8
   for (int k = 0; k < nsplit; ++k) s += part[(long)k * count + i];
-  out[i] = s;
+  out[o] = s;
 }
 
 // dE/dC = [4 h C_core | 2 h C_act D | 0] + Out   (Out = sum_L H_L W_L, n x op)
@@ -545,8 +548,9 @@ void launch_scale(double* p, long count, double a, cudaStream_t s) {
 }
 
 void launch_reduce_partials(const double* part, int nsplit, long count, double* out,
-                            int accumulate, cudaStream_t s) {
-  k_reduce_partials<<<nblk(count, 256), 256, 0, s>>>(part, nsplit, count, out, accumulate);
+                            int accumulate, cudaStream_t s, int cols, int ld) {
+  k_reduce_partials<<<nblk(count, 256), 256, 0, s>>>(part, nsplit, count, out, accumulate, cols,
+                                                     ld);
   las_count_launch();
 }
 
