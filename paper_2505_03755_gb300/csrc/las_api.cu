@@ -58,7 +58,7 @@ struct las_ctx {
   double* part;   // [ksplit][n][op]
   double* Out;    // [n][op]
   double* hC;     // [n][op]
-  double* hmo;    // [op][op]
+  double* e1;     // [E1_BLOCKS] partial sums of the one-electron energy
   double* M;      // [nmo][op]
   double* eps;    // [X]
   double* vc;     // [X]
@@ -120,7 +120,7 @@ static las_status dalloc(las_ctx* x, void** p, size_t bytes) {
 }
 
 static void free_all(las_ctx* x) {
-  void* ptrs[] = {x->Cocc, x->Ht, x->T, x->W, x->part, x->Out, x->hC, x->hmo, x->M, x->eps,
+  void* ptrs[] = {x->Cocc, x->Ht, x->T, x->W, x->part, x->Out, x->hC, x->e1, x->M, x->eps,
                   x->vc, x->va, x->Jp, x->Jt, x->Kt, x->widx, x->status, x->dC, x->dh, x->ddm1, x->ddm2,
                   x->dE, x->dG};
   for (void* p : ptrs)
@@ -197,7 +197,7 @@ extern "C" las_status las_create(las_ctx** out, const las_dims* d, const double*
   x->fi_c.ncore = d->ncore;
 
   // Workspace plan: the largest auxiliary chunk that fits the cap.
-  const size_t fixed = sizeof(double) * ((size_t)x->n * x->op * 4 + (size_t)x->op * x->op +
+  const size_t fixed = sizeof(double) * ((size_t)x->n * x->op * 4 + E1_BLOCKS +
                                          (size_t)x->nmo * x->op + 3 * (size_t)x->X + x->npair);
   size_t cap = max_ws ? max_ws : (size_t)64 << 30;
   int Lc = x->X;
@@ -231,7 +231,7 @@ extern "C" las_status las_create(las_ctx** out, const las_dims* d, const double*
   ALLOC(part, (size_t)x->ksplit * x->n * x->op);
   ALLOC(Out, (size_t)x->n * x->op);
   ALLOC(hC, (size_t)x->n * x->op);
-  ALLOC(hmo, (size_t)x->op * x->op);
+  ALLOC(e1, E1_BLOCKS);
   ALLOC(M, (size_t)x->nmo * x->op);
   ALLOC(eps, x->X);
   ALLOC(vc, x->X);
@@ -475,14 +475,12 @@ static las_status evaluate(las_ctx* x, const double* C, const double* h, const d
     if (with_grad && (st = project(x, nL, l0 > 0)) != LAS_OK) return st;
     if (l0 == 0) stage_mark(x, 4);
   }
-  if (x->prec == LAS_SPLIT_BF16) {  // one-electron pieces: hC = h C_occ, hmo = C_occ^T hC
-    if ((st = split_one_electron(x->split, h, x->hC, x->hmo, x->stream)) != LAS_OK) return st;
+  if (x->prec == LAS_SPLIT_BF16) {  // hC = h C_occ
+    if ((st = split_one_electron_hc(x->split, h, x->hC, x->stream)) != LAS_OK) return st;
   } else {
     gemm_f64_wide(x, n, op, n, StridedA{h, 0, n, 1}, StridedA{x->Cocc, 0, op, 1}, x->hC, op, 0);
-    gemm_f64_wide(x, op, op, n, StridedA{x->Cocc, 0, 1, op}, StridedA{x->hC, 0, op, 1}, x->hmo,
-                  op, 0);
   }
-  launch_energy_final(x->eps, x->X, x->hmo, op, dm1s, x->fi, E, x->stream);
+  launch_energy(x->eps, x->X, x->Cocc, x->hC, n, op, dm1s, x->fi, x->e1, E, x->stream);
   if (with_grad) {
     launch_assemble_grad(x->Out, x->hC, dm1s, x->fi, n, nmo, op, G, x->stream);
     if (gorb) {
@@ -940,7 +938,7 @@ static bool same_items(const las_batch_item& a, const las_batch_item& b) {
 // persistent grouped launch (tiles in the order the problems are visited: largest first), then
 // the next phase forks again.  Per auxiliary chunk c of each problem:
 //   A: [c = 0: C_occ and h digits]      products: S1 of chunk c (+ h C_occ at c = 0)
-//   B: digits of H                      products: S2 of chunk c (+ C_occ^T h C_occ at c = 0)
+//   B: digits of H                      products: S2 of chunk c
 //   C: per-aux contractions, W digits   products: projection of chunk c
 //   D: ordered sum of the projection's partials (run with the next round's A)
 // then the energy and gradient assembly.  Problems with fewer chunks drop out of later rounds.
@@ -1045,13 +1043,11 @@ static las_status capture_grouped(const BatchPlan& P, las_ctx* const* ctxs,
       return split_half(x->split, l0, nL, x->op, x->Ht, x->stream);
     }, true);
     if (rc != LAS_OK) break;
-    // B: digits of H; S2 of chunk c (and C_occ^T h C_occ at c = 0)
+    // B: digits of H; S2 of chunk c
     rc = phase([&](int i, las_ctx* x) -> las_status {
       if (c >= nchunks(x)) return LAS_OK;
       const int nL = std::min(x->Lc, x->X - c * x->Lc);
-      las_status r = split_full(x->split, nL, x->Ht, x->T, x->stream);
-      if (r == LAS_OK && c == 0) r = split_one_electron_hmo(x->split, x->hC, x->hmo, x->stream);
-      return r;
+      return split_full(x->split, nL, x->Ht, x->T, x->stream);
     }, true);
     if (rc != LAS_OK) break;
     // C: per-aux contractions and W digits; projection of chunk c
@@ -1070,8 +1066,8 @@ static las_status capture_grouped(const BatchPlan& P, las_ctx* const* ctxs,
     rc = phase([&](int i, las_ctx* x) -> las_status {
       const int last = nchunks(x) - 1;
       split_project_reduce(x->split, ks[i], x->Out, last > 0, x->stream);
-      launch_energy_final(x->eps, x->X, x->hmo, x->op, items[i].dm1s, x->fi, items[i].E,
-                          x->stream);
+      launch_energy(x->eps, x->X, x->Cocc, x->hC, x->n, x->op, items[i].dm1s, x->fi, x->e1,
+                    items[i].E, x->stream);
       launch_assemble_grad(x->Out, x->hC, items[i].dm1s, x->fi, x->n, x->nmo, x->op,
                            items[i].dEdC, x->stream);
       return check_launch();

@@ -103,8 +103,10 @@ void launch_reduce_partials(const double* part, int nsplit, long count, double* 
 void launch_assemble_grad(const double* Out, const double* hC, const double* dm1s,
                           const FragInfo& fi, int n, int nmo, int op, double* G,
                           cudaStream_t s);
-void launch_energy_final(const double* eps, int X, const double* hmo, int op,
-                         const double* dm1s, const FragInfo& fi, double* E, cudaStream_t s);
+// *E = one-electron energy of h (hC = h C_occ) + sum_L eps_L; e1: E1_BLOCKS doubles of scratch
+#define E1_BLOCKS 256
+void launch_energy(const double* eps, int X, const double* Cocc, const double* hC, int n, int op,
+                   const double* dm1s, const FragInfo& fi, double* e1, double* E, cudaStream_t s);
 void launch_antisym(const double* M, int nmo, int o, int op, double* g, cudaStream_t s);
 void launch_coulomb_packed(const double* Bp, const double* vc, int X, long npair,
                            double* Jp, cudaStream_t s);

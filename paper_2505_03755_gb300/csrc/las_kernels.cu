@@ -341,31 +341,51 @@ __global__ void k_assemble_grad(const double* __restrict__ Out, const double* __
   G[i] = g;
 }
 
-// E = 2 sum_i hmo(i,i) + sum_uv hmo(c+u,c+v) D_uv + sum_L eps_L  (one CTA, fixed order,
-// compensated summation).
+// One-electron energy sum_mu ( 2 sum_i C(mu,i) hC(mu,i) + sum_u C(mu,u) sum_v D_uv hC(mu,v) ): one
+// warp per row mu, one partial per block.  (Only these elements of C_occ^T h C_occ enter the
+// energy; forming the whole matrix took a slicing pass and a product of its own, 45 us at 400
+// orbitals against 4.)
 __global__ void __launch_bounds__(256)
-k_energy_final(const double* __restrict__ eps, int X, const double* __restrict__ hmo, int op,
-               const double* __restrict__ dm1s, FragInfo fi, double* __restrict__ E) {
-  __shared__ double red[256];
+k_energy_one(const double* __restrict__ Cocc, const double* __restrict__ hC, int n, int op,
+             const double* __restrict__ dm1s, FragInfo fi, double* __restrict__ e1) {
+  __shared__ double red[8];
+  const int lane = threadIdx.x & 31, c = fi.ncore, o = c + fi.nact;
+  double s[1] = {0.0};
+  for (long mu = blockIdx.x * 8L + (threadIdx.x >> 5); mu < n; mu += gridDim.x * 8L) {
+    const double* Cr = Cocc + mu * op;
+    const double* hr = hC + mu * op;
+    for (int p = lane; p < o; p += 32) {
+      if (p < c) {
+        s[0] += 2.0 * Cr[p] * hr[p];
+      } else {
+        const int u = p - c, K = frag_of(fi, u), oK = fi.off[K], m = fi.off[K + 1] - oK;
+        const double* g = dm1s + fi.dm1_off[K] + (u - oK) * m;
+        double t = 0.0;
+        for (int v = 0; v < m; ++v) t += (g[v] + g[m * m + v]) * hr[c + oK + v];
+        s[0] += Cr[p] * t;
+      }
+    }
+  }
+  block_sums<256, 1>(s, red);
+  if (threadIdx.x == 0) e1[blockIdx.x] = s[0];
+}
+
+// E = sum_b e1_b + sum_L eps_L  (one CTA, fixed order, compensated summation).
+__global__ void __launch_bounds__(1024)
+k_energy_final(const double* __restrict__ eps, int X, const double* __restrict__ e1, int ne1,
+               double* __restrict__ E) {
+  __shared__ double red[32];
   double s = 0.0, comp = 0.0;
   auto add = [&](double x) {  // Neumaier
     double t = s + x;
     if (fabs(s) >= fabs(x)) comp += (s - t) + x; else comp += (x - t) + s;
     s = t;
   };
-  for (int L = threadIdx.x; L < X; L += 256) add(eps[L]);
-  const int c = fi.ncore;
-  for (int i = threadIdx.x; i < c; i += 256) add(2.0 * hmo[(long)i * op + i]);
-  for (int K = 0; K < fi.nfrag; ++K) {
-    const int oK = fi.off[K], m = fi.off[K + 1] - oK;
-    const double* g = dm1s + fi.dm1_off[K];
-    for (int i = threadIdx.x; i < m * m; i += 256) {
-      const int u = i / m, v = i % m;
-      add(hmo[(long)(c + oK + u) * op + c + oK + v] * (g[i] + g[m * m + i]));
-    }
-  }
-  double tot = block_sum<256>(s + comp, red);
-  if (threadIdx.x == 0) *E = tot;
+  for (int L = threadIdx.x; L < X; L += 1024) add(eps[L]);
+  for (int i = threadIdx.x; i < ne1; i += 1024) add(e1[i]);
+  double tot[1] = {s + comp};
+  block_sums<1024, 1>(tot, red);
+  if (threadIdx.x == 0) *E = tot[0];
 }
 
 // g[p][q] = M'[p][q] - M'[q][p],  M'[p][q] = M[p][q] for q < o else 0  (M is nmo x op)
@@ -561,10 +581,13 @@ void launch_assemble_grad(const double* Out, const double* hC, const double* dm1
   las_count_launch();
 }
 
-void launch_energy_final(const double* eps, int X, const double* hmo, int op,
-                         const double* dm1s, const FragInfo& fi, double* E, cudaStream_t s) {
-  k_energy_final<<<1, 256, 0, s>>>(eps, X, hmo, op, dm1s, fi, E);
-  las_count_launch();
+void launch_energy(const double* eps, int X, const double* Cocc, const double* hC, int n, int op,
+                   const double* dm1s, const FragInfo& fi, double* e1, double* E,
+                   cudaStream_t s) {
+  const int nb = (int)std::min<long>(nblk(n, 8), E1_BLOCKS);
+  k_energy_one<<<nb, 256, 0, s>>>(Cocc, hC, n, op, dm1s, fi, e1);
+  k_energy_final<<<1, 1024, 0, s>>>(eps, X, e1, nb, E);
+  las_count_launch(2);
 }
 
 void launch_absmax_bits(const double* a, long count, unsigned long long* out, cudaStream_t s) {

@@ -1496,8 +1496,6 @@ struct SplitState {
   void* Mpblob;
   Planes hdig;           // rows mu of h, K = nu
   int* hexp;             // [n]
-  Planes hcdig;          // rows q of (h C_occ)^T, K = mu
-  int* hcexp;            // [op]
   int ksplit6;           // partial buffers allocated for this many K splits
   int ks;                // split-K factor of the projection GEMM (autotunable)
   int bn[SPLIT_NKIND];   // tile width of each product kind (autotunable): 64 or 96
@@ -1517,7 +1515,7 @@ static void split_free(SplitState* s) {
   void* ptrs[] = {s->Bdig.p, s->Bexp, s->Bpk.tiles.p, s->Bpk.rag.p, s->Bpk.exp, s->Bpk.mx,
                   s->Cdig.p, s->Cexp,
                   s->Hdig.p, s->Hexp, s->HdigT.p,
-                  s->Wdig.p, s->Wexp, s->part, s->mx, s->hdig.p, s->hexp, s->hcdig.p, s->hcexp};
+                  s->Wdig.p, s->Wexp, s->part, s->mx, s->hdig.p, s->hexp};
   for (void* q : ptrs)
     if (q) cudaFree(q);
 }
@@ -1599,14 +1597,10 @@ las_status split_create(SplitState** out, int n, int X, int op, int Lc, const do
   A((void**)&s->mx, (size_t)(op + n) * 8);
   A(&q, planes_bytes(n, n));         s->hdig = make_planes(q, n, n);    q = nullptr;
   A((void**)&s->hexp, (size_t)n * 4);
-  A(&q, planes_bytes(op, n));        s->hcdig = make_planes(q, op, n);  q = nullptr;
-  A((void**)&s->hcexp, (size_t)op * 4);
-  // rows mu >= n of the transposed planes and the padding rows of C, W, h and (h C)^T are never
-  // written by the per-evaluation slicers: make them zero once
+  // rows mu >= n of the transposed planes and the padding rows of C, W and h are never written by the per-evaluation slicers: make them zero once
   const struct { void* p; size_t b; } zero[] = {
       {s->HdigT.p, planes_bytes(n, R)}, {s->Wdig.p, planes_bytes(op, R)},
-      {s->Cdig.p, planes_bytes(op, n)}, {s->hdig.p, planes_bytes(n, n)},
-      {s->hcdig.p, planes_bytes(op, n)}};
+      {s->Cdig.p, planes_bytes(op, n)}, {s->hdig.p, planes_bytes(n, n)}};
   for (const auto& z : zero) {
     if (rc != LAS_OK) break;
     cudaError_t e = cudaMemsetAsync(z.p, 0, z.b, st);
@@ -1919,24 +1913,6 @@ las_status split_one_electron_hc(SplitState* s, const double* h, double* hC, cud
   if (rc == LAS_OK)
     rc = ozaki_gemm(s->hdig, 0, s->hexp, s->n, s->Cdig, 0, s->Cexp, s->op, s->n, 1, 0, hC, s->op,
                     0, 0, 0, s->status, st, 0, s->bn[SPLIT_ONE_ELECTRON]);
-  return rc;
-}
-
-las_status split_one_electron_hmo(SplitState* s, const double* hC, double* hmo,
-                                  cudaStream_t st) {
-  // hmo = C_occ^T hC  (rows p of C_occ^T are the C_occ digit rows; columns q of hC)
-  las_status rc =
-      slice_rows(RowsStrided{hC, 1, s->op, nullptr}, s->hcdig, s->hcexp, st, nullptr, true);
-  if (rc == LAS_OK)
-    rc = ozaki_gemm(s->Cdig, 0, s->Cexp, s->op, s->hcdig, 0, s->hcexp, s->op, s->n, 1, 0, hmo,
-                    s->op, 0, 0, 0, s->status, st, 0, s->bn[SPLIT_ONE_ELECTRON]);
-  return rc;
-}
-
-las_status split_one_electron(SplitState* s, const double* h, double* hC, double* hmo,
-                              cudaStream_t st) {
-  las_status rc = split_one_electron_hc(s, h, hC, st);
-  if (rc == LAS_OK) rc = split_one_electron_hmo(s, hC, hmo, st);
   return rc;
 }
 

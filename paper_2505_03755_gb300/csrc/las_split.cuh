@@ -27,7 +27,7 @@ las_status split_full(SplitState* s, int nL, const double* Ht, double* T, cudaSt
 las_status split_exchange(SplitState* s, int nL, int oc, const double* Ht, double* K, int accumulate,
                           cudaStream_t st);
 // Product kinds of an evaluation, each with its own tile width (64 or 96 columns; default 96):
-// S1, S2 (with its H slicer), the projection and the two one-electron products.
+// S1, S2 (with its H slicer), the projection and the one-electron product.
 enum { SPLIT_HALF = 0, SPLIT_FULL = 1, SPLIT_PROJECT = 2, SPLIT_ONE_ELECTRON = 3, SPLIT_NKIND = 4 };
 int split_get_tile(SplitState* s, int kind);
 las_status split_set_tile(SplitState* s, int kind, int bn);
@@ -36,9 +36,8 @@ int split_get_ksplit(SplitState* s);
 // split-K of the projection that shares its tiles out most evenly over the SMs for nL aux rows
 int split_balanced_ksplit(SplitState* s, int nL);
 void split_set_ksplit(SplitState* s, int ks);
-// hC = h C_occ and hmo = C_occ^T hC (split_prepare_C must have run for this C)
-las_status split_one_electron(SplitState* s, const double* h, double* hC, double* hmo,
-                              cudaStream_t st);
+// hC = h C_occ (split_prepare_C must have run for this C)
+las_status split_one_electron_hc(SplitState* s, const double* h, double* hC, cudaStream_t st);
 // Out (+)= sum_{(L,p)} H(mu,(L,p)) W((L,p),q) with Wt[q][(L,p)] = W_L(p,q) * 2^exp(L,p)
 las_status split_project(SplitState* s, int nL, const double* Wt, double* Out, int accumulate,
                          cudaStream_t st);
@@ -47,10 +46,6 @@ las_status split_project(SplitState* s, int nL, const double* Wt, double* Out, i
 las_status split_project_gemm(SplitState* s, int nL, const double* Wt, int* ks_used,
                               cudaStream_t st);
 void split_project_reduce(SplitState* s, int ks, double* Out, int accumulate, cudaStream_t st);
-// hC = h C_occ, then hmo = C_occ^T hC (split_one_electron = both)
-las_status split_one_electron_hc(SplitState* s, const double* h, double* hC, cudaStream_t st);
-las_status split_one_electron_hmo(SplitState* s, const double* hC, double* hmo,
-                                  cudaStream_t st);
 
 // Grouped launches: while a group is being recorded on the calling host thread, every split
 // product of the functions above is appended to it instead of being launched; ozgroup_launch then
@@ -93,7 +88,7 @@ las_status split_lpu(SplitState* s, int nL, const double* Ht, int c, int a, cons
 // adding its size to *bytes); per chunk: split_tangent_half (dH = b dC_occ), then, after
 // split_full of H, split_tangent_full (X = H^T dC and the digits of dH), and
 // split_tangent_project for each of the two projection terms; split_tangent_one_electron gives
-// h dC_occ (after split_one_electron of the same h).
+// h dC_occ (after split_one_electron_hc of the same h).
 las_status split_tangent_prepare(SplitState* s, const double* dCocc, cudaStream_t st,
                                  size_t* bytes);
 las_status split_tangent_half(SplitState* s, int l0, int nL, double* dHt, cudaStream_t st);
