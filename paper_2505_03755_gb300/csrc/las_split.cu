@@ -67,9 +67,6 @@ struct OzTile {
   static constexpr int STAGE_BYTES = A_BYTES + B_BYTES;
   static constexpr int NSTAGE = (220 * 1024) / STAGE_BYTES < 6 ? (220 * 1024) / STAGE_BYTES : 6;
   static constexpr int SMEM_BYTES = NSTAGE * STAGE_BYTES + 1024 + 256;
-  // epilogue: a tile's bn columns as 8-column blocks dealt round-robin to the 4 column groups
-  // (every TMEM load is 8 columns at an 8-aligned column)
-  static constexpr int MAXB = (BN / 8 + 3) / 4;  // blocks per epilogue thread, at most
   static_assert(STAGE_BYTES % 1024 == 0, "stages stay 1024-byte aligned");
 };
 
@@ -362,6 +359,13 @@ __device__ __forceinline__ void mma_exact(uint32_t tmem, uint32_t sa, uint32_t s
 // the A orientation of the launch's products as a compile-time constant (0: K-major, 1:
 // MN-major), or 2 when each tile reads its product's; the issuing thread runs measurably faster
 // with a constant.
+// f(tile width as a compile-time constant): the launch's fixed width, or the one of this tile.
+template <int FIXBN, class F>
+__device__ __forceinline__ bool with_width(int bn, F f) {
+  if constexpr (FIXBN != 0) return f(std::integral_constant<int, FIXBN>());
+  else return bn == 64 ? f(std::integral_constant<int, 64>()) : f(std::integral_constant<int, 96>());
+}
+
 template <int BN, bool GROUPED, int FIXBN, bool PACK, int AMN = 2>
 __global__ void __launch_bounds__(NTHREADS, 1)
 k_ozaki(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
@@ -370,7 +374,6 @@ k_ozaki(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtenso
         long ntiles) {
   using T = OzTile<BN>;
   constexpr int NSTAGE = T::NSTAGE;
-  constexpr int MAXB = T::MAXB;
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   uint64_t* bars = (uint64_t*)(smem + NSTAGE * T::STAGE_BYTES);
@@ -431,14 +434,14 @@ k_ozaki(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtenso
       cur.seek(t, p1, &tmA, &tmB, &tmA2, &tmA3, probs, nprob);
       const OzParams& p = *cur.P;
       const int nkb = cur.nkb;
-      const int bn = FIXBN ? FIXBN : p.bn;
-      const bool amn_tile = p.a_mn != 0;
+      [[maybe_unused]] const bool amn_tile = p.a_mn != 0;
       // packed-triangle A: K blocks of column blocks J > R (above the diagonal) are read MN-major
       const bool pack = PACK && p.a_pack != 0;
-      const int kb_mn = pack ? 8 * ((cur.m0 / BM) % p.pk_nb1 + 1) : 0;
+      [[maybe_unused]] const int kb_mn = pack ? 8 * ((cur.m0 / BM) % p.pk_nb1 + 1) : 0;
       // Stages [i0, i1) of the tile with one A orientation (a compile-time constant where the
-      // launch fixes it); false when a wait ran out.
-      auto stages = [&](auto amn, int i0, int i1) -> bool {
+      // launch fixes it) and one width; false when a wait ran out.
+      auto stages_of = [&](auto bn_c, auto amn, int i0, int i1) -> bool {
+        constexpr int bn = decltype(bn_c)::value;
         for (int i = i0; i < i1; ++i) {
           if (!sm100::mbar_wait(&full[st], phase, abort_flag, p.status, LAS_ERR_TIMEOUT))
             return false;
@@ -452,13 +455,8 @@ k_ozaki(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtenso
           sm100::tc_fence_after();
           const uint32_t sa = sm100::smem_u32(smem + st * T::STAGE_BYTES);
           const uint32_t sb = sa + A_BYTES;
-          if constexpr (exact) {
-            if (bn == 64) mma_exact<64>(tmem, sa, sb, first, amn);
-            else mma_exact<96>(tmem, sa, sb, first, amn);
-          } else {
-            if (bn == 64) mma_tail<64>(tmem + T::TAIL_COL, sa, sb, first, amn);
-            else mma_tail<96>(tmem + T::TAIL_COL, sa, sb, first, amn);
-          }
+          if constexpr (exact) mma_exact<bn>(tmem, sa, sb, first, amn);
+          else mma_tail<bn>(tmem + T::TAIL_COL, sa, sb, first, amn);
           sm100::mma_commit(&empty[st]);
           if (exact && ((i % CHUNK) == CHUNK - 1 || i == nkb - 1)) sm100::mma_commit(accf);
           if (++st == NSTAGE) {
@@ -467,6 +465,9 @@ k_ozaki(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtenso
           }
         }
         return true;
+      };
+      auto stages = [&](auto amn, int i0, int i1) -> bool {
+        return with_width<FIXBN>(p.bn, [&](auto bn_c) { return stages_of(bn_c, amn, i0, i1); });
       };
       using K_MAJOR = std::integral_constant<bool, false>;
       using MN_MAJOR = std::integral_constant<bool, true>;
@@ -566,11 +567,14 @@ k_ozaki(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtenso
     uint32_t gc = 0, tcount = 0;
     bool ok = true;
     OzCursor<GROUPED> cur;
-    for (long t = blockIdx.x; t < ntiles && ok; t += gridDim.x, ++tcount) {
-      cur.seek(t, p1, &tmA, &tmB, &tmA2, &tmA3, probs, nprob);
+    // One tile of a width: drains, then results; false when a wait ran out.
+    auto finish_tile = [&](auto bn_c) -> bool {
+      constexpr int bn = decltype(bn_c)::value;
+      // the tile's 8-column blocks are dealt round-robin to the 4 column groups (every TMEM load is
+      // 8 columns at an 8-aligned column): at most MAXB per thread
+      constexpr int MAXB = (bn / 8 + 3) / 4;
       const OzParams& p = *cur.P;
       const int m0 = cur.m0, n0 = cur.n0, kb0 = cur.kb0, nkb = cur.nkb;
-      const int bn = FIXBN ? FIXBN : p.bn;
       const int nb = (bn / 8 - cg + 3) / 4;   // this warp's column blocks (warp-uniform)
       const float tscale = __int_as_float((127 + 8 * (NEXACT - 1) + p.sh) << 23);  // 2^(24+sh)
       const int nchunks = (nkb + CHUNK - 1) / CHUNK;
@@ -581,10 +585,8 @@ k_ozaki(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtenso
         const bool fin = (c == nchunks - 1);
         if (!sm100::mbar_wait(accf, gc & 1, abort_flag, p.status, LAS_ERR_TIMEOUT, 256) ||
             (fin && !sm100::mbar_wait(tailf, tcount & 1, abort_flag, p.status, LAS_ERR_TIMEOUT,
-                                      64))) {
-          ok = false;
-          break;
-        }
+                                      64)))
+          return false;
         sm100::tc_fence_after();
         int extra = 0;
         if (fin) {
@@ -633,7 +635,6 @@ k_ozaki(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtenso
         __syncwarp();
         if (lane == 0) sm100::mbar_arrive(acce);   // exact accumulators free from here on
       }
-      if (!ok) break;
       // FP64 results (overlaps the next tile's MMAs)
       const int row = m0 + lq * 32 + lane - p.row_skip;
       bool live = row >= 0 && row < p.M;
@@ -672,6 +673,11 @@ k_ozaki(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtenso
           }
         }
       }
+      return true;
+    };
+    for (long t = blockIdx.x; t < ntiles && ok; t += gridDim.x, ++tcount) {
+      cur.seek(t, p1, &tmA, &tmB, &tmA2, &tmA3, probs, nprob);
+      ok = with_width<FIXBN>(cur.P->bn, finish_tile);
     }
     sm100::tc_fence_before();
   }
@@ -1126,26 +1132,30 @@ static las_status make_plane_map_mn(CUtensorMap* m, const Planes& P) {
 constexpr int OZ_BN = 96;
 static bool valid_bn(int bn) { return bn == 64 || bn == 96; }
 
+// Time of a stage of 96 and of 64 columns (clocks per 16 values of K, 50 to 75 stages a tile): the
+// narrow one pays nearly as much for its A planes, so it wins only where it saves a third of the
+// columns.  op = 128 (800 orbitals): 2 x 64 columns 2400, 96 + 64 2540 and B read twice.
+constexpr int STAGE96 = 1340, STAGE64 = 1200;
+static int pick_bn(long N) {
+  return (N + 63) / 64 * STAGE64 < (N + 95) / 96 * STAGE96 ? 64 : 96;
+}
+
 // The launch attribute is a per-device setting: set once for each device that uses the kernels
 // (a repeated set from two threads is harmless).
 template <bool GROUPED, int FIXBN>
 static cudaError_t ozaki_attr() {
-  cudaError_t e = cudaFuncSetAttribute(k_ozaki<OZ_BN, GROUPED, FIXBN, false>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       OzTile<OZ_BN>::SMEM_BYTES);
-  if (e != cudaSuccess) return e;
-  if constexpr (!GROUPED && FIXBN != 0) {
-    e = cudaFuncSetAttribute(k_ozaki<OZ_BN, GROUPED, FIXBN, false, 0>,
-                             cudaFuncAttributeMaxDynamicSharedMemorySize, OzTile<OZ_BN>::SMEM_BYTES);
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(k_ozaki<OZ_BN, GROUPED, FIXBN, false, 1>,
-                               cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               OzTile<OZ_BN>::SMEM_BYTES);
-    if (e != cudaSuccess) return e;
+  auto set = [](auto kern) {
+    return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                OzTile<OZ_BN>::SMEM_BYTES);
+  };
+  cudaError_t e;
+  if constexpr (GROUPED) {
+    e = set(k_ozaki<OZ_BN, true, FIXBN, false>);
+  } else {
+    e = set(k_ozaki<OZ_BN, false, FIXBN, false, 0>);
+    if (e == cudaSuccess) e = set(k_ozaki<OZ_BN, false, FIXBN, false, 1>);
   }
-  return cudaFuncSetAttribute(k_ozaki<OZ_BN, GROUPED, FIXBN, true>,
-                              cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              OzTile<OZ_BN>::SMEM_BYTES);
+  return e != cudaSuccess ? e : set(k_ozaki<OZ_BN, GROUPED, FIXBN, true>);
 }
 
 // Does the product need the instantiation with the packed-triangle logic (its A is the packed
@@ -1198,13 +1208,13 @@ static long ozaki_tiles(long M, long N, int lower, int bn = OZ_BN) {
 
 // K-split factor in [1, cap] that shares `tiles` output tiles of a product with kb K blocks out
 // most evenly over the persistent CTAs: ceil(tiles*ks / SMs) rounds, each of ceil(kb/ks) blocks
-// plus about two chunks of pipeline fill and drain.
+// plus about a chunk of pipeline fill and drain.
 static int balanced_ksplit(long tiles, long kb, long cap) {
   const long sms = num_sms();
   int best = 1;
   double best_t = 1e300;
   for (long ks = 1; ks <= cap; ++ks) {
-    const double t = (double)((tiles * ks + sms - 1) / sms) * (double)((kb + ks - 1) / ks + 2 * CHUNK);
+    const double t = (double)((tiles * ks + sms - 1) / sms) * (double)((kb + ks - 1) / ks + CHUNK);
     if (t < best_t * (1.0 - 1e-9)) {
       best_t = t;
       best = (int)ks;
@@ -1212,6 +1222,10 @@ static int balanced_ksplit(long tiles, long kb, long cap) {
   }
   return best;
 }
+
+// Shortest K of a split: one chunk.  (At 2048 the projection of the 48-orbital problem, K = 2560,
+// was one tile on one SM: 120 us.)
+constexpr long KSPLIT_MIN = CHUNK * BK;
 
 // Products recorded instead of launched while a group is being recorded on this host thread.
 struct OzGroup {
@@ -1367,8 +1381,9 @@ static las_status ozaki_setup(OzProblem& pr, const Planes& A, long a_row0, const
 las_status ozaki_gemm(const Planes& A, long a_row0, const int* ea, long M, const Planes& B,
                       long b_row0, const int* eb, long N, long K, int ksplit, int mode,
                       double* out, long ldc, long zstride, int ht_n, int ht_op, int* status,
-                      cudaStream_t st, int lower = 0, int bn = OZ_BN, int a_mn = 0) {
+                      cudaStream_t st, int lower = 0, int bn = 0, int a_mn = 0) {
   if (M <= 0 || N <= 0) return LAS_OK;
+  if (bn == 0) bn = lower && N > 64 ? OZ_BN : pick_bn(N);   // 0: the rule's width
   OzProblem pr;
   las_status s = ozaki_setup(pr, A, a_row0, ea, M, B, b_row0, eb, N, K, ksplit, mode, out, ldc,
                              zstride, ht_n, ht_op, status, lower, bn, a_mn);
@@ -1498,7 +1513,8 @@ struct SplitState {
   int* hexp;             // [n]
   int ksplit6;           // partial buffers allocated for this many K splits
   int ks;                // split-K factor of the projection GEMM (autotunable)
-  int bn[SPLIT_NKIND];   // tile width of each product kind (autotunable): 64 or 96
+  int bn[SPLIT_NKIND];   // tile width of each product kind: 64 or 96
+  int bn_set[SPLIT_NKIND];   // the width was chosen by the caller or the autotuner
   // tangent (Hessian-vector) scratch, allocated by the first split_tangent_prepare: digit planes
   // of dC_occ^T (rows p, K = nu) and of the chunk's dH (rows (L, p), K = mu)
   Planes dCdig;
@@ -1537,15 +1553,15 @@ las_status split_create(SplitState** out, int n, int X, int op, int Lc, const do
   s->Lc = Lc;
   s->status = status;
   s->ksplit6 = 64;
-  for (int k = 0; k < SPLIT_NKIND; ++k) s->bn[k] = OZ_BN;
+  for (int k = 0; k < SPLIT_NKIND; ++k) s->bn[k] = pick_bn(op);
+  s->bn[SPLIT_ONE_ELECTRON] = 64;   // fewer tiles than SMs: the shorter tile ends first
   // one-time launch attributes, so that later calls can be captured into CUDA graphs
   if (ozaki_prepare() != LAS_OK || num_sms() <= 0) {
     free(s);
     return LAS_ERR_CUDA;
   }
   // projection split-K (autotunable): output n x op, K = the (L, p) rows of one chunk
-  s->ks = balanced_ksplit(ozaki_tiles(n, op, 0), ((long)Lc * op + BK - 1) / BK,
-                          std::min<long>(s->ksplit6, std::max(1L, ((long)Lc * op) / 2048)));
+  s->ks = split_balanced_ksplit(s, Lc);
   size_t total = 0;
   las_status rc = LAS_OK;
   auto A = [&](void** p, size_t b) {
@@ -1658,12 +1674,21 @@ int split_get_ksplit(SplitState* s) { return s->ks; }
 int split_balanced_ksplit(SplitState* s, int nL) {
   return balanced_ksplit(ozaki_tiles(s->n, s->op, 0, s->bn[SPLIT_PROJECT]),
                          ((long)nL * s->op + BK - 1) / BK,
-                         std::min<long>(s->ksplit6, std::max(1L, ((long)nL * s->op) / 2048)));
+                         std::min<long>(s->ksplit6, std::max(1L, ((long)nL * s->op) / KSPLIT_MIN)));
+}
+// K splits of a projection over R rows (L, p): at most s->ks of at least KSPLIT_MIN each, counted
+// as ozaki_setup forms them (equal numbers of K blocks, none empty), so that every partial summed
+// afterwards has been written.
+static int project_ksplit(const SplitState* s, long R) {
+  const long kb = (R + BK - 1) / BK, ks = std::max(1L, std::min((long)s->ks, R / KSPLIT_MIN));
+  const long per = (kb + ks - 1) / ks;
+  return (int)((kb + per - 1) / per);
 }
 int split_get_tile(SplitState* s, int kind) { return s->bn[kind]; }
 las_status split_set_tile(SplitState* s, int kind, int bn) {
   if (kind < 0 || kind >= SPLIT_NKIND || !valid_bn(bn)) return LAS_ERR_ARG;
   s->bn[kind] = bn;
+  s->bn_set[kind] = 1;
   return LAS_OK;
 }
 void split_set_ksplit(SplitState* s, int ks) { s->ks = std::max(1, std::min(ks, s->ksplit6)); }
@@ -1679,6 +1704,30 @@ static las_status b_half(const SplitState* s, int l0, int nL, const Planes& Xd, 
   return ozaki_gemm(s->Bdig, (long)l0 * s->n, s->Bexp + (long)l0 * s->n, (long)nL * s->n, Xd,
                     x_row0, xexp, N, s->n, 1, 1, out, 0, 0, s->n, ht_op, s->status, st, 0, bn);
 }
+
+// The same with the widths of its column tiles chosen here.  In 96-column tiles, the columns beyond
+// the last whole tile may number at most 64 (the JK call's 150 core columns: 96 + 54): they then
+// form a second product of 64-column tiles, 160 columns computed instead of 192.  Not while
+// products are recorded for a grouped launch, which would then mix tile widths.  bn: 0 = by stage
+// times (pick_bn), or the width asked for.
+static las_status b_half_cols(const SplitState* s, int l0, int nL, const Planes& Xd,
+                              const int* xexp, long N, double* out, int ht_op, cudaStream_t st,
+                              int bn) {
+  const long whole = N / 96 * 96, rest = N - whole;
+  const bool ends = whole > 0 && rest > 0 && rest <= 64 && !g_record;   // 96s and one 64
+  if (bn == 0) {
+    bn = pick_bn(N);
+    if (ends && bn == 64 && whole / 96 * STAGE96 + STAGE64 < (N + 63) / 64 * STAGE64) bn = 96;
+  }
+  if (bn == 96 && ends) {
+    las_status rc = b_half(s, l0, nL, Xd, 0, xexp, whole, out, ht_op, st, 96);
+    if (rc != LAS_OK) return rc;
+    return b_half(s, l0, nL, Xd, whole, xexp + whole, rest, out + whole * s->n, ht_op, st, 64);
+  }
+  return b_half(s, l0, nL, Xd, 0, xexp, N, out, ht_op, st, bn);
+}
+
+static int half_bn(const SplitState* s) { return s->bn_set[SPLIT_HALF] ? s->bn[SPLIT_HALF] : 0; }
 
 las_status split_prepare_C(SplitState* s, const double* Cocc, cudaStream_t st) {
   // rows p of C_occ^T (K = nu): element (p, nu) = Cocc[nu*op + p]
@@ -1720,7 +1769,7 @@ las_status split_tangent_prepare(SplitState* s, const double* dCocc, cudaStream_
 
 // dH = b^L dC_occ for the chunk's aux rows (Ht layout [nL][op][n])
 las_status split_tangent_half(SplitState* s, int l0, int nL, double* dHt, cudaStream_t st) {
-  return b_half(s, l0, nL, s->dCdig, 0, s->dCexp, s->op, dHt, s->op, st, s->bn[SPLIT_HALF]);
+  return b_half_cols(s, l0, nL, s->dCdig, s->dCexp, s->op, dHt, s->op, st, half_bn(s));
 }
 
 // After split_full of the chunk: X[(L,p)][q] = sum_mu H_L(mu,p) dC(mu,q) (so that dT_L = X_L +
@@ -1752,7 +1801,7 @@ las_status split_tangent_project(SplitState* s, int nL, int which, const double*
   W.K = R;
   las_status rc = slice_rows(RowsStrided{Wt, R, 1, nullptr}, W, s->Wexp, st, s->mx, true);
   if (rc != LAS_OK) return rc;
-  const int ks = (int)std::max(1L, std::min((long)s->ks, (R + 32 * 64 - 1) / (32 * 64)));
+  const int ks = project_ksplit(s, R);
   rc = ozaki_gemm(which ? s->dHdig : s->Hdig, 0, nullptr, s->n, W, 0, s->Wexp, s->op, R, ks, 0,
                   s->part, s->op, (long)s->n * s->op, 0, 0, s->status, st, 0,
                   s->bn[SPLIT_PROJECT], 1);
@@ -1804,22 +1853,9 @@ las_status split_lpu(SplitState* s, int nL, const double* Ht, int c, int a, cons
   return rc;
 }
 
-// When the half transform runs in 96-column tiles and the columns beyond the last whole tile
-// number at most 64 (the JK call's 150 core columns: 96 + 54), those columns form a second product
-// of 64-column tiles: 160 columns computed instead of 192, and a 64-column stage costs about three
-// quarters of a 96-column one.  Not while products are recorded for a grouped launch, which would
-// then mix tile widths.
 las_status split_half(SplitState* s, int l0, int nL, int oc, double* Ht, cudaStream_t st) {
   if (oc < 1 || oc > s->op) return LAS_ERR_INTERNAL;
-  const int bn = s->bn[SPLIT_HALF];
-  const int whole = oc / 96 * 96, rest = oc - whole;
-  if (bn == 96 && whole > 0 && rest > 0 && rest <= 64 && !g_record) {
-    las_status rc = b_half(s, l0, nL, s->Cdig, 0, s->Cexp, whole, Ht, oc, st, 96);
-    if (rc != LAS_OK) return rc;
-    return b_half(s, l0, nL, s->Cdig, whole, s->Cexp + whole, rest, Ht + (size_t)whole * s->n,
-                  oc, st, 64);
-  }
-  return b_half(s, l0, nL, s->Cdig, 0, s->Cexp, oc, Ht, oc, st, bn);
+  return b_half_cols(s, l0, nL, s->Cdig, s->Cexp, oc, Ht, oc, st, half_bn(s));
 }
 
 las_status split_full(SplitState* s, int nL, const double* Ht, double* T, cudaStream_t st) {
@@ -1848,7 +1884,7 @@ las_status split_project_gemm(SplitState* s, int nL, const double* Wt, int* ks_u
   RowsStrided acc{Wt, R, 1, nullptr};
   las_status rc = slice_rows(acc, W, s->Wexp, st, s->mx, true);
   if (rc != LAS_OK) return rc;
-  const int ks = (int)std::max(1L, std::min((long)s->ks, (R + 32 * 64 - 1) / (32 * 64)));
+  const int ks = project_ksplit(s, R);
   *ks_used = ks;
   return ozaki_gemm(s->Hdig, 0, nullptr, s->n, W, 0, s->Wexp, s->op, R, ks, 0, s->part, s->op,
                     (long)s->n * s->op, 0, 0, s->status, st, 0, s->bn[SPLIT_PROJECT], 1);
@@ -1896,7 +1932,7 @@ las_status split_exchange(SplitState* s, int nL, int oc, const double* Ht, doubl
     }
   }
   // partials [ks][n][n] live in the projection's partial buffer (64 * n * op doubles)
-  const long cap = std::max(1L, std::min((64L * s->op) / n, (R + 32 * 64 - 1) / (32 * 64)));
+  const long cap = std::max(1L, std::min((64L * s->op) / n, R / KSPLIT_MIN));
   const int ks = balanced_ksplit(ozaki_tiles(n, n, 1), (R + BK - 1) / BK, cap);
   // symmetric product: only tiles touching the lower triangle; the caller mirrors the result
   rc = ozaki_gemm(HT, 0, s->hexp, n, HT, 0, s->hexp, n, R, ks, 0, s->part, n, n * n, 0, 0,
@@ -2077,7 +2113,7 @@ las_status frag_split_chunk(SplitState* s, FragSplit* f, int l0, int nL, double*
   const long n2 = (long)nmo * nmo, R1 = (long)nL * nmo;
   if (nL < 1 || nL > f->Lc || ma > f->ma) return LAS_ERR_INTERNAL;
   // Eq. ao2mo_1: H[L][p][e2] = sum_e1 b^L(e2, e1) M[e1][p]
-  las_status rc = b_half(s, l0, nL, f->Mdig, 0, f->Mexp, nmo, H, nmo, st, OZ_BN);
+  las_status rc = b_half_cols(s, l0, nL, f->Mdig, f->Mexp, nmo, H, nmo, st, 0);
   // Eq. ao2mo_2: T[L][p][q] = sum_e H[L][p][e] M[e][q]
   Planes Hd = f->Hd;
   Hd.R = R1;
