@@ -691,30 +691,33 @@ k_ozaki(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtenso
 // ------------------------------------------------------------------------------------------
 // Digit extraction (integer operations on the FP64 bit patterns)
 // ------------------------------------------------------------------------------------------
-struct RowsStrided {  // element (r, k) = base[r*sr + k*sk] * 2^(gexp ? gexp[k] : 0)
+struct RowsStrided {  // element (r, k) = base[r*sr + k*sk]
   const double* base;
   long sr, sk;
-  const int* gk;
   __device__ __forceinline__ double operator()(long r, long k) const {
-    double x = base[r * sr + k * sk];
-    if (gk) {
-      long long b = __double_as_longlong(x);
-      if ((b & 0x7FF0000000000000ll) != 0) b += ((long long)gk[k]) << 52;
-      else if (x != 0.0) return ldexp(x, gk[k]);
-      x = __longlong_as_double(b);
-    }
-    return x;
+    return base[r * sr + k * sk];
   }
+};
+
+// Rows that are contiguous in K: row r starts at base + r*sr.
+struct RowsContig {
+  const double* base;
+  long sr;
+  __host__ __device__ __forceinline__ const double* row(long r) const { return base + r * sr; }
+  bool aligned() const { return ((uintptr_t)base & 15) == 0 && (sr & 1) == 0; }
+  __device__ __forceinline__ double operator()(long r, long k) const { return row(r)[k]; }
 };
 
 // Row (L, u) of the active columns of the half transform, K = mu: Ht[(L op + c + u) n + mu]
 struct RowsHtAct {
   const double* Ht;
   int n, op, c, a;
-  __device__ __forceinline__ double operator()(long r, long k) const {
+  __host__ __device__ __forceinline__ const double* row(long r) const {
     const long L = r / a, u = r - L * a;
-    return Ht[(L * op + c + u) * n + k];
+    return Ht + (L * op + c + u) * n;
   }
+  bool aligned() const { return ((uintptr_t)Ht & 15) == 0 && (n & 1) == 0; }
+  __device__ __forceinline__ double operator()(long r, long k) const { return row(r)[k]; }
 };
 
 struct RowsPacked {   // element (r = L*n + mu, k = nu) of the packed symmetric b^L
@@ -728,50 +731,58 @@ struct RowsPacked {   // element (r = L*n + mu, k = nu) of the packed symmetric 
   }
 };
 
-// Six balanced base-256 digits of x * 2^-e rounded at 2^-47 (|x| < 2^e), returned as the BF16
-// plane values d_s * 2^-8s.  Integer operations on the bit pattern only.
-__device__ __forceinline__ void digits_of(double xv, int e, __nv_bfloat16 (&out)[NDIG]) {
-  const unsigned long long b = (unsigned long long)__double_as_longlong(xv);
-  const int bex = (int)((b >> 52) & 0x7FF);
-  unsigned long long m = b & 0xFFFFFFFFFFFFFull;
-  int ee = bex;
-  if (bex != 0) m |= (1ull << 52); else ee = 1;
-  // |x| * 2^(47 - e) = m * 2^(ee - 1075 + 47 - e), rounded to an integer below 2^47
-  const int shift = ee - 1028 - e;
-  unsigned long long y;
-  if (shift >= 0) y = m << shift;
-  else if (shift > -63) y = (m + (1ull << (-shift - 1))) >> (-shift);
-  else y = 0;
-  // balanced base-256 digits from the bottom, in 32-bit arithmetic on two 24-bit halves
-  int lo = (int)(y & 0xFFFFFF), hi = (int)(y >> 24);
-  if (b >> 63) {
-    lo = -lo;
-    hi = -hi;
-  }
-  int d[NDIG];
+// Six balanced base-256 digits of x * 2^-e rounded at 2^-47 (|x| < 2^e), returned as the floats
+// d_s * 2^-8s (exact in BF16: the upper halves of their bit patterns).  About 35 integer and FP32
+// instructions; a recurrence digit by digit with conversions took 100, and the slicers were bound
+// by them (3.3 to 4.4 ps per value over the chip).  With y = x 2^(47-e) rounded to an integer,
+// half a unit of every digit is added at once, Y = y + sum_k 128 * 256^k, so that the bytes of Y are
+// d_s + 128; a byte put under the exponent of 2^(23-8s) is the float 2^(23-8s) + (d_s + 128) 2^-8s.
+__device__ __forceinline__ void digits_of(double xv, int e, uint32_t (&f)[NDIG]) {
+  const uint32_t hi = (uint32_t)__double2hiint(xv), lo = (uint32_t)__double2loint(xv);
+  int ee = (int)(hi >> 20) & 0x7FF;
+  const uint32_t mh = (hi & 0xFFFFF) | (ee != 0 ? 0x100000u : 0u);
+  ee = max(ee, 1);
+  // |x| 2^(47-e) = m 2^(ee-1028-e); |x| < 2^e, so the shift is to the right.  Half up: shift by
+  // one less, add 1, halve.
+  const int sh = min(1027 + e - ee, 63);
+  const unsigned long long m = ((unsigned long long)mh << 32) | lo;
+  const unsigned long long y = ((m >> sh) + 1) >> 1;
+  const unsigned long long Y = ((int)hi < 0 ? 0ull - y : y) + 0x808080808080ull;
+  const uint32_t yl = (uint32_t)Y, yh = (uint32_t)(Y >> 32);
+  auto digit = [](uint32_t biased, int s) {   // bits of 2^(23-8s) + (d + 128) 2^-8s -> d 2^-8s
+    const float w = __int_as_float((127 - 8 * s) << 23);
+    return __float_as_uint(__uint_as_float(biased) - (8388608.0f + 128.0f) * w);
+  };
+  auto under = [](uint32_t word, int byte, int s) {
+    return __byte_perm(word, (uint32_t)(150 - 8 * s) << 23, 0x7540 | byte);
+  };
+  f[0] = digit(0x4B000000u | (yh >> 8), 0);   // d_0 + 128 in 0..256
+  f[1] = digit(under(yh, 0, 1), 1);
+  f[2] = digit(under(yl, 3, 2), 2);
+  f[3] = digit(under(yl, 2, 3), 3);
+  f[4] = digit(under(yl, 1, 4), 4);
+  f[5] = digit(under(yl, 0, 5), 5);
+}
+__device__ __forceinline__ __nv_bfloat16 digit_bf16(uint32_t f) {
+  return __ushort_as_bfloat16((unsigned short)(f >> 16));
+}
+
+// Digits of 8 values of one row (k0 a multiple of 8), one 16-byte store per plane.
+__device__ __forceinline__ void store_digits8(const Planes& P, long r, long k0,
+                                              const double (&x)[8], int e) {
+  uint32_t w[NDIG][4];
 #pragma unroll
-  for (int s = NDIG - 1; s >= 3; --s) {
-    const int t = ((lo + 128) & 255) - 128;
-    d[s] = t;
-    lo = (lo - t) >> 8;
-  }
-  hi += lo;   // carry out of the low half (-1, 0 or 1)
+  for (int j = 0; j < 4; ++j) {
+    uint32_t a[NDIG], b[NDIG];
+    digits_of(x[2 * j], e, a);
+    digits_of(x[2 * j + 1], e, b);
 #pragma unroll
-  for (int s = 2; s >= 1; --s) {
-    const int t = ((hi + 128) & 255) - 128;
-    d[s] = t;
-    hi = (hi - t) >> 8;
+    for (int s = 0; s < NDIG; ++s) w[s][j] = __byte_perm(a[s], b[s], 0x7632);   // upper halves
   }
-  d[0] = hi;
-  // d_s * 2^-8s as BF16 without conversion instructions: the float of d_s from the bit pattern
-  // of 1.5*2^23 + d_s (exact for |d_s| < 2^22), scaled by a power of two, and its upper half
-  // (exact: at most 8 significant bits)
+  __nv_bfloat16* p = P.p + P.idx(0, r, k0);
 #pragma unroll
-  for (int s = 0; s < NDIG; ++s) {
-    const float f = (__int_as_float(0x4B400000 + d[s]) - 12582912.0f) *
-                    __int_as_float((127 - 8 * s) << 23);
-    out[s] = __ushort_as_bfloat16((unsigned short)(__float_as_uint(f) >> 16));
-  }
+  for (int s = 0; s < NDIG; ++s)
+    *(uint4*)(p + s * P.plane) = make_uint4(w[s][0], w[s][1], w[s][2], w[s][3]);
 }
 
 __device__ __forceinline__ int exp_of_maxbits(unsigned long long mx) {
@@ -782,8 +793,129 @@ __device__ __forceinline__ unsigned long long absbits(double x) {
   return (unsigned long long)__double_as_longlong(x) & 0x7FFFFFFFFFFFFFFFull;
 }
 
-// Short rows: one warp per row r < rows (rows >= R are written as zeros); exponent e_r with
-// max|x| < 2^e_r for r < R, digit planes for every k < kb*BK (zero beyond K).
+// Rows contiguous in K, read once: rb rows (a power of two) go through shared memory (row stride S
+// doubles), their maxima taken on the way in, and are cut from there, 8 values and one 16-byte
+// store per plane at a time.  Rows >= R are written as zeros, and every k in [K, kb*BK).  The bytes
+// are the bound: 8 read and 12 written per value; reading the row a second time from memory took
+// 28 (2.34 ms for 2400 x 192 rows of 1200 against SLICE_NOW).  Few rows per block leave room for
+// five or more blocks per SM, whose loads and stores overlap.  S = 2 modulo 16: the 16-byte reads of
+// 8 neighbouring threads (rows, or 4 rows and two halves) fall into different banks.
+template <class Rows>
+__global__ void __launch_bounds__(256)
+k_slice_kmajor(Rows src, int vec, Planes P, long rows, long kb, int lg, int S, int* ex) {
+  extern __shared__ __align__(16) double rowbuf[];
+  __shared__ unsigned long long mxs[32];
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int rb = 1 << lg;
+  const long r0 = (long)blockIdx.x << lg;
+  const int n = (int)P.K, kend = (int)(kb * BK);
+  if (tid < rb) mxs[tid] = 0;
+  __syncthreads();
+  const int parts = rb < 8 ? 8 >> lg : 1, seg = ((kend + parts - 1) / parts + 63) / 64 * 64;
+  for (int i = warp; i < rb * parts; i += 8) {
+    const int row = i & (rb - 1), k0 = (i >> lg) * seg, k1 = min(kend, k0 + seg);
+    const long r = r0 + row;
+    const bool live = r < P.R;
+    const double* p = live ? src.row(r) : nullptr;
+    double* q = rowbuf + row * S;
+    unsigned long long m = 0;
+    auto take = [&](int k, double2 v) {
+      *(double2*)(q + k) = v;
+      const unsigned long long a = absbits(v.x), b = absbits(v.y), c = a > b ? a : b;
+      m = c > m ? c : m;
+    };
+    int k = k0 + 2 * lane;
+    const int kv = live && vec ? min(k1, n & ~1) : k0;
+#pragma unroll 5
+    for (; k < kv; k += 64) take(k, __ldg((const double2*)(p + k)));
+    for (; k < k1; k += 64)
+      take(k, make_double2(live && k < n ? p[k] : 0.0, live && k + 1 < n ? p[k + 1] : 0.0));
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      const unsigned long long v = __shfl_xor_sync(0xffffffffu, m, o);
+      m = v > m ? v : m;
+    }
+    if (lane == 0) atomicMax(&mxs[row], m);
+  }
+  __syncthreads();
+  if (tid < rb && r0 + tid < P.R) ex[r0 + tid] = exp_of_maxbits(mxs[tid]);
+  const int row = tid & (rb - 1);
+  const long r = r0 + row;
+  if (r >= rows) return;
+  const int e = exp_of_maxbits(mxs[row]);
+  const double* q = rowbuf + row * S;
+  for (int k = (tid >> lg) * 8; k < kend; k += (256 >> lg) * 8) {
+    double x[8];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const double2 t = *(const double2*)(q + k + 2 * j);
+      x[2 * j] = t.x;
+      x[2 * j + 1] = t.y;
+    }
+    store_digits8(P, r, k, x, e);
+  }
+}
+
+// Sources read along the rows r (neighbouring r are neighbours in memory, or nearly), 16 rows per
+// block over all of K: maxima first, then a warp cuts 16 rows x 16 values of K per step, whose
+// stores are 512 contiguous bytes per plane.  For products small enough to stay in L2 between the
+// two passes.  Rows >= R are written as zeros.
+template <class Acc>
+__global__ void __launch_bounds__(512)
+k_slice_cols(Acc acc, Planes P, long rows, long kb, int* ex) {
+  __shared__ unsigned long long red[16][16];
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, rl = lane & 15;
+  const long r = blockIdx.x * 16L + rl;
+  const bool live = r < P.R;
+  unsigned long long m = 0;
+  if (live) {
+#pragma unroll 4
+    for (long k = tid >> 4; k < P.K; k += 32) {
+      const unsigned long long b = absbits(acc(r, k));
+      m = b > m ? b : m;
+    }
+  }
+  const unsigned long long o = __shfl_xor_sync(0xffffffffu, m, 16);
+  m = o > m ? o : m;
+  if (lane < 16) red[warp][rl] = m;
+  __syncthreads();
+  for (int w = 0; w < 16; ++w) m = red[w][rl] > m ? red[w][rl] : m;
+  const int e = exp_of_maxbits(m);
+  if (tid < 16 && live) ex[r] = e;
+  if (r >= rows) return;
+  for (long b = warp; b < kb; b += 16) {
+    const long k0 = b * BK + (lane >> 4) * 8;
+    double x[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) x[j] = (live && k0 + j < P.K) ? acc(r, k0 + j) : 0.0;
+    store_digits8(P, r, k0, x, e);
+  }
+}
+
+// The second pass of such sources with the maxima given (mx): one warp per 16 rows x 16 values of
+// K, live rows only.
+template <class Acc>
+__global__ void __launch_bounds__(256)
+k_digits_cols(Acc acc, Planes P, long kb, const unsigned long long* __restrict__ mx, int* ex) {
+  const long groups = (P.R + 15) / 16;
+  const long w = blockIdx.x * 8L + (threadIdx.x >> 5);
+  if (w >= groups * kb) return;
+  const long b = w / groups;
+  const int lane = threadIdx.x & 31;
+  const long r = (w - b * groups) * 16 + (lane & 15);
+  if (r >= P.R) return;
+  const int e = exp_of_maxbits(mx[r]);
+  const long k0 = b * BK + (lane >> 4) * 8;
+  if (k0 == 0) ex[r] = e;
+  double x[8];
+#pragma unroll
+  for (int j = 0; j < 8; ++j) x[j] = k0 + j < P.K ? acc(r, k0 + j) : 0.0;
+  store_digits8(P, r, k0, x, e);
+}
+
+// Rows too long for k_slice_kmajor, and sources contiguous in neither index: one warp per row
+// r < rows (rows >= R are written as zeros); exponent e_r with max|x| < 2^e_r for r < R, digit
+// planes for every k < kb*BK (zero beyond K).
 template <class Acc>
 __global__ void __launch_bounds__(256)
 k_slice_rows(Acc acc, Planes P, long rows, long kb, int* ex) {
@@ -806,10 +938,10 @@ k_slice_rows(Acc acc, Planes P, long rows, long kb, int* ex) {
   if (lane == 0 && live) ex[r] = e;
   const long kend = kb * BK;
   for (long k = lane; k < kend; k += 32) {
-    __nv_bfloat16 d[NDIG];
+    uint32_t d[NDIG];
     digits_of((live && k < P.K) ? acc(r, k) : 0.0, e, d);
 #pragma unroll
-    for (int s = 0; s < NDIG; ++s) P.p[P.idx(s, r, k)] = d[s];
+    for (int s = 0; s < NDIG; ++s) P.p[P.idx(s, r, k)] = digit_bf16(d[s]);
   }
 }
 
@@ -838,23 +970,22 @@ k_rowmax_long(Acc acc, long K, long seg, unsigned long long* mx) {
   }
 }
 
-// Long rows, pass 2: element-parallel digits over rows x kb*BK (zeros outside R x K).
+// Long rows, pass 2: 8 values per thread over rows x kb*BK (zeros outside R x K); the source is
+// contiguous in K.  Neighbouring threads write neighbouring 16 bytes of a K block.
 template <class Acc>
 __global__ void __launch_bounds__(256)
 k_digits_long(Acc acc, Planes P, long rows, long kbc, const unsigned long long* mx, int* ex) {
-  const long kend = kbc * BK;
   const long i = blockIdx.x * (long)blockDim.x + threadIdx.x;
-  if (i >= rows * kend) return;
-  // thread order follows the K-blocked output: (k block, row, k within the block)
-  const long kb = i / (rows * BK), rem = i - kb * (rows * BK);
-  const long r = rem / BK, k = kb * BK + (rem - r * BK);
+  if (i >= rows * kbc * 2) return;
+  const long kb = i / (rows * 2), rem = i - kb * (rows * 2);
+  const long r = rem >> 1, k0 = kb * BK + (rem & 1) * 8;
   const bool live = r < P.R;
   const int e = live ? exp_of_maxbits(mx[r]) : 0;
-  if (k == 0 && live) ex[r] = e;
-  __nv_bfloat16 d[NDIG];
-  digits_of((live && k < P.K) ? acc(r, k) : 0.0, e, d);
+  if (k0 == 0 && live) ex[r] = e;
+  double x[8];
 #pragma unroll
-  for (int s = 0; s < NDIG; ++s) P.p[P.idx(s, r, k)] = d[s];
+  for (int j = 0; j < 8; ++j) x[j] = (live && k0 + j < P.K) ? acc(r, k0 + j) : 0.0;
+  store_digits8(P, r, k0, x, e);
 }
 
 // Packed-triangle digit planes of B (see BPacked).  Pass 1: max |b^L| over the packed triangle
@@ -901,11 +1032,11 @@ k_bpacked_tiles(const double* __restrict__ Bp, long npair, int T, const int* __r
   const int J = t - I * (I + 1) / 2;
   const long mu = 128L * I + row, nu = 128L * J + 16 * kk + c;
   const long hi = mu > nu ? mu : nu, lo = mu > nu ? nu : mu;
-  __nv_bfloat16 d[NDIG];
+  uint32_t d[NDIG];
   digits_of(Bp[L * npair + hi * (hi + 1) / 2 + lo], ex[L], d);
   const long o = (tt * 8 + kk) * (128L * BK) + Planes::swz(row, c);
 #pragma unroll
-  for (int s = 0; s < NDIG; ++s) P.p[s * P.plane + o] = d[s];
+  for (int s = 0; s < NDIG; ++s) P.p[s * P.plane + o] = digit_bf16(d[s]);
 }
 
 // Pass 3: the ragged rows mu = n1 + j (rows (L, j), j < rp, of all X rp, zeros for j >= r; then
@@ -929,79 +1060,10 @@ k_bpacked_ragged(const double* __restrict__ Bp, long npair, int n, int n1, int r
       x = Bp[L * npair + hi * (hi + 1) / 2 + lo];
     }
   }
-  __nv_bfloat16 d[NDIG];
+  uint32_t d[NDIG];
   digits_of(x, e, d);
 #pragma unroll
-  for (int s = 0; s < NDIG; ++s) P.p[P.idx(s, row, k)] = d[s];
-}
-
-// Half-transformed rows (L,p) of Ht [R][n]: exponents and digit planes Hd (rows (L,p),
-// K = mu); the full transform reads them K-major and the projection MN-major (rows mu, K =
-// (L,p)), so one layout serves both.  Block: 16 rows r, 256 threads.  The row maxima are read
-// first (warp per row); the digit pass then re-reads the block's rows: thread (r, c) cuts 8
-// consecutive columns of row r per 128-column step (a warp's 16-byte stores into Hd cover 512
-// contiguous bytes).  Rows of Hd beyond R and columns k >= n are written as zero digits within the
-// block's K range; rows beyond the blocks stay zero from set-up.
-__global__ void __launch_bounds__(256)
-k_slice_ht(const double* __restrict__ Ht, long R, int n, Planes Hd, int* __restrict__ ex) {
-  __shared__ int es[16];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const long r0 = (long)blockIdx.x * 16;
-  for (int i = 0; i < 2; ++i) {
-    const int row = warp * 2 + i;
-    const long r = r0 + row;
-    unsigned long long mx = 0;
-    if (r < R)
-      for (int k = lane; k < n; k += 32) {
-        const unsigned long long b = absbits(Ht[r * n + k]);
-        mx = b > mx ? b : mx;
-      }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      const unsigned long long v = __shfl_xor_sync(0xffffffffu, mx, o);
-      mx = v > mx ? v : mx;
-    }
-    if (lane == 0) {
-      es[row] = exp_of_maxbits(mx);
-      if (r < R) ex[r] = es[row];
-    }
-  }
-  __syncthreads();
-  const long kend = Hd.nkb * BK;            // a multiple of 16
-  const int rr = threadIdx.x & 15, kc = threadIdx.x >> 4;   // digit pass: row, 8-column group
-  const long r = r0 + rr;
-  if (r >= Hd.Rpad) return;
-  const bool live = r < R;
-  const int e = es[rr];
-  const double* hrow = Ht + r * n;
-  for (long k0 = 0; k0 < kend; k0 += 128) {
-    const long k = k0 + kc * 8;
-    if (k >= kend) break;
-    double x[8];
-    if (live && (n & 1) == 0 && k + 8 <= n) {
-      // 16-byte loads (rows start 16-byte aligned when n is even)
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const double2 t = *(const double2*)(hrow + k + 2 * j);
-        x[2 * j] = t.x;
-        x[2 * j + 1] = t.y;
-      }
-    } else {
-#pragma unroll
-      for (int j = 0; j < 8; ++j) x[j] = (live && k + j < n) ? hrow[k + j] : 0.0;
-    }
-    __nv_bfloat16 d[8][NDIG];
-#pragma unroll
-    for (int j = 0; j < 8; ++j) digits_of(x[j], e, d[j]);
-#pragma unroll
-    for (int s = 0; s < NDIG; ++s) {
-      uint4 v;
-      __nv_bfloat16* pv = (__nv_bfloat16*)&v;
-#pragma unroll
-      for (int j = 0; j < 8; ++j) pv[j] = d[j][s];
-      *(uint4*)(Hd.p + Hd.idx(s, r, k)) = v;
-    }
-  }
+  for (int s = 0; s < NDIG; ++s) P.p[P.idx(s, row, k)] = digit_bf16(d[s]);
 }
 
 // Column maxima of Ht [R][n] over its rows (coalesced along the columns): mx[mu] (atomic max of
@@ -1017,44 +1079,6 @@ k_colmax(const double* __restrict__ Ht, long R, int n, long seg, unsigned long l
     m = b > m ? b : m;
   }
   if (m) atomicMax(&mx[mu], m);
-}
-
-// Digits of H^T scaled per row mu (exponents from the column maxima): HdT[s](mu, k) for the
-// rows k = (L,p) of Ht, transposed through shared memory.  Block: 32 rows k x the columns
-// [blockIdx.y*COLS_PER_BLOCK, ...) of mu.
-constexpr int COLS_PER_BLOCK = 2048;
-__global__ void __launch_bounds__(256)
-k_slice_ht_cols(const double* __restrict__ Ht, long R, int n, const unsigned long long* mx,
-                Planes HdT, int* __restrict__ ex) {
-  __shared__ __nv_bfloat16 tile[NDIG][32][34];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const long r0 = (long)blockIdx.x * 32;
-  const int c0 = blockIdx.y * COLS_PER_BLOCK, c1 = min(n, c0 + COLS_PER_BLOCK);
-  if (blockIdx.x == 0)
-    for (int mu = c0 + threadIdx.x; mu < c1; mu += 256) ex[mu] = exp_of_maxbits(mx[mu]);
-  for (int k0 = c0; k0 < c1; k0 += 32) {
-    const int mu = k0 + lane;
-    const int e = mu < c1 ? exp_of_maxbits(mx[mu]) : 0;
-    for (int i = 0; i < 4; ++i) {
-      const int row = warp + 8 * i;
-      const long r = r0 + row;
-      __nv_bfloat16 d[NDIG];
-      digits_of((r < R && mu < c1) ? Ht[r * n + mu] : 0.0, e, d);
-#pragma unroll
-      for (int s = 0; s < NDIG; ++s) tile[s][row][lane] = d[s];
-    }
-    __syncthreads();
-    for (int i = 0; i < 4; ++i) {
-      const int kk = warp * 4 + i;
-      const int m2 = k0 + kk;
-      const long r = r0 + lane;
-      if (m2 < c1 && r < HdT.nkb * BK) {
-#pragma unroll
-        for (int s = 0; s < NDIG; ++s) HdT.p[HdT.idx(s, m2, r)] = tile[s][lane][kk];
-      }
-    }
-    __syncthreads();
-  }
 }
 
 }  // namespace lasdf_split
@@ -1455,40 +1479,91 @@ static las_status bpacked_half(const BPacked& b, int l0, int nL, const Planes& X
   return rc;
 }
 
-// live_only: only rows < R and the K blocks that hold K are written (planes whose padding rows
-// were zeroed at set-up); otherwise every padded row and K block of the layout is written.
-template <class Acc>
-static las_status slice_rows(Acc acc, const Planes& P, int* ex, cudaStream_t st,
-                             unsigned long long* mx_ws = nullptr, bool live_only = false) {
-  if (P.R <= 0) return LAS_OK;
-  const long rows = live_only ? P.R : P.Rpad;
-  const long kbc = live_only ? std::min(P.nkb, planes_nkb(P.K)) : P.nkb;
-  if (P.K > 8192 && mx_ws && P.R <= 65535) {
-    // long rows: block-parallel maxima, then element-parallel digits
-    cudaError_t e0 = cudaMemsetAsync(mx_ws, 0, P.R * sizeof(unsigned long long), st);
-    if (e0 != cudaSuccess) {
-      las_record_cuda_error(e0, "cudaMemsetAsync(rowmax)", __FILE__, __LINE__);
-      return LAS_ERR_CUDA;
-    }
-    const long seg = 8192;
-    dim3 g1((unsigned)((P.K + seg - 1) / seg), (unsigned)P.R);
-    k_rowmax_long<Acc><<<g1, 256, 0, st>>>(acc, P.K, seg, mx_ws);
-    las_count_launch();
-    const long tot = rows * kbc * BK;
-    k_digits_long<Acc><<<(unsigned)((tot + 255) / 256), 256, 0, st>>>(acc, P, rows, kbc, mx_ws,
-                                                                       ex);
-    las_count_launch();
-  } else {
-    const long threads = rows * 32;
-    k_slice_rows<Acc><<<(unsigned)((threads + 255) / 256), 256, 0, st>>>(acc, P, rows, kbc, ex);
-    las_count_launch();
-  }
+// Digit planes P and row exponents ex of a source.  live_only: only rows < R and the K blocks that
+// hold K are written (planes whose padding rows were zeroed at set-up); otherwise every padded row
+// and K block of the layout is written.
+static las_status slice_done(const char* what) {
+  las_count_launch();
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) {
-    las_record_cuda_error(e, "k_slice_rows launch", __FILE__, __LINE__);
+    las_record_cuda_error(e, what, __FILE__, __LINE__);
     return LAS_ERR_CUDA;
   }
   return LAS_OK;
+}
+static long slice_extent(const Planes& P, bool live_only, long* kb) {
+  *kb = live_only ? std::min(P.nkb, planes_nkb(P.K)) : P.nkb;
+  return live_only ? P.R : P.Rpad;
+}
+
+// Any source: one warp per row.
+template <class Acc>
+static las_status slice_rows(Acc acc, const Planes& P, int* ex, cudaStream_t st,
+                             bool live_only = false) {
+  if (P.R <= 0) return LAS_OK;
+  long kb;
+  const long rows = slice_extent(P, live_only, &kb);
+  k_slice_rows<Acc><<<(unsigned)((rows * 32 + 255) / 256), 256, 0, st>>>(acc, P, rows, kb, ex);
+  return slice_done("k_slice_rows launch");
+}
+
+// Rows contiguous in K (RowsContig, RowsHtAct).  Rows per block: up to 40 KB of shared memory, and
+// no more than leaves two blocks per SM; a single row has to fit 48 KB (K <= 6128).
+template <class Rows>
+static las_status slice_contig(Rows src, const Planes& P, int* ex, cudaStream_t st,
+                               bool live_only = false) {
+  if (P.R <= 0) return LAS_OK;
+  long kb;
+  const long rows = slice_extent(P, live_only, &kb);
+  const long S = kb * BK + 2;
+  if (S * 8 > 48 * 1024 - 512) return slice_rows(src, P, ex, st, live_only);
+  int lg = 0;
+  while (lg < 5 && (S * 8 << (lg + 1)) <= 40 * 1024 && (rows >> (lg + 1)) >= 2 * num_sms()) ++lg;
+  k_slice_kmajor<Rows><<<(unsigned)((rows + (1 << lg) - 1) >> lg), 256, (size_t)(S * 8) << lg,
+                         st>>>(src, src.aligned(), P, rows, kb, lg, (int)S, ex);
+  return slice_done("k_slice_kmajor launch");
+}
+
+// Sources read along the rows, small enough that both passes of a block of 16 rows find them in L2.
+template <class Acc>
+static las_status slice_cols(Acc acc, const Planes& P, int* ex, cudaStream_t st,
+                             bool live_only = false) {
+  if (P.R <= 0) return LAS_OK;
+  long kb;
+  const long rows = slice_extent(P, live_only, &kb);
+  k_slice_cols<Acc><<<(unsigned)((rows + 15) / 16), 512, 0, st>>>(acc, P, rows, kb, ex);
+  return slice_done("k_slice_cols launch");
+}
+
+// Long rows contiguous in K (the projection's W): block-parallel maxima in mx, then the digits of
+// the live rows.
+static las_status slice_long(RowsContig src, const Planes& P, int* ex, unsigned long long* mx,
+                             cudaStream_t st) {
+  if (P.R <= 0) return LAS_OK;
+  LAS_CUDA_TRY(cudaMemsetAsync(mx, 0, P.R * sizeof(unsigned long long), st));
+  const long seg = 8192;
+  dim3 g1((unsigned)((P.K + seg - 1) / seg), (unsigned)P.R);
+  k_rowmax_long<RowsContig><<<g1, 256, 0, st>>>(src, P.K, seg, mx);
+  las_count_launch();
+  const long kb = std::min(P.nkb, planes_nkb(P.K)), tot = P.R * kb * 2;
+  k_digits_long<RowsContig><<<(unsigned)((tot + 255) / 256), 256, 0, st>>>(src, P, P.R, kb, mx, ex);
+  return slice_done("k_digits_long launch");
+}
+
+// Large sources read along the rows ([K][R] in memory, rows of the planes = columns of the source):
+// column maxima in mx, then the digits of the live rows.
+static las_status slice_transposed(const double* src, const Planes& P, int* ex,
+                                   unsigned long long* mx, cudaStream_t st) {
+  if (P.R <= 0) return LAS_OK;
+  LAS_CUDA_TRY(cudaMemsetAsync(mx, 0, P.R * sizeof(unsigned long long), st));
+  const long seg = 512;
+  dim3 g1((unsigned)((P.R + 255) / 256), (unsigned)((P.K + seg - 1) / seg));
+  k_colmax<<<g1, 256, 0, st>>>(src, P.K, (int)P.R, seg, mx);
+  las_count_launch();
+  const long kb = planes_nkb(P.K), warps = (P.R + 15) / 16 * kb;
+  k_digits_cols<RowsStrided><<<(unsigned)((warps + 7) / 8), 256, 0, st>>>(
+      RowsStrided{src, 1, P.R}, P, kb, mx, ex);
+  return slice_done("k_digits_cols launch");
 }
 
 struct SplitState {
@@ -1731,8 +1806,7 @@ static int half_bn(const SplitState* s) { return s->bn_set[SPLIT_HALF] ? s->bn[S
 
 las_status split_prepare_C(SplitState* s, const double* Cocc, cudaStream_t st) {
   // rows p of C_occ^T (K = nu): element (p, nu) = Cocc[nu*op + p]
-  RowsStrided acc{Cocc, 1, s->op, nullptr};
-  return slice_rows(acc, s->Cdig, s->Cexp, st, nullptr, true);
+  return slice_cols(RowsStrided{Cocc, 1, s->op}, s->Cdig, s->Cexp, st, true);
 }
 
 // ------------------------------------------------------------------------------------------
@@ -1763,8 +1837,7 @@ las_status split_tangent_prepare(SplitState* s, const double* dCocc, cudaStream_
     s->dHexp = (int*)(w + b0 + b1 + b2);
     *bytes += b0 + b1 + b2 + b3;
   }
-  RowsStrided acc{dCocc, 1, s->op, nullptr};
-  return slice_rows(acc, s->dCdig, s->dCexp, st, nullptr, true);
+  return slice_cols(RowsStrided{dCocc, 1, s->op}, s->dCdig, s->dCexp, st, true);
 }
 
 // dH = b^L dC_occ for the chunk's aux rows (Ht layout [nL][op][n])
@@ -1780,14 +1853,9 @@ las_status split_tangent_full(SplitState* s, int nL, const double* dHt, double* 
   las_status rc = ozaki_gemm(s->Hdig, 0, s->Hexp, R, s->dCdig, 0, s->dCexp, s->op, s->n, 1, 0, X,
                              s->op, 0, 0, 0, s->status, st, 0, s->bn[SPLIT_FULL]);
   if (rc != LAS_OK) return rc;
-  k_slice_ht<<<(unsigned)((R + 15) / 16), 256, 0, st>>>(dHt, R, s->n, s->dHdig, s->dHexp);
-  las_count_launch();
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) {
-    las_record_cuda_error(e, "k_slice_ht launch", __FILE__, __LINE__);
-    return LAS_ERR_CUDA;
-  }
-  return LAS_OK;
+  Planes dH = s->dHdig;
+  dH.R = R;
+  return slice_contig(RowsContig{dHt, s->n}, dH, s->dHexp, st, true);
 }
 
 const int* split_tangent_dhexp(SplitState* s) { return s->dHexp; }
@@ -1799,7 +1867,7 @@ las_status split_tangent_project(SplitState* s, int nL, int which, const double*
   const long R = (long)nL * s->op;
   Planes W = s->Wdig;
   W.K = R;
-  las_status rc = slice_rows(RowsStrided{Wt, R, 1, nullptr}, W, s->Wexp, st, s->mx, true);
+  las_status rc = slice_long(RowsContig{Wt, R}, W, s->Wexp, s->mx, st);
   if (rc != LAS_OK) return rc;
   const int ks = project_ksplit(s, R);
   rc = ozaki_gemm(which ? s->dHdig : s->Hdig, 0, nullptr, s->n, W, 0, s->Wexp, s->op, R, ks, 0,
@@ -1841,12 +1909,11 @@ las_status split_lpu(SplitState* s, int nL, const double* Ht, int c, int a, cons
   }
   Planes Mp = s->Mpd;
   Mp.R = np;
-  las_status rc = slice_rows(RowsStrided{C + p0, 1, nmo, nullptr}, Mp, s->Mpexp, st, nullptr,
-                             true);
+  las_status rc = slice_cols(RowsStrided{C + p0, 1, nmo}, Mp, s->Mpexp, st, true);
   // the active rows (L,u) of this chunk, sliced into the H digit planes (capacity Lc*op rows)
   Planes Hd = s->Hdig;
   Hd.R = (long)nL * a;
-  if (rc == LAS_OK) rc = slice_rows(RowsHtAct{Ht, n, s->op, c, a}, Hd, s->Hexp, st, nullptr, true);
+  if (rc == LAS_OK) rc = slice_contig(RowsHtAct{Ht, n, s->op, c, a}, Hd, s->Hexp, st, true);
   if (rc == LAS_OK)
     rc = ozaki_gemm(Hd, 0, s->Hexp, (long)nL * a, Mp, 0, s->Mpexp, np, n, 1, 1, Lpu, 0, 0, a, np,
                     s->status, st);
@@ -1860,15 +1927,10 @@ las_status split_half(SplitState* s, int l0, int nL, int oc, double* Ht, cudaStr
 
 las_status split_full(SplitState* s, int nL, const double* Ht, double* T, cudaStream_t st) {
   const long R = (long)nL * s->op;
-  k_slice_ht<<<(unsigned)((R + 15) / 16), 256, 0, st>>>(Ht, R, s->n, s->Hdig, s->Hexp);
-  las_count_launch();
-  {
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) {
-      las_record_cuda_error(e, "k_slice_ht launch", __FILE__, __LINE__);
-      return LAS_ERR_CUDA;
-    }
-  }
+  Planes Hd = s->Hdig;
+  Hd.R = R;
+  las_status rc = slice_contig(RowsContig{Ht, s->n}, Hd, s->Hexp, st, true);
+  if (rc != LAS_OK) return rc;
   return ozaki_gemm(s->Hdig, 0, s->Hexp, R, s->Cdig, 0, s->Cexp, s->op, s->n, 1, 0, T, s->op, 0,
                     0, 0, s->status, st, 0, s->bn[SPLIT_FULL]);
 }
@@ -1881,8 +1943,7 @@ las_status split_project_gemm(SplitState* s, int nL, const double* Wt, int* ks_u
   // W rows q (K = (L,p)), already scaled by 2^Hexp[(L,p)] and stored transposed: Wt[q][R]
   Planes W = s->Wdig;
   W.K = R;
-  RowsStrided acc{Wt, R, 1, nullptr};
-  las_status rc = slice_rows(acc, W, s->Wexp, st, s->mx, true);
+  las_status rc = slice_long(RowsContig{Wt, R}, W, s->Wexp, s->mx, st);
   if (rc != LAS_OK) return rc;
   const int ks = project_ksplit(s, R);
   *ks_used = ks;
@@ -1911,26 +1972,8 @@ las_status split_exchange(SplitState* s, int nL, int oc, const double* Ht, doubl
   if (oc < 1 || oc > s->op) return LAS_ERR_INTERNAL;
   Planes HT = s->HdigT;
   HT.K = R;
-  las_status rc = LAS_OK;
-  {
-    cudaError_t e = cudaMemsetAsync(s->mx, 0, n * sizeof(unsigned long long), st);
-    if (e != cudaSuccess) {
-      las_record_cuda_error(e, "cudaMemsetAsync(colmax)", __FILE__, __LINE__);
-      return LAS_ERR_CUDA;
-    }
-    const long seg = 512;
-    dim3 g1((unsigned)((n + 255) / 256), (unsigned)((R + seg - 1) / seg));
-    k_colmax<<<g1, 256, 0, st>>>(Ht, R, (int)n, seg, s->mx);
-    las_count_launch();
-    dim3 g2((unsigned)((R + 31) / 32), (unsigned)((n + COLS_PER_BLOCK - 1) / COLS_PER_BLOCK));
-    k_slice_ht_cols<<<g2, 256, 0, st>>>(Ht, R, (int)n, s->mx, HT, s->hexp);
-    las_count_launch();
-    e = cudaGetLastError();
-    if (e != cudaSuccess) {
-      las_record_cuda_error(e, "k_slice_ht_cols launch", __FILE__, __LINE__);
-      return LAS_ERR_CUDA;
-    }
-  }
+  las_status rc = slice_transposed(Ht, HT, s->hexp, s->mx, st);
+  if (rc != LAS_OK) return rc;
   // partials [ks][n][n] live in the projection's partial buffer (64 * n * op doubles)
   const long cap = std::max(1L, std::min((64L * s->op) / n, R / KSPLIT_MIN));
   const int ks = balanced_ksplit(ozaki_tiles(n, n, 1), (R + BK - 1) / BK, cap);
@@ -1944,8 +1987,7 @@ las_status split_exchange(SplitState* s, int nL, int oc, const double* Ht, doubl
 
 las_status split_one_electron_hc(SplitState* s, const double* h, double* hC, cudaStream_t st) {
   // hC = h C_occ  (rows mu of h, columns p of C_occ: the digits of C_occ are already sliced)
-  las_status rc = slice_rows(RowsStrided{h, s->n, 1, nullptr}, s->hdig, s->hexp, st, nullptr,
-                             true);
+  las_status rc = slice_contig(RowsContig{h, s->n}, s->hdig, s->hexp, st, true);
   if (rc == LAS_OK)
     rc = ozaki_gemm(s->hdig, 0, s->hexp, s->n, s->Cdig, 0, s->Cexp, s->op, s->n, 1, 0, hC, s->op,
                     0, 0, 0, s->status, st, 0, s->bn[SPLIT_ONE_ELECTRON]);
@@ -1991,8 +2033,8 @@ extern "C" las_status las_split_gemm(long M, long N, long K, const double* A, lo
   w += rup(N * 4, 256);
   int* status = (int*)w;
   LAS_CUDA_TRY(cudaMemsetAsync(status, 0, 4, st));
-  las_status rc = slice_rows(RowsStrided{A, lda, 1, nullptr}, Ad, ea, st);
-  if (rc == LAS_OK) rc = slice_rows(RowsStrided{B, 1, ldb, nullptr}, Bd, eb, st);
+  las_status rc = slice_contig(RowsContig{A, lda}, Ad, ea, st);
+  if (rc == LAS_OK) rc = slice_cols(RowsStrided{B, 1, ldb}, Bd, eb, st);
   if (rc == LAS_OK)
     rc = ozaki_gemm(Ad, 0, ea, M, Bd, 0, eb, N, K, 1, 0, C, ldc, 0, 0, 0, status, st);
   if (rc != LAS_OK) return rc;
@@ -2103,7 +2145,7 @@ int frag_split_fits(const FragSplit* f, int n, int nmo, int ma, int Lc) {
 
 las_status frag_split_prepare_M(FragSplit* f, const double* M, cudaStream_t st) {
   // rows p of M^T (K = e): element (p, e) = M[e][p]
-  return slice_rows(RowsStrided{M, 1, f->nmo, nullptr}, f->Mdig, f->Mexp, st, nullptr, true);
+  return slice_cols(RowsStrided{M, 1, f->nmo}, f->Mdig, f->Mexp, st, true);
 }
 
 las_status frag_split_chunk(SplitState* s, FragSplit* f, int l0, int nL, double* H, double* T,
@@ -2117,7 +2159,7 @@ las_status frag_split_chunk(SplitState* s, FragSplit* f, int l0, int nL, double*
   // Eq. ao2mo_2: T[L][p][q] = sum_e H[L][p][e] M[e][q]
   Planes Hd = f->Hd;
   Hd.R = R1;
-  if (rc == LAS_OK) rc = slice_rows(RowsStrided{H, n, 1, nullptr}, Hd, f->Hexp, st, nullptr, true);
+  if (rc == LAS_OK) rc = slice_contig(RowsContig{H, n}, Hd, f->Hexp, st, true);
   if (rc == LAS_OK)
     rc = ozaki_gemm(Hd, 0, f->Hexp, R1, f->Mdig, 0, f->Mexp, nmo, n, 1, 0, T, nmo, 0, 0, 0,
                     s->status, st);
@@ -2129,27 +2171,10 @@ las_status frag_split_chunk(SplitState* s, FragSplit* f, int l0, int nL, double*
     A.K = nL;
     B.R = (long)ma * ma;
     B.K = nL;
-    // rows (p,q) of T^T with per-row exponents: column maxima of T [nL][n2], then a transposing
-    // slicer (coalesced reads along (p,q))
-    cudaError_t e = cudaMemsetAsync(f->mx, 0, (size_t)n2 * 8, st);
-    if (e != cudaSuccess) {
-      las_record_cuda_error(e, "cudaMemsetAsync(frag colmax)", __FILE__, __LINE__);
-      return LAS_ERR_CUDA;
-    }
-    const long seg = 512;
-    dim3 g1((unsigned)((n2 + 255) / 256), (unsigned)((nL + seg - 1) / seg));
-    k_colmax<<<g1, 256, 0, st>>>(T, nL, (int)n2, seg, f->mx);
-    las_count_launch();
-    dim3 g2((unsigned)((nL + 31) / 32), (unsigned)((n2 + COLS_PER_BLOCK - 1) / COLS_PER_BLOCK));
-    k_slice_ht_cols<<<g2, 256, 0, st>>>(T, nL, (int)n2, f->mx, A, f->Texp);
-    las_count_launch();
-    e = cudaGetLastError();
-    if (e != cudaSuccess) {
-      las_record_cuda_error(e, "frag slicer launch", __FILE__, __LINE__);
-      return LAS_ERR_CUDA;
-    }
+    // rows (p,q) of T^T with per-row exponents
+    rc = slice_transposed(T, A, f->Texp, f->mx, st);
     if (rc == LAS_OK)
-      rc = slice_rows(RowsAA{T, n2, nmo, a0, ma}, B, f->Taaexp, st, nullptr, true);
+      rc = slice_cols(RowsAA{T, n2, nmo, a0, ma}, B, f->Taaexp, st, true);
     const long out = n2 * ma * ma;
     const int ks = balanced_ksplit(ozaki_tiles(n2, (long)ma * ma, 0), kb,
                                    std::max(1L, std::min(kb, part_elems / out)));
@@ -2165,7 +2190,7 @@ las_status frag_split_chunk(SplitState* s, FragSplit* f, int l0, int nL, double*
     Planes A = f->Tpa;
     A.R = (long)nmo * ma;
     A.K = nL;
-    rc = slice_rows(RowsPA{T, n2, nmo, a0, ma}, A, f->Tpaexp, st, nullptr, true);
+    rc = slice_cols(RowsPA{T, n2, nmo, a0, ma}, A, f->Tpaexp, st, true);
     const long m = (long)nmo * ma, out = m * m;
     const int ks = balanced_ksplit(ozaki_tiles(m, m, 1), kb,
                                    std::max(1L, std::min(kb, part_elems / out)));
