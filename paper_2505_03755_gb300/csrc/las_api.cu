@@ -69,6 +69,7 @@ struct las_ctx {
   int* status;    // device status word
   // staging for the host-buffer call
   double *dC, *dh, *ddm1, *ddm2, *dE, *dG;
+  double* dm2t;   // pair-transposed fragment 2-RDMs of the evaluation in progress
   long ndm1, ndm2;
   size_t bytes;
   // split-precision state (owned)
@@ -122,7 +123,7 @@ static las_status dalloc(las_ctx* x, void** p, size_t bytes) {
 static void free_all(las_ctx* x) {
   void* ptrs[] = {x->Cocc, x->Ht, x->T, x->W, x->part, x->Out, x->hC, x->e1, x->M, x->eps,
                   x->vc, x->va, x->Jp, x->Jt, x->Kt, x->widx, x->status, x->dC, x->dh, x->ddm1, x->ddm2,
-                  x->dE, x->dG};
+                  x->dE, x->dG, x->dm2t};
   for (void* p : ptrs)
     if (p) cudaFree(p);
   if (x->split) split_destroy(x->split);
@@ -245,6 +246,7 @@ extern "C" las_status las_create(las_ctx** out, const las_dims* d, const double*
   ALLOC(dh, (size_t)x->n * x->n);
   ALLOC(ddm1, std::max(1L, x->ndm1));
   ALLOC(ddm2, std::max(1L, x->ndm2));
+  ALLOC(dm2t, std::max(1L, x->ndm2));
   ALLOC(dE, 1);
   ALLOC(dG, (size_t)x->n * x->nmo);
 #undef ALLOC
@@ -256,7 +258,7 @@ extern "C" las_status las_create(las_ctx** out, const las_dims* d, const double*
     }
   }
   if (st == LAS_OK) {
-    st = per_aux_prepare(a);
+    st = per_aux_prepare();
   }
   if (st == LAS_OK && prec == LAS_SPLIT_BF16) {
     st = split_create(&x->split, x->n, x->X, x->op, x->Lc, B_packed, packed, x->status,
@@ -458,7 +460,8 @@ static las_status evaluate(las_ctx* x, const double* C, const double* h, const d
   if (gorb && !G) G = x->dG;
   las_status st;
   stage_mark(x, 0);
-  launch_pack_cocc(C, n, nmo, x->o, op, x->Cocc, x->stream);
+  launch_pack_cocc(C, n, nmo, x->o, op, x->Cocc, x->stream, x->a > 0 ? dm2 : nullptr, &x->fi,
+                   x->dm2t);
   if (x->prec == LAS_SPLIT_BF16) {
     st = split_prepare_C(x->split, x->Cocc, x->stream);
     if (st != LAS_OK) return st;
@@ -468,8 +471,8 @@ static las_status evaluate(las_ctx* x, const double* C, const double* h, const d
     if ((st = half_and_full(x, l0, nL, 1, l0 == 0 ? 1 : -1)) != LAS_OK) return st;
     if (l0 == 0) stage_mark(x, 2);
     // split mode: W is written transposed and row-scaled for the split projection GEMM
-    launch_per_aux(x->T, nL, op, dm1s, dm2, x->fi, x->W, x->eps + l0, x->vc + l0, x->va + l0,
-                   with_grad, x->split ? split_hexp(x->split) : nullptr, x->status, x->stream);
+    launch_per_aux(x->T, nL, op, dm1s, x->dm2t, x->fi, x->W, x->eps + l0, x->vc + l0, x->va + l0,
+                   with_grad, x->split ? split_hexp(x->split) : nullptr, x->stream);
     if ((st = check_launch()) != LAS_OK) return st;
     if (l0 == 0) stage_mark(x, 3);
     if (with_grad && (st = project(x, nL, l0 > 0)) != LAS_OK) return st;
@@ -702,8 +705,7 @@ extern "C" las_status las_veff(las_ctx* x, const double* Ca, const double* wa, i
 // one more half transform (dH), one more full-transform product (X), two per-aux passes and two
 // projections; in split precision W(T_L) is scaled by the row exponents of dH and W(dT_L) by those
 // of H, the operand each is projected against.  G(C) itself (for Dg) is one plain evaluation.
-static las_status tangent_grad(las_ctx* x, const double* h, const double* dm1s,
-                               const double* dm2, double* dG) {
+static las_status tangent_grad(las_ctx* x, const double* h, const double* dm1s, double* dG) {
   const int n = x->n, op = x->op, nmo = x->nmo;   // x->tCocc holds dC_occ
   const bool split = x->prec == LAS_SPLIT_BF16;
   las_status st;
@@ -733,10 +735,10 @@ static las_status tangent_grad(las_ctx* x, const double* h, const double* dm1s,
     // W(T) against dH and W(dT) against H (the per-aux outputs eps, vc, va are not needed)
     const int* hexp = split ? split_hexp(x->split) : nullptr;
     const int* dhexp = split ? split_tangent_dhexp(x->split) : nullptr;
-    launch_per_aux(x->T, nL, op, dm1s, dm2, x->fi, x->tWd, x->eps + l0, x->vc + l0, x->va + l0, 1,
-                   dhexp, x->status, x->stream);
-    launch_per_aux(x->tdT, nL, op, dm1s, dm2, x->fi, x->tdW, x->eps + l0, x->vc + l0, x->va + l0,
-                   1, hexp, x->status, x->stream);
+    launch_per_aux(x->T, nL, op, dm1s, x->dm2t, x->fi, x->tWd, x->eps + l0, x->vc + l0, x->va + l0,
+                   1, dhexp, x->stream);
+    launch_per_aux(x->tdT, nL, op, dm1s, x->dm2t, x->fi, x->tdW, x->eps + l0, x->vc + l0,
+                   x->va + l0, 1, hexp, x->stream);
     if ((st = check_launch()) != LAS_OK) return st;
     if (split) {
       if ((st = split_tangent_project(x->split, nL, 0, x->tdW, x->tOut, l0 > 0, x->stream)) !=
@@ -782,9 +784,9 @@ extern "C" las_status las_orbital_hvp(las_ctx* x, const double* C, const double*
   // dC_occ = C X_occ (only the occupied columns of C X are ever needed); zero padding columns
   LAS_CUDA_TRY(cudaMemsetAsync(x->tCocc, 0, sizeof(double) * n * op, x->stream));
   gemm_f64_wide(x, n, o, nmo, StridedA{C, 0, nmo, 1}, StridedA{X, 0, nmo, 1}, x->tCocc, op, 0);
-  // G(C): C_occ, its digits and those of h stay in place for the tangent chain
+  // G(C): C_occ, its digits, those of h and dm2t stay in place for the tangent chain
   if ((st = evaluate(x, C, h, dm1s, dm2, x->dE, x->hG, nullptr)) != LAS_OK) return st;
-  if ((st = tangent_grad(x, h, dm1s, dm2, dG)) != LAS_OK) return st;
+  if ((st = tangent_grad(x, h, dm1s, dG)) != LAS_OK) return st;
   if (Dg) {
     // Dg = (C X)^T G + C^T dG - transpose = X^T (C^T G) + C^T dG - transpose  (virtual columns
     // of G and dG are zero)
@@ -1034,7 +1036,8 @@ static las_status capture_grouped(const BatchPlan& P, las_ctx* const* ctxs,
       if (c >= nchunks(x)) return LAS_OK;
       las_status r = LAS_OK;
       if (c == 0) {
-        launch_pack_cocc(items[i].C, x->n, x->nmo, x->o, x->op, x->Cocc, x->stream);
+        launch_pack_cocc(items[i].C, x->n, x->nmo, x->o, x->op, x->Cocc, x->stream,
+                         x->a > 0 ? items[i].dm2 : nullptr, &x->fi, x->dm2t);
         if ((r = split_prepare_C(x->split, x->Cocc, x->stream)) != LAS_OK) return r;
         if ((r = split_one_electron_hc(x->split, items[i].h, x->hC, x->stream)) != LAS_OK)
           return r;
@@ -1054,8 +1057,8 @@ static las_status capture_grouped(const BatchPlan& P, las_ctx* const* ctxs,
     rc = phase([&](int i, las_ctx* x) -> las_status {
       if (c >= nchunks(x)) return LAS_OK;
       const int l0 = c * x->Lc, nL = std::min(x->Lc, x->X - l0);
-      launch_per_aux(x->T, nL, x->op, items[i].dm1s, items[i].dm2, x->fi, x->W, x->eps + l0,
-                     x->vc + l0, x->va + l0, 1, split_hexp(x->split), x->status, x->stream);
+      launch_per_aux(x->T, nL, x->op, items[i].dm1s, x->dm2t, x->fi, x->W, x->eps + l0,
+                     x->vc + l0, x->va + l0, 1, split_hexp(x->split), x->stream);
       las_status r = check_launch();
       if (r == LAS_OK) r = split_project_gemm(x->split, nL, x->W, &ks[i], x->stream);
       return r;

@@ -72,18 +72,21 @@ struct StridedC {  // C[b*sb + m*sm + n*sn] (=|+=) alpha * acc
 };
 
 // Small helpers implemented in las_kernels.cu
+// Cocc[n][op] = the first o columns of C (zero padding); with dm2 also the pair-transposed
+// fragment 2-RDMs dm2t that launch_per_aux reads
 void launch_pack_cocc(const double* C, int n, int nmo, int o, int op, double* Cocc,
-                      cudaStream_t s);
-las_status per_aux_prepare(int nact);
+                      cudaStream_t s, const double* dm2 = nullptr, const FragInfo* fi = nullptr,
+                      double* dm2t = nullptr);
+las_status per_aux_prepare();
 // gexp == nullptr: W[L][p][q];  otherwise W is written as Wt[q][L*op + p] * 2^gexp[L*op + p]
 // CT[k][mu] = Cocc[mu][k] for k < r (Cocc is n x op)
 void launch_transpose_cols(const double* Cocc, int n, int op, int r, double* CT, cudaStream_t s);
 // vc[b] = 2 sum_{k<r} sum_mu Ht[(b*r + k)*n + mu] * CT[k*n + mu], b < nL (fixed summation order)
 void launch_trace_ht(const double* Ht, const double* CT, int nL, int r, int n, double* vc,
                      cudaStream_t s);
-void launch_per_aux(const double* T, int nL, int op, const double* dm1s, const double* dm2,
+void launch_per_aux(const double* T, int nL, int op, const double* dm1s, const double* dm2t,
                     const FragInfo& fi, double* W, double* eps, double* vc, double* va,
-                    int with_grad, const int* gexp, int* status, cudaStream_t s);
+                    int with_grad, const int* gexp, cudaStream_t s);
 void launch_scale(double* p, long count, double a, cudaStream_t s);
 void launch_mirror_lower(double* K, int n, cudaStream_t s);
 void launch_axpy(double* y, const double* x, double a, long count, cudaStream_t s);

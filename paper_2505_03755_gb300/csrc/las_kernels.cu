@@ -1,32 +1,28 @@
 // Small FP64 kernels of the LAS energy/gradient chain: per-auxiliary-index contractions with the
 // block-product RDMs, energy reduction, gradient assembly and layout helpers.
+#include <string.h>
+
 #include <algorithm>
 
 #include "las_common.cuh"
 
 namespace lasdf {
 
-// Deterministic block sums of K doubles per thread: warp butterflies (lane 0's order is fixed),
-// then the warp partials in warp order; every thread returns the K totals.  red: NT/32*K doubles.
-template <int NT, int K>
-__device__ void block_sums(double (&v)[K], double* red) {
-  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-#pragma unroll
-  for (int k = 0; k < K; ++k)
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v[k] += __shfl_xor_sync(0xffffffffu, v[k], o);
-  if (lane == 0)
-#pragma unroll
-    for (int k = 0; k < K; ++k) red[w * K + k] = v[k];
+// Deterministic block sum of one double per thread, on thread 0 only: the warps' values of a lane
+// added in warp order by the first warp, then a butterfly.  FP64 adds are slow on this part (a
+// warp's add takes some 18 clocks of the SM), so no thread adds what another one has added.
+template <int NT>
+__device__ double block_sum0(double v, double* red) {   // red: NT doubles
+  red[threadIdx.x] = v;
   __syncthreads();
+  double t = 0.0;
+  if (threadIdx.x < 32) {
 #pragma unroll
-  for (int k = 0; k < K; ++k) {
-    double t = 0.0;
+    for (int w = 0; w < NT / 32; ++w) t += red[w * 32 + threadIdx.x];
 #pragma unroll
-    for (int i = 0; i < NT / 32; ++i) t += red[i * K + k];
-    v[k] = t;
+    for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
   }
-  __syncthreads();
+  return t;
 }
 
 // Deterministic block reduction of one double per thread (fixed tree order).
@@ -44,13 +40,28 @@ __device__ double block_sum(double v, double* red) {
   return r;
 }
 
+// Cocc[mu][p] = C[mu][p] for p < o, 0 for o <= p < op; and, with dm2, the pair-transposed fragment
+// 2-RDMs dm2t_K[wx][uv] = Gamma^K[uv][wx] that k_per_aux reads along uv.
 __global__ void k_pack_cocc(const double* __restrict__ C, int n, int nmo, int o, int op,
-                            double* __restrict__ Cocc) {
+                            double* __restrict__ Cocc, const double* __restrict__ dm2,
+                            FragInfo fi, double* __restrict__ dm2t) {
   long i = blockIdx.x * (long)blockDim.x + threadIdx.x;
-  long total = (long)n * op;
-  if (i >= total) return;
-  int mu = (int)(i / op), p = (int)(i % op);
-  Cocc[i] = (p < o) ? C[(long)mu * nmo + p] : 0.0;
+  const long total = (long)n * op;
+  if (i < total) {
+    int mu = (int)(i / op), p = (int)(i % op);
+    Cocc[i] = (p < o) ? C[(long)mu * nmo + p] : 0.0;
+    return;
+  }
+  if (!dm2) return;
+  i -= total;
+  for (int K = 0; K < fi.nfrag; ++K) {
+    const long m = fi.off[K + 1] - fi.off[K], m2 = m * m;
+    if (i < m2 * m2) {
+      dm2t[fi.dm2_off[K] + (i % m2) * m2 + i / m2] = dm2[fi.dm2_off[K] + i];
+      return;
+    }
+    i -= m2 * m2;
+  }
 }
 
 __device__ __forceinline__ int frag_of(const FragInfo& fi, int u) {
@@ -67,183 +78,245 @@ __device__ __forceinline__ int frag_of(const FragInfo& fi, int u) {
 //   eps_L  = vc^2/2 - sum_ij T(i,j)^2 + vc va - sum_{i,u} Z(i,u) T(i,u) + 1/2 sum_uv T(u,v) Y(u,v)
 //            with Z = T(core,act) D  (the L-th term of the two-electron energy)
 //   W_L(p,q): the matrix with  dE/dC(two-electron part) = sum_L H_L W_L, H_L = b^L C_occ.
-// x * 2^g for normal or zero x (exponent-field arithmetic; no FP64 multiply)
+// x * 2^g, and -x * 2^g, in exponent-field and sign-bit arithmetic: an FP64 multiply, comparison or
+// negation would each take a slot of the FP64 pipe (and so would those of ldexp, even on a branch
+// that no thread takes).
 __device__ __forceinline__ double scale2(double x, int g) {
-  long long b = __double_as_longlong(x);
-  if ((b & 0x7FF0000000000000ll) == 0) return x == 0.0 ? x : ldexp(x, g);
-  return __longlong_as_double(b + (((long long)g) << 52));
+  unsigned long long b = (unsigned long long)__double_as_longlong(x);
+  if ((b & 0x7FF0000000000000ull) == 0) {   // zero, or subnormal: bring the leading one to bit 52
+    const unsigned long long m = b << 12 >> 12;
+    const int lz = __clzll((long long)m) - 11;
+    if (m == 0) return x;
+    if (1 - lz + g < 1) return __longlong_as_double((long long)(b - m));   // (nearly) 0
+    b = b - m + (m << lz) + (((long long)-lz) << 52);
+  }
+  return __longlong_as_double((long long)b + (((long long)g) << 52));
+}
+__device__ __forceinline__ double neg_scale2(double x, int g) {
+  return scale2(__longlong_as_double(__double_as_longlong(x) ^ (long long)(1ull << 63)), g);
 }
 
-__global__ void __launch_bounds__(256)
+// FP64 arithmetic is the bound (about 1.75 multiply-adds per clock and SM, a warp's instruction at
+// 18 clocks however few of its lanes are live): at 150 core and 5 x 8 active orbitals 1.5e5 of them
+// per L, 0.65 ms for 2400 L.  So the loops run over exactly the elements that have work (the
+// intra-fragment pairs as one list), signs and powers of two are exponent arithmetic, and sums are
+// combined by one warp.  (As one loop over all a x a elements with the fragment test inside, a
+// warp's FMAs were four fifths masked: 1.59 ms; now 0.92.)  The rest of the time is the
+// phases' latency, overlapped by the other blocks of the SM.
+// Element (r, l) of W_L, r the row that is contiguous: FP64 mode W[L][p = r][q = l]; split mode
+// (gexp) Wt[q = r][(L, p = l)] * 2^gexp(L, p), in which T(p, q) of the core block is read as
+// T(q, p) (T_L is symmetric).
+__global__ void __launch_bounds__(256, 5)
 k_per_aux(const double* __restrict__ T, int nL, int op, const double* __restrict__ dm1s,
-          const double* __restrict__ dm2, FragInfo fi, double* __restrict__ W,
+          const double* __restrict__ dm2t, FragInfo fi, double* __restrict__ W,
           double* __restrict__ eps, double* __restrict__ vcv, double* __restrict__ vav,
-          int with_grad, const int* __restrict__ gexp, int* status, int use_p) {
+          int with_grad, const int* __restrict__ gexp, int use_p) {
   extern __shared__ double sm[];
-  const int a = fi.nact, c = fi.ncore, o = c + a;
-  double* Taa = sm;             // a*a
-  double* Ds = Taa + a * a;     // a*a (block diagonal D)
-  double* Y = Ds + a * a;       // a*a
-  double* red = Y + a * a;      // 256
-  double* cK = red + 256;       // nfrag
-  double* P = cK + LAS_MAX_FRAG;  // a*a when the launch provides it (fast cross-fragment path)
+  const int a = fi.nact, c = fi.ncore, o = c + a, nf = fi.nfrag;
+  // fragment offsets, offsets of their D blocks (doff[nf] = size of all), fragment of an orbital
+  __shared__ int off[LAS_MAX_FRAG + 1], doff[LAS_MAX_FRAG + 1];
+  __shared__ unsigned char fk[LAS_MAX_ACT];
+  __shared__ double vs[2];                 // vc, va
+  double* Taa = sm;               // a*a
+  double* Y = Taa + a * a;        // a*a: Y, then Y + vc D^T
+  double* red = Y + a * a;        // 256
+  double* cK = red + 256;         // nfrag
+  double* Ds = cK + LAS_MAX_FRAG; // sum of m_K^2: the blocks of D
   const long Lb = blockIdx.x;
   const double* TL = T + Lb * (long)op * op;
-  const int tid = threadIdx.x;
-
-  for (int i = tid; i < a * a; i += 256) {
-    int u = i / a, v = i % a;
-    Taa[i] = TL[(long)(c + u) * op + c + v];
-    int K = frag_of(fi, u);
-    double d = 0.0;
-    if (v >= fi.off[K] && v < fi.off[K + 1]) {
-      int m = fi.off[K + 1] - fi.off[K];
-      int uu = u - fi.off[K], vv = v - fi.off[K];
-      const double* g = dm1s + fi.dm1_off[K];
-      d = g[uu * m + vv] + g[m * m + uu * m + vv];
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  if (tid == 0) {
+    int s = 0;
+    off[0] = 0;
+    for (int K = 0; K < nf; ++K) {
+      const int o0 = fi.off[K], o1 = fi.off[K + 1];
+      doff[K] = s;
+      off[K + 1] = o1;
+      s += (o1 - o0) * (o1 - o0);
+      for (int u = o0; u < o1; ++u) fk[u] = (unsigned char)K;
     }
-    Ds[i] = d;
+    doff[nf] = s;
   }
-  __syncthreads();
-
-  double pvc = 0.0, pcore = 0.0;
-  for (int i = tid; i < c; i += 256) pvc += TL[(long)i * op + i];
-  for (long i = tid; i < (long)c * c; i += 256) {
-    double x = TL[(i / c) * op + (i % c)];
-    pcore += x * x;
-  }
-  double pva = 0.0;
-  for (int i = tid; i < a * a; i += 256) pva += Ds[i] * Taa[i];
-  double r3[3] = {pvc, pcore, pva};
-  block_sums<256, 3>(r3, red);
-  const double vc = 2.0 * r3[0], fro = r3[1], va = r3[2];
-  if (tid < fi.nfrag) {
-    int K = tid, o0 = fi.off[K], m = fi.off[K + 1] - o0;
-    double s = 0.0;
-    for (int u = 0; u < m; ++u)
-      for (int v = 0; v < m; ++v) s += Ds[(o0 + u) * a + o0 + v] * Taa[(o0 + u) * a + o0 + v];
-    cK[K] = s;
-  }
-  __syncthreads();
-
-  // Y = Gamma . T over the active block, fragment structure of Eq. las_wfn.
   for (int i = tid; i < a * a; i += 256) {
-    const int u = i / a, v = i % a;
-    const int K = frag_of(fi, u), Kp = frag_of(fi, v);
-    const int oK = fi.off[K], mK = fi.off[K + 1] - oK;
-    double y = 0.0;
-    if (K != Kp && use_p) {
-      // cross-fragment blocks come from the factored form below
-    } else if (K == Kp) {
-      const double* g2 = dm2 + fi.dm2_off[K];
-      const int uu = u - oK, vv = v - oK;
-      const double* gr = g2 + ((long)uu * mK + vv) * mK * mK;
-      for (int w = 0; w < mK; ++w)
-        for (int x = 0; x < mK; ++x) y += gr[w * mK + x] * Taa[(oK + w) * a + oK + x];
-      y += Ds[i] * (va - cK[K]);
+    const int u = i / a;
+    Taa[i] = TL[(long)(c + u) * op + c + i - u * a];
+  }
+  __syncthreads();
+  const int nd = doff[nf];
+  double* P = Ds + nd;            // a*a when the launch provides it (cross-fragment path)
+  // fragment of element j of the list of intra-fragment pairs
+  auto frag_of_pair = [&](int j) {
+    int K = 0;
+    while (K + 1 < nf && doff[K + 1] <= j) ++K;
+    return K;
+  };
+  for (int j = tid; j < nd; j += 256) {
+    const int K = frag_of_pair(j), m = off[K + 1] - off[K];
+    const double* g = dm1s + fi.dm1_off[K] + (j - doff[K]);
+    Ds[j] = g[0] + g[m * m];
+  }
+  __syncthreads();
+  // cK = sum of D_K T_KK (one warp per fragment), vc = 2 sum_i T(i,i) (the first warp)
+  for (int K = warp - 1; K < nf; K += 8) {
+    double t = 0.0;
+    if (K < 0) {
+      for (int i = lane; i < c; i += 32) t += TL[(long)i * op + i];
     } else {
-      // -sum_sigma sum_{x in K, w in K'} gK_s[u,x] T(x,w) gK'_s[w,v]
-      const int oP = fi.off[Kp], mP = fi.off[Kp + 1] - oP;
-      const double* gK = dm1s + fi.dm1_off[K];
-      const double* gP = dm1s + fi.dm1_off[Kp];
-      const int uu = u - oK, vv = v - oP;
-      for (int s = 0; s < 2; ++s) {
-        const double* gKs = gK + s * mK * mK;
-        const double* gPs = gP + s * mP * mP;
-        for (int x = 0; x < mK; ++x) {
-          double gux = gKs[uu * mK + x];
-          if (gux == 0.0) continue;
-          double t = 0.0;
-          for (int w = 0; w < mP; ++w) t += Taa[(oK + x) * a + oP + w] * gPs[w * mP + vv];
-          y -= gux * t;
-        }
+      const int oK = off[K], m = off[K + 1] - oK;
+      for (int j = lane; j < m * m; j += 32) {
+        const int u = j / m;
+        t += Ds[doff[K] + j] * Taa[(oK + u) * a + oK + j - u * m];
       }
     }
-    Y[i] = y;
+#pragma unroll
+    for (int q = 16; q > 0; q >>= 1) t += __shfl_xor_sync(0xffffffffu, t, q);
+    if (lane == 0) {
+      if (K < 0) vs[0] = 2.0 * t;
+      else cK[K] = t;
+    }
   }
-  if (use_p) {
-    // -sum_sigma gK_s (T_KK' gK'_s) for K != K': P_s = T_aa blockdiag(g_s) first (a*a*m work),
-    // then the left factor, instead of the inner sum per (u, v)
+  __syncthreads();
+  if (tid == 0) {
+    double va = 0.0;
+    for (int K = 0; K < nf; ++K) va += cK[K];
+    vs[1] = va;
+  }
+
+  // Y = Gamma . T over the active block, fragment structure of Eq. las_wfn; qy += T Y.
+  // Cross-fragment blocks: -sum_sigma gK_s (T_KK' gK'_s), P_s = T_aa blockdiag(g_s) first
+  double qy = 0.0;
+  if (nf > 1 && use_p) {
     for (int sg = 0; sg < 2; ++sg) {
-      __syncthreads();
+      if (sg) __syncthreads();
       for (int i = tid; i < a * a; i += 256) {
-        const int x = i / a, v = i % a;
-        const int Kp = frag_of(fi, v), oP = fi.off[Kp], mP = fi.off[Kp + 1] - oP;
-        const double* gPs = dm1s + fi.dm1_off[Kp] + sg * mP * mP;
-        const int vv = v - oP;
+        const int x = i / a, v = i - x * a;
+        const int Kp = fk[v], oP = off[Kp], mP = off[Kp + 1] - oP;
+        if (x >= oP && x < oP + mP) continue;
+        const double* g = dm1s + fi.dm1_off[Kp] + sg * mP * mP + v - oP;
         double t = 0.0;
-        for (int w = 0; w < mP; ++w) t += Taa[x * a + oP + w] * gPs[w * mP + vv];
+        for (int w = 0; w < mP; ++w) t += Taa[x * a + oP + w] * g[w * mP];
         P[i] = t;
       }
       __syncthreads();
       for (int i = tid; i < a * a; i += 256) {
-        const int u = i / a, v = i % a;
-        const int K = frag_of(fi, u), Kp = frag_of(fi, v);
-        if (K == Kp) continue;
-        const int oK = fi.off[K], mK = fi.off[K + 1] - oK;
-        const double* gKs = dm1s + fi.dm1_off[K] + sg * mK * mK;
-        const int uu = u - oK;
-        double t = 0.0;
-        for (int x = 0; x < mK; ++x) t += gKs[uu * mK + x] * P[(oK + x) * a + v];
-        Y[i] -= t;
+        const int u = i / a, v = i - u * a;
+        const int K = fk[u], oK = off[K], mK = off[K + 1] - oK;
+        if (v >= oK && v < oK + mK) continue;
+        const double* g = dm1s + fi.dm1_off[K] + sg * mK * mK + (u - oK) * mK;
+        double t = sg ? Y[i] : 0.0;
+        for (int x = 0; x < mK; ++x) t -= g[x] * P[(oK + x) * a + v];
+        Y[i] = t;
+        if (sg) qy += Taa[i] * t;
       }
+    }
+  } else if (nf > 1) {
+    for (int i = tid; i < a * a; i += 256) {
+      const int u = i / a, v = i - u * a;
+      const int K = fk[u], oK = off[K], mK = off[K + 1] - oK;
+      if (v >= oK && v < oK + mK) continue;
+      const int Kp = fk[v], oP = off[Kp], mP = off[Kp + 1] - oP;
+      double y = 0.0;
+      for (int s = 0; s < 2; ++s) {
+        const double* gK = dm1s + fi.dm1_off[K] + s * mK * mK + (u - oK) * mK;
+        const double* gP = dm1s + fi.dm1_off[Kp] + s * mP * mP + v - oP;
+        for (int x = 0; x < mK; ++x) {
+          double t = 0.0;
+          for (int w = 0; w < mP; ++w) t += Taa[(oK + x) * a + oP + w] * gP[w * mP];
+          y -= gK[x] * t;
+        }
+      }
+      Y[i] = y;
+      qy += Taa[i] * y;
     }
   }
   __syncthreads();
+  const double vc = vs[0], va = vs[1];
+  // intra-fragment pairs: Gamma^K . T_KK + D (va - cK)
+  for (int j = tid; j < nd; j += 256) {
+    const int K = frag_of_pair(j), oK = off[K], m = off[K + 1] - oK, m2 = m * m;
+    const int r = j - doff[K], uu = r / m, vv = r - uu * m;
+    const double* g2 = dm2t + fi.dm2_off[K] + r;
+    double y0 = 0.0, y1 = 0.0;
+    for (int w = 0; w < m; ++w) {
+      const double* t = Taa + (oK + w) * a + oK;
+      const double* g = g2 + (long)w * m * m2;
+      int x = 0;
+      for (; x + 1 < m; x += 2) {
+        y0 += g[(long)x * m2] * t[x];
+        y1 += g[(long)(x + 1) * m2] * t[x + 1];
+      }
+      if (x < m) y0 += g[(long)x * m2] * t[x];
+    }
+    const double y = y0 + y1 + Ds[j] * (va - cK[K]);
+    const int i = (oK + uu) * a + oK + vv;
+    qy += Taa[i] * y;
+    Y[i] = y + vc * Ds[doff[K] + vv * m + uu];
+  }
+  __syncthreads();
 
-  // Z(i,u) = sum_v T(i, c+v) D(v,u) over core i and active u; its contraction with T(i,u).
-  double pz = 0.0;
+  // Z(i,u) = sum_v T(i, c+v) D(v,u) over core i and active u; q -= Z T.  W(i,u) = W(u,i) = -2 Z.
+  double q = 0.5 * qy;
   double* WL = W + Lb * (long)op * op;
   const long wld = (long)nL * op;
-  // W_L(p,q) -> its storage slot (plain, or transposed and scaled by 2^gexp for split mode)
-  auto putW = [&](int p, int q, double w) {
-    if (gexp) {
-      const long k = Lb * (long)op + p;
-      W[(long)q * wld + k] = scale2(w, gexp[k]);
-    } else {
-      WL[(long)p * op + q] = w;
-    }
-  };
-  for (long idx = tid; idx < (long)c * a; idx += 256) {
-    const int i = (int)(idx / a), u = (int)(idx % a);
-    const int K = frag_of(fi, u), oK = fi.off[K], mK = fi.off[K + 1] - oK;
-    const double* Ti = TL + (long)i * op + c;
-    double z = 0.0;
-    for (int v = oK; v < oK + mK; ++v) z += Ti[v] * Ds[v * a + u];
-    pz += z * Ti[u];
-    if (with_grad) {
-      putW(i, c + u, -2.0 * z);
-      putW(c + u, i, -2.0 * z);
+  const int* gL = gexp ? gexp + Lb * (long)op : nullptr;
+  if (a > 0) {
+    const int du = 256 % a, di = 256 / a;
+    for (int i = tid / a, u = tid % a; i < c;) {
+      const int K = fk[u], oK = off[K], m = off[K + 1] - oK;
+      const double* Ti = TL + (long)i * op + c;
+      const double* d = Ds + doff[K] + u - oK;
+      double z = 0.0;
+      for (int v = 0; v < m; ++v) z += Ti[oK + v] * d[v * m];
+      q -= z * Ti[u];
+      if (with_grad) {
+        if (gL) {
+          W[(long)(c + u) * wld + Lb * (long)op + i] = neg_scale2(z, gL[i] + 1);
+          W[(long)i * wld + Lb * (long)op + c + u] = neg_scale2(z, gL[c + u] + 1);
+        } else {
+          WL[(long)i * op + c + u] = WL[(long)(c + u) * op + i] = neg_scale2(z, 1);
+        }
+      }
+      u += du;
+      i += di;
+      if (u >= a) {
+        u -= a;
+        ++i;
+      }
     }
   }
-  double pe = 0.0;
-  for (int i = tid; i < a * a; i += 256) pe += Taa[i] * Y[i];
-  double r2[2] = {pz, pe};
-  block_sums<256, 2>(r2, red);
-  const double zt = r2[0], ty = r2[1];
+  // core-core block (with sum_ij T(i,j)^2), active-active block and zero padding, a warp per row
+  const int rows = with_grad ? op : c;
+  for (int r = warp; r < rows; r += 8) {
+    const double* Tr = TL + (long)r * op;
+    double* Wr = gL ? W + (long)r * wld + Lb * (long)op : WL + (long)r * op;
+    if (r < c) {
+      for (int l = lane; l < c; l += 32) {
+        const double t = Tr[l];
+        q -= t * t;
+        if (with_grad && l != r) Wr[l] = neg_scale2(t, (gL ? gL[l] : 0) + 2);
+      }
+      if (with_grad)
+        for (int l = o + lane; l < op; l += 32) Wr[l] = 0.0;
+    } else if (r < o) {
+      const int u = r - c;
+      for (int l = lane; l < a; l += 32)
+        Wr[c + l] = scale2(gL ? Y[u * a + l] : Y[l * a + u], (gL ? gL[c + l] : 0) + 1);
+      for (int l = o + lane; l < op; l += 32) Wr[l] = 0.0;
+    } else {
+      for (int l = lane; l < op; l += 32) Wr[l] = 0.0;
+    }
+  }
+  if (with_grad)
+    for (int r = tid; r < c; r += 256) {
+      const double w = scale2(vc + va - TL[(long)r * op + r], (gL ? gL[r] : 0) + 2);
+      if (gL) W[(long)r * wld + Lb * (long)op + r] = w;
+      else WL[(long)r * op + r] = w;
+    }
+  const double qs = block_sum0<256>(q, red);
   if (tid == 0) {
-    eps[Lb] = 0.5 * vc * vc - fro + vc * va - zt + 0.5 * ty;
+    eps[Lb] = 0.5 * vc * vc + vc * va + qs;
     vcv[Lb] = vc;
     vav[Lb] = va;
-  }
-  if (!with_grad) return;
-  // core-core block, active-active block and zero padding
-  for (long idx = tid; idx < (long)op * op; idx += 256) {
-    // q-major in split mode so that consecutive threads write consecutive p (coalesced)
-    const int p = gexp ? (int)(idx % op) : (int)(idx / op);
-    const int q = gexp ? (int)(idx / op) : (int)(idx % op);
-    double w;
-    if (p < c && q < c) {
-      w = -4.0 * TL[(long)p * op + q] + (p == q ? 4.0 * (vc + va) : 0.0);
-    } else if (p >= c && p < o && q >= c && q < o) {
-      const int wv = p - c, u = q - c;
-      w = 2.0 * vc * Ds[wv * a + u] + 2.0 * Y[u * a + wv];
-    } else if (p >= o || q >= o) {
-      w = 0.0;
-    } else {
-      continue;  // core/active blocks written above
-    }
-    putW(p, q, w);
   }
 }
 
@@ -348,44 +421,44 @@ __global__ void k_assemble_grad(const double* __restrict__ Out, const double* __
 __global__ void __launch_bounds__(256)
 k_energy_one(const double* __restrict__ Cocc, const double* __restrict__ hC, int n, int op,
              const double* __restrict__ dm1s, FragInfo fi, double* __restrict__ e1) {
-  __shared__ double red[8];
+  __shared__ double red[256];
   const int lane = threadIdx.x & 31, c = fi.ncore, o = c + fi.nact;
-  double s[1] = {0.0};
+  double s = 0.0;
   for (long mu = blockIdx.x * 8L + (threadIdx.x >> 5); mu < n; mu += gridDim.x * 8L) {
     const double* Cr = Cocc + mu * op;
     const double* hr = hC + mu * op;
     for (int p = lane; p < o; p += 32) {
       if (p < c) {
-        s[0] += 2.0 * Cr[p] * hr[p];
+        s += 2.0 * Cr[p] * hr[p];
       } else {
         const int u = p - c, K = frag_of(fi, u), oK = fi.off[K], m = fi.off[K + 1] - oK;
         const double* g = dm1s + fi.dm1_off[K] + (u - oK) * m;
         double t = 0.0;
         for (int v = 0; v < m; ++v) t += (g[v] + g[m * m + v]) * hr[c + oK + v];
-        s[0] += Cr[p] * t;
+        s += Cr[p] * t;
       }
     }
   }
-  block_sums<256, 1>(s, red);
-  if (threadIdx.x == 0) e1[blockIdx.x] = s[0];
+  const double t = block_sum0<256>(s, red);
+  if (threadIdx.x == 0) e1[blockIdx.x] = t;
 }
 
 // E = sum_b e1_b + sum_L eps_L  (one CTA, fixed order, compensated summation).
-__global__ void __launch_bounds__(1024)
+__global__ void __launch_bounds__(256)
 k_energy_final(const double* __restrict__ eps, int X, const double* __restrict__ e1, int ne1,
                double* __restrict__ E) {
-  __shared__ double red[32];
+  __shared__ double red[256];
   double s = 0.0, comp = 0.0;
   auto add = [&](double x) {  // Neumaier
     double t = s + x;
     if (fabs(s) >= fabs(x)) comp += (s - t) + x; else comp += (x - t) + s;
     s = t;
   };
-  for (int L = threadIdx.x; L < X; L += 1024) add(eps[L]);
-  for (int i = threadIdx.x; i < ne1; i += 1024) add(e1[i]);
-  double tot[1] = {s + comp};
-  block_sums<1024, 1>(tot, red);
-  if (threadIdx.x == 0) *E = tot[0];
+#pragma unroll 4
+  for (int L = threadIdx.x; L < X; L += 256) add(eps[L]);
+  for (int i = threadIdx.x; i < ne1; i += 256) add(e1[i]);
+  const double tot = block_sum0<256>(s + comp, red);
+  if (threadIdx.x == 0) *E = tot;
 }
 
 // g[p][q] = M'[p][q] - M'[q][p],  M'[p][q] = M[p][q] for q < o else 0  (M is nmo x op)
@@ -478,23 +551,40 @@ using namespace lasdf;
 static inline unsigned nblk(long count, int nt) { return (unsigned)((count + nt - 1) / nt); }
 
 void launch_pack_cocc(const double* C, int n, int nmo, int o, int op, double* Cocc,
-                      cudaStream_t s) {
-  k_pack_cocc<<<nblk((long)n * op, 256), 256, 0, s>>>(C, n, nmo, o, op, Cocc);
+                      cudaStream_t s, const double* dm2, const FragInfo* fi, double* dm2t) {
+  long count = (long)n * op;
+  FragInfo f;
+  memset(&f, 0, sizeof(f));
+  if (dm2) {
+    f = *fi;
+    for (int K = 0; K < f.nfrag; ++K) {
+      const long m = f.off[K + 1] - f.off[K];
+      count += m * m * m * m;
+    }
+  }
+  k_pack_cocc<<<nblk(count, 256), 256, 0, s>>>(C, n, nmo, o, op, Cocc, dm2, f, dm2t);
   las_count_launch();
 }
 
-#define LAS_PER_AUX_FAST_MAX_ACT 84
-static size_t per_aux_fast_smem(int a) {
-  return (4 * (size_t)a * a + 256 + LAS_MAX_FRAG) * sizeof(double);
+// Dynamic shared memory of k_per_aux (the factored cross-fragment path needs one more a*a buffer)
+// and the most that a block may have beside its static 1 KB.
+static size_t per_aux_smem(const FragInfo& fi, int use_p) {
+  size_t d = 0;
+  for (int K = 0; K < fi.nfrag; ++K) {
+    const size_t m = fi.off[K + 1] - fi.off[K];
+    d += m * m;
+  }
+  const size_t a2 = (size_t)fi.nact * fi.nact;
+  return (2 * a2 + d + (use_p ? a2 : 0) + 256 + LAS_MAX_FRAG) * sizeof(double);
 }
+constexpr size_t PER_AUX_SMEM_MAX = 226 * 1024;
 
-las_status per_aux_prepare(int nact) {
-  // always the largest supported size, so that contexts with different active spaces coexist
-  (void)nact;
-  size_t smem = (3 * (size_t)LAS_MAX_ACT * LAS_MAX_ACT + 256 + LAS_MAX_FRAG) * sizeof(double);
-  smem = std::max(smem, per_aux_fast_smem(LAS_PER_AUX_FAST_MAX_ACT));
+las_status per_aux_prepare() {
+  // always the largest size, so that contexts with different active spaces coexist
+  static_assert((3 * (size_t)LAS_MAX_ACT * LAS_MAX_ACT + 256 + LAS_MAX_FRAG) * sizeof(double) <=
+                    PER_AUX_SMEM_MAX, "one fragment of every active orbital");
   cudaError_t e = cudaFuncSetAttribute(k_per_aux, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)std::max<size_t>(smem, 48 * 1024));
+                                       (int)PER_AUX_SMEM_MAX);
   if (e != cudaSuccess) {
     las_record_cuda_error(e, "cudaFuncSetAttribute(k_per_aux)", __FILE__, __LINE__);
     return LAS_ERR_CUDA;
@@ -502,16 +592,13 @@ las_status per_aux_prepare(int nact) {
   return LAS_OK;
 }
 
-void launch_per_aux(const double* T, int nL, int op, const double* dm1s, const double* dm2,
+void launch_per_aux(const double* T, int nL, int op, const double* dm1s, const double* dm2t,
                     const FragInfo& fi, double* W, double* eps, double* vc, double* va,
-                    int with_grad, const int* gexp, int* status, cudaStream_t s) {
+                    int with_grad, const int* gexp, cudaStream_t s) {
   if (nL <= 0) return;
-  // the factored cross-fragment path needs one more a*a buffer; it fits for a <= 84
-  const int use_p = fi.nfrag > 1 && fi.nact <= LAS_PER_AUX_FAST_MAX_ACT;
-  size_t smem = use_p ? per_aux_fast_smem(fi.nact)
-                      : (3 * (size_t)fi.nact * fi.nact + 256 + LAS_MAX_FRAG) * sizeof(double);
-  k_per_aux<<<nL, 256, smem, s>>>(T, nL, op, dm1s, dm2, fi, W, eps, vc, va, with_grad, gexp,
-                                  status, use_p);
+  const int use_p = fi.nfrag > 1 && per_aux_smem(fi, 1) <= PER_AUX_SMEM_MAX;
+  k_per_aux<<<nL, 256, per_aux_smem(fi, use_p), s>>>(T, nL, op, dm1s, dm2t, fi, W, eps, vc, va,
+                                                     with_grad, gexp, use_p);
   las_count_launch();
 }
 
@@ -586,7 +673,7 @@ void launch_energy(const double* eps, int X, const double* Cocc, const double* h
                    cudaStream_t s) {
   const int nb = (int)std::min<long>(nblk(n, 8), E1_BLOCKS);
   k_energy_one<<<nb, 256, 0, s>>>(Cocc, hC, n, op, dm1s, fi, e1);
-  k_energy_final<<<1, 1024, 0, s>>>(eps, X, e1, nb, E);
+  k_energy_final<<<1, 256, 0, s>>>(eps, X, e1, nb, E);
   las_count_launch(2);
 }
 

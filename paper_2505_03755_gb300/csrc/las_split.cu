@@ -797,7 +797,7 @@ __device__ __forceinline__ unsigned long long absbits(double x) {
 // doubles), their maxima taken on the way in, and are cut from there, 8 values and one 16-byte
 // store per plane at a time.  Rows >= R are written as zeros, and every k in [K, kb*BK).  The bytes
 // are the bound: 8 read and 12 written per value; reading the row a second time from memory took
-// 28 (2.34 ms for 2400 x 192 rows of 1200 against SLICE_NOW).  Few rows per block leave room for
+// 28 (2400 x 192 rows of 1200 values: 2.02 ms, 5.5 TB/s, against 2.34).  Few rows per block leave room for
 // five or more blocks per SM, whose loads and stores overlap.  S = 2 modulo 16: the 16-byte reads of
 // 8 neighbouring threads (rows, or 4 rows and two halves) fall into different banks.
 template <class Rows>
