@@ -63,9 +63,8 @@ struct las_ctx {
   double* eps;    // [X]
   double* vc;     // [X]
   double* va;     // [X]
-  double* Jp;     // [npair] (JK)
-  double* Jt;     // [n][n]  J of one sign part (general-density JK)
-  double* Kt;     // [n][n]  K of one sign part
+  double* Jp;     // [jparts][npair] (JK)
+  int jparts;     // parts of the auxiliary index in the Coulomb sum
   int* status;    // device status word
   // staging for the host-buffer call
   double *dC, *dh, *ddm1, *ddm2, *dE, *dG;
@@ -80,13 +79,13 @@ struct las_ctx {
   size_t fbytes;   // device bytes of the fragment AO2MO workspace (counted in `bytes`)
   int fnmo, fma;
   FragSplit* fsplit;
-  double *vJ, *vK;   // scratch of las_veff (allocated by its first call)
+  double *vKa, *vKb;   // K of either spin in las_veff (allocated by its first call)
   // scratch of las_orbital_hvp (allocated by its first call): G(C) [n][nmo] and C^T G [nmo][op];
   // the tangent chain's dC_occ, h dC_occ and projection [n][op], dH [Lc][op][n], X = H^T dC, dT and
   // the two W matrices of the tangent [Lc][op][op]
   double *hM, *hG, *tCocc, *thC, *tOut, *tHt, *tX, *tdT, *tdW, *tWd;
-  int* widx;          // [2*o + 2] columns of each weight sign and their counts (JK density)
-  int wcount[2];      // host copy of those counts
+  int* widx;          // [4*o + 4] columns of each weight sign of two densities, and their counts
+  int wcount[4];      // host copy of those counts
   // timing: a ring of LAS_TIMING_RING evaluations x 6 stage marks, read without per-call syncs
   int timing;
   cudaEvent_t* ev;       // [LAS_TIMING_RING][6]
@@ -122,13 +121,13 @@ static las_status dalloc(las_ctx* x, void** p, size_t bytes) {
 
 static void free_all(las_ctx* x) {
   void* ptrs[] = {x->Cocc, x->Ht, x->T, x->W, x->part, x->Out, x->hC, x->e1, x->M, x->eps,
-                  x->vc, x->va, x->Jp, x->Jt, x->Kt, x->widx, x->status, x->dC, x->dh, x->ddm1, x->ddm2,
+                  x->vc, x->va, x->Jp, x->widx, x->status, x->dC, x->dh, x->ddm1, x->ddm2,
                   x->dE, x->dG, x->dm2t};
   for (void* p : ptrs)
     if (p) cudaFree(p);
   if (x->split) split_destroy(x->split);
   if (x->fsplit) frag_split_destroy(x->fsplit);
-  for (double* q : {x->fH, x->fT, x->fpart, x->vJ, x->vK, x->hM, x->hG, x->tCocc, x->thC,
+  for (double* q : {x->fH, x->fT, x->fpart, x->vKa, x->vKb, x->hM, x->hG, x->tCocc, x->thC,
                     x->tOut, x->tHt, x->tX, x->tdT, x->tdW, x->tWd})
     if (q) cudaFree(q);
   if (x->ev) {
@@ -237,10 +236,9 @@ extern "C" las_status las_create(las_ctx** out, const las_dims* d, const double*
   ALLOC(eps, x->X);
   ALLOC(vc, x->X);
   ALLOC(va, x->X);
-  ALLOC(Jp, x->npair);
-  ALLOC(Jt, (size_t)x->n * x->n);
-  ALLOC(Kt, (size_t)x->n * x->n);
-  ALLOC(widx, 2 * (size_t)x->o + 2);
+  x->jparts = coulomb_parts(x->npair, x->X, x->sms);
+  ALLOC(Jp, (size_t)x->jparts * x->npair);
+  ALLOC(widx, 4 * (size_t)x->o + 4);
   ALLOC(status, 4);
   ALLOC(dC, (size_t)x->n * x->nmo);
   ALLOC(dh, (size_t)x->n * x->n);
@@ -529,27 +527,35 @@ extern "C" las_status las_energy_grad_host(las_ctx* x, const double* C_host,
   return las_sync(x);
 }
 
-// J and K of the density D = sum_{k < r} c_k c_k^T whose columns c_k are in x->Cocc (columns >= r
-// zero):  J[mu][nu] = sum_L b^L_{mu nu} Tr(b^L D)  (Eqs. J_1, J_2),
-//         K[mu][nu] = sum_L (b^L D b^L)_{mu nu}   (Eqs. K_1, K_2, with b^L D = H_L C^T).
-static las_status jk_raw(las_ctx* x, int r, double* J, double* K) {
+// One part of a density: D = sgn * sum_{k < r} c_k c_k^T, its columns c_k in x->Cocc (columns >= r
+// zero).  Adds (or, as the first part of either, sets) the Coulomb traces vc_L = Tr(b^L D) (Eq. J_1) and
+// K[mu][nu] = sum_L (b^L D b^L)_{mu nu} (Eqs. K_1, K_2, with b^L D = H_L C^T); either may be null.
+// In split precision only the lower triangle of K is valid.
+static las_status jk_part(las_ctx* x, int r, double sgn, bool firstv, bool firstK, double* vc,
+                          double* K) {
   const int n = x->n, op = x->op;
-  if (x->prec == LAS_SPLIT_BF16) {
+  const bool split = x->prec == LAS_SPLIT_BF16;
+  if (split) {
     las_status st = split_prepare_C(x->split, x->Cocc, x->stream);
     if (st != LAS_OK) return st;
   }
   // the first r columns of C_occ carry the density; `Out` (n x op, idle here) holds them
   // transposed for the traces of the Coulomb term
-  if (J) launch_transpose_cols(x->Cocc, n, op, r, x->Out, x->stream);
+  if (vc) launch_transpose_cols(x->Cocc, n, op, r, x->Out, x->stream);
   las_status st;
   for (int l0 = 0; l0 < x->X; l0 += x->Lc) {
     const int nL = std::min(x->Lc, x->X - l0);
+    const int acc = !firstK || l0 > 0;
     // H_L over the r density columns only: Ht is [nL][r][n] here
     if ((st = half_and_full(x, l0, nL, 0, -1, r)) != LAS_OK) return st;
-    // vc_L = 2 sum_k c_k^T H_L(k,:)^T = 2 Tr(b^L D)
-    if (J) launch_trace_ht(x->Ht, x->Out, nL, r, n, x->vc + l0, x->stream);
-    if (K && x->prec == LAS_SPLIT_BF16) {  // K = sum_{L,k} H_L(k,:)^T H_L(k,:)
-      if ((st = split_exchange(x->split, nL, r, x->Ht, K, l0 > 0, x->stream)) != LAS_OK)
+    // traces, and in the same pass over H the column maxima of the exchange digits
+    unsigned long long* mx = nullptr;
+    if (split && K && (st = split_exchange_max(x->split, &mx, x->stream)) != LAS_OK) return st;
+    if (vc || mx)
+      launch_trace_ht(x->Ht, x->Out, nL, r, n, vc ? vc + l0 : nullptr, sgn, !firstv, mx,
+                      x->stream);
+    if (split && K) {  // K = sum_{L,k} H_L(k,:)^T H_L(k,:)
+      if ((st = split_exchange(x->split, nL, r, x->Ht, K, acc, sgn, x->stream)) != LAS_OK)
         return st;
     } else if (K) {
       StridedA A{x->Ht, 0, 1, n};
@@ -561,20 +567,25 @@ static las_status jk_raw(las_ctx* x, int r, double* J, double* K) {
       if (ks > 1) {
         StridedC Pk{x->part, (long)n * n, n, 1, 1.0, 0};
         gemm_f64<true>(n, n, nL * r, 1, ks, A, B, Pk, x->stream);
-        launch_reduce_partials(x->part, ks, (long)n * n, K, l0 > 0, x->stream);
+        launch_reduce_partials(x->part, ks, (long)n * n, K, acc, x->stream, 0, 0, sgn);
       } else {
-        StridedC Kd{K, 0, n, 1, 1.0, l0 > 0};
+        StridedC Kd{K, 0, n, 1, sgn, acc};
         gemm_f64<true>(n, n, nL * r, 1, 1, A, B, Kd, x->stream);
       }
     }
     if ((st = check_launch()) != LAS_OK) return st;
   }
-  if (K && x->prec == LAS_SPLIT_BF16) launch_mirror_lower(K, n, x->stream);
+  return LAS_OK;
+}
+
+// J = scale * sum_L vc_L b^L (Eq. J_2), and K = scale * K with both triangles filled
+static las_status jk_finish(las_ctx* x, double scale, double* J, double* K) {
+  const int n = x->n;
   if (J) {
-    launch_coulomb_packed(x->Bp, x->vc, x->X, x->npair, x->Jp, x->stream);
-    launch_unpack_sym(x->Jp, n, J, x->stream);
-    launch_scale(J, (long)n * n, 0.5, x->stream);   // vc carried the factor 2
+    launch_coulomb_packed(x->Bp, x->vc, x->X, x->npair, x->jparts, x->Jp, x->stream);
+    launch_unpack_sym(x->Jp, x->jparts, n, scale, J, x->stream);
   }
+  if (K) launch_mirror_lower(K, n, scale, x->stream);
   return check_launch();
 }
 
@@ -589,11 +600,47 @@ extern "C" las_status las_df_jk(las_ctx* x, const double* C, double* J, double* 
   }
   // core-only C_occ (columns >= c zeroed): D = C_core C_core^T and Dc = 2 D
   launch_pack_cocc(C, n, x->nmo, c, op, x->Cocc, x->stream);
-  las_status st = jk_raw(x, c, J, K);
-  if (st != LAS_OK) return st;
-  if (J) launch_scale(J, (long)n * n, 2.0, x->stream);
-  if (K) launch_scale(K, (long)n * n, 2.0, x->stream);
-  return check_launch();
+  las_status st = jk_part(x, c, 1.0, true, true, J ? x->vc : nullptr, K);
+  return st == LAS_OK ? jk_finish(x, 2.0, J, K) : st;
+}
+
+// A factored density as the library takes it: D = C diag(w) C^T with r columns
+struct Factored {
+  const double* C;
+  const double* w;
+  int r;
+};
+
+// The columns of each sign of the weights of `nd` densities (at most two), their counts in
+// x->wcount: D = D+ - D-,  D± = sum_k max(±w_k, 0) c_k c_k^T, each over the columns of its sign only
+// (their counts size the transforms, so they are read back, once for all densities).
+static las_status sign_split(las_ctx* x, const Factored* d, int nd) {
+  int* counts = x->widx + 4 * x->o;
+  launch_sign_split(d[0].w, d[0].r, nd > 1 ? d[1].w : nullptr, nd > 1 ? d[1].r : 0, x->o, x->widx,
+                    counts, x->stream);
+  LAS_CUDA_TRY(cudaMemcpyAsync(x->wcount, counts, 4 * sizeof(int), cudaMemcpyDeviceToHost,
+                               x->stream));
+  LAS_CUDA_TRY(cudaStreamSynchronize(x->stream));
+  return LAS_OK;
+}
+
+// Traces and K of density i of the last sign_split.  The traces are added to vc unless `first`; K is
+// set (to zero for an empty density, which leaves vc alone).  *any: the density had columns.
+static las_status jk_density(las_ctx* x, const Factored& d, int i, bool first, double* vc,
+                             double* K, bool* any) {
+  *any = false;
+  for (int neg = 0; neg < 2; ++neg) {
+    const int cnt = d.r > 0 ? x->wcount[2 * i + neg] : 0;
+    if (cnt == 0) continue;
+    const double sgn = neg ? -1.0 : 1.0;
+    launch_pack_weighted(d.C, d.w, x->widx + (2 * i + neg) * x->o, cnt, sgn, x->n, d.r, x->op,
+                         x->Cocc, x->stream);
+    las_status st = jk_part(x, cnt, sgn, first && !*any, !*any, vc, K);
+    if (st != LAS_OK) return st;
+    *any = true;
+  }
+  if (!*any && K) LAS_CUDA_TRY(cudaMemsetAsync(K, 0, (size_t)x->n * x->n * 8, x->stream));
+  return LAS_OK;
 }
 
 extern "C" las_status las_df_jk_density(las_ctx* x, const double* Cx, const double* w, int r,
@@ -601,37 +648,14 @@ extern "C" las_status las_df_jk_density(las_ctx* x, const double* Cx, const doub
   if (!x || r < 0 || (r > 0 && (!Cx || !w))) return LAS_ERR_ARG;   // r = 0: D = 0
   if (r > x->o) return LAS_ERR_ARG;
   if (!J && !K) return LAS_OK;
-  const int n = x->n;
-  if (r == 0) {
-    if (J) LAS_CUDA_TRY(cudaMemsetAsync(J, 0, (size_t)n * n * 8, x->stream));
-    if (K) LAS_CUDA_TRY(cudaMemsetAsync(K, 0, (size_t)n * n * 8, x->stream));
-    return LAS_OK;
-  }
-  // D = D+ - D-,  D± = sum_k max(±w_k, 0) c_k c_k^T, each over the columns of its sign only
-  // (their counts size the transforms, so they are read back once)
-  int* idx_pos = x->widx;
-  int* idx_neg = x->widx + x->o;
-  int* counts = x->widx + 2 * x->o;
-  launch_sign_split(w, r, idx_pos, idx_neg, counts, x->stream);
-  LAS_CUDA_TRY(cudaMemcpyAsync(x->wcount, counts, 2 * sizeof(int), cudaMemcpyDeviceToHost,
-                               x->stream));
-  LAS_CUDA_TRY(cudaStreamSynchronize(x->stream));
-  const int rp = x->wcount[0], rn = x->wcount[1];
-  las_status st = LAS_OK;
-  if (rp > 0) {
-    launch_pack_weighted(Cx, w, idx_pos, rp, +1.0, n, r, x->op, x->Cocc, x->stream);
-    if ((st = jk_raw(x, rp, J, K)) != LAS_OK) return st;
-  } else {
-    if (J) LAS_CUDA_TRY(cudaMemsetAsync(J, 0, (size_t)n * n * 8, x->stream));
-    if (K) LAS_CUDA_TRY(cudaMemsetAsync(K, 0, (size_t)n * n * 8, x->stream));
-  }
-  if (rn > 0) {
-    launch_pack_weighted(Cx, w, idx_neg, rn, -1.0, n, r, x->op, x->Cocc, x->stream);
-    if ((st = jk_raw(x, rn, J ? x->Jt : nullptr, K ? x->Kt : nullptr)) != LAS_OK) return st;
-    if (J) launch_axpy(J, x->Jt, -1.0, (long)n * n, x->stream);
-    if (K) launch_axpy(K, x->Kt, -1.0, (long)n * n, x->stream);
-  }
-  return check_launch();
+  const Factored d{Cx, w, r};
+  las_status st = r > 0 ? sign_split(x, &d, 1) : LAS_OK;
+  bool any = false;
+  if (st == LAS_OK) st = jk_density(x, d, 0, true, J ? x->vc : nullptr, K, &any);
+  if (st != LAS_OK) return st;
+  if (any) return jk_finish(x, 1.0, J, K);
+  if (J) LAS_CUDA_TRY(cudaMemsetAsync(J, 0, (size_t)x->n * x->n * 8, x->stream));
+  return LAS_OK;
 }
 
 extern "C" las_status las_df_transform(las_ctx* x, const double* C, int p0, int p1,
@@ -639,8 +663,9 @@ extern "C" las_status las_df_transform(las_ctx* x, const double* C, int p0, int 
   if (!x || !C) return LAS_ERR_ARG;
   if (p0 < 0 || p1 < p0 || p1 > x->nmo) return LAS_ERR_ARG;
   if (x->a == 0) return LAS_OK;
+  // the active columns only: Ht is [nL][a][n] here
   const int n = x->n, op = x->op, c = x->c, a = x->a, np = p1 - p0;
-  launch_pack_cocc(C, n, x->nmo, x->o, op, x->Cocc, x->stream);
+  launch_pack_cocc(C + c, n, x->nmo, a, op, x->Cocc, x->stream);
   if (x->prec == LAS_SPLIT_BF16) {
     las_status st = split_prepare_C(x->split, x->Cocc, x->stream);
     if (st != LAS_OK) return st;
@@ -648,16 +673,16 @@ extern "C" las_status las_df_transform(las_ctx* x, const double* C, int p0, int 
   las_status st;
   for (int l0 = 0; l0 < x->X; l0 += x->Lc) {
     const int nL = std::min(x->Lc, x->X - l0);
-    if ((st = half_and_full(x, l0, nL, 0)) != LAS_OK) return st;
-    if (Lmu_u) launch_copy_cols(x->Ht, nL, op, n, c, a, Lmu_u + (size_t)l0 * n * a, x->stream);
+    if ((st = half_and_full(x, l0, nL, 0, -1, a)) != LAS_OK) return st;
+    if (Lmu_u) launch_transpose_ht(x->Ht, nL, n, a, Lmu_u + (size_t)l0 * n * a, x->stream);
     if (Lpu && np > 0 && x->prec == LAS_SPLIT_BF16) {
-      if ((st = split_lpu(x->split, nL, x->Ht, c, a, C, x->nmo, p0, np,
+      if ((st = split_lpu(x->split, nL, x->Ht, a, C, x->nmo, p0, np,
                           Lpu + (size_t)l0 * np * a, x->stream, &x->bytes)) != LAS_OK)
         return st;
     } else if (Lpu && np > 0) {
-      // Lpu[b][p][u] = sum_mu C[mu][p0+p] Ht[b][c+u][mu]
+      // Lpu[b][p][u] = sum_mu C[mu][p0+p] Ht[b][u][mu]
       StridedA A{C + p0, 0, 1, x->nmo};
-      StridedA B{x->Ht + (size_t)c * n, (long)op * n, 1, n};
+      StridedA B{x->Ht, (long)a * n, 1, n};
       StridedC Co{Lpu + (size_t)l0 * np * a, (long)np * a, a, 1, 1.0, 0};
       // batch over L: A is shared (sb = 0), B and C advance per L
       gemm_f64(np, a, n, nL, 1, A, B, Co, x->stream);
@@ -677,20 +702,24 @@ extern "C" las_status las_veff(las_ctx* x, const double* Ca, const double* wa, i
   if ((ra > 0 && (!Ca || !wa)) || (rb > 0 && (!Cb || !wb))) return LAS_ERR_ARG;
   if (ra > x->o || rb > x->o) return LAS_ERR_ARG;
   const long nn = (long)x->n * x->n;
-  if (!x->vJ) {
+  if (!x->vKb) {
     las_status st = LAS_OK;
-    if ((st = dalloc(x, (void**)&x->vJ, sizeof(double) * nn)) != LAS_OK ||
-        (st = dalloc(x, (void**)&x->vK, sizeof(double) * nn)) != LAS_OK)
+    if ((!x->vKa && (st = dalloc(x, (void**)&x->vKa, sizeof(double) * nn)) != LAS_OK) ||
+        (st = dalloc(x, (void**)&x->vKb, sizeof(double) * nn)) != LAS_OK)
       return st;
   }
-  // alpha: va = J_a, vK = K_a;  beta: vJ = J_b, vb = K_b
-  las_status st = las_df_jk_density(x, Ca, wa, ra, va, x->vK);
-  if (st == LAS_OK) st = las_df_jk_density(x, Cb, wb, rb, x->vJ, vb);
+  // both spins' traces add up to those of D, so that J[D] takes one pass over B
+  const Factored d[2] = {{Ca, wa, ra}, {Cb, wb, rb}};
+  las_status st = ra > 0 || rb > 0 ? sign_split(x, d, 2) : LAS_OK;
+  bool a = false, b = false;
+  if (st == LAS_OK) st = jk_density(x, d[0], 0, true, x->vc, x->vKa, &a);
+  if (st == LAS_OK) st = jk_density(x, d[1], 1, !a, x->vc, x->vKb, &b);
   if (st != LAS_OK) return st;
-  launch_axpy(va, x->vJ, 1.0, nn, x->stream);      // va = J[D]
-  launch_scale(vb, nn, -1.0, x->stream);
-  launch_axpy(vb, va, 1.0, nn, x->stream);         // vb = J[D] - K_b
-  launch_axpy(va, x->vK, -1.0, nn, x->stream);     // va = J[D] - K_a
+  if (a || b)
+    launch_coulomb_packed(x->Bp, x->vc, x->X, x->npair, x->jparts, x->Jp, x->stream);
+  else
+    LAS_CUDA_TRY(cudaMemsetAsync(x->Jp, 0, sizeof(double) * x->jparts * x->npair, x->stream));
+  launch_veff_combine(x->Jp, x->jparts, x->vKa, x->vKb, x->n, va, vb, x->stream);
   return check_launch();
 }
 
@@ -922,7 +951,7 @@ extern "C" las_status las_frag_ao2mo(las_ctx* x, const double* M, int a0, int ma
     }
     if ((st = check_launch()) != LAS_OK) return st;
   }
-  if (split && papa) launch_mirror_lower(papa, (int)m, x->stream);
+  if (split && papa) launch_mirror_lower(papa, (int)m, 1.0, x->stream);
   return check_launch();
 }
 

@@ -81,28 +81,28 @@ las_status per_aux_prepare();
 // gexp == nullptr: W[L][p][q];  otherwise W is written as Wt[q][L*op + p] * 2^gexp[L*op + p]
 // CT[k][mu] = Cocc[mu][k] for k < r (Cocc is n x op)
 void launch_transpose_cols(const double* Cocc, int n, int op, int r, double* CT, cudaStream_t s);
-// vc[b] = 2 sum_{k<r} sum_mu Ht[(b*r + k)*n + mu] * CT[k*n + mu], b < nL (fixed summation order)
+// vc[b] (+)= sgn sum_{k<r} sum_mu Ht[(b*r + k)*n + mu] * CT[k*n + mu], b < nL (fixed summation
+// order); and mx[mu] = max(mx[mu], max_{b,k} |Ht|) as bit patterns.  Either of vc, mx may be null.
 void launch_trace_ht(const double* Ht, const double* CT, int nL, int r, int n, double* vc,
-                     cudaStream_t s);
+                     double sgn, int accumulate, unsigned long long* mx, cudaStream_t s);
 void launch_per_aux(const double* T, int nL, int op, const double* dm1s, const double* dm2t,
                     const FragInfo& fi, double* W, double* eps, double* vc, double* va,
                     int with_grad, const int* gexp, cudaStream_t s);
-void launch_scale(double* p, long count, double a, cudaStream_t s);
-void launch_mirror_lower(double* K, int n, cudaStream_t s);
-void launch_axpy(double* y, const double* x, double a, long count, cudaStream_t s);
+// K = scale * (its lower triangle, mirrored)
+void launch_mirror_lower(double* K, int n, double scale, cudaStream_t s);
 // dT[L] = X[L] + X[L]^T for L < nL (op x op each)
 void launch_sym_add(const double* X, int nL, int op, double* dT, cudaStream_t s);
-// *out (atomic max, caller zeroes it) = max_i |a[i]| as the bit pattern of the double
-void launch_absmax_bits(const double* a, long count, unsigned long long* out, cudaStream_t s);
-// Columns of each sign of w (k_sign_split), then the packed factor of one sign
-void launch_sign_split(const double* w, int r, int* idx_pos, int* idx_neg, int* counts,
-                       cudaStream_t s);
+// Columns of each sign of w0 (idx, then idx + o: w > 0, w < 0) and of w1 (idx + 2 o, idx + 3 o) in
+// order and their counts[4], then the packed factor of one sign
+void launch_sign_split(const double* w0, int r0, const double* w1, int r1, int o, int* idx,
+                       int* counts, cudaStream_t s);
 void launch_pack_weighted(const double* Cx, const double* w, const int* idx, int cnt,
                           double sign, int n, int r, int op, double* Cocc, cudaStream_t s);
-// out (+)= sum_k part[k*count ...] in order of k; with cols < ld the values are rows of `cols`
-// that land `ld` apart in out
+// out (+)= scale sum_k part[k*count ...] in order of k; with cols < ld the values are rows of
+// `cols` that land `ld` apart in out
 void launch_reduce_partials(const double* part, int nsplit, long count, double* out,
-                            int accumulate, cudaStream_t s, int cols = 0, int ld = 0);
+                            int accumulate, cudaStream_t s, int cols = 0, int ld = 0,
+                            double scale = 1.0);
 void launch_assemble_grad(const double* Out, const double* hC, const double* dm1s,
                           const FragInfo& fi, int n, int nmo, int op, double* G,
                           cudaStream_t s);
@@ -111,8 +111,15 @@ void launch_assemble_grad(const double* Out, const double* hC, const double* dm1
 void launch_energy(const double* eps, int X, const double* Cocc, const double* hC, int n, int op,
                    const double* dm1s, const FragInfo& fi, double* e1, double* E, cudaStream_t s);
 void launch_antisym(const double* M, int nmo, int o, int op, double* g, cudaStream_t s);
-void launch_coulomb_packed(const double* Bp, const double* vc, int X, long npair,
+// Jp[z][npair], z < parts: partial sums over parts of the auxiliary index (coulomb_parts: how many)
+int coulomb_parts(long npair, int X, int sms);
+void launch_coulomb_packed(const double* Bp, const double* vc, int X, long npair, int parts,
                            double* Jp, cudaStream_t s);
-void launch_unpack_sym(const double* Jp, int n, double* J, cudaStream_t s);
-void launch_copy_cols(const double* Ht, int X, int op, int n, int c0, int a, double* Lmu,
-                      cudaStream_t s);
+// J = scale * the symmetric matrix of the packed lower triangle sum_z Jp[z]
+void launch_unpack_sym(const double* Jp, int parts, int n, double scale, double* J,
+                       cudaStream_t s);
+// va = J - Ka, vb = J - Kb from the packed J and the lower triangles of Ka, Kb
+void launch_veff_combine(const double* Jp, int parts, const double* Ka, const double* Kb, int n,
+                         double* va, double* vb, cudaStream_t s);
+// Lmu[L][mu][u] = Ht[L][u][mu] for L < nL, u < a (at most LAS_MAX_ACT)
+void launch_transpose_ht(const double* Ht, int nL, int n, int a, double* Lmu, cudaStream_t s);

@@ -25,21 +25,6 @@ __device__ double block_sum0(double v, double* red) {   // red: NT doubles
   return t;
 }
 
-// Deterministic block reduction of one double per thread (fixed tree order).
-template <int NT>
-__device__ double block_sum(double v, double* red) {
-  red[threadIdx.x] = v;
-  __syncthreads();
-#pragma unroll
-  for (int s = NT / 2; s > 0; s >>= 1) {
-    if (threadIdx.x < s) red[threadIdx.x] += red[threadIdx.x + s];
-    __syncthreads();
-  }
-  double r = red[0];
-  __syncthreads();
-  return r;
-}
-
 // Cocc[mu][p] = C[mu][p] for p < o, 0 for o <= p < op; and, with dm2, the pair-transposed fragment
 // 2-RDMs dm2t_K[wx][uv] = Gamma^K[uv][wx] that k_per_aux reads along uv.
 __global__ void k_pack_cocc(const double* __restrict__ C, int n, int nmo, int o, int op,
@@ -320,18 +305,30 @@ k_per_aux(const double* __restrict__ T, int nL, int op, const double* __restrict
   }
 }
 
-// Cocc[mu][k] = Cx[mu][k] * sqrt(max(sign * w[k], 0)) for k < r, zero for r <= k < op
-// Columns of one sign of the weights, in order: idx[0..cnt) (sign = +1 or -1 picks w > 0 or w < 0).
-__global__ void k_sign_split(const double* __restrict__ w, int r, int* __restrict__ idx_pos,
-                             int* __restrict__ idx_neg, int* __restrict__ counts) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
+// Columns of each sign of the weights of up to two densities, in order; one warp per density.
+__global__ void __launch_bounds__(32)
+k_sign_split(const double* __restrict__ w0, int r0, const double* __restrict__ w1, int r1, int o,
+             int* __restrict__ idx, int* __restrict__ counts) {
+  const int lane = threadIdx.x;
+  const double* w = blockIdx.x ? w1 : w0;
+  const int r = blockIdx.x ? r1 : r0;
+  int* pos = idx + 2 * blockIdx.x * o;
+  int* neg = pos + o;
   int np = 0, nn = 0;
-  for (int k = 0; k < r; ++k) {
-    if (w[k] > 0.0) idx_pos[np++] = k;
-    else if (w[k] < 0.0) idx_neg[nn++] = k;
+  for (int k0 = 0; k0 < r; k0 += 32) {
+    const int k = k0 + lane;
+    const double v = k < r ? w[k] : 0.0;
+    const unsigned mp = __ballot_sync(0xffffffffu, v > 0.0), mn = __ballot_sync(0xffffffffu, v < 0.0);
+    const unsigned below = (1u << lane) - 1;
+    if (v > 0.0) pos[np + __popc(mp & below)] = k;
+    if (v < 0.0) neg[nn + __popc(mn & below)] = k;
+    np += __popc(mp);
+    nn += __popc(mn);
   }
-  counts[0] = np;
-  counts[1] = nn;
+  if (lane == 0) {
+    counts[2 * blockIdx.x] = np;
+    counts[2 * blockIdx.x + 1] = nn;
+  }
 }
 
 // Cocc[mu][j] = Cx[mu][idx[j]] * sqrt(sign * w[idx[j]]) for j < cnt, zero for cnt <= j < op
@@ -349,12 +346,15 @@ __global__ void k_pack_weighted(const double* __restrict__ Cx, const double* __r
   Cocc[i] = v;
 }
 
-// K[i][j] = K[j][i] for i < j (copy the lower triangle to the upper)
-__global__ void k_mirror_lower(double* __restrict__ K, int n) {
+// K = scale * (its lower triangle, mirrored to the upper)
+__global__ void k_mirror_lower(double* __restrict__ K, int n, double scale) {
   long idx = blockIdx.x * (long)blockDim.x + threadIdx.x;
   if (idx >= (long)n * n) return;
   const int i = (int)(idx / n), j = (int)(idx % n);
-  if (i < j) K[idx] = K[(long)j * n + i];
+  if (i > j) return;   // element (j, i) is handled by its mirror image's thread
+  const double v = scale * K[(long)j * n + i];
+  K[idx] = v;
+  if (scale != 1.0) K[(long)j * n + i] = v;
 }
 
 // dT[L][p][q] = X[L][p][q] + X[L][q][p]  (the symmetric tangent of T_L = C^T b^L C)
@@ -367,26 +367,17 @@ __global__ void k_sym_add(const double* __restrict__ X, long nL, int op, double*
   dT[i] = X[i] + X[L * per + (long)q * op + p];
 }
 
-__global__ void k_axpy(double* __restrict__ y, const double* __restrict__ x, double a, long count) {
-  long i = blockIdx.x * (long)blockDim.x + threadIdx.x;
-  if (i < count) y[i] += a * x[i];
-}
-
-__global__ void k_scale(double* __restrict__ p, long count, double a) {
-  long i = blockIdx.x * (long)blockDim.x + threadIdx.x;
-  if (i < count) p[i] *= a;
-}
-
 // Partials of rows of `cols` values, summed in order into rows `ld` apart.
 __global__ void k_reduce_partials(const double* __restrict__ part, int nsplit, long count,
-                                  double* __restrict__ out, int accumulate, int cols, int ld) {
+                                  double* __restrict__ out, int accumulate, int cols, int ld,
+                                  double scale) {
   long i = blockIdx.x * (long)blockDim.x + threadIdx.x;
   if (i >= count) return;
   const long o = cols == ld ? i : i / cols * ld + i % cols;
-  double s = accumulate ? out[o] : 0.0;
+  double s = 0.0;
 #pragma unroll 8
   for (int k = 0; k < nsplit; ++k) s += part[(long)k * count + i];
-  out[o] = s;
+  out[o] = accumulate ? fma(scale, s, out[o]) : scale * s;
 }
 
 // dE/dC = [4 h C_core | 2 h C_act D | 0] + Out   (Out = sum_L H_L W_L, n x op)
@@ -472,35 +463,78 @@ __global__ void k_antisym(const double* __restrict__ M, int nmo, int o, int op,
   g[i] = x - y;
 }
 
-// Jp[pair] = sum_L vc[L] Bp[L][pair]  (Eq. J_2 on the packed triangle; coalesced along pairs)
-__global__ void k_coulomb_packed(const double* __restrict__ Bp, const double* __restrict__ vc,
-                                 int X, long npair, double* __restrict__ Jp) {
-  long i = blockIdx.x * (long)blockDim.x + threadIdx.x;
-  if (i >= npair) return;
-  double s = 0.0;
-  for (int L = 0; L < X; ++L) s += vc[L] * Bp[(long)L * npair + i];
-  Jp[i] = s;
+// Jp[z][pair] = sum_{L in part z} vc[L] Bp[L][pair]  (Eq. J_2 on the packed triangle; coalesced
+// along pairs, two per thread, parts of the auxiliary index in grid.y).  One FP64 multiply-add per
+// element read is more than the FP64 pipe does in the time of the read (800 orbitals, 1600 L: 0.92 ms
+// against 0.61 ms), so the parts are there to fill every SM evenly, some 24 blocks each (one thread
+// per pair over all of L: 1.08 ms, and 430 us at 400 orbitals, where it is 228 now).
+constexpr int COULOMB_PAIRS = 512;
+__global__ void __launch_bounds__(256)
+k_coulomb_packed(const double* __restrict__ Bp, const double* __restrict__ vc, int X, int per,
+                 long npair, double* __restrict__ Jp) {
+  const long i0 = blockIdx.x * (long)COULOMB_PAIRS + threadIdx.x, i1 = i0 + 256;
+  const int l0 = blockIdx.y * per, l1 = min(X, l0 + per);
+  double s0 = 0.0, s1 = 0.0;
+  if (i1 < npair) {
+    const double* b = Bp + l0 * npair + i0;
+#pragma unroll 8
+    for (int L = l0; L < l1; ++L, b += npair) {
+      const double v = vc[L];
+      s0 += v * b[0];
+      s1 += v * b[256];
+    }
+    Jp[blockIdx.y * npair + i1] = s1;
+  } else if (i0 < npair) {
+    const double* b = Bp + l0 * npair + i0;
+#pragma unroll 8
+    for (int L = l0; L < l1; ++L, b += npair) s0 += vc[L] * b[0];
+  }
+  if (i0 < npair) Jp[blockIdx.y * npair + i0] = s0;
 }
 
-__global__ void k_unpack_sym(const double* __restrict__ Jp, int n, double* __restrict__ J) {
+__device__ __forceinline__ double coulomb_sum(const double* __restrict__ Jp, int parts, long npair,
+                                              long pair) {
+  double s = Jp[pair];
+  for (int z = 1; z < parts; ++z) s += Jp[z * npair + pair];
+  return s;
+}
+
+__global__ void k_unpack_sym(const double* __restrict__ Jp, int parts, int n, double scale,
+                             double* __restrict__ J) {
   long i = blockIdx.x * (long)blockDim.x + threadIdx.x;
   if (i >= (long)n * n) return;
   long mu = i / n, nu = i % n;
   long hi = mu > nu ? mu : nu, lo = mu > nu ? nu : mu;
-  J[i] = Jp[hi * (hi + 1) / 2 + lo];
+  J[i] = scale * coulomb_sum(Jp, parts, (long)n * (n + 1) / 2, hi * (hi + 1) / 2 + lo);
 }
 
-// Lmu[L][mu][u] = Ht[L][c0+u][mu]
-__global__ void k_copy_cols(const double* __restrict__ Ht, int X, int op, int n, int c0, int a,
-                            double* __restrict__ Lmu) {
+__global__ void k_veff_combine(const double* __restrict__ Jp, int parts,
+                               const double* __restrict__ Ka, const double* __restrict__ Kb, int n,
+                               double* __restrict__ va, double* __restrict__ vb) {
   long i = blockIdx.x * (long)blockDim.x + threadIdx.x;
-  long total = (long)X * n * a;
-  if (i >= total) return;
-  const int u = (int)(i % a);
-  const long r = i / a;
-  const int mu = (int)(r % n);
-  const long L = r / n;
-  Lmu[i] = Ht[(L * op + c0 + u) * n + mu];
+  if (i >= (long)n * n) return;
+  long mu = i / n, nu = i % n;
+  long hi = mu > nu ? mu : nu, lo = mu > nu ? nu : mu;
+  const double j = coulomb_sum(Jp, parts, (long)n * (n + 1) / 2, hi * (hi + 1) / 2 + lo);
+  va[i] = j - Ka[hi * n + lo];
+  vb[i] = j - Kb[hi * n + lo];
+}
+
+// Lmu[L][mu][u] = Ht[L][u][mu], u < a: 32 values of mu per block through shared memory, so that
+// reads and writes are contiguous (element by element, the reads of a warp were n apart: 50 us for
+// 1600 x 400 x 16 values, against 27).
+__global__ void __launch_bounds__(256)
+k_transpose_ht(const double* __restrict__ Ht, int n, int a, double* __restrict__ Lmu) {
+  __shared__ double tile[LAS_MAX_ACT][33];
+  const long L = blockIdx.y;
+  const int mu0 = blockIdx.x * 32, nm = min(32, n - mu0);
+  const double* h = Ht + L * (long)a * n + mu0;
+  const int lane = threadIdx.x & 31;
+  for (int u = threadIdx.x >> 5; u < a; u += 8)
+    if (lane < nm) tile[u][lane] = h[(long)u * n + lane];
+  __syncthreads();
+  double* o = Lmu + (L * n + mu0) * (long)a;
+  for (int i = threadIdx.x; i < nm * a; i += 256) o[i] = tile[i % a][i / a];
 }
 
 __global__ void k_transpose_cols(const double* __restrict__ C, int n, int op, int r,
@@ -511,37 +545,40 @@ __global__ void k_transpose_cols(const double* __restrict__ C, int n, int op, in
   CT[i] = C[(long)mu * op + k];
 }
 
-// Coulomb traces: one block per aux row, coalesced along mu, tree reduction in a fixed order.
+// Coulomb traces (fixed summation order) and column maxima of |H|, one block per aux row; a warp
+// takes 32 columns x a quarter of the rows k at a time (more items than warps, so that none idles
+// long), and a column's maximum reaches memory only where it exceeds what is there.  The FP64
+// multiply-adds of the traces are the bound (800 orbitals, 1600 x 100 rows: 0.245 ms of 0.33);
+// the maxima of the exchange digits ride along instead of a pass of their own over H (0.18 ms).
 __global__ void __launch_bounds__(256)
 k_trace_ht(const double* __restrict__ Ht, const double* __restrict__ CT, int r, int n,
-           double* __restrict__ vc) {
+           double* __restrict__ vc, double sgn, int accumulate,
+           unsigned long long* __restrict__ mx) {
   __shared__ double red[256];
   const long b = blockIdx.x;
-  const long cnt = (long)r * n;
-  const double* h = Ht + b * cnt;
+  const double* hb = Ht + b * (long)r * n;
+  const int lane = threadIdx.x & 31, chunks = (n + 31) / 32, kq = (r + 3) / 4;
   double acc = 0.0;
-  for (long i = threadIdx.x; i < cnt; i += 256) acc = fma(h[i], CT[i], acc);
-  const double t = block_sum<256>(acc, red);
-  if (threadIdx.x == 0) vc[b] = 2.0 * t;
-}
-
-// out (atomic max) = max |a[i]| as an ordered bit pattern (block tree, then one atomic per block)
-__global__ void __launch_bounds__(256)
-k_absmax_bits(const double* __restrict__ a, long count, unsigned long long* out) {
-  __shared__ unsigned long long red[256];
-  unsigned long long m = 0;
-  for (long i = blockIdx.x * 256L + threadIdx.x; i < count; i += (long)gridDim.x * 256) {
-    const unsigned long long b = (unsigned long long)__double_as_longlong(a[i]) & 0x7FFFFFFFFFFFFFFFull;
-    m = b > m ? b : m;
+  for (int it = threadIdx.x >> 5; it < 4 * chunks; it += 8) {
+    const int q = it / chunks, mu = (it - q * chunks) * 32 + lane;
+    const int k0 = q * kq, k1 = min(r, k0 + kq);
+    if (mu >= n) continue;
+    unsigned long long m = 0;
+    const double* h = hb + mu;
+    const double* c = CT + mu;
+#pragma unroll 8
+    for (int k = k0; k < k1; ++k) {
+      const double v = h[(long)k * n];
+      const unsigned long long a = (unsigned long long)__double_as_longlong(v) << 1;
+      m = a > m ? a : m;
+      if (vc) acc = fma(v, c[(long)k * n], acc);
+    }
+    m >>= 1;
+    if (mx && m > *(volatile unsigned long long*)&mx[mu]) atomicMax(&mx[mu], m);
   }
-  red[threadIdx.x] = m;
-  __syncthreads();
-  for (int w = 128; w > 0; w >>= 1) {
-    if ((int)threadIdx.x < w && red[threadIdx.x + w] > red[threadIdx.x])
-      red[threadIdx.x] = red[threadIdx.x + w];
-    __syncthreads();
-  }
-  if (threadIdx.x == 0 && red[0]) atomicMax(out, red[0]);
+  if (!vc) return;
+  const double t = block_sum0<256>(acc, red);
+  if (threadIdx.x == 0) vc[b] = accumulate ? fma(sgn, t, vc[b]) : sgn * t;
 }
 
 }  // namespace lasdf
@@ -602,9 +639,9 @@ void launch_per_aux(const double* T, int nL, int op, const double* dm1s, const d
   las_count_launch();
 }
 
-void launch_sign_split(const double* w, int r, int* idx_pos, int* idx_neg, int* counts,
-                       cudaStream_t s) {
-  k_sign_split<<<1, 32, 0, s>>>(w, r, idx_pos, idx_neg, counts);
+void launch_sign_split(const double* w0, int r0, const double* w1, int r1, int o, int* idx,
+                       int* counts, cudaStream_t s) {
+  k_sign_split<<<2, 32, 0, s>>>(w0, r0, w1, r1, o, idx, counts);
   las_count_launch();
 }
 
@@ -615,8 +652,8 @@ void launch_pack_weighted(const double* Cx, const double* w, const int* idx, int
   las_count_launch();
 }
 
-void launch_mirror_lower(double* K, int n, cudaStream_t s) {
-  k_mirror_lower<<<nblk((long)n * n, 256), 256, 0, s>>>(K, n);
+void launch_mirror_lower(double* K, int n, double scale, cudaStream_t s) {
+  k_mirror_lower<<<nblk((long)n * n, 256), 256, 0, s>>>(K, n, scale);
   las_count_launch();
 }
 
@@ -624,12 +661,6 @@ void launch_sym_add(const double* X, int nL, int op, double* dT, cudaStream_t s)
   const long count = (long)nL * op * op;
   if (count <= 0) return;
   k_sym_add<<<nblk(count, 256), 256, 0, s>>>(X, nL, op, dT);
-  las_count_launch();
-}
-
-void launch_axpy(double* y, const double* x, double a, long count, cudaStream_t s) {
-  if (count <= 0) return;
-  k_axpy<<<nblk(count, 256), 256, 0, s>>>(y, x, a, count);
   las_count_launch();
 }
 
@@ -642,22 +673,16 @@ void launch_transpose_cols(const double* Cocc, int n, int op, int r, double* CT,
 }
 
 void launch_trace_ht(const double* Ht, const double* CT, int nL, int r, int n, double* vc,
-                     cudaStream_t s) {
+                     double sgn, int accumulate, unsigned long long* mx, cudaStream_t s) {
   if (nL <= 0) return;
-  k_trace_ht<<<nL, 256, 0, s>>>(Ht, CT, r, n, vc);
-  las_count_launch();
-}
-
-void launch_scale(double* p, long count, double a, cudaStream_t s) {
-  if (count <= 0) return;
-  k_scale<<<nblk(count, 256), 256, 0, s>>>(p, count, a);
+  k_trace_ht<<<nL, 256, 0, s>>>(Ht, CT, r, n, vc, sgn, accumulate, mx);
   las_count_launch();
 }
 
 void launch_reduce_partials(const double* part, int nsplit, long count, double* out,
-                            int accumulate, cudaStream_t s, int cols, int ld) {
+                            int accumulate, cudaStream_t s, int cols, int ld, double scale) {
   k_reduce_partials<<<nblk(count, 256), 256, 0, s>>>(part, nsplit, count, out, accumulate, cols,
-                                                     ld);
+                                                     ld, scale);
   las_count_launch();
 }
 
@@ -677,30 +702,40 @@ void launch_energy(const double* eps, int X, const double* Cocc, const double* h
   las_count_launch(2);
 }
 
-void launch_absmax_bits(const double* a, long count, unsigned long long* out, cudaStream_t s) {
-  if (count <= 0) return;
-  k_absmax_bits<<<(unsigned)std::min<long>(nblk(count, 256), 1024), 256, 0, s>>>(a, count, out);
-  las_count_launch();
-}
-
 void launch_antisym(const double* M, int nmo, int o, int op, double* g, cudaStream_t s) {
   k_antisym<<<nblk((long)nmo * nmo, 256), 256, 0, s>>>(M, nmo, o, op, g);
   las_count_launch();
 }
 
-void launch_coulomb_packed(const double* Bp, const double* vc, int X, long npair, double* Jp,
-                           cudaStream_t s) {
-  k_coulomb_packed<<<nblk(npair, 256), 256, 0, s>>>(Bp, vc, X, npair, Jp);
+int coulomb_parts(long npair, int X, int sms) {
+  const long blocks = (npair + COULOMB_PAIRS - 1) / COULOMB_PAIRS;
+  return (int)std::max(1L, std::min({24L, (24L * sms + blocks - 1) / blocks, (long)X / 32}));
+}
+
+void launch_coulomb_packed(const double* Bp, const double* vc, int X, long npair, int parts,
+                           double* Jp, cudaStream_t s) {
+  dim3 grid(nblk(npair, COULOMB_PAIRS), parts);
+  k_coulomb_packed<<<grid, 256, 0, s>>>(Bp, vc, X, (X + parts - 1) / parts, npair, Jp);
   las_count_launch();
 }
 
-void launch_unpack_sym(const double* Jp, int n, double* J, cudaStream_t s) {
-  k_unpack_sym<<<nblk((long)n * n, 256), 256, 0, s>>>(Jp, n, J);
+void launch_unpack_sym(const double* Jp, int parts, int n, double scale, double* J,
+                       cudaStream_t s) {
+  k_unpack_sym<<<nblk((long)n * n, 256), 256, 0, s>>>(Jp, parts, n, scale, J);
   las_count_launch();
 }
 
-void launch_copy_cols(const double* Ht, int X, int op, int n, int c0, int a, double* Lmu,
-                      cudaStream_t s) {
-  k_copy_cols<<<nblk((long)X * n * a, 256), 256, 0, s>>>(Ht, X, op, n, c0, a, Lmu);
+void launch_veff_combine(const double* Jp, int parts, const double* Ka, const double* Kb, int n,
+                         double* va, double* vb, cudaStream_t s) {
+  k_veff_combine<<<nblk((long)n * n, 256), 256, 0, s>>>(Jp, parts, Ka, Kb, n, va, vb);
   las_count_launch();
+}
+
+void launch_transpose_ht(const double* Ht, int nL, int n, int a, double* Lmu, cudaStream_t s) {
+  for (int l0 = 0; l0 < nL; l0 += 32768) {   // the grid's y extent
+    const int m = std::min(nL - l0, 32768);
+    k_transpose_ht<<<dim3((n + 31) / 32, m), 256, 0, s>>>(Ht + (size_t)l0 * a * n, n, a,
+                                                          Lmu + (size_t)l0 * n * a);
+    las_count_launch();
+  }
 }

@@ -708,18 +708,6 @@ struct RowsContig {
   __device__ __forceinline__ double operator()(long r, long k) const { return row(r)[k]; }
 };
 
-// Row (L, u) of the active columns of the half transform, K = mu: Ht[(L op + c + u) n + mu]
-struct RowsHtAct {
-  const double* Ht;
-  int n, op, c, a;
-  __host__ __device__ __forceinline__ const double* row(long r) const {
-    const long L = r / a, u = r - L * a;
-    return Ht + (L * op + c + u) * n;
-  }
-  bool aligned() const { return ((uintptr_t)Ht & 15) == 0 && (n & 1) == 0; }
-  __device__ __forceinline__ double operator()(long r, long k) const { return row(r)[k]; }
-};
-
 struct RowsPacked {   // element (r = L*n + mu, k = nu) of the packed symmetric b^L
   const double* Bp;
   long npair;
@@ -800,9 +788,8 @@ __device__ __forceinline__ unsigned long long absbits(double x) {
 // 28 (2400 x 192 rows of 1200 values: 2.02 ms, 5.5 TB/s, against 2.34).  Few rows per block leave room for
 // five or more blocks per SM, whose loads and stores overlap.  S = 2 modulo 16: the 16-byte reads of
 // 8 neighbouring threads (rows, or 4 rows and two halves) fall into different banks.
-template <class Rows>
 __global__ void __launch_bounds__(256)
-k_slice_kmajor(Rows src, int vec, Planes P, long rows, long kb, int lg, int S, int* ex) {
+k_slice_kmajor(RowsContig src, int vec, Planes P, long rows, long kb, int lg, int S, int* ex) {
   extern __shared__ __align__(16) double rowbuf[];
   __shared__ unsigned long long mxs[32];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -894,9 +881,8 @@ k_slice_cols(Acc acc, Planes P, long rows, long kb, int* ex) {
 
 // The second pass of such sources with the maxima given (mx): one warp per 16 rows x 16 values of
 // K, live rows only.
-template <class Acc>
 __global__ void __launch_bounds__(256)
-k_digits_cols(Acc acc, Planes P, long kb, const unsigned long long* __restrict__ mx, int* ex) {
+k_digits_cols(RowsStrided acc, Planes P, long kb, const unsigned long long* __restrict__ mx, int* ex) {
   const long groups = (P.R + 15) / 16;
   const long w = blockIdx.x * 8L + (threadIdx.x >> 5);
   if (w >= groups * kb) return;
@@ -946,9 +932,8 @@ k_slice_rows(Acc acc, Planes P, long rows, long kb, int* ex) {
 }
 
 // Long rows, pass 1: mx[r] = max_k |x(r,k)| as ordered bit patterns (grid: segments x rows).
-template <class Acc>
 __global__ void __launch_bounds__(256)
-k_rowmax_long(Acc acc, long K, long seg, unsigned long long* mx) {
+k_rowmax_long(RowsContig acc, long K, long seg, unsigned long long* mx) {
   __shared__ unsigned long long red[8];
   const long r = blockIdx.y;
   const long k0 = (long)blockIdx.x * seg, k1 = min(K, k0 + seg);
@@ -972,9 +957,8 @@ k_rowmax_long(Acc acc, long K, long seg, unsigned long long* mx) {
 
 // Long rows, pass 2: 8 values per thread over rows x kb*BK (zeros outside R x K); the source is
 // contiguous in K.  Neighbouring threads write neighbouring 16 bytes of a K block.
-template <class Acc>
 __global__ void __launch_bounds__(256)
-k_digits_long(Acc acc, Planes P, long rows, long kbc, const unsigned long long* mx, int* ex) {
+k_digits_long(RowsContig acc, Planes P, long rows, long kbc, const unsigned long long* mx, int* ex) {
   const long i = blockIdx.x * (long)blockDim.x + threadIdx.x;
   if (i >= rows * kbc * 2) return;
   const long kb = i / (rows * 2), rem = i - kb * (rows * 2);
@@ -1507,10 +1491,9 @@ static las_status slice_rows(Acc acc, const Planes& P, int* ex, cudaStream_t st,
   return slice_done("k_slice_rows launch");
 }
 
-// Rows contiguous in K (RowsContig, RowsHtAct).  Rows per block: up to 40 KB of shared memory, and
+// Rows contiguous in K.  Rows per block: up to 40 KB of shared memory, and
 // no more than leaves two blocks per SM; a single row has to fit 48 KB (K <= 6128).
-template <class Rows>
-static las_status slice_contig(Rows src, const Planes& P, int* ex, cudaStream_t st,
+static las_status slice_contig(RowsContig src, const Planes& P, int* ex, cudaStream_t st,
                                bool live_only = false) {
   if (P.R <= 0) return LAS_OK;
   long kb;
@@ -1519,7 +1502,7 @@ static las_status slice_contig(Rows src, const Planes& P, int* ex, cudaStream_t 
   if (S * 8 > 48 * 1024 - 512) return slice_rows(src, P, ex, st, live_only);
   int lg = 0;
   while (lg < 5 && (S * 8 << (lg + 1)) <= 40 * 1024 && (rows >> (lg + 1)) >= 2 * num_sms()) ++lg;
-  k_slice_kmajor<Rows><<<(unsigned)((rows + (1 << lg) - 1) >> lg), 256, (size_t)(S * 8) << lg,
+  k_slice_kmajor<<<(unsigned)((rows + (1 << lg) - 1) >> lg), 256, (size_t)(S * 8) << lg,
                          st>>>(src, src.aligned(), P, rows, kb, lg, (int)S, ex);
   return slice_done("k_slice_kmajor launch");
 }
@@ -1543,25 +1526,27 @@ static las_status slice_long(RowsContig src, const Planes& P, int* ex, unsigned 
   LAS_CUDA_TRY(cudaMemsetAsync(mx, 0, P.R * sizeof(unsigned long long), st));
   const long seg = 8192;
   dim3 g1((unsigned)((P.K + seg - 1) / seg), (unsigned)P.R);
-  k_rowmax_long<RowsContig><<<g1, 256, 0, st>>>(src, P.K, seg, mx);
+  k_rowmax_long<<<g1, 256, 0, st>>>(src, P.K, seg, mx);
   las_count_launch();
   const long kb = std::min(P.nkb, planes_nkb(P.K)), tot = P.R * kb * 2;
-  k_digits_long<RowsContig><<<(unsigned)((tot + 255) / 256), 256, 0, st>>>(src, P, P.R, kb, mx, ex);
+  k_digits_long<<<(unsigned)((tot + 255) / 256), 256, 0, st>>>(src, P, P.R, kb, mx, ex);
   return slice_done("k_digits_long launch");
 }
 
 // Large sources read along the rows ([K][R] in memory, rows of the planes = columns of the source):
-// column maxima in mx, then the digits of the live rows.
+// column maxima in mx (have_max: already there), then the digits of the live rows.
 static las_status slice_transposed(const double* src, const Planes& P, int* ex,
-                                   unsigned long long* mx, cudaStream_t st) {
+                                   unsigned long long* mx, bool have_max, cudaStream_t st) {
   if (P.R <= 0) return LAS_OK;
-  LAS_CUDA_TRY(cudaMemsetAsync(mx, 0, P.R * sizeof(unsigned long long), st));
-  const long seg = 512;
-  dim3 g1((unsigned)((P.R + 255) / 256), (unsigned)((P.K + seg - 1) / seg));
-  k_colmax<<<g1, 256, 0, st>>>(src, P.K, (int)P.R, seg, mx);
-  las_count_launch();
+  if (!have_max) {
+    LAS_CUDA_TRY(cudaMemsetAsync(mx, 0, P.R * sizeof(unsigned long long), st));
+    const long seg = 512;
+    dim3 g1((unsigned)((P.R + 255) / 256), (unsigned)((P.K + seg - 1) / seg));
+    k_colmax<<<g1, 256, 0, st>>>(src, P.K, (int)P.R, seg, mx);
+    las_count_launch();
+  }
   const long kb = planes_nkb(P.K), warps = (P.R + 15) / 16 * kb;
-  k_digits_cols<RowsStrided><<<(unsigned)((warps + 7) / 8), 256, 0, st>>>(
+  k_digits_cols<<<(unsigned)((warps + 7) / 8), 256, 0, st>>>(
       RowsStrided{src, 1, P.R}, P, kb, mx, ex);
   return slice_done("k_digits_cols launch");
 }
@@ -1884,9 +1869,9 @@ las_status split_tangent_one_electron(SplitState* s, double* hdC, cudaStream_t s
                     s->op, 0, 0, 0, s->status, st, 0, s->bn[SPLIT_ONE_ELECTRON]);
 }
 
-las_status split_lpu(SplitState* s, int nL, const double* Ht, int c, int a, const double* C,
-                     int nmo, int p0, int np, double* Lpu, cudaStream_t st, size_t* bytes) {
-  // Lpu[L][p][u] = sum_mu C[mu][p0+p] Ht[L][c+u][mu]: rows (L,u) of the half transform times the
+las_status split_lpu(SplitState* s, int nL, const double* Ht, int a, const double* C, int nmo,
+                     int p0, int np, double* Lpu, cudaStream_t st, size_t* bytes) {
+  // Lpu[L][p][u] = sum_mu C[mu][p0+p] Ht[L][u][mu]: rows (L,u) of the half transform times the
   // rows p of C[:, p0:p1]^T, written in the (L, p, u) layout by the half-transform epilogue mode
   const int n = s->n;
   if (a < 1 || np < 1) return LAS_OK;
@@ -1913,7 +1898,7 @@ las_status split_lpu(SplitState* s, int nL, const double* Ht, int c, int a, cons
   // the active rows (L,u) of this chunk, sliced into the H digit planes (capacity Lc*op rows)
   Planes Hd = s->Hdig;
   Hd.R = (long)nL * a;
-  if (rc == LAS_OK) rc = slice_contig(RowsHtAct{Ht, n, s->op, c, a}, Hd, s->Hexp, st, true);
+  if (rc == LAS_OK) rc = slice_contig(RowsContig{Ht, n}, Hd, s->Hexp, st, true);
   if (rc == LAS_OK)
     rc = ozaki_gemm(Hd, 0, s->Hexp, (long)nL * a, Mp, 0, s->Mpexp, np, n, 1, 1, Lpu, 0, 0, a, np,
                     s->status, st);
@@ -1964,15 +1949,21 @@ las_status split_project(SplitState* s, int nL, const double* Wt, double* Out, i
   return LAS_OK;
 }
 
+las_status split_exchange_max(SplitState* s, unsigned long long** mx, cudaStream_t st) {
+  LAS_CUDA_TRY(cudaMemsetAsync(s->mx, 0, s->n * sizeof(unsigned long long), st));
+  *mx = s->mx;
+  return LAS_OK;
+}
+
 las_status split_exchange(SplitState* s, int nL, int oc, const double* Ht, double* K, int accumulate,
-                          cudaStream_t st) {
+                          double sgn, cudaStream_t st) {
   // K(mu,nu) (+)= sum_{(L,p)} Ht[(L,p)][mu] Ht[(L,p)][nu]: rows mu of H^T, scaled per row over
   // the long index (L,p), serve as both operands
   const long R = (long)nL * oc, n = s->n;
   if (oc < 1 || oc > s->op) return LAS_ERR_INTERNAL;
   Planes HT = s->HdigT;
   HT.K = R;
-  las_status rc = slice_transposed(Ht, HT, s->hexp, s->mx, st);
+  las_status rc = slice_transposed(Ht, HT, s->hexp, s->mx, true, st);
   if (rc != LAS_OK) return rc;
   // partials [ks][n][n] live in the projection's partial buffer (64 * n * op doubles)
   const long cap = std::max(1L, std::min((64L * s->op) / n, R / KSPLIT_MIN));
@@ -1981,7 +1972,7 @@ las_status split_exchange(SplitState* s, int nL, int oc, const double* Ht, doubl
   rc = ozaki_gemm(HT, 0, s->hexp, n, HT, 0, s->hexp, n, R, ks, 0, s->part, n, n * n, 0, 0,
                   s->status, st, 1);
   if (rc != LAS_OK) return rc;
-  launch_reduce_partials(s->part, ks, n * n, K, accumulate, st);
+  launch_reduce_partials(s->part, ks, n * n, K, accumulate, st, 0, 0, sgn);
   return LAS_OK;
 }
 
@@ -2172,7 +2163,7 @@ las_status frag_split_chunk(SplitState* s, FragSplit* f, int l0, int nL, double*
     B.R = (long)ma * ma;
     B.K = nL;
     // rows (p,q) of T^T with per-row exponents
-    rc = slice_transposed(T, A, f->Texp, f->mx, st);
+    rc = slice_transposed(T, A, f->Texp, f->mx, false, st);
     if (rc == LAS_OK)
       rc = slice_cols(RowsAA{T, n2, nmo, a0, ma}, B, f->Taaexp, st, true);
     const long out = n2 * ma * ma;

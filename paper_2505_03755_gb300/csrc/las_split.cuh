@@ -22,10 +22,12 @@ las_status split_prepare_C(SplitState* s, const double* Cocc, cudaStream_t st);
 las_status split_half(SplitState* s, int l0, int nL, int oc, double* Ht, cudaStream_t st);
 // S2: T[b] = Ht[b] C_occ   (op x op per b)
 las_status split_full(SplitState* s, int nL, const double* Ht, double* T, cudaStream_t st);
-// K (+)= sum_{(L,p)} H(mu,(L,p)) H(nu,(L,p)) over the chunk's half transform Ht[(L,p)][mu];
-// only the lower triangle (mu >= nu) is valid: mirror it afterwards
+// K (+)= sgn sum_{(L,p)} H(mu,(L,p)) H(nu,(L,p)) over the chunk's half transform Ht[(L,p)][mu];
+// only the lower triangle (mu >= nu) is valid: mirror it afterwards.  split_exchange_max first
+// clears *mx[n], into which the caller then puts max_{(L,p)} |Ht| of every column mu.
+las_status split_exchange_max(SplitState* s, unsigned long long** mx, cudaStream_t st);
 las_status split_exchange(SplitState* s, int nL, int oc, const double* Ht, double* K, int accumulate,
-                          cudaStream_t st);
+                          double sgn, cudaStream_t st);
 // Product kinds of an evaluation, each with its own tile width (64 or 96 columns; default 96):
 // S1, S2 (with its H slicer), the projection and the one-electron product.
 enum { SPLIT_HALF = 0, SPLIT_FULL = 1, SPLIT_PROJECT = 2, SPLIT_ONE_ELECTRON = 3, SPLIT_NKIND = 4 };
@@ -77,11 +79,11 @@ las_status frag_split_chunk(SplitState* s, FragSplit* f, int l0, int nL, double*
                             int a0, int ma, double* ppaa, double* papa, double* part,
                             long part_elems, int accumulate, cudaStream_t st);
 
-// (L|pu) of las_df_transform for a chunk: Lpu[L][p][u] = sum_mu C[mu][p0+p] Ht[L][c+u][mu]
+// (L|pu) of las_df_transform for a chunk: Lpu[L][p][u] = sum_mu C[mu][p0+p] Ht[L][u][mu], u < a
 // (C: [n][nmo]; Lpu points at the chunk's first row).  The digit planes of C^T are allocated on
 // the first call and their size is added to *bytes.
-las_status split_lpu(SplitState* s, int nL, const double* Ht, int c, int a, const double* C,
-                     int nmo, int p0, int np, double* Lpu, cudaStream_t st, size_t* bytes);
+las_status split_lpu(SplitState* s, int nL, const double* Ht, int a, const double* C, int nmo,
+                     int p0, int np, double* Lpu, cudaStream_t st, size_t* bytes);
 
 // Tangent of the evaluation along dC (orbital Hessian-vector product), split precision.
 // split_tangent_prepare slices dC_occ (and allocates the tangent scratch on its first call,
