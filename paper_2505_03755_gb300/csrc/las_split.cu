@@ -161,6 +161,7 @@ struct OzParams {
   const int* eb;           // column exponents [N]
   double* out;
   int mode;                // 0: out[z*zstride + r*ldc + c]; 1: Ht layout (rows (L,mu))
+  int vec;                 // mode 0: rows of out are 32-byte aligned at multiples of 4 columns
   long ldc, zstride;
   int ht_n, ht_op;
   int lower;               // symmetric product: only tiles that touch the lower triangle
@@ -656,19 +657,31 @@ k_ozaki(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtenso
         }
       }
       const int z = kb0 / p.kb_per_split;
+      const int e0 = ea - 14 - 8 * (NEXACT - 1) - p.sh;
+      double* const orow = p.mode == 0 ? p.out + (long)z * p.zstride + (long)row * p.ldc
+                                       : p.out + L * p.ht_op * (long)p.ht_n + mu;
 #pragma unroll
       for (int b = 0; b < MAXB; ++b) {
-        if (b < nb) {
+        const int c0 = n0 + (cg + 4 * b) * 8;
+        if (b >= nb || !live || c0 >= p.N) continue;
+        if (p.vec && c0 + 8 <= p.N) {
+          // a thread's 8 columns are 64 bytes of its row: two 32-byte stores (8-byte ones of a warp
+          // are 32 partial sectors each, and a tile's took 18000 clocks)
+#pragma unroll
+          for (int h = 0; h < 8; h += 4) {
+            double v[4];
+#pragma unroll
+            for (int e = 0; e < 4; ++e)
+              v[e] = make_double((long long)acc[b * 8 + h + e], e0 + p.eb[c0 + h + e]);
+            sm100::st_global_32b(orow + c0 + h, v);
+          }
+        } else {
 #pragma unroll
           for (int e = 0; e < 8; ++e) {
-            const int col = n0 + (cg + 4 * b) * 8 + e;
-            if (live && col < p.N) {
-              const int E = ea + p.eb[col] - 14 - 8 * (NEXACT - 1) - p.sh;
-              const double v = make_double((long long)acc[b * 8 + e], E);
-              if (p.mode == 0)
-                p.out[(long)z * p.zstride + (long)row * p.ldc + col] = v;
-              else
-                p.out[(L * p.ht_op + col) * (long)p.ht_n + mu] = v;
+            const int col = c0 + e;
+            if (col < p.N) {
+              const double v = make_double((long long)acc[b * 8 + e], e0 + p.eb[col]);
+              orow[p.mode == 0 ? (long)col : col * (long)p.ht_n] = v;
             }
           }
         }
@@ -1371,6 +1384,7 @@ static las_status ozaki_setup(OzProblem& pr, const Planes& A, long a_row0, const
   p.eb = eb;
   p.out = out;
   p.mode = mode;
+  p.vec = mode == 0 && ((uintptr_t)out & 31) == 0 && ldc % 4 == 0 && zstride % 4 == 0;
   p.ldc = ldc;
   p.zstride = zstride;
   p.ht_n = ht_n;
