@@ -53,7 +53,7 @@ constexpr int NTHREADS = 32 * (EPI_WARP0 + EPI_WARPS);
 // accumulators are still being drained (every accumulator starts at a multiple of 32).  The
 // six B digit planes of a stage lie back to back in shared memory (plane t at t*bn rows), so
 // that one MMA of A_s against planes t0..t1 of B (N = (t1-t0+1)*bn <= 256) lands every product
-// A_s B_t in the accumulator of its own exact group s + t (mma_slab): the ten exact products of a
+// A_s B_t in the accumulator of its own exact group s + t: the ten exact products of a
 // stage take six MMAs at bn = 96 (four of N = 192) and four at bn = 64 (N = 256, 192, 128, 64).
 // (Tiles with a second tail accumulator, so that the tail products could be merged the same way,
 // measured slower: a shorter stage carries the same waits for data and for the exact drains.)
@@ -287,36 +287,48 @@ struct OzCursor {
   }
 };
 
-// D[groups s+t0 .. s+t0+nt-1] (+)= A_s * [B_t0 .. B_t0+nt-1]^T: nt consecutive B planes (tile
-// width BNV, planes BNV*32 bytes apart) against one A plane, as ceil(nt / maxp) MMAs of balanced
-// width (N = np * BNV <= 256).  Everything is a compile-time constant once inlined: the single
-// issuing thread must not spend its time on address arithmetic.
-// Descriptor of A plane s of a stage: K-major, or MN-major (amn) when the stage holds the
-// transposed access of planes stored with rows along K.
-__device__ __forceinline__ uint64_t a_desc(uint32_t sa, int s, bool amn) {
-  return amn ? sm100::smem_desc_sw32_mn(sa + s * A_PLANE) : sm100::smem_desc_sw32(sa + s * A_PLANE);
+// Descriptor of plane `plane` of an operand whose planes lie `bytes` apart: formed for each MMA, or
+// (BASE) as the first plane's plus an offset.  Which is faster depends on the issuing code around it
+// (issue_converged).
+template <bool BASE>
+__device__ __forceinline__ uint64_t plane_desc(uint32_t addr, int plane, int bytes, bool mn) {
+  if constexpr (BASE)
+    return (mn ? sm100::smem_desc_sw32_mn(addr) : sm100::smem_desc_sw32(addr)) +
+           (uint64_t)(plane * (bytes >> 4));
+  else
+    return mn ? sm100::smem_desc_sw32_mn(addr + plane * bytes)
+              : sm100::smem_desc_sw32(addr + plane * bytes);
 }
 
-template <int BNV>
-__device__ __forceinline__ void mma_slab(uint32_t tmem, uint32_t sa, uint32_t sb, int s, int t0,
-                                         int nt, bool accumulate, bool amn) {
+// One stage's exact products (groups 0..3): A_s against planes 0 .. 3-s of B, nt consecutive planes
+// (tile width BNV, planes BNV*32 bytes apart) against one A plane as ceil(nt / maxp) MMAs of balanced
+// width (N = np * BNV <= 256), which land in the accumulators of groups s .. 3; s = 0 spans all four
+// groups and starts them at a chunk's first stage.  amn: the stage holds the transposed access of
+// planes stored with rows along K (A MN-major).  Everything is a compile-time constant once
+// inlined: the issuing thread must not spend its time on address arithmetic.
+template <int BNV, bool BASE>
+__device__ __forceinline__ void mma_exact(uint32_t tmem, uint32_t sa, uint32_t sb,
+                                          bool first_in_chunk, bool amn) {
   constexpr int maxp = 256 / BNV;
-  const int nm = (nt + maxp - 1) / maxp;
-  int t = t0;
 #pragma unroll
-  for (int j = 0; j < nm; ++j) {
-    const int np = (t0 + nt - t) / (nm - j);
-    sm100::mma_bf16(tmem + (uint32_t)((s + t) * BNV), a_desc(sa, s, amn),
-                    sm100::smem_desc_sw32(sb + t * BNV * BK * 2),
-                    sm100::idesc_bf16(BM, np * BNV) | (amn ? sm100::IDESC_A_MN : 0u),
-                    accumulate ? 1u : 0u);
-    t += np;
+  for (int s = 0; s < NEXACT; ++s) {
+    const int nt = NEXACT - s, nm = (nt + maxp - 1) / maxp;
+    int t = 0;
+#pragma unroll
+    for (int j = 0; j < nm; ++j) {
+      const int np = (nt - t) / (nm - j);
+      sm100::mma_bf16(tmem + (uint32_t)((s + t) * BNV), plane_desc<BASE>(sa, s, A_PLANE, amn),
+                      plane_desc<BASE>(sb, t, BNV * BK * 2, false),
+                      sm100::idesc_bf16(BM, np * BNV) | (amn ? sm100::IDESC_A_MN : 0u),
+                      s > 0 || !first_in_chunk ? 1u : 0u);
+      t += np;
+    }
   }
 }
 
-// One stage's tail products (groups 4 and 5, eleven MMAs into the tail accumulator at tail_col),
-// started at the first stage of a tile.
-template <int BNV>
+// One stage's tail products (groups 4 and 5, eleven MMAs into the tail accumulator), started at the
+// first stage of a tile.
+template <int BNV, bool BASE>
 __device__ __forceinline__ void mma_tail(uint32_t tmem_tail, uint32_t sa, uint32_t sb,
                                          bool first_stage, bool amn) {
   bool acc = !first_stage;
@@ -325,20 +337,20 @@ __device__ __forceinline__ void mma_tail(uint32_t tmem_tail, uint32_t sa, uint32
   for (int s = 0; s < NDIG; ++s)
 #pragma unroll
     for (int t = (s >= NEXACT ? 0 : NEXACT - s); s + t < NGROUP; ++t) {
-      sm100::mma_bf16(tmem_tail, a_desc(sa, s, amn), sm100::smem_desc_sw32(sb + t * BNV * BK * 2),
-                      idesc, acc ? 1u : 0u);
+      sm100::mma_bf16(tmem_tail, plane_desc<BASE>(sa, s, A_PLANE, amn),
+                      plane_desc<BASE>(sb, t, BNV * BK * 2, false), idesc, acc ? 1u : 0u);
       acc = true;
     }
 }
 
-// One stage's exact products (groups 0..3): A_s against planes 0 .. 3-s; s = 0 spans all four
-// groups and starts them at a chunk's first stage.
-template <int BNV>
-__device__ __forceinline__ void mma_exact(uint32_t tmem, uint32_t sa, uint32_t sb,
-                                          bool first_in_chunk, bool amn) {
-#pragma unroll
-  for (int s = 0; s < NEXACT; ++s)
-    mma_slab<BNV>(tmem, sa, sb, s, 0, NEXACT - s, s > 0 || !first_in_chunk, amn);
+// Whether an issuer runs as a converged warp that elects the issuing thread (its addresses then stay
+// in uniform registers, and it issues an MMA in 48 clocks instead of 56) or as a single thread.  At
+// 64 columns, where the issue bounds the tail, the converged form takes 1130 to 1170 clocks a stage
+// instead of 1240 (800-orbital autograd 13.0 -> 12.2 ms); at 96 columns, where shared memory is the
+// bound, its bursts cost 5 % (1200-orbital half 23.7 -> 24.9 ms), and in grouped launches of short
+// tiles 20 % (batch of 8: 3.6 -> 4.3 ms).
+__host__ __device__ constexpr bool issue_converged(bool grouped, int fixbn, bool exact) {
+  return !grouped && fixbn == 64;
 }
 
 // Persistent CTAs (one per SM) walk the tiles (row tile, column tile, K split).  Roles:
@@ -346,8 +358,9 @@ __device__ __forceinline__ void mma_exact(uint32_t tmem, uint32_t sa, uint32_t s
 // warp 2 those of the tail, warps 3.. drain the TMEM accumulators.  Stage, chunk and tile counters
 // run on across tiles so that the loads of the next tile overlap the last MMAs of the current one,
 // and its MMAs overlap the current tile's conversion and stores.
-// One thread issues an MMA about every 65 clocks (descriptors and all), so a single issuer's 17 MMAs
-// took as long at 64 columns as at 96: the issue, not the tensor pipe, set the stage time.  The
+// One thread issues an MMA in 56 clocks at best (descriptors and all; 65 in this loop), so a single
+// issuer's 17 MMAs took as long at 64 columns as at 96: the issue, not the tensor pipe, set the
+// stage time.  The
 // two issuers write disjoint accumulators and each wait only for what they overwrite: the exact
 // issuer for the drain of the previous chunk, the tail issuer for the read-out of the previous
 // tile's tail, so that tail products of up to NSTAGE stages run during a drain.
@@ -388,7 +401,11 @@ k_ozaki(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtenso
   uint32_t* tmem_slot = (uint32_t*)(bars + 2 * NSTAGE + 6);
   volatile int* abort_flag = (volatile int*)(tmem_slot + 1);
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  constexpr bool CONV_E = issue_converged(GROUPED, FIXBN, true);
+  constexpr bool CONV_T = issue_converged(GROUPED, FIXBN, false);
+  const int warp = CONV_E || CONV_T ? __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0)
+                                    : (int)threadIdx.x >> 5;
+  const int lane = threadIdx.x & 31;
   // status word for waits outside any tile (the first product's)
   int* const status0 = GROUPED ? probs[0].p.status : p1.status;
 
@@ -426,6 +443,12 @@ k_ozaki(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtenso
   // ---------------- MMA issuers: the exact groups (warp 1) or the tail (warp 2) ----------------
   auto issue = [&](auto exact_c) {
     constexpr bool exact = decltype(exact_c)::value;
+    constexpr bool conv = exact ? CONV_E : CONV_T;   // all lanes are here, one is elected to issue
+    auto issuing = [&]() { return !conv || sm100::elect_one(); };
+    auto wait = [&](uint64_t* bar, uint32_t parity, int* status) -> bool {
+      const bool got = sm100::mbar_wait(bar, parity, abort_flag, status, LAS_ERR_TIMEOUT);
+      return conv ? __all_sync(0xffffffffu, got) : got;
+    };
     int st = 0;
     uint32_t phase = 0;
     uint32_t nstart = 0;   // accumulations started so far (exact: chunks; tail: tiles)
@@ -444,22 +467,22 @@ k_ozaki(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtenso
       auto stages_of = [&](auto bn_c, auto amn, int i0, int i1) -> bool {
         constexpr int bn = decltype(bn_c)::value;
         for (int i = i0; i < i1; ++i) {
-          if (!sm100::mbar_wait(&full[st], phase, abort_flag, p.status, LAS_ERR_TIMEOUT))
-            return false;
+          if (!wait(&full[st], phase, p.status)) return false;
           const bool first = exact ? (i % CHUNK) == 0 : i == 0;
           if (first) {   // the accumulators this stage starts must have been read out
-            if (nstart > 0 && !sm100::mbar_wait(exact ? acce : accT, (nstart - 1) & 1,
-                                                abort_flag, p.status, LAS_ERR_TIMEOUT))
-              return false;
+            if (nstart > 0 && !wait(exact ? acce : accT, (nstart - 1) & 1, p.status)) return false;
             ++nstart;
           }
           sm100::tc_fence_after();
           const uint32_t sa = sm100::smem_u32(smem + st * T::STAGE_BYTES);
           const uint32_t sb = sa + A_BYTES;
-          if constexpr (exact) mma_exact<bn>(tmem, sa, sb, first, amn);
-          else mma_tail<bn>(tmem + T::TAIL_COL, sa, sb, first, amn);
-          sm100::mma_commit(&empty[st]);
-          if (exact && ((i % CHUNK) == CHUNK - 1 || i == nkb - 1)) sm100::mma_commit(accf);
+          if (issuing()) {
+            if constexpr (exact) mma_exact<bn, conv>(tmem, sa, sb, first, amn);
+            else mma_tail<bn, conv>(tmem + T::TAIL_COL, sa, sb, first, amn);
+            sm100::mma_commit(&empty[st]);
+            if (exact && ((i % CHUNK) == CHUNK - 1 || i == nkb - 1)) sm100::mma_commit(accf);
+          }
+          if (conv) __syncwarp();
           if (++st == NSTAGE) {
             st = 0;
             phase ^= 1;
@@ -481,10 +504,10 @@ k_ozaki(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtenso
       } else {
         ok = stages(std::integral_constant<bool, AMN == 1>(), 0, nkb);
       }
-      if (ok && !exact) sm100::mma_commit(tailf);
+      if (ok && !exact && issuing()) sm100::mma_commit(tailf);
     }
     // make sure no MMA is still writing TMEM when the CTA tears down
-    sm100::mma_commit(&drain[exact]);
+    if (issuing()) sm100::mma_commit(&drain[exact]);
     sm100::mbar_wait(&drain[exact], 0, abort_flag, status0, LAS_ERR_TIMEOUT);
   };
 
@@ -556,9 +579,9 @@ k_ozaki(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtenso
     for (int k = 0; k < filled; ++k)
       sm100::mbar_wait(&full[k], k < st ? phase : phase ^ 1, abort_flag, status0,
                        LAS_ERR_TIMEOUT);
-  } else if (warp == 1 && lane == 0) {
+  } else if (warp == 1 && (CONV_E || lane == 0)) {
     issue(std::true_type());    // exact groups
-  } else if (warp == 2 && lane == 0) {
+  } else if (warp == 2 && (CONV_T || lane == 0)) {
     issue(std::false_type());   // tail
   } else if (warp >= EPI_WARP0) {
     // ---------------- epilogue (16 warps) ----------------
@@ -1155,8 +1178,8 @@ static bool valid_bn(int bn) { return bn == 64 || bn == 96; }
 
 // Time of a stage of 96 and of 64 columns (clocks per 16 values of K, 50 to 75 stages a tile): the
 // narrow one pays nearly as much for its A planes, so it wins only where it saves a third of the
-// columns.  op = 128 (800 orbitals): 2 x 64 columns 2400, 96 + 64 2540 and B read twice.
-constexpr int STAGE96 = 1340, STAGE64 = 1200;
+// columns.  op = 128 (800 orbitals): 2 x 64 columns 2300, 96 + 64 2490 and B read twice.
+constexpr int STAGE96 = 1340, STAGE64 = 1150;
 static int pick_bn(long N) {
   return (N + 63) / 64 * STAGE64 < (N + 95) / 96 * STAGE96 ? 64 : 96;
 }
