@@ -28,6 +28,7 @@ __device__ __forceinline__ void dmma_16x8x4(double (&c)[4], double a0, double a1
 template <int NJ, bool SYM, class LA, class LB, class SC>
 __global__ void __launch_bounds__(128)
 k_gemm_f64(int M, int N, int K, int ksplit, int kchunk, LA la, LB lb, SC sc) {
+  pdl_begin();
   constexpr int BN = 8 * NJ, PA = 8, PB = BN / 8;   // A and B elements per thread and K step
   __shared__ double As[2][16][64 + 2];
   __shared__ double Bs[2][16][BN + 2];
@@ -144,6 +145,8 @@ void gemm_f64(int M, int N, int K, int batch, int ksplit, LA a, LB b, SC c, cuda
   const int kchunk = f64_kchunk(K, ksplit);
   const int nj = f64_nj(N);
   dim3 grid((M + 63) / 64, (N + 8 * nj - 1) / (8 * nj), batch * ksplit);
+  // an ordinary launch: blocks placed while the launch before drains would gather on the SMs that
+  // are free first, and the fullest SM is the time (a chained C^T G at 400 orbitals lost 45 us)
   auto go = [&](auto kern) { kern<<<grid, 128, 0, s>>>(M, N, K, ksplit, kchunk, a, b, c); };
   switch (nj) {
     case 4: go(lasdf::k_gemm_f64<4, SYM, LA, LB, SC>); break;

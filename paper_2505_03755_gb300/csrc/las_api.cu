@@ -29,6 +29,8 @@
 static thread_local char g_last_error[512];
 static std::atomic<long> g_launches{0};
 
+thread_local bool g_chain_launches = false;
+
 void las_count_launch(long k) { g_launches.fetch_add(k, std::memory_order_relaxed); }
 
 extern "C" long las_kernel_launches(void) { return g_launches.load(std::memory_order_relaxed); }
@@ -481,13 +483,11 @@ static las_status evaluate(las_ctx* x, const double* C, const double* h, const d
   } else {
     gemm_f64_wide(x, n, op, n, StridedA{h, 0, n, 1}, StridedA{x->Cocc, 0, op, 1}, x->hC, op, 0);
   }
-  launch_energy(x->eps, x->X, x->Cocc, x->hC, n, op, dm1s, x->fi, x->e1, E, x->stream);
-  if (with_grad) {
-    launch_assemble_grad(x->Out, x->hC, dm1s, x->fi, n, nmo, op, G, x->stream);
-    if (gorb) {
-      gemm_f64_wide(x, nmo, x->o, n, StridedA{C, 0, 1, nmo}, StridedA{G, 0, nmo, 1}, x->M, op, 0);
-      launch_antisym(x->M, nmo, x->o, op, gorb, x->stream);
-    }
+  launch_energy(x->eps, x->X, x->Cocc, x->hC, n, op, dm1s, x->fi, x->e1, E, x->stream, x->Out, nmo,
+                with_grad ? G : nullptr);
+  if (gorb) {
+    gemm_f64_wide(x, nmo, x->o, n, StridedA{C, 0, 1, nmo}, StridedA{G, 0, nmo, 1}, x->M, op, 0);
+    launch_antisym(x->M, nmo, x->o, op, gorb, x->stream);
   }
   stage_mark(x, 5);
   return check_launch();
@@ -495,12 +495,16 @@ static las_status evaluate(las_ctx* x, const double* C, const double* h, const d
 
 extern "C" las_status las_energy(las_ctx* x, const double* C, const double* h,
                                  const double* dm1s, const double* dm2, double* E) {
+  if (!x) return LAS_ERR_ARG;
+  ChainScope chain(x->stream);
   return evaluate(x, C, h, dm1s, dm2, E, nullptr, nullptr);
 }
 
 extern "C" las_status las_energy_grad(las_ctx* x, const double* C, const double* h,
                                       const double* dm1s, const double* dm2, double* E,
                                       double* dEdC, double* gorb) {
+  if (!x) return LAS_ERR_ARG;
+  ChainScope chain(x->stream);
   if (!dEdC && !gorb) return LAS_ERR_ARG;
   return evaluate(x, C, h, dm1s, dm2, E, dEdC, gorb);
 }
@@ -509,6 +513,8 @@ extern "C" las_status las_energy_grad_host(las_ctx* x, const double* C_host,
                                            const double* h_host, const double* dm1s_host,
                                            const double* dm2_host, double* E_host,
                                            double* dEdC_host) {
+  if (!x) return LAS_ERR_ARG;
+  ChainScope chain(x->stream);
   if (!x || !C_host || !h_host || !E_host) return LAS_ERR_ARG;
   if (x->a > 0 && (!dm1s_host || !dm2_host)) return LAS_ERR_ARG;
   cudaStream_t s = x->stream;
@@ -590,6 +596,8 @@ static las_status jk_finish(las_ctx* x, double scale, double* J, double* K) {
 }
 
 extern "C" las_status las_df_jk(las_ctx* x, const double* C, double* J, double* K) {
+  if (!x) return LAS_ERR_ARG;
+  ChainScope chain(x->stream);
   if (!x || !C) return LAS_ERR_ARG;
   if (!J && !K) return LAS_OK;
   const int n = x->n, op = x->op, c = x->c;
@@ -645,6 +653,8 @@ static las_status jk_density(las_ctx* x, const Factored& d, int i, bool first, d
 
 extern "C" las_status las_df_jk_density(las_ctx* x, const double* Cx, const double* w, int r,
                                         double* J, double* K) {
+  if (!x) return LAS_ERR_ARG;
+  ChainScope chain(x->stream);
   if (!x || r < 0 || (r > 0 && (!Cx || !w))) return LAS_ERR_ARG;   // r = 0: D = 0
   if (r > x->o) return LAS_ERR_ARG;
   if (!J && !K) return LAS_OK;
@@ -660,6 +670,8 @@ extern "C" las_status las_df_jk_density(las_ctx* x, const double* Cx, const doub
 
 extern "C" las_status las_df_transform(las_ctx* x, const double* C, int p0, int p1,
                                        double* Lmu_u, double* Lpu) {
+  if (!x) return LAS_ERR_ARG;
+  ChainScope chain(x->stream);
   if (!x || !C) return LAS_ERR_ARG;
   if (p0 < 0 || p1 < p0 || p1 > x->nmo) return LAS_ERR_ARG;
   if (x->a == 0) return LAS_OK;
@@ -698,6 +710,8 @@ extern "C" las_status las_df_transform(las_ctx* x, const double* C, int p0, int 
 extern "C" las_status las_veff(las_ctx* x, const double* Ca, const double* wa, int ra,
                                const double* Cb, const double* wb, int rb, double* va,
                                double* vb) {
+  if (!x) return LAS_ERR_ARG;
+  ChainScope chain(x->stream);
   if (!x || !va || !vb || ra < 0 || rb < 0) return LAS_ERR_ARG;
   if ((ra > 0 && (!Ca || !wa)) || (rb > 0 && (!Cb || !wb))) return LAS_ERR_ARG;
   if (ra > x->o || rb > x->o) return LAS_ERR_ARG;
@@ -795,6 +809,8 @@ static las_status tangent_grad(las_ctx* x, const double* h, const double* dm1s, 
 extern "C" las_status las_orbital_hvp(las_ctx* x, const double* C, const double* h,
                                       const double* dm1s, const double* dm2, const double* X,
                                       double* dG, double* Dg) {
+  if (!x) return LAS_ERR_ARG;
+  ChainScope chain(x->stream);
   if (!x || !C || !h || !X || !dG) return LAS_ERR_ARG;
   if (x->a > 0 && (!dm1s || !dm2)) return LAS_ERR_ARG;
   const int n = x->n, nmo = x->nmo, op = x->op, o = x->o;
@@ -899,6 +915,8 @@ static las_status frag_workspace(las_ctx* x, int ma) {
 
 extern "C" las_status las_frag_ao2mo(las_ctx* x, const double* M, int a0, int ma, double* ppaa,
                                      double* papa) {
+  if (!x) return LAS_ERR_ARG;
+  ChainScope chain(x->stream);
   if (!x || !M) return LAS_ERR_ARG;
   if (ma < 1 || a0 < 0 || a0 + ma > x->nmo) return LAS_ERR_ARG;
   if (!ppaa && !papa) return LAS_OK;
@@ -1099,9 +1117,7 @@ static las_status capture_grouped(const BatchPlan& P, las_ctx* const* ctxs,
       const int last = nchunks(x) - 1;
       split_project_reduce(x->split, ks[i], x->Out, last > 0, x->stream);
       launch_energy(x->eps, x->X, x->Cocc, x->hC, x->n, x->op, items[i].dm1s, x->fi, x->e1,
-                    items[i].E, x->stream);
-      launch_assemble_grad(x->Out, x->hC, items[i].dm1s, x->fi, x->n, x->nmo, x->op,
-                           items[i].dEdC, x->stream);
+                    items[i].E, x->stream, x->Out, x->nmo, items[i].dEdC);
       return check_launch();
     }, false);
   return rc;
@@ -1239,6 +1255,8 @@ extern "C" las_status las_energy_grad_batched(int nsys, las_ctx* const* ctxs,
 extern "C" las_status las_autotune(las_ctx* x, const double* C, const double* h,
                                    const double* dm1s, const double* dm2, double* E,
                                    double* dEdC) {
+  if (!x) return LAS_ERR_ARG;
+  ChainScope chain(x->stream);
   if (!x || !C || !h || !E || !dEdC) return LAS_ERR_ARG;
   if (x->prec != LAS_SPLIT_BF16) return LAS_OK;   // the FP64 path is bound by FP64 arithmetic
   las_status st = las_set_timing(x, 1);

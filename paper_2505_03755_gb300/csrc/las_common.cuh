@@ -26,6 +26,55 @@ void las_record_cuda_error(cudaError_t e, const char* what, const char* file, in
 // Process-wide count of kernels this library has launched (diagnostics).
 void las_count_launch(long k = 1);
 
+// Programmatic dependent launches.  A kernel launched by launch_chained may start while the launch
+// before it in the stream still runs: its blocks are placed as soon as all blocks of that one have
+// begun, and wait in pdl_wait until it has completed and its writes are visible.  Every kernel
+// launched this way calls pdl_wait (or pdl_begin) in all threads before it touches global memory,
+// so completion is transitive along a chain.  An evaluation of a small problem is 16 launches of a
+// few microseconds each, and this hides their launch latency and set-up (48 orbitals: 125 -> 104 us).
+__device__ __forceinline__ void pdl_trigger() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_begin() {
+  pdl_trigger();
+  pdl_wait();
+}
+// Launches of this thread are chained while a ChainScope of an uncaptured stream is alive (under
+// stream capture they are ordinary launches).
+extern thread_local bool g_chain_launches;
+struct ChainScope {
+  bool saved;
+  explicit ChainScope(cudaStream_t s) : saved(g_chain_launches) {
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    g_chain_launches =
+        cudaStreamIsCapturing(s, &st) == cudaSuccess && st == cudaStreamCaptureStatusNone;
+  }
+  ~ChainScope() { g_chain_launches = saved; }
+  ChainScope(const ChainScope&) = delete;
+  ChainScope& operator=(const ChainScope&) = delete;
+};
+// kern<<<grid, block, smem, s>>>(args...); errors are left to cudaGetLastError as with <<<>>>
+template <class... P, class... A>
+void launch_chained(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
+                    A... args) {
+  if (!g_chain_launches) {
+    kern<<<grid, block, smem, s>>>(P(args)...);
+    return;
+  }
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  cudaLaunchKernelEx(&cfg, kern, P(args)...);
+}
+
 // Fragment description in constant-size form (passed by value to kernels).
 struct FragInfo {
   int nfrag;
@@ -106,10 +155,12 @@ void launch_reduce_partials(const double* part, int nsplit, long count, double* 
 void launch_assemble_grad(const double* Out, const double* hC, const double* dm1s,
                           const FragInfo& fi, int n, int nmo, int op, double* G,
                           cudaStream_t s);
-// *E = one-electron energy of h (hC = h C_occ) + sum_L eps_L; e1: E1_BLOCKS doubles of scratch
+// *E = one-electron energy of h (hC = h C_occ) + sum_L eps_L; e1: E1_BLOCKS doubles of scratch; with
+// G also launch_assemble_grad, in the same launch as the energy's sum
 #define E1_BLOCKS 256
 void launch_energy(const double* eps, int X, const double* Cocc, const double* hC, int n, int op,
-                   const double* dm1s, const FragInfo& fi, double* e1, double* E, cudaStream_t s);
+                   const double* dm1s, const FragInfo& fi, double* e1, double* E, cudaStream_t s,
+                   const double* Out = nullptr, int nmo = 0, double* G = nullptr);
 void launch_antisym(const double* M, int nmo, int o, int op, double* g, cudaStream_t s);
 // Jp[z][npair], z < parts: partial sums over parts of the auxiliary index (coulomb_parts: how many)
 int coulomb_parts(long npair, int X, int sms);

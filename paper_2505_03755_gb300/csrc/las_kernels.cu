@@ -30,6 +30,7 @@ __device__ double block_sum0(double v, double* red) {   // red: NT doubles
 __global__ void k_pack_cocc(const double* __restrict__ C, int n, int nmo, int o, int op,
                             double* __restrict__ Cocc, const double* __restrict__ dm2,
                             FragInfo fi, double* __restrict__ dm2t) {
+  pdl_begin();
   long i = blockIdx.x * (long)blockDim.x + threadIdx.x;
   const long total = (long)n * op;
   if (i < total) {
@@ -96,6 +97,7 @@ k_per_aux(const double* __restrict__ T, int nL, int op, const double* __restrict
           const double* __restrict__ dm2t, FragInfo fi, double* __restrict__ W,
           double* __restrict__ eps, double* __restrict__ vcv, double* __restrict__ vav,
           int with_grad, const int* __restrict__ gexp, int use_p) {
+  pdl_begin();
   extern __shared__ double sm[];
   const int a = fi.nact, c = fi.ncore, o = c + a, nf = fi.nfrag;
   // fragment offsets, offsets of their D blocks (doff[nf] = size of all), fragment of an orbital
@@ -309,6 +311,7 @@ k_per_aux(const double* __restrict__ T, int nL, int op, const double* __restrict
 __global__ void __launch_bounds__(32)
 k_sign_split(const double* __restrict__ w0, int r0, const double* __restrict__ w1, int r1, int o,
              int* __restrict__ idx, int* __restrict__ counts) {
+  pdl_begin();
   const int lane = threadIdx.x;
   const double* w = blockIdx.x ? w1 : w0;
   const int r = blockIdx.x ? r1 : r0;
@@ -335,6 +338,7 @@ k_sign_split(const double* __restrict__ w0, int r0, const double* __restrict__ w
 __global__ void k_pack_weighted(const double* __restrict__ Cx, const double* __restrict__ w,
                                 const int* __restrict__ idx, int cnt, double sign, int n, int r,
                                 int op, double* __restrict__ Cocc) {
+  pdl_begin();
   long i = blockIdx.x * (long)blockDim.x + threadIdx.x;
   if (i >= (long)n * op) return;
   const int mu = (int)(i / op), j = (int)(i % op);
@@ -348,6 +352,7 @@ __global__ void k_pack_weighted(const double* __restrict__ Cx, const double* __r
 
 // K = scale * (its lower triangle, mirrored to the upper)
 __global__ void k_mirror_lower(double* __restrict__ K, int n, double scale) {
+  pdl_begin();
   long idx = blockIdx.x * (long)blockDim.x + threadIdx.x;
   if (idx >= (long)n * n) return;
   const int i = (int)(idx / n), j = (int)(idx % n);
@@ -359,6 +364,7 @@ __global__ void k_mirror_lower(double* __restrict__ K, int n, double scale) {
 
 // dT[L][p][q] = X[L][p][q] + X[L][q][p]  (the symmetric tangent of T_L = C^T b^L C)
 __global__ void k_sym_add(const double* __restrict__ X, long nL, int op, double* __restrict__ dT) {
+  pdl_begin();
   const long i = blockIdx.x * (long)blockDim.x + threadIdx.x;
   const long per = (long)op * op;
   if (i >= nL * per) return;
@@ -371,6 +377,7 @@ __global__ void k_sym_add(const double* __restrict__ X, long nL, int op, double*
 __global__ void k_reduce_partials(const double* __restrict__ part, int nsplit, long count,
                                   double* __restrict__ out, int accumulate, int cols, int ld,
                                   double scale) {
+  pdl_begin();
   long i = blockIdx.x * (long)blockDim.x + threadIdx.x;
   if (i >= count) return;
   const long o = cols == ld ? i : i / cols * ld + i % cols;
@@ -380,31 +387,6 @@ __global__ void k_reduce_partials(const double* __restrict__ part, int nsplit, l
   out[o] = accumulate ? fma(scale, s, out[o]) : scale * s;
 }
 
-// dE/dC = [4 h C_core | 2 h C_act D | 0] + Out   (Out = sum_L H_L W_L, n x op)
-__global__ void k_assemble_grad(const double* __restrict__ Out, const double* __restrict__ hC,
-                                const double* __restrict__ dm1s, FragInfo fi, int n, int nmo,
-                                int op, double* __restrict__ G) {
-  long i = blockIdx.x * (long)blockDim.x + threadIdx.x;
-  if (i >= (long)n * nmo) return;
-  const int mu = (int)(i / nmo), q = (int)(i % nmo);
-  const int c = fi.ncore, o = c + fi.nact;
-  double g = 0.0;
-  if (q < c) {
-    g = 4.0 * hC[(long)mu * op + q] + Out[(long)mu * op + q];
-  } else if (q < o) {
-    const int u = q - c;
-    const int K = frag_of(fi, u), oK = fi.off[K], m = fi.off[K + 1] - oK;
-    const double* gK = dm1s + fi.dm1_off[K];
-    double s = 0.0;
-    for (int v = 0; v < m; ++v) {
-      double d = gK[v * m + (u - oK)] + gK[m * m + v * m + (u - oK)];
-      s += hC[(long)mu * op + c + oK + v] * d;
-    }
-    g = 2.0 * s + Out[(long)mu * op + q];
-  }
-  G[i] = g;
-}
-
 // One-electron energy sum_mu ( 2 sum_i C(mu,i) hC(mu,i) + sum_u C(mu,u) sum_v D_uv hC(mu,v) ): one
 // warp per row mu, one partial per block.  (Only these elements of C_occ^T h C_occ enter the
 // energy; forming the whole matrix took a slicing pass and a product of its own, 45 us at 400
@@ -412,6 +394,7 @@ __global__ void k_assemble_grad(const double* __restrict__ Out, const double* __
 __global__ void __launch_bounds__(256)
 k_energy_one(const double* __restrict__ Cocc, const double* __restrict__ hC, int n, int op,
              const double* __restrict__ dm1s, FragInfo fi, double* __restrict__ e1) {
+  pdl_begin();
   __shared__ double red[256];
   const int lane = threadIdx.x & 31, c = fi.ncore, o = c + fi.nact;
   double s = 0.0;
@@ -434,10 +417,15 @@ k_energy_one(const double* __restrict__ Cocc, const double* __restrict__ hC, int
   if (threadIdx.x == 0) e1[blockIdx.x] = t;
 }
 
-// E = sum_b e1_b + sum_L eps_L  (one CTA, fixed order, compensated summation).
-__global__ void __launch_bounds__(256)
-k_energy_final(const double* __restrict__ eps, int X, const double* __restrict__ e1, int ne1,
-               double* __restrict__ E) {
+// E = sum_b e1_b + sum_L eps_L  (one block of 256, fixed order, compensated summation).
+struct EnergySum {
+  const double* eps;
+  int X;
+  const double* e1;
+  int ne1;
+  double* E;
+};
+__device__ void energy_sum(const EnergySum& a) {
   __shared__ double red[256];
   double s = 0.0, comp = 0.0;
   auto add = [&](double x) {  // Neumaier
@@ -446,15 +434,52 @@ k_energy_final(const double* __restrict__ eps, int X, const double* __restrict__
     s = t;
   };
 #pragma unroll 4
-  for (int L = threadIdx.x; L < X; L += 256) add(eps[L]);
-  for (int i = threadIdx.x; i < ne1; i += 256) add(e1[i]);
+  for (int L = threadIdx.x; L < a.X; L += 256) add(a.eps[L]);
+  for (int i = threadIdx.x; i < a.ne1; i += 256) add(a.e1[i]);
   const double tot = block_sum0<256>(s + comp, red);
-  if (threadIdx.x == 0) *E = tot;
+  if (threadIdx.x == 0) *a.E = tot;
+}
+__global__ void __launch_bounds__(256) k_energy_final(EnergySum a) {
+  pdl_begin();
+  energy_sum(a);
+}
+
+// dE/dC = [4 h C_core | 2 h C_act D | 0] + Out   (Out = sum_L H_L W_L, n x op); with es.E, the last
+// block sums the energy instead.
+__global__ void __launch_bounds__(256)
+k_assemble_grad(const double* __restrict__ Out, const double* __restrict__ hC,
+                const double* __restrict__ dm1s, FragInfo fi, int n, int nmo, int op,
+                double* __restrict__ G, EnergySum es) {
+  pdl_begin();
+  if (es.E && blockIdx.x == gridDim.x - 1) {
+    energy_sum(es);
+    return;
+  }
+  long i = blockIdx.x * 256L + threadIdx.x;
+  if (i >= (long)n * nmo) return;
+  const int mu = (int)(i / nmo), q = (int)(i % nmo);
+  const int c = fi.ncore, o = c + fi.nact;
+  double g = 0.0;
+  if (q < c) {
+    g = 4.0 * hC[(long)mu * op + q] + Out[(long)mu * op + q];
+  } else if (q < o) {
+    const int u = q - c;
+    const int K = frag_of(fi, u), oK = fi.off[K], m = fi.off[K + 1] - oK;
+    const double* gK = dm1s + fi.dm1_off[K];
+    double s = 0.0;
+    for (int v = 0; v < m; ++v) {
+      double d = gK[v * m + (u - oK)] + gK[m * m + v * m + (u - oK)];
+      s += hC[(long)mu * op + c + oK + v] * d;
+    }
+    g = 2.0 * s + Out[(long)mu * op + q];
+  }
+  G[i] = g;
 }
 
 // g[p][q] = M'[p][q] - M'[q][p],  M'[p][q] = M[p][q] for q < o else 0  (M is nmo x op)
 __global__ void k_antisym(const double* __restrict__ M, int nmo, int o, int op,
                           double* __restrict__ g) {
+  pdl_begin();
   long i = blockIdx.x * (long)blockDim.x + threadIdx.x;
   if (i >= (long)nmo * nmo) return;
   const int p = (int)(i / nmo), q = (int)(i % nmo);
@@ -472,6 +497,7 @@ constexpr int COULOMB_PAIRS = 512;
 __global__ void __launch_bounds__(256)
 k_coulomb_packed(const double* __restrict__ Bp, const double* __restrict__ vc, int X, int per,
                  long npair, double* __restrict__ Jp) {
+  pdl_begin();
   const long i0 = blockIdx.x * (long)COULOMB_PAIRS + threadIdx.x, i1 = i0 + 256;
   const int l0 = blockIdx.y * per, l1 = min(X, l0 + per);
   double s0 = 0.0, s1 = 0.0;
@@ -501,6 +527,7 @@ __device__ __forceinline__ double coulomb_sum(const double* __restrict__ Jp, int
 
 __global__ void k_unpack_sym(const double* __restrict__ Jp, int parts, int n, double scale,
                              double* __restrict__ J) {
+  pdl_begin();
   long i = blockIdx.x * (long)blockDim.x + threadIdx.x;
   if (i >= (long)n * n) return;
   long mu = i / n, nu = i % n;
@@ -511,6 +538,7 @@ __global__ void k_unpack_sym(const double* __restrict__ Jp, int parts, int n, do
 __global__ void k_veff_combine(const double* __restrict__ Jp, int parts,
                                const double* __restrict__ Ka, const double* __restrict__ Kb, int n,
                                double* __restrict__ va, double* __restrict__ vb) {
+  pdl_begin();
   long i = blockIdx.x * (long)blockDim.x + threadIdx.x;
   if (i >= (long)n * n) return;
   long mu = i / n, nu = i % n;
@@ -525,6 +553,7 @@ __global__ void k_veff_combine(const double* __restrict__ Jp, int parts,
 // 1600 x 400 x 16 values, against 27).
 __global__ void __launch_bounds__(256)
 k_transpose_ht(const double* __restrict__ Ht, int n, int a, double* __restrict__ Lmu) {
+  pdl_begin();
   __shared__ double tile[LAS_MAX_ACT][33];
   const long L = blockIdx.y;
   const int mu0 = blockIdx.x * 32, nm = min(32, n - mu0);
@@ -539,6 +568,7 @@ k_transpose_ht(const double* __restrict__ Ht, int n, int a, double* __restrict__
 
 __global__ void k_transpose_cols(const double* __restrict__ C, int n, int op, int r,
                                  double* __restrict__ CT) {
+  pdl_begin();
   const long i = blockIdx.x * (long)blockDim.x + threadIdx.x;   // over r*n, mu fastest
   if (i >= (long)r * n) return;
   const int k = (int)(i / n), mu = (int)(i - (long)k * n);
@@ -554,6 +584,7 @@ __global__ void __launch_bounds__(256)
 k_trace_ht(const double* __restrict__ Ht, const double* __restrict__ CT, int r, int n,
            double* __restrict__ vc, double sgn, int accumulate,
            unsigned long long* __restrict__ mx) {
+  pdl_begin();
   __shared__ double red[256];
   const long b = blockIdx.x;
   const double* hb = Ht + b * (long)r * n;
@@ -599,7 +630,7 @@ void launch_pack_cocc(const double* C, int n, int nmo, int o, int op, double* Co
       count += m * m * m * m;
     }
   }
-  k_pack_cocc<<<nblk(count, 256), 256, 0, s>>>(C, n, nmo, o, op, Cocc, dm2, f, dm2t);
+  launch_chained(k_pack_cocc, nblk(count, 256), 256, 0, s, C, n, nmo, o, op, Cocc, dm2, f, dm2t);
   las_count_launch();
 }
 
@@ -634,6 +665,7 @@ void launch_per_aux(const double* T, int nL, int op, const double* dm1s, const d
                     int with_grad, const int* gexp, cudaStream_t s) {
   if (nL <= 0) return;
   const int use_p = fi.nfrag > 1 && per_aux_smem(fi, 1) <= PER_AUX_SMEM_MAX;
+  // an ordinary launch, as the FP64 GEMM's: its FP64 work is to be even over the SMs
   k_per_aux<<<nL, 256, per_aux_smem(fi, use_p), s>>>(T, nL, op, dm1s, dm2t, fi, W, eps, vc, va,
                                                      with_grad, gexp, use_p);
   las_count_launch();
@@ -641,26 +673,26 @@ void launch_per_aux(const double* T, int nL, int op, const double* dm1s, const d
 
 void launch_sign_split(const double* w0, int r0, const double* w1, int r1, int o, int* idx,
                        int* counts, cudaStream_t s) {
-  k_sign_split<<<2, 32, 0, s>>>(w0, r0, w1, r1, o, idx, counts);
+  launch_chained(k_sign_split, 2, 32, 0, s, w0, r0, w1, r1, o, idx, counts);
   las_count_launch();
 }
 
 void launch_pack_weighted(const double* Cx, const double* w, const int* idx, int cnt,
                           double sign, int n, int r, int op, double* Cocc, cudaStream_t s) {
-  k_pack_weighted<<<nblk((long)n * op, 256), 256, 0, s>>>(Cx, w, idx, cnt, sign, n, r, op,
+  launch_chained(k_pack_weighted, nblk((long)n * op, 256), 256, 0, s, Cx, w, idx, cnt, sign, n, r, op,
                                                          Cocc);
   las_count_launch();
 }
 
 void launch_mirror_lower(double* K, int n, double scale, cudaStream_t s) {
-  k_mirror_lower<<<nblk((long)n * n, 256), 256, 0, s>>>(K, n, scale);
+  launch_chained(k_mirror_lower, nblk((long)n * n, 256), 256, 0, s, K, n, scale);
   las_count_launch();
 }
 
 void launch_sym_add(const double* X, int nL, int op, double* dT, cudaStream_t s) {
   const long count = (long)nL * op * op;
   if (count <= 0) return;
-  k_sym_add<<<nblk(count, 256), 256, 0, s>>>(X, nL, op, dT);
+  launch_chained(k_sym_add, nblk(count, 256), 256, 0, s, X, nL, op, dT);
   las_count_launch();
 }
 
@@ -668,20 +700,20 @@ void launch_transpose_cols(const double* Cocc, int n, int op, int r, double* CT,
                            cudaStream_t s) {
   const long cnt = (long)r * n;
   if (cnt <= 0) return;
-  k_transpose_cols<<<nblk(cnt, 256), 256, 0, s>>>(Cocc, n, op, r, CT);
+  launch_chained(k_transpose_cols, nblk(cnt, 256), 256, 0, s, Cocc, n, op, r, CT);
   las_count_launch();
 }
 
 void launch_trace_ht(const double* Ht, const double* CT, int nL, int r, int n, double* vc,
                      double sgn, int accumulate, unsigned long long* mx, cudaStream_t s) {
   if (nL <= 0) return;
-  k_trace_ht<<<nL, 256, 0, s>>>(Ht, CT, r, n, vc, sgn, accumulate, mx);
+  launch_chained(k_trace_ht, nL, 256, 0, s, Ht, CT, r, n, vc, sgn, accumulate, mx);
   las_count_launch();
 }
 
 void launch_reduce_partials(const double* part, int nsplit, long count, double* out,
                             int accumulate, cudaStream_t s, int cols, int ld, double scale) {
-  k_reduce_partials<<<nblk(count, 256), 256, 0, s>>>(part, nsplit, count, out, accumulate, cols,
+  launch_chained(k_reduce_partials, nblk(count, 256), 256, 0, s, part, nsplit, count, out, accumulate, cols,
                                                      ld, scale);
   las_count_launch();
 }
@@ -689,21 +721,27 @@ void launch_reduce_partials(const double* part, int nsplit, long count, double* 
 void launch_assemble_grad(const double* Out, const double* hC, const double* dm1s,
                           const FragInfo& fi, int n, int nmo, int op, double* G,
                           cudaStream_t s) {
-  k_assemble_grad<<<nblk((long)n * nmo, 256), 256, 0, s>>>(Out, hC, dm1s, fi, n, nmo, op, G);
+  launch_chained(k_assemble_grad, nblk((long)n * nmo, 256), 256, 0, s, Out, hC, dm1s, fi, n, nmo,
+                 op, G, EnergySum{});
   las_count_launch();
 }
 
 void launch_energy(const double* eps, int X, const double* Cocc, const double* hC, int n, int op,
                    const double* dm1s, const FragInfo& fi, double* e1, double* E,
-                   cudaStream_t s) {
+                   cudaStream_t s, const double* Out, int nmo, double* G) {
   const int nb = (int)std::min<long>(nblk(n, 8), E1_BLOCKS);
-  k_energy_one<<<nb, 256, 0, s>>>(Cocc, hC, n, op, dm1s, fi, e1);
-  k_energy_final<<<1, 256, 0, s>>>(eps, X, e1, nb, E);
+  launch_chained(k_energy_one, nb, 256, 0, s, Cocc, hC, n, op, dm1s, fi, e1);
+  const EnergySum es{eps, X, e1, nb, E};
+  if (G)
+    launch_chained(k_assemble_grad, nblk((long)n * nmo, 256) + 1, 256, 0, s, Out, hC, dm1s, fi, n,
+                   nmo, op, G, es);
+  else
+    launch_chained(k_energy_final, 1, 256, 0, s, es);
   las_count_launch(2);
 }
 
 void launch_antisym(const double* M, int nmo, int o, int op, double* g, cudaStream_t s) {
-  k_antisym<<<nblk((long)nmo * nmo, 256), 256, 0, s>>>(M, nmo, o, op, g);
+  launch_chained(k_antisym, nblk((long)nmo * nmo, 256), 256, 0, s, M, nmo, o, op, g);
   las_count_launch();
 }
 
@@ -715,26 +753,26 @@ int coulomb_parts(long npair, int X, int sms) {
 void launch_coulomb_packed(const double* Bp, const double* vc, int X, long npair, int parts,
                            double* Jp, cudaStream_t s) {
   dim3 grid(nblk(npair, COULOMB_PAIRS), parts);
-  k_coulomb_packed<<<grid, 256, 0, s>>>(Bp, vc, X, (X + parts - 1) / parts, npair, Jp);
+  launch_chained(k_coulomb_packed, grid, 256, 0, s, Bp, vc, X, (X + parts - 1) / parts, npair, Jp);
   las_count_launch();
 }
 
 void launch_unpack_sym(const double* Jp, int parts, int n, double scale, double* J,
                        cudaStream_t s) {
-  k_unpack_sym<<<nblk((long)n * n, 256), 256, 0, s>>>(Jp, parts, n, scale, J);
+  launch_chained(k_unpack_sym, nblk((long)n * n, 256), 256, 0, s, Jp, parts, n, scale, J);
   las_count_launch();
 }
 
 void launch_veff_combine(const double* Jp, int parts, const double* Ka, const double* Kb, int n,
                          double* va, double* vb, cudaStream_t s) {
-  k_veff_combine<<<nblk((long)n * n, 256), 256, 0, s>>>(Jp, parts, Ka, Kb, n, va, vb);
+  launch_chained(k_veff_combine, nblk((long)n * n, 256), 256, 0, s, Jp, parts, Ka, Kb, n, va, vb);
   las_count_launch();
 }
 
 void launch_transpose_ht(const double* Ht, int nL, int n, int a, double* Lmu, cudaStream_t s) {
   for (int l0 = 0; l0 < nL; l0 += 32768) {   // the grid's y extent
     const int m = std::min(nL - l0, 32768);
-    k_transpose_ht<<<dim3((n + 31) / 32, m), 256, 0, s>>>(Ht + (size_t)l0 * a * n, n, a,
+    launch_chained(k_transpose_ht, dim3((n + 31) / 32, m), 256, 0, s, Ht + (size_t)l0 * a * n, n, a,
                                                           Lmu + (size_t)l0 * n * a);
     las_count_launch();
   }

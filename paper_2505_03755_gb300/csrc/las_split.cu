@@ -401,6 +401,7 @@ k_ozaki(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtenso
   uint32_t* tmem_slot = (uint32_t*)(bars + 2 * NSTAGE + 6);
   volatile int* abort_flag = (volatile int*)(tmem_slot + 1);
 
+  pdl_trigger();
   constexpr bool CONV_E = issue_converged(GROUPED, FIXBN, true);
   constexpr bool CONV_T = issue_converged(GROUPED, FIXBN, false);
   const int warp = CONV_E || CONV_T ? __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0)
@@ -439,6 +440,7 @@ k_ozaki(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtenso
   __syncthreads();
   sm100::tc_fence_after();
   const uint32_t tmem = *tmem_slot;
+  pdl_wait();   // nothing before this reads what an earlier launch wrote
 
   // ---------------- MMA issuers: the exact groups (warp 1) or the tail (warp 2) ----------------
   auto issue = [&](auto exact_c) {
@@ -826,6 +828,7 @@ __device__ __forceinline__ unsigned long long absbits(double x) {
 // 8 neighbouring threads (rows, or 4 rows and two halves) fall into different banks.
 __global__ void __launch_bounds__(256)
 k_slice_kmajor(RowsContig src, int vec, Planes P, long rows, long kb, int lg, int S, int* ex) {
+  pdl_begin();
   extern __shared__ __align__(16) double rowbuf[];
   __shared__ unsigned long long mxs[32];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -886,6 +889,7 @@ k_slice_kmajor(RowsContig src, int vec, Planes P, long rows, long kb, int lg, in
 template <class Acc>
 __global__ void __launch_bounds__(512)
 k_slice_cols(Acc acc, Planes P, long rows, long kb, int* ex) {
+  pdl_begin();
   __shared__ unsigned long long red[16][16];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, rl = lane & 15;
   const long r = blockIdx.x * 16L + rl;
@@ -919,6 +923,7 @@ k_slice_cols(Acc acc, Planes P, long rows, long kb, int* ex) {
 // K, live rows only.
 __global__ void __launch_bounds__(256)
 k_digits_cols(RowsStrided acc, Planes P, long kb, const unsigned long long* __restrict__ mx, int* ex) {
+  pdl_begin();
   const long groups = (P.R + 15) / 16;
   const long w = blockIdx.x * 8L + (threadIdx.x >> 5);
   if (w >= groups * kb) return;
@@ -941,6 +946,7 @@ k_digits_cols(RowsStrided acc, Planes P, long kb, const unsigned long long* __re
 template <class Acc>
 __global__ void __launch_bounds__(256)
 k_slice_rows(Acc acc, Planes P, long rows, long kb, int* ex) {
+  pdl_begin();
   const long r = (blockIdx.x * (long)blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   if (r >= rows) return;
@@ -970,6 +976,7 @@ k_slice_rows(Acc acc, Planes P, long rows, long kb, int* ex) {
 // Long rows, pass 1: mx[r] = max_k |x(r,k)| as ordered bit patterns (grid: segments x rows).
 __global__ void __launch_bounds__(256)
 k_rowmax_long(RowsContig acc, long K, long seg, unsigned long long* mx) {
+  pdl_begin();
   __shared__ unsigned long long red[8];
   const long r = blockIdx.y;
   const long k0 = (long)blockIdx.x * seg, k1 = min(K, k0 + seg);
@@ -995,6 +1002,7 @@ k_rowmax_long(RowsContig acc, long K, long seg, unsigned long long* mx) {
 // contiguous in K.  Neighbouring threads write neighbouring 16 bytes of a K block.
 __global__ void __launch_bounds__(256)
 k_digits_long(RowsContig acc, Planes P, long rows, long kbc, const unsigned long long* mx, int* ex) {
+  pdl_begin();
   const long i = blockIdx.x * (long)blockDim.x + threadIdx.x;
   if (i >= rows * kbc * 2) return;
   const long kb = i / (rows * 2), rem = i - kb * (rows * 2);
@@ -1090,6 +1098,7 @@ k_bpacked_ragged(const double* __restrict__ Bp, long npair, int n, int n1, int r
 // |x| bit patterns).  Grid: (ceil(n/256), row segments).
 __global__ void __launch_bounds__(256)
 k_colmax(const double* __restrict__ Ht, long R, int n, long seg, unsigned long long* mx) {
+  pdl_begin();
   const int mu = blockIdx.x * 256 + threadIdx.x;
   if (mu >= n) return;
   const long r0 = (long)blockIdx.y * seg, r1 = min(R, r0 + seg);
@@ -1304,7 +1313,7 @@ las_status ozgroup_launch(const OzGroup* g, void* dev, cudaStream_t st) {
   const int np = (int)g->probs.size();
   constexpr int SM = OzTile<OZ_BN>::SMEM_BYTES;
   auto go = [&](auto kern) {
-    kern<<<grid, NTHREADS, SM, st>>>(m0, m0, m0, m0, dummy, probs, np, g->tiles);
+    launch_chained(kern, grid, NTHREADS, SM, st, m0, m0, m0, m0, dummy, probs, np, g->tiles);
   };
   if (bn == 96) pack ? go(k_ozaki<OZ_BN, true, 96, true>) : go(k_ozaki<OZ_BN, true, 96, false>);
   else if (bn == 64) pack ? go(k_ozaki<OZ_BN, true, 64, true>) : go(k_ozaki<OZ_BN, true, 64, false>);
@@ -1338,7 +1347,7 @@ static las_status ozaki_submit(OzProblem& pr, cudaStream_t st) {
   dim3 grid((unsigned)std::min<long>(tiles, num_sms()), 1, 1);
   constexpr int SM = OzTile<OZ_BN>::SMEM_BYTES;
   auto go = [&](auto kern) {
-    kern<<<grid, NTHREADS, SM, st>>>(pr.tmA, pr.tmB, pr.tmA2, pr.tmA3, p, nullptr, 0, tiles);
+    launch_chained(kern, grid, NTHREADS, SM, st, pr.tmA, pr.tmB, pr.tmA2, pr.tmA3, p, nullptr, 0, tiles);
   };
   const bool pack = needs_pack(p);
   // full-row products take an instantiation with their A orientation as a compile-time constant
@@ -1524,9 +1533,11 @@ static las_status slice_rows(Acc acc, const Planes& P, int* ex, cudaStream_t st,
   if (P.R <= 0) return LAS_OK;
   long kb;
   const long rows = slice_extent(P, live_only, &kb);
-  k_slice_rows<Acc><<<(unsigned)((rows * 32 + 255) / 256), 256, 0, st>>>(acc, P, rows, kb, ex);
+  launch_chained(k_slice_rows<Acc>, (unsigned)((rows * 32 + 255) / 256), 256, 0, st, acc, P, rows, kb, ex);
   return slice_done("k_slice_rows launch");
 }
+
+static bool slice_fits(long kb) { return (kb * BK + 2) * 8 <= 48 * 1024 - 512; }
 
 // Rows contiguous in K.  Rows per block: up to 40 KB of shared memory, and
 // no more than leaves two blocks per SM; a single row has to fit 48 KB (K <= 6128).
@@ -1536,11 +1547,10 @@ static las_status slice_contig(RowsContig src, const Planes& P, int* ex, cudaStr
   long kb;
   const long rows = slice_extent(P, live_only, &kb);
   const long S = kb * BK + 2;
-  if (S * 8 > 48 * 1024 - 512) return slice_rows(src, P, ex, st, live_only);
+  if (!slice_fits(kb)) return slice_rows(src, P, ex, st, live_only);
   int lg = 0;
   while (lg < 5 && (S * 8 << (lg + 1)) <= 40 * 1024 && (rows >> (lg + 1)) >= 2 * num_sms()) ++lg;
-  k_slice_kmajor<<<(unsigned)((rows + (1 << lg) - 1) >> lg), 256, (size_t)(S * 8) << lg,
-                         st>>>(src, src.aligned(), P, rows, kb, lg, (int)S, ex);
+  launch_chained(k_slice_kmajor, (unsigned)((rows + (1 << lg) - 1) >> lg), 256, (size_t)(S * 8) << lg, st, src, src.aligned(), P, rows, kb, lg, (int)S, ex);
   return slice_done("k_slice_kmajor launch");
 }
 
@@ -1551,22 +1561,23 @@ static las_status slice_cols(Acc acc, const Planes& P, int* ex, cudaStream_t st,
   if (P.R <= 0) return LAS_OK;
   long kb;
   const long rows = slice_extent(P, live_only, &kb);
-  k_slice_cols<Acc><<<(unsigned)((rows + 15) / 16), 512, 0, st>>>(acc, P, rows, kb, ex);
+  launch_chained(k_slice_cols<Acc>, (unsigned)((rows + 15) / 16), 512, 0, st, acc, P, rows, kb, ex);
   return slice_done("k_slice_cols launch");
 }
 
-// Long rows contiguous in K (the projection's W): block-parallel maxima in mx, then the digits of
-// the live rows.
+// Few long rows contiguous in K (the projection's W): a block per row while a row fits shared
+// memory (one launch); else block-parallel maxima in mx, then the digits of the live rows.
 static las_status slice_long(RowsContig src, const Planes& P, int* ex, unsigned long long* mx,
                              cudaStream_t st) {
   if (P.R <= 0) return LAS_OK;
+  if (slice_fits(planes_nkb(P.K))) return slice_contig(src, P, ex, st, true);
   LAS_CUDA_TRY(cudaMemsetAsync(mx, 0, P.R * sizeof(unsigned long long), st));
   const long seg = 8192;
   dim3 g1((unsigned)((P.K + seg - 1) / seg), (unsigned)P.R);
-  k_rowmax_long<<<g1, 256, 0, st>>>(src, P.K, seg, mx);
+  launch_chained(k_rowmax_long, g1, 256, 0, st, src, P.K, seg, mx);
   las_count_launch();
   const long kb = std::min(P.nkb, planes_nkb(P.K)), tot = P.R * kb * 2;
-  k_digits_long<<<(unsigned)((tot + 255) / 256), 256, 0, st>>>(src, P, P.R, kb, mx, ex);
+  launch_chained(k_digits_long, (unsigned)((tot + 255) / 256), 256, 0, st, src, P, P.R, kb, mx, ex);
   return slice_done("k_digits_long launch");
 }
 
@@ -1579,11 +1590,11 @@ static las_status slice_transposed(const double* src, const Planes& P, int* ex,
     LAS_CUDA_TRY(cudaMemsetAsync(mx, 0, P.R * sizeof(unsigned long long), st));
     const long seg = 512;
     dim3 g1((unsigned)((P.R + 255) / 256), (unsigned)((P.K + seg - 1) / seg));
-    k_colmax<<<g1, 256, 0, st>>>(src, P.K, (int)P.R, seg, mx);
+    launch_chained(k_colmax, g1, 256, 0, st, src, P.K, (int)P.R, seg, mx);
     las_count_launch();
   }
   const long kb = planes_nkb(P.K), warps = (P.R + 15) / 16 * kb;
-  k_digits_cols<<<(unsigned)((warps + 7) / 8), 256, 0, st>>>(
+  launch_chained(k_digits_cols, (unsigned)((warps + 7) / 8), 256, 0, st, 
       RowsStrided{src, 1, P.R}, P, kb, mx, ex);
   return slice_done("k_digits_cols launch");
 }
@@ -2060,6 +2071,7 @@ extern "C" las_status las_split_gemm(long M, long N, long K, const double* A, lo
   int* eb = (int*)w;
   w += rup(N * 4, 256);
   int* status = (int*)w;
+  ChainScope chain(st);
   LAS_CUDA_TRY(cudaMemsetAsync(status, 0, 4, st));
   las_status rc = slice_contig(RowsContig{A, lda}, Ad, ea, st);
   if (rc == LAS_OK) rc = slice_cols(RowsStrided{B, 1, ldb}, Bd, eb, st);
