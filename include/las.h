@@ -258,7 +258,8 @@ int las_stage_times(las_ctx* ctx, float* ms, int cap);
  * The method has no counterpart in the paper (which runs FP64 GEMMs and names reduced precision
  * only as an outlook, section "Outlook"); it implements that outlook for this hardware.
  * workspace: device buffer of at least las_split_gemm_workspace(M, N, K) bytes, 256-byte
- * aligned, owned by the caller.  Synchronous: returns after C is written (or an error). */
+ * aligned, owned by the caller: the digit planes, and where few tiles would leave SMs idle the
+ * partial sums of a K split (a buffer that holds only the planes is accepted too).  Synchronous: returns after C is written (or an error). */
 size_t las_split_gemm_workspace(long M, long N, long K);
 las_status las_split_gemm(long M, long N, long K, const double* A, long lda, const double* B,
                           long ldb, double* C, long ldc, void* workspace,
@@ -271,8 +272,9 @@ las_status las_split_gemm(long M, long N, long K, const double* A, long lda, con
  * has no counterpart; this is a service of this library.
  * Scratch: a fixed LAS_NOALLOC_SCRATCH_BYTES device array inside the library image (held by
  * every GPU that loads the library until the process exits); nothing is allocated or freed.
- * Sizes whose digit planes do not fit the array, i.e. las_split_gemm_workspace(M, N, K) >
- * LAS_NOALLOC_SCRATCH_BYTES, are rejected with LAS_ERR_WORKSPACE before any GPU work.
+ * Sizes whose digit planes do not fit the array are rejected with LAS_ERR_WORKSPACE before any
+ * GPU work.  (las_split_gemm_workspace may ask for more: it counts the partial sums of a K split,
+ * which is shortened to what is left of the array.)
  * The first call on each device looks up the array's device address (with that device
  * current) and keeps it for later calls; make that first call before any stream capture
  * begins.  A reset of the device's primary context (cudaDeviceReset) invalidates the kept

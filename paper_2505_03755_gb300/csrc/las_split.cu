@@ -826,14 +826,15 @@ __device__ __forceinline__ unsigned long long absbits(double x) {
 // 28 (2400 x 192 rows of 1200 values: 2.02 ms, 5.5 TB/s, against 2.34).  Few rows per block leave room for
 // five or more blocks per SM, whose loads and stores overlap.  S = 2 modulo 16: the 16-byte reads of
 // 8 neighbouring threads (rows, or 4 rows and two halves) fall into different banks.
-__global__ void __launch_bounds__(256)
-k_slice_kmajor(RowsContig src, int vec, Planes P, long rows, long kb, int lg, int S, int* ex) {
-  pdl_begin();
+// Blocks of 256 threads.
+__device__ __forceinline__ void slice_kmajor_block(const RowsContig& src, int vec, const Planes& P,
+                                                   long rows, long kb, int lg, int S, int* ex,
+                                                   long block) {
   extern __shared__ __align__(16) double rowbuf[];
   __shared__ unsigned long long mxs[32];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int rb = 1 << lg;
-  const long r0 = (long)blockIdx.x << lg;
+  const long r0 = block << lg;
   const int n = (int)P.K, kend = (int)(kb * BK);
   if (tid < rb) mxs[tid] = 0;
   __syncthreads();
@@ -885,19 +886,19 @@ k_slice_kmajor(RowsContig src, int vec, Planes P, long rows, long kb, int lg, in
 // Sources read along the rows r (neighbouring r are neighbours in memory, or nearly), 16 rows per
 // block over all of K: maxima first, then a warp cuts 16 rows x 16 values of K per step, whose
 // stores are 512 contiguous bytes per plane.  For products small enough to stay in L2 between the
-// two passes.  Rows >= R are written as zeros.
-template <class Acc>
-__global__ void __launch_bounds__(512)
-k_slice_cols(Acc acc, Planes P, long rows, long kb, int* ex) {
-  pdl_begin();
-  __shared__ unsigned long long red[16][16];
+// two passes.  Rows >= R are written as zeros.  Blocks of NT threads.
+template <int NT, class Acc>
+__device__ __forceinline__ void slice_cols_block(const Acc& acc, const Planes& P, long rows,
+                                                 long kb, int* ex, long block) {
+  constexpr int NW = NT / 32;
+  __shared__ unsigned long long red[NW][16];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, rl = lane & 15;
-  const long r = blockIdx.x * 16L + rl;
+  const long r = block * 16 + rl;
   const bool live = r < P.R;
   unsigned long long m = 0;
   if (live) {
 #pragma unroll 4
-    for (long k = tid >> 4; k < P.K; k += 32) {
+    for (long k = tid >> 4; k < P.K; k += NT / 16) {
       const unsigned long long b = absbits(acc(r, k));
       m = b > m ? b : m;
     }
@@ -906,17 +907,43 @@ k_slice_cols(Acc acc, Planes P, long rows, long kb, int* ex) {
   m = o > m ? o : m;
   if (lane < 16) red[warp][rl] = m;
   __syncthreads();
-  for (int w = 0; w < 16; ++w) m = red[w][rl] > m ? red[w][rl] : m;
+  for (int w = 0; w < NW; ++w) m = red[w][rl] > m ? red[w][rl] : m;
   const int e = exp_of_maxbits(m);
   if (tid < 16 && live) ex[r] = e;
   if (r >= rows) return;
-  for (long b = warp; b < kb; b += 16) {
+  for (long b = warp; b < kb; b += NW) {
     const long k0 = b * BK + (lane >> 4) * 8;
     double x[8];
 #pragma unroll
     for (int j = 0; j < 8; ++j) x[j] = (live && k0 + j < P.K) ? acc(r, k0 + j) : 0.0;
     store_digits8(P, r, k0, x, e);
   }
+}
+
+__global__ void __launch_bounds__(256)
+k_slice_kmajor(RowsContig src, int vec, Planes P, long rows, long kb, int lg, int S, int* ex) {
+  pdl_begin();
+  slice_kmajor_block(src, vec, P, rows, kb, lg, S, ex, blockIdx.x);
+}
+
+template <class Acc>
+__global__ void __launch_bounds__(512)
+k_slice_cols(Acc acc, Planes P, long rows, long kb, int* ex) {
+  pdl_begin();
+  slice_cols_block<512>(acc, P, rows, kb, ex, blockIdx.x);
+}
+
+// Both operands of a product A B, A contiguous in K, B along its columns, in one launch: the first
+// ncols blocks cut B (each of them takes longest), the others A; and the status word is cleared.
+__global__ void __launch_bounds__(256)
+k_slice_operands(RowsContig a, int vec, Planes Pa, long kb, int lg, int S, int* ea, RowsStrided b,
+                 Planes Pb, int* eb, int ncols, int* status) {
+  pdl_begin();
+  if (blockIdx.x == 0 && threadIdx.x == 0) *status = 0;
+  if ((int)blockIdx.x < ncols)
+    slice_cols_block<256>(b, Pb, Pb.R, kb, eb, blockIdx.x);
+  else
+    slice_kmajor_block(a, vec, Pa, Pa.R, kb, lg, S, ea, (long)blockIdx.x - ncols);
 }
 
 // The second pass of such sources with the maxima given (mx): one warp per 16 rows x 16 values of
@@ -1538,6 +1565,11 @@ static las_status slice_rows(Acc acc, const Planes& P, int* ex, cudaStream_t st,
 }
 
 static bool slice_fits(long kb) { return (kb * BK + 2) * 8 <= 48 * 1024 - 512; }
+static int slice_lg(long S, long rows) {
+  int lg = 0;
+  while (lg < 5 && (S * 8 << (lg + 1)) <= 40 * 1024 && (rows >> (lg + 1)) >= 2 * num_sms()) ++lg;
+  return lg;
+}
 
 // Rows contiguous in K.  Rows per block: up to 40 KB of shared memory, and
 // no more than leaves two blocks per SM; a single row has to fit 48 KB (K <= 6128).
@@ -1548,8 +1580,7 @@ static las_status slice_contig(RowsContig src, const Planes& P, int* ex, cudaStr
   const long rows = slice_extent(P, live_only, &kb);
   const long S = kb * BK + 2;
   if (!slice_fits(kb)) return slice_rows(src, P, ex, st, live_only);
-  int lg = 0;
-  while (lg < 5 && (S * 8 << (lg + 1)) <= 40 * 1024 && (rows >> (lg + 1)) >= 2 * num_sms()) ++lg;
+  const int lg = slice_lg(S, rows);
   launch_chained(k_slice_kmajor, (unsigned)((rows + (1 << lg) - 1) >> lg), 256, (size_t)(S * 8) << lg, st, src, src.aligned(), P, rows, kb, lg, (int)S, ex);
   return slice_done("k_slice_kmajor launch");
 }
@@ -2041,9 +2072,28 @@ static size_t sgemm_ws(long M, long N, long K) {
          rup(N * 4, 256) + 256;
 }
 
+// K splits of the product: few tiles leave SMs idle, and a split costs the sum of its partials (about
+// 6 K blocks' time).  2999 x 1201 x 187: 48 tiles in 3 parts.
+static int sgemm_ksplit(long M, long N, long K, size_t room) {
+  const long tiles = ozaki_tiles(M, N, 0, pick_bn(N)), kb = planes_nkb(K), sms = num_sms();
+  const long cap = std::min<long>({16, kb / 4, (long)(room / ((size_t)M * N * 8))});
+  int best = 1;
+  long best_t = (tiles + sms - 1) / sms * (kb + CHUNK);
+  for (long ks = 2; ks <= cap; ++ks) {
+    const long per = (kb + ks - 1) / ks;
+    const long t = (tiles * ks + sms - 1) / sms * (per + CHUNK) + 6;
+    if (t < best_t && (kb + per - 1) / per == ks) {
+      best_t = t;
+      best = (int)ks;
+    }
+  }
+  return best;
+}
+
 extern "C" size_t las_split_gemm_workspace(long M, long N, long K) {
   if (M <= 0 || N <= 0 || K <= 0) return 0;
-  return sgemm_ws(M, N, K);
+  const int ks = sgemm_ksplit(M, N, K, ~(size_t)0 >> 1);
+  return sgemm_ws(M, N, K) + (ks > 1 ? (size_t)ks * M * N * 8 : 0);
 }
 
 extern "C" las_status las_split_gemm(long M, long N, long K, const double* A, long lda,
@@ -2071,12 +2121,33 @@ extern "C" las_status las_split_gemm(long M, long N, long K, const double* A, lo
   int* eb = (int*)w;
   w += rup(N * 4, 256);
   int* status = (int*)w;
+  w += 256;
   ChainScope chain(st);
-  LAS_CUDA_TRY(cudaMemsetAsync(status, 0, 4, st));
-  las_status rc = slice_contig(RowsContig{A, lda}, Ad, ea, st);
-  if (rc == LAS_OK) rc = slice_cols(RowsStrided{B, 1, ldb}, Bd, eb, st);
-  if (rc == LAS_OK)
+  // the planes' padding rows stay unwritten: they only feed rows and columns that are not stored
+  las_status rc = LAS_OK;
+  const RowsContig ra{A, lda};
+  const RowsStrided rb{B, 1, ldb};
+  if (slice_fits(Ad.nkb)) {
+    const long S = Ad.nkb * BK + 2;
+    const int lg = slice_lg(S, M), ncols = (int)((N + 15) / 16);
+    launch_chained(k_slice_operands, (unsigned)(ncols + ((M + (1 << lg) - 1) >> lg)), 256,
+                   (size_t)(S * 8) << lg, st, ra, (int)ra.aligned(), Ad, Ad.nkb, lg, (int)S, ea, rb,
+                   Bd, eb, ncols, status);
+    rc = slice_done("k_slice_operands launch");
+  } else {
+    LAS_CUDA_TRY(cudaMemsetAsync(status, 0, 4, st));
+    rc = slice_rows(ra, Ad, ea, st, true);
+    if (rc == LAS_OK) rc = slice_cols(rb, Bd, eb, st, true);
+  }
+  if (rc != LAS_OK) return rc;
+  const int ks = sgemm_ksplit(M, N, K, workspace_bytes - sgemm_ws(M, N, K));
+  double* part = (double*)w;
+  if (ks == 1) {
     rc = ozaki_gemm(Ad, 0, ea, M, Bd, 0, eb, N, K, 1, 0, C, ldc, 0, 0, 0, status, st);
+  } else {
+    rc = ozaki_gemm(Ad, 0, ea, M, Bd, 0, eb, N, K, ks, 0, part, N, M * N, 0, 0, status, st);
+    if (rc == LAS_OK) launch_reduce_partials(part, ks, M * N, C, 0, st, (int)N, (int)ldc);
+  }
   if (rc != LAS_OK) return rc;
   int h = 0;
   LAS_CUDA_TRY(cudaMemcpyAsync(&h, status, 4, cudaMemcpyDeviceToHost, st));
