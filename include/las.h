@@ -233,8 +233,9 @@ las_status las_autotune(las_ctx* ctx, const double* C, const double* h, const do
                         const double* dm2, double* E, double* dEdC);
 
 /* Tile widths of the split products of a context (bn4: host int[4], for S1, S2, projection and
- * one-electron products; each 64 or 96), as chosen by las_autotune or set by hand.  Split mode
- * only (LAS_ERR_UNSUPPORTED otherwise). */
+ * one-electron products; each 64 or 96), as chosen by las_autotune or set by hand; products left to
+ * the library may run narrower tiles (results do not depend on the width).  Split mode only
+ * (LAS_ERR_UNSUPPORTED otherwise). */
 las_status las_get_tiles(const las_ctx* ctx, int* bn4);
 las_status las_set_tiles(las_ctx* ctx, const int* bn4);
 

@@ -1277,9 +1277,9 @@ extern "C" las_status las_autotune(las_ctx* x, const double* C, const double* h,
   // tile width of each product kind, judged by the stage that holds it: [0] S1, [1] S2 and the
   // H slicer, [3] the projection, [4] the one-electron products, energy and assembly
   const int stage_of[SPLIT_NKIND] = {0, 1, 3, 4};
-  const int widths[] = {96, 64};
+  const int widths[] = {0, 96, 64};   // 0: by the rule of the columns
   for (int kind = 0; kind < SPLIT_NKIND && st == LAS_OK; ++kind) {
-    int best = split_get_tile(x->split, kind);
+    int best = 0;
     float best_ms = 1e30f;
     for (int bn : widths) {
       if ((st = split_set_tile(x->split, kind, bn)) != LAS_OK) break;

@@ -45,12 +45,12 @@ constexpr int EPI_WARPS = 16;    // epilogue warps: 4 column groups x 4 TMEM lan
 constexpr int EPI_WARP0 = 3;     // warp 0 TMA, warps 1 and 2 MMA, then the epilogue warps
 constexpr int NTHREADS = 32 * (EPI_WARP0 + EPI_WARPS);
 
-// Tile width bn (columns of the output per CTA tile, a product's parameter: 64 or 96) and the
+// Tile width bn (columns of the output per CTA tile, a product's parameter: 48, 64, 80 or 96) and the
 // stage layout, sized for the widest tile BN.  The exact weight groups q = 0..3 each own one
 // FP32 accumulator of bn TMEM columns, at column q*bn, and the tail groups 4 and 5 share one
 // more, at the fixed column TAIL_COL = 4*BN whatever the tile width, so that consecutive tiles
 // of different widths in one launch never put one tile's tail where the previous tile's exact
-// accumulators are still being drained (every accumulator starts at a multiple of 32).  The
+// accumulators are still being drained (every accumulator starts at a multiple of 16).  The
 // six B digit planes of a stage lie back to back in shared memory (plane t at t*bn rows), so
 // that one MMA of A_s against planes t0..t1 of B (N = (t1-t0+1)*bn <= 256) lands every product
 // A_s B_t in the accumulator of its own exact group s + t: the ten exact products of a
@@ -167,7 +167,7 @@ struct OzParams {
   int lower;               // symmetric product: only tiles that touch the lower triangle
   long tiles_z;            // tiles per K split (the lower-triangle ones only when lower != 0)
   int sh;                  // fractional bits kept when merging the tail
-  int bn;                  // tile width: 64 or 96 columns
+  int bn;                  // tile width: 48, 64, 80 or 96 columns
   int a_mn;                // A read MN-major: rows of the stored planes are K, their K is M
   // A = the Cholesky vectors in packed-triangle digit form (a_pack != 0; see BPacked): the
   // product's row tiles are the full 128-row blocks R of each b^L (tile m = L * pk_nb1 + R of the
@@ -346,11 +346,11 @@ __device__ __forceinline__ void mma_tail(uint32_t tmem_tail, uint32_t sa, uint32
 // Whether an issuer runs as a converged warp that elects the issuing thread (its addresses then stay
 // in uniform registers, and it issues an MMA in 48 clocks instead of 56) or as a single thread.  At
 // 64 columns, where the issue bounds the tail, the converged form takes 1130 to 1170 clocks a stage
-// instead of 1240 (800-orbital autograd 13.0 -> 12.2 ms); at 96 columns, where shared memory is the
-// bound, its bursts cost 5 % (1200-orbital half 23.7 -> 24.9 ms), and in grouped launches of short
-// tiles 20 % (batch of 8: 3.6 -> 4.3 ms).
+// instead of 1240 (800-orbital autograd 13.0 -> 12.2 ms); at 96 and 80 columns, where shared memory is
+// the bound, its bursts cost 5 % (1200-orbital half 23.7 -> 24.9 ms, 400 orbitals 1.41 -> 1.46 ms),
+// and in grouped launches of short tiles 20 % (batch of 8: 3.6 -> 4.3 ms).
 __host__ __device__ constexpr bool issue_converged(bool grouped, int fixbn, bool exact) {
-  return !grouped && fixbn == 64;
+  return !grouped && (fixbn == 64 || fixbn == 48);
 }
 
 // Persistent CTAs (one per SM) walk the tiles (row tile, column tile, K split).  Roles:
@@ -366,8 +366,8 @@ __host__ __device__ constexpr bool issue_converged(bool grouped, int fixbn, bool
 // tile's tail, so that tail products of up to NSTAGE stages run during a drain.
 // GROUPED: the launch walks the concatenated tiles of nprob products described in global
 // memory (probs); otherwise the one product of the kernel parameters.  FIXBN: the tile width of
-// every product of the launch as a compile-time constant (64 or 96), or 0 when products of both
-// widths share a grouped launch (each tile then reads its product's width).  PACK: the launch
+// every product of the launch as a compile-time constant, or 0 when a grouped launch holds other
+// widths than 64 or 96 alone (each tile then reads its product's width).  PACK: the launch
 // may hold products whose A is the packed-triangle form of the Cholesky vectors (a_pack); the
 // other instantiations leave that logic out of the issuing and loading threads entirely.  AMN:
 // the A orientation of the launch's products as a compile-time constant (0: K-major, 1:
@@ -376,8 +376,14 @@ __host__ __device__ constexpr bool issue_converged(bool grouped, int fixbn, bool
 // f(tile width as a compile-time constant): the launch's fixed width, or the one of this tile.
 template <int FIXBN, class F>
 __device__ __forceinline__ bool with_width(int bn, F f) {
-  if constexpr (FIXBN != 0) return f(std::integral_constant<int, FIXBN>());
-  else return bn == 64 ? f(std::integral_constant<int, 64>()) : f(std::integral_constant<int, 96>());
+  if constexpr (FIXBN != 0) {
+    return f(std::integral_constant<int, FIXBN>());
+  } else {
+    if (bn == 48) return f(std::integral_constant<int, 48>());
+    if (bn == 64) return f(std::integral_constant<int, 64>());
+    if (bn == 80) return f(std::integral_constant<int, 80>());
+    return f(std::integral_constant<int, 96>());
+  }
 }
 
 template <int BN, bool GROUPED, int FIXBN, bool PACK, int AMN = 2>
@@ -1206,22 +1212,24 @@ static las_status make_plane_map_mn(CUtensorMap* m, const Planes& P) {
   return r == CUDA_SUCCESS ? LAS_OK : LAS_ERR_INTERNAL;
 }
 
-// Widest tile (the stage layout's B region) and the default tile width of a product: 96
-// columns, so that the four exact accumulators and the tail take 480 of the 512 TMEM columns.
-// A product may run with 64-column tiles instead (las_autotune chooses per product kind).
+// Widest tile (the stage layout's B region): 96 columns, so that the four exact accumulators and the
+// tail take 480 of the 512 TMEM columns.  A product runs with tiles of 48, 64, 80 or 96 columns.
 constexpr int OZ_BN = 96;
-static bool valid_bn(int bn) { return bn == 64 || bn == 96; }
-
-// Time of a stage of 96 and of 64 columns (clocks per 16 values of K, 50 to 75 stages a tile): the
-// narrow one pays nearly as much for its A planes, so it wins only where it saves a third of the
-// columns.  op = 128 (800 orbitals): 2 x 64 columns 2300, 96 + 64 2490 and B read twice.
-constexpr int STAGE96 = 1340, STAGE64 = 1150;
+constexpr int TILE_WIDTHS[] = {48, 64, 80, 96};
+// Measured time of a stage of each width (clocks per 16 values of K, 50 to 75 stages a tile): what a
+// narrow one saves is its B planes only, so the width that wins is the one that fits.  op = 128
+// (800 orbitals): 2 x 64 columns 2340, 96 + 64 2600 and B read twice.
+constexpr int STAGE_TIME[] = {1060, 1170, 1310, 1430};
+static bool valid_bn(int bn) { return bn == 48 || bn == 64 || bn == 80 || bn == 96; }
+static int stage_time(int bn) { return STAGE_TIME[(bn - 48) / 16]; }
+static long cols_time(long N, int bn) { return (N + bn - 1) / bn * stage_time(bn); }
 static int pick_bn(long N) {
-  return (N + 63) / 64 * STAGE64 < (N + 95) / 96 * STAGE96 ? 64 : 96;
+  int best = 96;
+  for (int w : TILE_WIDTHS)
+    if (cols_time(N, w) < cols_time(N, best)) best = w;
+  return best;
 }
 
-// The launch attribute is a per-device setting: set once for each device that uses the kernels
-// (a repeated set from two threads is harmless).
 template <bool GROUPED, int FIXBN>
 static cudaError_t ozaki_attr() {
   auto set = [](auto kern) {
@@ -1248,7 +1256,9 @@ static las_status ozaki_prepare() {
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return LAS_ERR_CUDA;
   if (done[dev]) return LAS_OK;
   cudaError_t e = ozaki_attr<false, 96>();
+  if (e == cudaSuccess) e = ozaki_attr<false, 80>();
   if (e == cudaSuccess) e = ozaki_attr<false, 64>();
+  if (e == cudaSuccess) e = ozaki_attr<false, 48>();
   if (e == cudaSuccess) e = ozaki_attr<true, 96>();
   if (e == cudaSuccess) e = ozaki_attr<true, 64>();
   if (e == cudaSuccess) e = ozaki_attr<true, 0>();
@@ -1378,15 +1388,17 @@ static las_status ozaki_submit(OzProblem& pr, cudaStream_t st) {
   };
   const bool pack = needs_pack(p);
   // full-row products take an instantiation with their A orientation as a compile-time constant
-  if (pack) {
-    if (p.bn == 64) go(k_ozaki<OZ_BN, false, 64, true>);
-    else go(k_ozaki<OZ_BN, false, 96, true>);
-  } else if (p.a_mn) {
-    if (p.bn == 64) go(k_ozaki<OZ_BN, false, 64, false, 1>);
-    else go(k_ozaki<OZ_BN, false, 96, false, 1>);
-  } else {
-    if (p.bn == 64) go(k_ozaki<OZ_BN, false, 64, false, 0>);
-    else go(k_ozaki<OZ_BN, false, 96, false, 0>);
+  auto width = [&](auto bn_c) {
+    constexpr int bn = decltype(bn_c)::value;
+    if (pack) go(k_ozaki<OZ_BN, false, bn, true>);
+    else if (p.a_mn) go(k_ozaki<OZ_BN, false, bn, false, 1>);
+    else go(k_ozaki<OZ_BN, false, bn, false, 0>);
+  };
+  switch (p.bn) {
+    case 48: width(std::integral_constant<int, 48>()); break;
+    case 64: width(std::integral_constant<int, 64>()); break;
+    case 80: width(std::integral_constant<int, 80>()); break;
+    default: width(std::integral_constant<int, 96>()); break;
   }
   las_count_launch();
   cudaError_t e = cudaGetLastError();
@@ -1652,8 +1664,8 @@ struct SplitState {
   int* hexp;             // [n]
   int ksplit6;           // partial buffers allocated for this many K splits
   int ks;                // split-K factor of the projection GEMM (autotunable)
-  int bn[SPLIT_NKIND];   // tile width of each product kind: 64 or 96
-  int bn_set[SPLIT_NKIND];   // the width was chosen by the caller or the autotuner
+  int bn[SPLIT_NKIND];   // tile width of each product kind (64 or 96) as chosen by the caller or the
+                         // autotuner, or 0: by the rule of its columns
   // tangent (Hessian-vector) scratch, allocated by the first split_tangent_prepare: digit planes
   // of dC_occ^T (rows p, K = nu) and of the chunk's dH (rows (L, p), K = mu)
   Planes dCdig;
@@ -1692,8 +1704,6 @@ las_status split_create(SplitState** out, int n, int X, int op, int Lc, const do
   s->Lc = Lc;
   s->status = status;
   s->ksplit6 = 64;
-  for (int k = 0; k < SPLIT_NKIND; ++k) s->bn[k] = pick_bn(op);
-  s->bn[SPLIT_ONE_ELECTRON] = 64;   // fewer tiles than SMs: the shorter tile ends first
   // one-time launch attributes, so that later calls can be captured into CUDA graphs
   if (ozaki_prepare() != LAS_OK || num_sms() <= 0) {
     free(s);
@@ -1811,10 +1821,16 @@ const int* split_hexp(SplitState* s) { return s->Hexp; }
 
 int split_get_ksplit(SplitState* s) { return s->ks; }
 int split_balanced_ksplit(SplitState* s, int nL) {
-  return balanced_ksplit(ozaki_tiles(s->n, s->op, 0, s->bn[SPLIT_PROJECT]),
+  const int bn = s->bn[SPLIT_PROJECT] ? s->bn[SPLIT_PROJECT] : pick_bn(s->op);
+  return balanced_ksplit(ozaki_tiles(s->n, s->op, 0, bn),
                          ((long)nL * s->op + BK - 1) / BK,
                          std::min<long>(s->ksplit6, std::max(1L, ((long)nL * s->op) / KSPLIT_MIN)));
 }
+// The one-electron products are fewer tiles than SMs: the shorter tile ends first.
+static int one_electron_bn(const SplitState* s) {
+  return s->bn[SPLIT_ONE_ELECTRON] ? s->bn[SPLIT_ONE_ELECTRON] : s->op <= 48 ? 48 : 64;
+}
+
 // K splits of a projection over R rows (L, p): at most s->ks of at least KSPLIT_MIN each, counted
 // as ozaki_setup forms them (equal numbers of K blocks, none empty), so that every partial summed
 // afterwards has been written.
@@ -1823,11 +1839,13 @@ static int project_ksplit(const SplitState* s, long R) {
   const long per = (kb + ks - 1) / ks;
   return (int)((kb + per - 1) / per);
 }
-int split_get_tile(SplitState* s, int kind) { return s->bn[kind]; }
+int split_get_tile(SplitState* s, int kind) {
+  if (s->bn[kind]) return s->bn[kind];
+  return kind == SPLIT_ONE_ELECTRON || cols_time(s->op, 64) < cols_time(s->op, 96) ? 64 : 96;
+}
 las_status split_set_tile(SplitState* s, int kind, int bn) {
-  if (kind < 0 || kind >= SPLIT_NKIND || !valid_bn(bn)) return LAS_ERR_ARG;
+  if (kind < 0 || kind >= SPLIT_NKIND || (bn != 0 && bn != 64 && bn != 96)) return LAS_ERR_ARG;
   s->bn[kind] = bn;
-  s->bn_set[kind] = 1;
   return LAS_OK;
 }
 void split_set_ksplit(SplitState* s, int ks) { s->ks = std::max(1, std::min(ks, s->ksplit6)); }
@@ -1844,29 +1862,30 @@ static las_status b_half(const SplitState* s, int l0, int nL, const Planes& Xd, 
                     x_row0, xexp, N, s->n, 1, 1, out, 0, 0, s->n, ht_op, s->status, st, 0, bn);
 }
 
-// The same with the widths of its column tiles chosen here.  In 96-column tiles, the columns beyond
-// the last whole tile may number at most 64 (the JK call's 150 core columns: 96 + 54): they then
-// form a second product of 64-column tiles, 160 columns computed instead of 192.  Not while
-// products are recorded for a grouped launch, which would then mix tile widths.  bn: 0 = by stage
-// times (pick_bn), or the width asked for.
+// The same with the widths of its column tiles chosen here.  The columns beyond the last whole
+// 96-column tile may form a second product of a narrower tile (150 columns as 96 + 54: 160 computed
+// instead of 192); not while products are recorded for a grouped launch, which would then hold
+// more of them.  bn: 0 = by stage times, or the width asked for.
 static las_status b_half_cols(const SplitState* s, int l0, int nL, const Planes& Xd,
                               const int* xexp, long N, double* out, int ht_op, cudaStream_t st,
                               int bn) {
   const long whole = N / 96 * 96, rest = N - whole;
-  const bool ends = whole > 0 && rest > 0 && rest <= 64 && !g_record;   // 96s and one 64
+  const bool ends = whole > 0 && rest > 0 && rest <= 64 && !g_record;   // 96s and a narrower one
+  int last = 64;
+  bool two = bn == 96 && ends;
   if (bn == 0) {
     bn = pick_bn(N);
-    if (ends && bn == 64 && whole / 96 * STAGE96 + STAGE64 < (N + 63) / 64 * STAGE64) bn = 96;
+    last = pick_bn(rest);
+    // a second launch reads B once more: it has to save a twentieth
+    two = ends && (cols_time(whole, 96) + stage_time(last)) * 20 < cols_time(N, bn) * 19;
   }
-  if (bn == 96 && ends) {
+  if (two) {
     las_status rc = b_half(s, l0, nL, Xd, 0, xexp, whole, out, ht_op, st, 96);
     if (rc != LAS_OK) return rc;
-    return b_half(s, l0, nL, Xd, whole, xexp + whole, rest, out + whole * s->n, ht_op, st, 64);
+    return b_half(s, l0, nL, Xd, whole, xexp + whole, rest, out + whole * s->n, ht_op, st, last);
   }
   return b_half(s, l0, nL, Xd, 0, xexp, N, out, ht_op, st, bn);
 }
-
-static int half_bn(const SplitState* s) { return s->bn_set[SPLIT_HALF] ? s->bn[SPLIT_HALF] : 0; }
 
 las_status split_prepare_C(SplitState* s, const double* Cocc, cudaStream_t st) {
   // rows p of C_occ^T (K = nu): element (p, nu) = Cocc[nu*op + p]
@@ -1906,7 +1925,7 @@ las_status split_tangent_prepare(SplitState* s, const double* dCocc, cudaStream_
 
 // dH = b^L dC_occ for the chunk's aux rows (Ht layout [nL][op][n])
 las_status split_tangent_half(SplitState* s, int l0, int nL, double* dHt, cudaStream_t st) {
-  return b_half_cols(s, l0, nL, s->dCdig, s->dCexp, s->op, dHt, s->op, st, half_bn(s));
+  return b_half_cols(s, l0, nL, s->dCdig, s->dCexp, s->op, dHt, s->op, st, s->bn[SPLIT_HALF]);
 }
 
 // After split_full of the chunk: X[(L,p)][q] = sum_mu H_L(mu,p) dC(mu,q) (so that dT_L = X_L +
@@ -1945,7 +1964,7 @@ las_status split_tangent_project(SplitState* s, int nL, int which, const double*
 // hdC = h dC_occ (the digits of h from split_one_electron_hc of the same h)
 las_status split_tangent_one_electron(SplitState* s, double* hdC, cudaStream_t st) {
   return ozaki_gemm(s->hdig, 0, s->hexp, s->n, s->dCdig, 0, s->dCexp, s->op, s->n, 1, 0, hdC,
-                    s->op, 0, 0, 0, s->status, st, 0, s->bn[SPLIT_ONE_ELECTRON]);
+                    s->op, 0, 0, 0, s->status, st, 0, one_electron_bn(s));
 }
 
 las_status split_lpu(SplitState* s, int nL, const double* Ht, int a, const double* C, int nmo,
@@ -1986,7 +2005,7 @@ las_status split_lpu(SplitState* s, int nL, const double* Ht, int a, const doubl
 
 las_status split_half(SplitState* s, int l0, int nL, int oc, double* Ht, cudaStream_t st) {
   if (oc < 1 || oc > s->op) return LAS_ERR_INTERNAL;
-  return b_half_cols(s, l0, nL, s->Cdig, s->Cexp, oc, Ht, oc, st, half_bn(s));
+  return b_half_cols(s, l0, nL, s->Cdig, s->Cexp, oc, Ht, oc, st, s->bn[SPLIT_HALF]);
 }
 
 las_status split_full(SplitState* s, int nL, const double* Ht, double* T, cudaStream_t st) {
@@ -2060,7 +2079,7 @@ las_status split_one_electron_hc(SplitState* s, const double* h, double* hC, cud
   las_status rc = slice_contig(RowsContig{h, s->n}, s->hdig, s->hexp, st, true);
   if (rc == LAS_OK)
     rc = ozaki_gemm(s->hdig, 0, s->hexp, s->n, s->Cdig, 0, s->Cexp, s->op, s->n, 1, 0, hC, s->op,
-                    0, 0, 0, s->status, st, 0, s->bn[SPLIT_ONE_ELECTRON]);
+                    0, 0, 0, s->status, st, 0, one_electron_bn(s));
   return rc;
 }
 
