@@ -169,9 +169,9 @@ las_status las_veff(las_ctx* ctx, const double* C_alpha, const double* w_alpha, 
  *   Dg = d/dt g(C exp(tX)) at t = 0 = (C X)^T G + C^T dG - transpose   (device [nmo][nmo],
  *        NULL to skip; g = C^T dE/dC - transpose is the orbital-rotation gradient)
  * dG is the tangent of the evaluation chain (dE/dC = one-electron terms + sum_L H_L W(T_L), W
- * linear in T): one more half transform b^L dC, one more full-transform product, two per-aux
- * passes and two projections, next to one plain evaluation for G.  Asynchronous.  The first
- * call allocates the tangent's scratch (about the evaluation's per-chunk workspace again). */
+ * linear in T): one more half transform b^L dC, one more full-transform product, one more per-aux
+ * pass and two projections, in the same pass over the auxiliary index as G (formed for Dg only).
+ * Asynchronous.  The first call allocates the tangent's scratch (about the evaluation's per-chunk workspace again). */
 las_status las_orbital_hvp(las_ctx* ctx, const double* C, const double* h, const double* dm1s,
                            const double* dm2, const double* X, double* dG, double* Dg);
 

@@ -745,64 +745,80 @@ extern "C" las_status las_veff(las_ctx* x, const double* Ca, const double* wa, i
 // dC is the tangent chain
 //     dG = [4 h dC_c | 2 h dC_a D | 0] + sum_L ( dH_L W(T_L) + H_L W(dT_L) ),
 //     dH_L = b^L dC_occ,   dT_L = X_L + X_L^T,   X_L = H_L^T dC_occ   (b^L symmetric):
-// one more half transform (dH), one more full-transform product (X), two per-aux passes and two
+// one more half transform (dH), one more full-transform product (X), one more per-aux pass and two
 // projections; in split precision W(T_L) is scaled by the row exponents of dH and W(dT_L) by those
-// of H, the operand each is projected against.  G(C) itself (for Dg) is one plain evaluation.
-static las_status tangent_grad(las_ctx* x, const double* h, const double* dm1s, double* dG) {
-  const int n = x->n, op = x->op, nmo = x->nmo;   // x->tCocc holds dC_occ
+// of H, the operand each is projected against.  G(C) itself is formed for Dg.  One pass over the auxiliary index serves both gradients: H, its digits and T of a chunk are formed
+// once (as an evaluation followed by its tangent they were formed twice, a fifth of the call at 400
+// orbitals).  dC_occ is in x->tCocc; G (into x->hG) is left out unless want_G.
+static las_status grad_and_tangent(las_ctx* x, const double* C, const double* h,
+                                   const double* dm1s, const double* dm2, double* dG,
+                                   bool want_G) {
+  const int n = x->n, op = x->op, nmo = x->nmo;
   const bool split = x->prec == LAS_SPLIT_BF16;
   las_status st;
-  if (split && (st = split_tangent_prepare(x->split, x->tCocc, x->stream, &x->bytes)) != LAS_OK)
+  stage_mark(x, 0);
+  launch_pack_cocc(C, n, nmo, x->o, op, x->Cocc, x->stream, x->a > 0 ? dm2 : nullptr, &x->fi,
+                   x->dm2t);
+  if (split && ((st = split_prepare_C(x->split, x->Cocc, x->stream)) != LAS_OK ||
+                (st = split_tangent_prepare(x->split, x->tCocc, x->stream, &x->bytes)) != LAS_OK))
     return st;
-  if (split && (st = split_prepare_C(x->split, x->Cocc, x->stream)) != LAS_OK) return st;
   for (int l0 = 0; l0 < x->X; l0 += x->Lc) {
     const int nL = std::min(x->Lc, x->X - l0);
+    if ((st = half_and_full(x, l0, nL, 1, l0 == 0 ? 1 : -1)) != LAS_OK) return st;   // H, T
     if (split) {
-      if ((st = split_half(x->split, l0, nL, op, x->Ht, x->stream)) != LAS_OK ||
-          (st = split_tangent_half(x->split, l0, nL, x->tHt, x->stream)) != LAS_OK ||
-          (st = split_full(x->split, nL, x->Ht, x->T, x->stream)) != LAS_OK ||
+      if ((st = split_tangent_half(x->split, l0, nL, x->tHt, x->stream)) != LAS_OK ||
           (st = split_tangent_full(x->split, nL, x->tHt, x->tX, x->stream)) != LAS_OK)
         return st;
     } else {
-      PackedSymA A{x->Bp, x->npair, l0};
-      StridedA Bc{x->Cocc, 0, op, 1}, Bd{x->tCocc, 0, op, 1};
-      gemm_f64(n, op, n, nL, 1, A, Bc, StridedC{x->Ht, (long)op * n, 1, n, 1.0, 0}, x->stream);
-      gemm_f64(n, op, n, nL, 1, A, Bd, StridedC{x->tHt, (long)op * n, 1, n, 1.0, 0}, x->stream);
-      StridedA Ah{x->Ht, (long)op * n, n, 1};
-      gemm_f64<true>(op, op, n, nL, 1, Ah, Bc, StridedC{x->T, (long)op * op, op, 1, 1.0, 0},
-                     x->stream);
+      const StridedA Bd{x->tCocc, 0, op, 1}, Ah{x->Ht, (long)op * n, n, 1};
+      gemm_f64(n, op, n, nL, 1, PackedSymA{x->Bp, x->npair, l0}, Bd,
+               StridedC{x->tHt, (long)op * n, 1, n, 1.0, 0}, x->stream);
       gemm_f64(op, op, n, nL, 1, Ah, Bd, StridedC{x->tX, (long)op * op, op, 1, 1.0, 0},
                x->stream);
     }
     launch_sym_add(x->tX, nL, op, x->tdT, x->stream);
-    // W(T) against dH and W(dT) against H (the per-aux outputs eps, vc, va are not needed)
+    if (l0 == 0) stage_mark(x, 2);
+    // W(T) against H (for G) and against dH, W(dT) against H; in split precision each scaled by the
+    // row exponents of its operand (the per-aux outputs eps, vc, va are not needed)
     const int* hexp = split ? split_hexp(x->split) : nullptr;
     const int* dhexp = split ? split_tangent_dhexp(x->split) : nullptr;
-    launch_per_aux(x->T, nL, op, dm1s, x->dm2t, x->fi, x->tWd, x->eps + l0, x->vc + l0, x->va + l0,
-                   1, dhexp, x->stream);
+    const double* Wd = x->W;   // W(T) for dH
+    launch_per_aux(x->T, nL, op, dm1s, x->dm2t, x->fi, x->W, x->eps + l0, x->vc + l0, x->va + l0,
+                   1, hexp, x->stream);
+    if (split) {
+      launch_rescale_w(x->W, (long)nL * op, op, hexp, dhexp, x->tWd, x->stream);
+      Wd = x->tWd;
+    }
     launch_per_aux(x->tdT, nL, op, dm1s, x->dm2t, x->fi, x->tdW, x->eps + l0, x->vc + l0,
                    x->va + l0, 1, hexp, x->stream);
     if ((st = check_launch()) != LAS_OK) return st;
+    if (l0 == 0) stage_mark(x, 3);
+    if (want_G && (st = project(x, nL, l0 > 0)) != LAS_OK) return st;
     if (split) {
       if ((st = split_tangent_project(x->split, nL, 0, x->tdW, x->tOut, l0 > 0, x->stream)) !=
               LAS_OK ||
-          (st = split_tangent_project(x->split, nL, 1, x->tWd, x->tOut, 1, x->stream)) != LAS_OK)
+          (st = split_tangent_project(x->split, nL, 1, Wd, x->tOut, 1, x->stream)) != LAS_OK)
         return st;
     } else {
       project_f64(x, nL, x->Ht, x->tdW, x->tOut, l0 > 0);
-      project_f64(x, nL, x->tHt, x->tWd, x->tOut, 1);
+      project_f64(x, nL, x->tHt, Wd, x->tOut, 1);
     }
     if ((st = check_launch()) != LAS_OK) return st;
+    if (l0 == 0) stage_mark(x, 4);
   }
-  // h dC_occ
+  // h C_occ and h dC_occ
   if (split) {
     if ((st = split_one_electron_hc(x->split, h, x->hC, x->stream)) != LAS_OK ||
         (st = split_tangent_one_electron(x->split, x->thC, x->stream)) != LAS_OK)
       return st;
   } else {
-    gemm_f64_wide(x, n, op, n, StridedA{h, 0, n, 1}, StridedA{x->tCocc, 0, op, 1}, x->thC, op, 0);
+    const StridedA Ah{h, 0, n, 1};
+    if (want_G) gemm_f64_wide(x, n, op, n, Ah, StridedA{x->Cocc, 0, op, 1}, x->hC, op, 0);
+    gemm_f64_wide(x, n, op, n, Ah, StridedA{x->tCocc, 0, op, 1}, x->thC, op, 0);
   }
+  if (want_G) launch_assemble_grad(x->Out, x->hC, dm1s, x->fi, n, nmo, op, x->hG, x->stream);
   launch_assemble_grad(x->tOut, x->thC, dm1s, x->fi, n, nmo, op, dG, x->stream);
+  stage_mark(x, 5);
   return check_launch();
 }
 
@@ -829,9 +845,7 @@ extern "C" las_status las_orbital_hvp(las_ctx* x, const double* C, const double*
   // dC_occ = C X_occ (only the occupied columns of C X are ever needed); zero padding columns
   LAS_CUDA_TRY(cudaMemsetAsync(x->tCocc, 0, sizeof(double) * n * op, x->stream));
   gemm_f64_wide(x, n, o, nmo, StridedA{C, 0, nmo, 1}, StridedA{X, 0, nmo, 1}, x->tCocc, op, 0);
-  // G(C): C_occ, its digits, those of h and dm2t stay in place for the tangent chain
-  if ((st = evaluate(x, C, h, dm1s, dm2, x->dE, x->hG, nullptr)) != LAS_OK) return st;
-  if ((st = tangent_grad(x, h, dm1s, dG)) != LAS_OK) return st;
+  if ((st = grad_and_tangent(x, C, h, dm1s, dm2, dG, Dg != nullptr)) != LAS_OK) return st;
   if (Dg) {
     // Dg = (C X)^T G + C^T dG - transpose = X^T (C^T G) + C^T dG - transpose  (virtual columns
     // of G and dG are zero)

@@ -139,6 +139,9 @@ void launch_per_aux(const double* T, int nL, int op, const double* dm1s, const d
                     int with_grad, const int* gexp, cudaStream_t s);
 // K = scale * (its lower triangle, mirrored)
 void launch_mirror_lower(double* K, int n, double scale, cudaStream_t s);
+// out[q][k] = Wt[q][k] * 2^(g1[k] - g0[k]) for k < wld, q < rows: Wt scaled by 2^g1 instead of 2^g0
+void launch_rescale_w(const double* Wt, long wld, int rows, const int* g0, const int* g1,
+                      double* out, cudaStream_t s);
 // dT[L] = X[L] + X[L]^T for L < nL (op x op each)
 void launch_sym_add(const double* X, int nL, int op, double* dT, cudaStream_t s);
 // Columns of each sign of w0 (idx, then idx + o: w > 0, w < 0) and of w1 (idx + 2 o, idx + 3 o) in

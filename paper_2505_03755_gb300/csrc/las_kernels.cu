@@ -307,6 +307,16 @@ k_per_aux(const double* __restrict__ T, int nL, int op, const double* __restrict
   }
 }
 
+__global__ void __launch_bounds__(256)
+k_rescale_w(const double* __restrict__ Wt, long wld, const int* __restrict__ g0,
+            const int* __restrict__ g1, double* __restrict__ out) {
+  pdl_begin();
+  const long k = blockIdx.x * 256L + threadIdx.x;
+  if (k >= wld) return;
+  const long i = blockIdx.y * wld + k;
+  out[i] = scale2(Wt[i], g1[k] - g0[k]);
+}
+
 // Columns of each sign of the weights of up to two densities, in order; one warp per density.
 __global__ void __launch_bounds__(32)
 k_sign_split(const double* __restrict__ w0, int r0, const double* __restrict__ w1, int r1, int o,
@@ -668,6 +678,13 @@ void launch_per_aux(const double* T, int nL, int op, const double* dm1s, const d
   // an ordinary launch, as the FP64 GEMM's: its FP64 work is to be even over the SMs
   k_per_aux<<<nL, 256, per_aux_smem(fi, use_p), s>>>(T, nL, op, dm1s, dm2t, fi, W, eps, vc, va,
                                                      with_grad, gexp, use_p);
+  las_count_launch();
+}
+
+void launch_rescale_w(const double* Wt, long wld, int rows, const int* g0, const int* g1,
+                      double* out, cudaStream_t s) {
+  if (wld <= 0 || rows <= 0) return;
+  launch_chained(k_rescale_w, dim3(nblk(wld, 256), rows), 256, 0, s, Wt, wld, g0, g1, out);
   las_count_launch();
 }
 
