@@ -160,7 +160,8 @@ struct OzParams {
   const int* ea;           // row exponents [M] (nullptr: 0)
   const int* eb;           // column exponents [N]
   double* out;
-  int mode;                // 0: out[z*zstride + r*ldc + c]; 1: Ht layout (rows (L,mu))
+  int mode;                // 0: out[z*zstride + r*ldc + c]; 1: Ht layout out[z*zstride +
+                           // (L*ht_op + c)*ht_n + mu] (rows (L,mu))
   int vec;                 // mode 0: rows of out are 32-byte aligned at multiples of 4 columns
   long ldc, zstride;
   int ht_n, ht_op;
@@ -690,7 +691,8 @@ k_ozaki(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtenso
       const int z = kb0 / p.kb_per_split;
       const int e0 = ea - 14 - 8 * (NEXACT - 1) - p.sh;
       double* const orow = p.mode == 0 ? p.out + (long)z * p.zstride + (long)row * p.ldc
-                                       : p.out + L * p.ht_op * (long)p.ht_n + mu;
+                                       : p.out + (long)z * p.zstride +
+                                             L * p.ht_op * (long)p.ht_n + mu;
 #pragma unroll
       for (int b = 0; b < MAXB; ++b) {
         const int c0 = n0 + (cg + 4 * b) * 8;
@@ -1296,14 +1298,14 @@ static long ozaki_tiles(long M, long N, int lower, int bn = OZ_BN) {
   return t;
 }
 
-// K-split factor in [1, cap] that shares `tiles` output tiles of a product with kb K blocks out
+// K-split factor in [lo, cap] that shares `tiles` output tiles of a product with kb K blocks out
 // most evenly over the persistent CTAs: ceil(tiles*ks / SMs) rounds, each of ceil(kb/ks) blocks
 // plus about a chunk of pipeline fill and drain.
-static int balanced_ksplit(long tiles, long kb, long cap) {
+static int balanced_ksplit(long tiles, long kb, long cap, long lo = 1) {
   const long sms = num_sms();
-  int best = 1;
+  int best = (int)lo;
   double best_t = 1e300;
-  for (long ks = 1; ks <= cap; ++ks) {
+  for (long ks = lo; ks <= cap; ++ks) {
     const double t = (double)((tiles * ks + sms - 1) / sms) * (double)((kb + ks - 1) / ks + CHUNK);
     if (t < best_t * (1.0 - 1e-9)) {
       best_t = t;
@@ -2063,14 +2065,45 @@ las_status split_exchange(SplitState* s, int nL, int oc, const double* Ht, doubl
   HT.K = R;
   las_status rc = slice_transposed(Ht, HT, s->hexp, s->mx, true, st);
   if (rc != LAS_OK) return rc;
-  // partials [ks][n][n] live in the projection's partial buffer (64 * n * op doubles)
-  const long cap = std::max(1L, std::min((64L * s->op) / n, R / KSPLIT_MIN));
-  const int ks = balanced_ksplit(ozaki_tiles(n, n, 1), (R + BK - 1) / BK, cap);
-  // symmetric product: only tiles touching the lower triangle; the caller mirrors the result
-  rc = ozaki_gemm(HT, 0, s->hexp, n, HT, 0, s->hexp, n, R, ks, 0, s->part, n, n * n, 0, 0,
-                  s->status, st, 1);
+  // Partials live in the projection's partial buffer (64 * n * op doubles).  Only tiles that touch
+  // the lower triangle are computed; the caller mirrors the result.  When the rows past the last
+  // whole 128-row tile are few, their row tile is mostly padding: they then go as the columns of a
+  // second product instead, stored transposed, if that ends sooner (800 orbitals: 30 row-column
+  // tiles and 7 narrow ones instead of 39).
+  const long kb = (R + BK - 1) / BK, n1 = n / BM * BM, r = n - n1, room = 64L * s->op;
+  auto rounds = [&](long tiles, long ks) {
+    return (tiles * ks + num_sms() - 1) / num_sms() * ((kb + ks - 1) / ks + CHUNK);
+  };
+  auto cap = [&](long rows) { return std::max(1L, std::min(rows, R / KSPLIT_MIN)); };
+  long n0 = n, tiles = ozaki_tiles(n, n, 1);
+  int ks = balanced_ksplit(tiles, kb, cap(room / n)), ksr = 0;
+  if (n1 > 0 && r > 0) {
+    const int bn = pick_bn(r);
+    const long t1 = ozaki_tiles(n1, n1, 1), t2 = ozaki_tiles(n, r, 0, bn);
+    const int k2 = balanced_ksplit(t2, kb, cap(std::min(64L, room / 4 / r)));
+    // no fewer splits than the one product has: the tail's FP32 sums run over a split's K
+    const int k1 = balanced_ksplit(t1, kb, cap((room - k2 * r) / n1), ks);
+    if (k2 >= ks && k2 * r + k1 * n1 <= room && (kb + k1 - 1) / k1 * (k1 - 1) < kb &&
+        (kb + k2 - 1) / k2 * (k2 - 1) < kb &&
+        rounds(t1, k1) * stage_time(OZ_BN) + rounds(t2, k2) * stage_time(bn) <
+            rounds(tiles, ks) * stage_time(OZ_BN)) {
+      n0 = n1;
+      ks = k1;
+      ksr = k2;
+    }
+  }
+  rc = ozaki_gemm(HT, 0, s->hexp, n0, HT, 0, s->hexp, n0, R, ks, 0, s->part, n, n0 * n, 0, 0,
+                  s->status, st, 1, OZ_BN);
   if (rc != LAS_OK) return rc;
-  launch_reduce_partials(s->part, ks, n * n, K, accumulate, st, 0, 0, sgn);
+  launch_reduce_partials(s->part, ks, n0 * n, K, accumulate, st, 0, 0, sgn);
+  if (ksr > 0) {
+    // rows n1.. of K: element (n1 + c, mu) = sum over (mu, c) of the product, written along mu
+    double* part = s->part + (size_t)ks * n1 * n;
+    rc = ozaki_gemm(HT, 0, s->hexp, n, HT, n1, s->hexp + n1, r, R, ksr, 1, part, 0, r * n, (int)n,
+                    (int)r, s->status, st);
+    if (rc != LAS_OK) return rc;
+    launch_reduce_partials(part, ksr, r * n, K + n1 * n, accumulate, st, 0, 0, sgn);
+  }
   return LAS_OK;
 }
 
