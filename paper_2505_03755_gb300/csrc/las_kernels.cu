@@ -66,7 +66,10 @@ __device__ __forceinline__ int frag_of(const FragInfo& fi, int u) {
 //   W_L(p,q): the matrix with  dE/dC(two-electron part) = sum_L H_L W_L, H_L = b^L C_occ.
 // x * 2^g, and -x * 2^g, in exponent-field and sign-bit arithmetic: an FP64 multiply, comparison or
 // negation would each take a slot of the FP64 pipe (and so would those of ldexp, even on a branch
-// that no thread takes).
+// that no thread takes).  The sign is flipped by the same addition as the exponent: an exclusive or
+// with the sign bit is what the compiler takes for a negation and gives to the FP64 pipe (a fifth of
+// k_per_aux's FP64 instructions).
+template <bool NEG = false>
 __device__ __forceinline__ double scale2(double x, int g) {
   unsigned long long b = (unsigned long long)__double_as_longlong(x);
   if ((b & 0x7FF0000000000000ull) == 0) {   // zero, or subnormal: bring the leading one to bit 52
@@ -76,11 +79,9 @@ __device__ __forceinline__ double scale2(double x, int g) {
     if (1 - lz + g < 1) return __longlong_as_double((long long)(b - m));   // (nearly) 0
     b = b - m + (m << lz) + (((long long)-lz) << 52);
   }
-  return __longlong_as_double((long long)b + (((long long)g) << 52));
+  return __longlong_as_double((long long)b + (((long long)(g + (NEG ? 2048 : 0))) << 52));
 }
-__device__ __forceinline__ double neg_scale2(double x, int g) {
-  return scale2(__longlong_as_double(__double_as_longlong(x) ^ (long long)(1ull << 63)), g);
-}
+__device__ __forceinline__ double neg_scale2(double x, int g) { return scale2<true>(x, g); }
 
 // FP64 arithmetic is the bound (about 1.75 multiply-adds per clock and SM, a warp's instruction at
 // 18 clocks however few of its lanes are live): at 150 core and 5 x 8 active orbitals 1.5e5 of them
@@ -124,6 +125,7 @@ k_per_aux(const double* __restrict__ T, int nL, int op, const double* __restrict
     }
     doff[nf] = s;
   }
+#pragma unroll 4
   for (int i = tid; i < a * a; i += 256) {
     const int u = i / a;
     Taa[i] = TL[(long)(c + u) * op + c + i - u * a];
@@ -248,6 +250,7 @@ k_per_aux(const double* __restrict__ T, int nL, int op, const double* __restrict
   const int* gL = gexp ? gexp + Lb * (long)op : nullptr;
   if (a > 0) {
     const int du = 256 % a, di = 256 / a;
+#pragma unroll 2
     for (int i = tid / a, u = tid % a; i < c;) {
       const int K = fk[u], oK = off[K], m = off[K + 1] - oK;
       const double* Ti = TL + (long)i * op + c;
@@ -277,6 +280,7 @@ k_per_aux(const double* __restrict__ T, int nL, int op, const double* __restrict
     const double* Tr = TL + (long)r * op;
     double* Wr = gL ? W + (long)r * wld + Lb * (long)op : WL + (long)r * op;
     if (r < c) {
+#pragma unroll 4
       for (int l = lane; l < c; l += 32) {
         const double t = Tr[l];
         q -= t * t;
