@@ -68,17 +68,37 @@ __device__ __forceinline__ int frag_of(const FragInfo& fi, int u) {
 // negation would each take a slot of the FP64 pipe (and so would those of ldexp, even on a branch
 // that no thread takes).  The sign is flipped by the same addition as the exponent: an exclusive or
 // with the sign bit is what the compiler takes for a negation and gives to the FP64 pipe (a fifth of
-// k_per_aux's FP64 instructions).
+// k_per_aux's FP64 instructions).  Zeros, infinities, NaN and whatever is subnormal before or after
+// the scaling (rounded to even) or overflows in it go through scale2_edge.
+__device__ __forceinline__ double scale2_edge(unsigned long long b, int g) {
+  const unsigned long long sign = b >> 63 << 63, inf = 0x7FF0000000000000ull;
+  unsigned long long m = b << 12 >> 12;
+  int ex = (int)(b >> 52) & 0x7FF;
+  if (ex == 0x7FF || (ex == 0 && m == 0)) return __longlong_as_double((long long)b);
+  if (ex == 0) {   // bring the leading one to bit 52
+    const int lz = __clzll((long long)m) - 11;
+    m <<= lz;
+    ex = 1 - lz;
+  } else {
+    m |= 1ull << 52;
+  }
+  ex += g;
+  if (ex >= 0x7FF) {
+    m = inf;
+  } else if (ex >= 1) {
+    m += (unsigned long long)(ex - 1) << 52;
+  } else {
+    const int sh = 1 - ex;
+    m = sh > 54 ? 0 : (m + (1ull << (sh - 1)) - 1 + ((m >> sh) & 1)) >> sh;
+  }
+  return __longlong_as_double((long long)(sign | m));
+}
 template <bool NEG = false>
 __device__ __forceinline__ double scale2(double x, int g) {
-  unsigned long long b = (unsigned long long)__double_as_longlong(x);
-  if ((b & 0x7FF0000000000000ull) == 0) {   // zero, or subnormal: bring the leading one to bit 52
-    const unsigned long long m = b << 12 >> 12;
-    const int lz = __clzll((long long)m) - 11;
-    if (m == 0) return x;
-    if (1 - lz + g < 1) return __longlong_as_double((long long)(b - m));   // (nearly) 0
-    b = b - m + (m << lz) + (((long long)-lz) << 52);
-  }
+  const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+  const int ex = (int)(b >> 52) & 0x7FF;
+  if (min(ex, ex + g) < 1 || max(ex, ex + g) > 2046)
+    return scale2_edge(b + (NEG ? 1ull << 63 : 0), g);
   return __longlong_as_double((long long)b + (((long long)(g + (NEG ? 2048 : 0))) << 52));
 }
 __device__ __forceinline__ double neg_scale2(double x, int g) { return scale2<true>(x, g); }

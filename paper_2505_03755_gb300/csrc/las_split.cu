@@ -354,6 +354,19 @@ __host__ __device__ constexpr bool issue_converged(bool grouped, int fixbn, bool
   return !grouped && (fixbn == 64 || fixbn == 48);
 }
 
+// f(tile width as a compile-time constant): the launch's fixed width, or the one of this tile.
+template <int FIXBN, class F>
+__device__ __forceinline__ bool with_width(int bn, F f) {
+  if constexpr (FIXBN != 0) {
+    return f(std::integral_constant<int, FIXBN>());
+  } else {
+    if (bn == 48) return f(std::integral_constant<int, 48>());
+    if (bn == 64) return f(std::integral_constant<int, 64>());
+    if (bn == 80) return f(std::integral_constant<int, 80>());
+    return f(std::integral_constant<int, 96>());
+  }
+}
+
 // Persistent CTAs (one per SM) walk the tiles (row tile, column tile, K split).  Roles:
 // warp 0 streams digit-plane stages with TMA, warp 1 issues the tcgen05.mma of the exact groups and
 // warp 2 those of the tail, warps 3.. drain the TMEM accumulators.  Stage, chunk and tile counters
@@ -374,19 +387,6 @@ __host__ __device__ constexpr bool issue_converged(bool grouped, int fixbn, bool
 // the A orientation of the launch's products as a compile-time constant (0: K-major, 1:
 // MN-major), or 2 when each tile reads its product's; the issuing thread runs measurably faster
 // with a constant.
-// f(tile width as a compile-time constant): the launch's fixed width, or the one of this tile.
-template <int FIXBN, class F>
-__device__ __forceinline__ bool with_width(int bn, F f) {
-  if constexpr (FIXBN != 0) {
-    return f(std::integral_constant<int, FIXBN>());
-  } else {
-    if (bn == 48) return f(std::integral_constant<int, 48>());
-    if (bn == 64) return f(std::integral_constant<int, 64>());
-    if (bn == 80) return f(std::integral_constant<int, 80>());
-    return f(std::integral_constant<int, 96>());
-  }
-}
-
 template <int BN, bool GROUPED, int FIXBN, bool PACK, int AMN = 2>
 __global__ void __launch_bounds__(NTHREADS, 1)
 k_ozaki(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,

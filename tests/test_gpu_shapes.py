@@ -179,3 +179,33 @@ def test_hvp_without_rotation_gradient(precision):
         las.close()
     for x, y in zip(*out):
         assert np.abs(x - y).max() <= 1e-9 * np.abs(x).max()
+
+
+@pytest.mark.parametrize("precision", ["fp64", "split", "split_packed"])
+def test_auxiliary_rows_of_extreme_scale(precision):
+    """Auxiliary rows of 2^-560 (their products underflow), 2^-1010 (some elements subnormal) and zeros
+    beside ordinary ones: the scaling of W by powers of two ends in zero there, with no wrap of the
+    exponent field."""
+    s = make_system(37, 12, 5, [(2, 3), (3, 2)], seed=78)
+    Bp = s.Bp.reshape(12, -1).copy()
+    Bp[3] *= 2.0 ** -560
+    Bp[5] *= 2.0 ** -1010
+    Bp[7] = 0.0
+    s.Bp = Bp.reshape(s.Bp.shape)
+    ref = O.system_energy_grad(s)
+    E, G, _ = gpu_energy_grad(s, precision)
+    assert abs(E - ref["E"]) <= (1e-10 * abs(ref["E"]) if precision == "fp64" else 1e-8)
+    assert np.abs(G - ref["G"]).max() <= (1e-9 if precision == "fp64" else 1e-8)
+
+
+def test_fp64_nan_and_infinity_reach_every_result():
+    """One NaN or infinity in B makes the energy and every occupied column of dE/dC non-finite: T_L
+    has no finite element, and neither has W_L."""
+    for bad in (np.nan, np.inf, -np.inf):
+        s = make_system(37, 12, 5, [(2, 3), (3, 2)], seed=79)
+        Bp = s.Bp.reshape(12, -1).copy()
+        Bp[4, 100] = bad
+        s.Bp = Bp.reshape(s.Bp.shape)
+        E, G, _ = gpu_energy_grad(s, "fp64")
+        assert not np.isfinite(E)
+        assert not np.isfinite(G[:, :s.nocc]).any()
