@@ -41,6 +41,7 @@ constexpr int CHUNK = 16;        // stages per exact chunk (256 values of k)
 constexpr int A_PLANE = BM * BK * 2;                 // 4096 B
 constexpr int A_BYTES = NDIG * A_PLANE;              // 24576
 constexpr int TMEM_COLS = 512;
+constexpr int HEAD = 4;          // stages of a chunk's first turn (issue_turns)
 constexpr int EPI_WARPS = 16;    // epilogue warps: 4 column groups x 4 TMEM lane quarters
 constexpr int EPI_WARP0 = 3;     // warp 0 TMA, warps 1 and 2 MMA, then the epilogue warps
 constexpr int NTHREADS = 32 * (EPI_WARP0 + EPI_WARPS);
@@ -289,8 +290,8 @@ struct OzCursor {
 };
 
 // Descriptor of plane `plane` of an operand whose planes lie `bytes` apart: formed for each MMA, or
-// (BASE) as the first plane's plus an offset.  Which is faster depends on the issuing code around it
-// (issue_converged).
+// (BASE) as the first plane's plus an offset, which is faster where addresses stay in uniform
+// registers (issue_in_turn; 800-orbital autograd 11.2 -> 11.0 ms).
 template <bool BASE>
 __device__ __forceinline__ uint64_t plane_desc(uint32_t addr, int plane, int bytes, bool mn) {
   if constexpr (BASE)
@@ -301,56 +302,62 @@ __device__ __forceinline__ uint64_t plane_desc(uint32_t addr, int plane, int byt
               : sm100::smem_desc_sw32(addr + plane * bytes);
 }
 
-// One stage's exact products (groups 0..3): A_s against planes 0 .. 3-s of B, nt consecutive planes
-// (tile width BNV, planes BNV*32 bytes apart) against one A plane as ceil(nt / maxp) MMAs of balanced
-// width (N = np * BNV <= 256), which land in the accumulators of groups s .. 3; s = 0 spans all four
-// groups and starts them at a chunk's first stage.  amn: the stage holds the transposed access of
+// One stage's products, A plane by A plane.  EXACT: groups 0..3, A_s against planes 0 .. 3-s of B as
+// few MMAs of balanced width (N = np * BNV <= 256) that land in the accumulators of groups s .. 3;
+// s = 0 spans all four and starts them when start_exact.  TAIL: groups 4 and 5 (eleven MMAs into the
+// tail accumulator), started when start_tail.  KEEP: the MMAs of one A plane, which follow one
+// another, read it from shared memory once, the first keeping it in the collector buffer; only
+// where no other thread's MMAs come between them.  amn: the stage holds the transposed access of
 // planes stored with rows along K (A MN-major).  Everything is a compile-time constant once
 // inlined: the issuing thread must not spend its time on address arithmetic.
-template <int BNV, bool BASE>
-__device__ __forceinline__ void mma_exact(uint32_t tmem, uint32_t sa, uint32_t sb,
-                                          bool first_in_chunk, bool amn) {
+template <int BNV, bool EXACT, bool TAIL, bool KEEP>
+__device__ __forceinline__ void mma_stage(uint32_t tmem, uint32_t tmem_tail, uint32_t sa,
+                                          uint32_t sb, bool start_exact, bool start_tail, bool amn) {
   constexpr int maxp = 256 / BNV;
+  const uint32_t ia = amn ? sm100::IDESC_A_MN : 0u;
 #pragma unroll
-  for (int s = 0; s < NEXACT; ++s) {
-    const int nt = NEXACT - s, nm = (nt + maxp - 1) / maxp;
+  for (int s = 0; s < NDIG; ++s) {
+    const int nt = EXACT && s < NEXACT ? NEXACT - s : 0, nm = (nt + maxp - 1) / maxp;
+    const int t_tail = s < NEXACT ? NEXACT - s : 0;
+    const int all = nm + (TAIL ? NGROUP - s - t_tail : 0);
     int t = 0;
 #pragma unroll
-    for (int j = 0; j < nm; ++j) {
-      const int np = (nt - t) / (nm - j);
-      sm100::mma_bf16(tmem + (uint32_t)((s + t) * BNV), plane_desc<BASE>(sa, s, A_PLANE, amn),
-                      plane_desc<BASE>(sb, t, BNV * BK * 2, false),
-                      sm100::idesc_bf16(BM, np * BNV) | (amn ? sm100::IDESC_A_MN : 0u),
-                      s > 0 || !first_in_chunk ? 1u : 0u);
-      t += np;
+    for (int m = 0; m < all; ++m) {
+      const uint64_t a = plane_desc<KEEP>(sa, s, A_PLANE, amn);
+      uint32_t d, id, acc;
+      uint64_t b;
+      if (m < nm) {
+        const int np = (nt - t) / (nm - m);
+        d = tmem + (uint32_t)((s + t) * BNV);
+        b = plane_desc<KEEP>(sb, t, BNV * BK * 2, false);
+        id = sm100::idesc_bf16(BM, np * BNV) | ia;
+        acc = s > 0 || !start_exact ? 1u : 0u;
+        t += np;
+      } else {
+        d = tmem_tail;
+        b = plane_desc<KEEP>(sb, t_tail + m - nm, BNV * BK * 2, false);
+        id = sm100::idesc_bf16(BM, BNV) | ia;
+        acc = s > 0 || m > nm || !start_tail ? 1u : 0u;
+      }
+      if (!KEEP || all == 1) sm100::mma_bf16(d, a, b, id, acc);
+      else if (m == 0) sm100::mma_bf16<sm100::FILL>(d, a, b, id, acc);
+      else if (m < all - 1) sm100::mma_bf16<sm100::USE>(d, a, b, id, acc);
+      else sm100::mma_bf16<sm100::LAST_USE>(d, a, b, id, acc);
     }
   }
 }
 
-// One stage's tail products (groups 4 and 5, eleven MMAs into the tail accumulator), started at the
-// first stage of a tile.
-template <int BNV, bool BASE>
-__device__ __forceinline__ void mma_tail(uint32_t tmem_tail, uint32_t sa, uint32_t sb,
-                                         bool first_stage, bool amn) {
-  bool acc = !first_stage;
-  const uint32_t idesc = sm100::idesc_bf16(BM, BNV) | (amn ? sm100::IDESC_A_MN : 0u);
-#pragma unroll
-  for (int s = 0; s < NDIG; ++s)
-#pragma unroll
-    for (int t = (s >= NEXACT ? 0 : NEXACT - s); s + t < NGROUP; ++t) {
-      sm100::mma_bf16(tmem_tail, plane_desc<BASE>(sa, s, A_PLANE, amn),
-                      plane_desc<BASE>(sb, t, BNV * BK * 2, false), idesc, acc ? 1u : 0u);
-      acc = true;
-    }
-}
-
-// Whether an issuer runs as a converged warp that elects the issuing thread (its addresses then stay
-// in uniform registers, and it issues an MMA in 48 clocks instead of 56) or as a single thread.  At
-// 64 columns, where the issue bounds the tail, the converged form takes 1130 to 1170 clocks a stage
-// instead of 1240 (800-orbital autograd 13.0 -> 12.2 ms); at 96 and 80 columns, where shared memory is
-// the bound, its bursts cost 5 % (1200-orbital half 23.7 -> 24.9 ms, 400 orbitals 1.41 -> 1.46 ms),
-// and in grouped launches of short tiles 20 % (batch of 8: 3.6 -> 4.3 ms).
-__host__ __device__ constexpr bool issue_converged(bool grouped, int fixbn, bool exact) {
+// How a launch's two issuers share the work.  In turn: each issues all 21 products of every other
+// stage, as a converged warp that elects the issuing thread (its addresses stay in uniform registers:
+// an MMA in 48 clocks instead of 56), so that an A plane is read from shared memory once for its
+// two to four MMAs.  By group: one issues the exact products, the other the tail's, each as a single
+// thread.  In turn a stage at 64
+// columns takes about 990 clocks, by group 1130 to 1170 (800-orbital autograd 12.2 -> 11.0 ms, JK 7.2 ->
+// 6.7 ms; with the MMAs and copies alone 750 and 950).  At 96 and 80 columns the exact drains (4900 clocks each) set the pace and
+// in turn they leave fewer products to run meanwhile (1200-orbital half 23.7 ms by group, 24.0 in
+// turn; 400 orbitals 1.39 and 1.44); grouped launches hold several widths' code and spill (batch of 8:
+// 3.6 and 4.7 ms).
+__host__ __device__ constexpr bool issue_in_turn(bool grouped, int fixbn) {
   return !grouped && (fixbn == 64 || fixbn == 48);
 }
 
@@ -368,16 +375,24 @@ __device__ __forceinline__ bool with_width(int bn, F f) {
 }
 
 // Persistent CTAs (one per SM) walk the tiles (row tile, column tile, K split).  Roles:
-// warp 0 streams digit-plane stages with TMA, warp 1 issues the tcgen05.mma of the exact groups and
-// warp 2 those of the tail, warps 3.. drain the TMEM accumulators.  Stage, chunk and tile counters
-// run on across tiles so that the loads of the next tile overlap the last MMAs of the current one,
-// and its MMAs overlap the current tile's conversion and stores.
-// One thread issues an MMA in 56 clocks at best (descriptors and all; 65 in this loop), so a single
-// issuer's 17 MMAs took as long at 64 columns as at 96: the issue, not the tensor pipe, set the
-// stage time.  The
-// two issuers write disjoint accumulators and each wait only for what they overwrite: the exact
-// issuer for the drain of the previous chunk, the tail issuer for the read-out of the previous
-// tile's tail, so that tail products of up to NSTAGE stages run during a drain.
+// warp 0 streams digit-plane stages with TMA, warps 1 and 2 issue the tcgen05.mma (by group, or a
+// stage each in turn: issue_in_turn), warps 3.. drain the TMEM accumulators.  Stage, chunk and tile
+// counters run on across tiles so that the loads of the next tile overlap the last MMAs of the current
+// one, and its MMAs overlap the current tile's conversion and stores.
+// Two issuers, because one thread issues an MMA in 56 clocks at best (descriptors and all; 65 in
+// this loop), so a single issuer's 17 MMAs took as long at 64 columns as at 96: the issue, not the
+// tensor pipe, set the stage time.
+// By group, the issuers write disjoint accumulators and each waits only for what it overwrites: the
+// exact issuer for the drain of the previous chunk, the tail issuer for the read-out of the previous
+// tile's tail, so that tail products of up to NSTAGE stages run during a drain.  Shared memory is
+// the bound: the MMAs' reads of A and B and the stage's own bytes are 173 KB at 96 columns, 1352
+// clocks at 128 bytes a clock.
+// In turn, both write all accumulators, one after the other: a turn is handed on through an
+// mbarrier between tcgen05 fences.  A chunk's first turn takes up to HEAD stages, whose tail
+// products run while the last chunk is drained; the others take one.  accf counts one commit by the
+// issuer of each of the chunk's last two turns (both by the first when there is only one), since a
+// commit covers the MMAs of its own thread; the earlier of the two comes before its turn is handed
+// on, so that no arrival of the next chunk can precede it.
 // GROUPED: the launch walks the concatenated tiles of nprob products described in global
 // memory (probs); otherwise the one product of the kernel parameters.  FIXBN: the tile width of
 // every product of the launch as a compile-time constant, or 0 when a grouped launch holds other
@@ -404,15 +419,15 @@ k_ozaki(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtenso
   uint64_t* acce = bars + 2 * NSTAGE + 1;
   uint64_t* drain = bars + 2 * NSTAGE + 2;  // [2] teardown of the two issuers
   uint64_t* accT = bars + 2 * NSTAGE + 4;   // tail accumulator read out (once per tile)
-  uint64_t* tailf = bars + 2 * NSTAGE + 5;  // tail accumulator complete (once per tile)
-  uint32_t* tmem_slot = (uint32_t*)(bars + 2 * NSTAGE + 6);
+  uint64_t* tailf = bars + 2 * NSTAGE + 5;  // by group: tail accumulator complete (once per tile)
+  uint64_t* turn = bars + 2 * NSTAGE + 6;   // [2] in turn: the issuer's go
+  uint32_t* tmem_slot = (uint32_t*)(bars + 2 * NSTAGE + 8);
   volatile int* abort_flag = (volatile int*)(tmem_slot + 1);
 
   pdl_trigger();
-  constexpr bool CONV_E = issue_converged(GROUPED, FIXBN, true);
-  constexpr bool CONV_T = issue_converged(GROUPED, FIXBN, false);
-  const int warp = CONV_E || CONV_T ? __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0)
-                                    : (int)threadIdx.x >> 5;
+  constexpr bool IN_TURN = issue_in_turn(GROUPED, FIXBN);
+  const int warp = IN_TURN ? __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0)
+                           : (int)threadIdx.x >> 5;
   const int lane = threadIdx.x & 31;
   // status word for waits outside any tile (the first product's)
   int* const status0 = GROUPED ? probs[0].p.status : p1.status;
@@ -420,13 +435,15 @@ k_ozaki(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtenso
   if (threadIdx.x == 0) {
     for (int s = 0; s < NSTAGE; ++s) {
       sm100::mbar_init(&full[s], 1);
-      sm100::mbar_init(&empty[s], 2);   // both issuers
+      sm100::mbar_init(&empty[s], IN_TURN ? 1 : 2);
     }
-    sm100::mbar_init(accf, 1);
+    sm100::mbar_init(accf, IN_TURN ? 2 : 1);
     sm100::mbar_init(acce, EPI_WARPS);
     sm100::mbar_init(accT, EPI_WARPS);
-    sm100::mbar_init(&drain[0], 1);
-    sm100::mbar_init(&drain[1], 1);
+    for (int w = 0; w < 2; ++w) {
+      sm100::mbar_init(&drain[w], 1);
+      sm100::mbar_init(&turn[w], 1);
+    }
     sm100::mbar_init(tailf, 1);
     *abort_flag = 0;
     sm100::fence_mbar_init();
@@ -449,14 +466,11 @@ k_ozaki(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtenso
   const uint32_t tmem = *tmem_slot;
   pdl_wait();   // nothing before this reads what an earlier launch wrote
 
-  // ---------------- MMA issuers: the exact groups (warp 1) or the tail (warp 2) ----------------
-  auto issue = [&](auto exact_c) {
+  // ---------------- MMA issuers by group: exact (warp 1) or tail (warp 2) ----------------
+  [[maybe_unused]] auto issue_group = [&](auto exact_c) {
     constexpr bool exact = decltype(exact_c)::value;
-    constexpr bool conv = exact ? CONV_E : CONV_T;   // all lanes are here, one is elected to issue
-    auto issuing = [&]() { return !conv || sm100::elect_one(); };
     auto wait = [&](uint64_t* bar, uint32_t parity, int* status) -> bool {
-      const bool got = sm100::mbar_wait(bar, parity, abort_flag, status, LAS_ERR_TIMEOUT);
-      return conv ? __all_sync(0xffffffffu, got) : got;
+      return sm100::mbar_wait(bar, parity, abort_flag, status, LAS_ERR_TIMEOUT);
     };
     int st = 0;
     uint32_t phase = 0;
@@ -484,14 +498,10 @@ k_ozaki(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtenso
           }
           sm100::tc_fence_after();
           const uint32_t sa = sm100::smem_u32(smem + st * T::STAGE_BYTES);
-          const uint32_t sb = sa + A_BYTES;
-          if (issuing()) {
-            if constexpr (exact) mma_exact<bn, conv>(tmem, sa, sb, first, amn);
-            else mma_tail<bn, conv>(tmem + T::TAIL_COL, sa, sb, first, amn);
-            sm100::mma_commit(&empty[st]);
-            if (exact && ((i % CHUNK) == CHUNK - 1 || i == nkb - 1)) sm100::mma_commit(accf);
-          }
-          if (conv) __syncwarp();
+          mma_stage<bn, exact, !exact, false>(tmem, tmem + T::TAIL_COL, sa, sa + A_BYTES, first,
+                                              first, amn);
+          sm100::mma_commit(&empty[st]);
+          if (exact && ((i % CHUNK) == CHUNK - 1 || i == nkb - 1)) sm100::mma_commit(accf);
           if (++st == NSTAGE) {
             st = 0;
             phase ^= 1;
@@ -513,11 +523,130 @@ k_ozaki(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtenso
       } else {
         ok = stages(std::integral_constant<bool, AMN == 1>(), 0, nkb);
       }
-      if (ok && !exact && issuing()) sm100::mma_commit(tailf);
+      if (ok && !exact) sm100::mma_commit(tailf);
     }
     // make sure no MMA is still writing TMEM when the CTA tears down
-    if (issuing()) sm100::mma_commit(&drain[exact]);
+    sm100::mma_commit(&drain[exact]);
     sm100::mbar_wait(&drain[exact], 0, abort_flag, status0, LAS_ERR_TIMEOUT);
+  };
+
+  // ---------------- MMA issuers in turn (warps 1 and 2) ----------------
+  [[maybe_unused]] auto issue_turns = [&](const int who) {
+    auto wait = [&](uint64_t* bar, uint32_t parity, int* status) -> bool {
+      return __all_sync(0xffffffffu,
+                        sm100::mbar_wait(bar, parity, abort_flag, status, LAS_ERR_TIMEOUT));
+    };
+    int st = 0;
+    uint32_t phase = 0;
+    uint32_t turns = 0, chunks = 0, tiles = 0;   // turns, exact chunks and tiles so far
+    bool ok = true;
+    OzCursor<GROUPED> cur;
+    for (long t = blockIdx.x; t < ntiles && ok; t += gridDim.x) {
+      cur.seek(t, p1, &tmA, &tmB, &tmA2, &tmA3, probs, nprob);
+      const OzParams& p = *cur.P;
+      const int nkb = cur.nkb;
+      [[maybe_unused]] const bool amn_tile = p.a_mn != 0;
+      // packed-triangle A: K blocks of column blocks J > R (above the diagonal) are read MN-major
+      const bool pack = PACK && p.a_pack != 0;
+      [[maybe_unused]] const int kb_mn = pack ? 8 * ((cur.m0 / BM) % p.pk_nb1 + 1) : 0;
+      // Stages [i0, i1) of the tile with one A orientation (a compile-time constant where the
+      // launch fixes it) and one width; false when a wait ran out.
+      auto stages_of = [&](auto bn_c, auto amn, int i0, int i1) -> bool {
+        constexpr int bn = decltype(bn_c)::value;
+        const uint32_t tail = tmem + T::TAIL_COL, ring = sm100::smem_u32(smem);
+        auto my_turn = [&]() -> bool {
+          return turns == 0 || wait(&turn[who], ((turns - 1) >> 1) & 1, p.status);
+        };
+        // after the last MMA of a turn that ends at stage e: the other issuer's go, the chunk's
+        // commits before it (one by each issuer of the chunk's last two turns)
+        auto pass_turn = [&](int i, int e) {
+          const int ce = min(nkb, (i & ~(CHUNK - 1)) + CHUNK);
+          if (e + 1 >= ce) {
+            sm100::mma_commit(accf);
+            if (e == ce && (i & (CHUNK - 1)) == 0) sm100::mma_commit(accf);
+          }
+          sm100::tc_fence_before();
+          sm100::mbar_arrive(&turn[who ^ 1]);
+        };
+#pragma unroll 1
+        for (int i = i0; i < i1; ++turns) {
+          const bool head = (i & (CHUNK - 1)) == 0;
+          const int len = head ? min(HEAD, i1 - i) : 1;
+          const bool mine = (turns & 1) == (uint32_t)who;
+          if (mine && head) {
+            // A chunk's first stages: tail products while the last chunk is drained, then the exact
+            // products (which start the accumulators)
+            int slot = st;
+            uint32_t ph = phase;
+#pragma unroll 1
+            for (int j = 0; j < len; ++j) {
+              if (!wait(&full[slot], ph, p.status) || (j == 0 && !my_turn()) ||
+                  (i + j == 0 && tiles > 0 && !wait(accT, (tiles - 1) & 1, p.status)))
+                return false;
+              sm100::tc_fence_after();
+              const uint32_t sa = ring + slot * T::STAGE_BYTES;
+              if (sm100::elect_one())
+                mma_stage<bn, false, true, true>(tmem, tail, sa, sa + A_BYTES, false, i + j == 0, amn);
+              __syncwarp();
+              if (++slot == NSTAGE) {
+                slot = 0;
+                ph ^= 1;
+              }
+            }
+            if (chunks > 0 && !wait(acce, (chunks - 1) & 1, p.status)) return false;
+            sm100::tc_fence_after();
+            slot = st;
+#pragma unroll 1
+            for (int j = 0; j < len; ++j) {
+              const uint32_t sa = ring + slot * T::STAGE_BYTES;
+              if (sm100::elect_one()) {
+                mma_stage<bn, true, false, true>(tmem, tail, sa, sa + A_BYTES, j == 0, false, amn);
+                sm100::mma_commit(&empty[slot]);
+                if (j == len - 1) pass_turn(i, i + len);
+              }
+              __syncwarp();
+              if (++slot == NSTAGE) slot = 0;
+            }
+          } else if (mine) {
+            if (!wait(&full[st], phase, p.status) || !my_turn()) return false;
+            sm100::tc_fence_after();
+            const uint32_t sa = ring + st * T::STAGE_BYTES;
+            if (sm100::elect_one()) {
+              mma_stage<bn, true, true, true>(tmem, tail, sa, sa + A_BYTES, false, false, amn);
+              pass_turn(i, i + 1);
+              sm100::mma_commit(&empty[st]);
+            }
+            __syncwarp();
+          }
+          if (head) ++chunks;
+          i += len;
+          st += len;
+          if (st >= NSTAGE) {
+            st -= NSTAGE;
+            phase ^= 1;
+          }
+        }
+        return true;
+      };
+      auto stages = [&](auto amn, int i0, int i1) -> bool {
+        return with_width<FIXBN>(p.bn, [&](auto bn_c) { return stages_of(bn_c, amn, i0, i1); });
+      };
+      using K_MAJOR = std::integral_constant<bool, false>;
+      using MN_MAJOR = std::integral_constant<bool, true>;
+      if constexpr (PACK) {
+        // packed-triangle A: the K-major stages (up to the diagonal block), then the MN-major ones
+        const int isplit = pack ? min(nkb, max(0, kb_mn - cur.kb0)) : amn_tile ? 0 : nkb;
+        ok = stages(K_MAJOR(), 0, isplit) && stages(MN_MAJOR(), isplit, nkb);
+      } else if constexpr (AMN == 2) {
+        ok = stages(amn_tile, 0, nkb);
+      } else {
+        ok = stages(std::integral_constant<bool, AMN == 1>(), 0, nkb);
+      }
+      ++tiles;
+    }
+    // make sure no MMA is still writing TMEM when the CTA tears down
+    if (sm100::elect_one()) sm100::mma_commit(&drain[who]);
+    sm100::mbar_wait(&drain[who], 0, abort_flag, status0, LAS_ERR_TIMEOUT);
   };
 
   if (warp == 0 && lane == 0) {
@@ -588,10 +717,10 @@ k_ozaki(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtenso
     for (int k = 0; k < filled; ++k)
       sm100::mbar_wait(&full[k], k < st ? phase : phase ^ 1, abort_flag, status0,
                        LAS_ERR_TIMEOUT);
-  } else if (warp == 1 && (CONV_E || lane == 0)) {
-    issue(std::true_type());    // exact groups
-  } else if (warp == 2 && (CONV_T || lane == 0)) {
-    issue(std::false_type());   // tail
+  } else if (warp == 1 || warp == 2) {
+    if constexpr (IN_TURN) issue_turns(warp - 1);
+    else if (lane == 0 && warp == 1) issue_group(std::true_type());
+    else if (lane == 0) issue_group(std::false_type());
   } else if (warp >= EPI_WARP0) {
     // ---------------- epilogue (16 warps) ----------------
     const int lq = warp & 3;                 // TMEM lane quarter this warp may access
@@ -617,7 +746,7 @@ k_ozaki(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtenso
       for (int c = 0; c < nchunks; ++c, ++gc) {
         const bool fin = (c == nchunks - 1);
         if (!sm100::mbar_wait(accf, gc & 1, abort_flag, p.status, LAS_ERR_TIMEOUT, 256) ||
-            (fin && !sm100::mbar_wait(tailf, tcount & 1, abort_flag, p.status, LAS_ERR_TIMEOUT,
+            (!IN_TURN && fin && !sm100::mbar_wait(tailf, tcount & 1, abort_flag, p.status, LAS_ERR_TIMEOUT,
                                       64)))
           return false;
         sm100::tc_fence_after();
@@ -1219,9 +1348,10 @@ static las_status make_plane_map_mn(CUtensorMap* m, const Planes& P) {
 constexpr int OZ_BN = 96;
 constexpr int TILE_WIDTHS[] = {48, 64, 80, 96};
 // Measured time of a stage of each width (clocks per 16 values of K, 50 to 75 stages a tile): what a
-// narrow one saves is its B planes only, so the width that wins is the one that fits.  op = 128
-// (800 orbitals): 2 x 64 columns 2340, 96 + 64 2600 and B read twice.
-constexpr int STAGE_TIME[] = {1060, 1170, 1310, 1430};
+// narrow one saves is its B planes and, at 48 and 64 columns, the issue in turn, so the width that
+// wins is mostly the one that fits.  op = 128 (800 orbitals): 2 x 64 columns 2040, 96 + 64 2450 and B
+// read twice.
+constexpr int STAGE_TIME[] = {1000, 1020, 1310, 1430};
 static bool valid_bn(int bn) { return bn == 48 || bn == 64 || bn == 80 || bn == 96; }
 static int stage_time(int bn) { return STAGE_TIME[(bn - 48) / 16]; }
 static long cols_time(long N, int bn) { return (N + bn - 1) / bn * stage_time(bn); }

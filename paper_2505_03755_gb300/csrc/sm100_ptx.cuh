@@ -132,24 +132,25 @@ __device__ __forceinline__ void tc_fence_after() {
 }
 
 // D[tmem] (+)= A[smem desc] * B[smem desc]^T, kind::f16 (BF16 inputs, FP32 accumulate).
+// Collector buffer of the A operand: an MMA may keep the A it read (FILL) for the MMAs that follow
+// it with the same A and instruction-descriptor A fields (USE, the last one LAST_USE).
+enum Collect { DISCARD, FILL, USE, LAST_USE };
+
+template <Collect C = DISCARD>
 __device__ __forceinline__ void mma_bf16(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc,
                                          uint32_t idesc, uint32_t accumulate) {
-  asm volatile(
-      "{\n .reg .pred p;\n setp.ne.u32 p, %4, 0;\n"
-      " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(d_tmem),
-      "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
-      : "memory");
-}
-
-// D[tmem] (+)= A[tmem] * B[smem desc]^T, kind::f16; A holds 128 rows (lanes) x 16 BF16 in 8
-// consecutive 32-bit columns.
-__device__ __forceinline__ void mma_bf16_ta(uint32_t d_tmem, uint32_t a_tmem, uint64_t bdesc,
-                                            uint32_t idesc, uint32_t accumulate) {
-  asm volatile(
-      "{\n .reg .pred p;\n setp.ne.u32 p, %4, 0;\n"
-      " tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n}\n" ::"r"(d_tmem),
-      "r"(a_tmem), "l"(bdesc), "r"(idesc), "r"(accumulate)
-      : "memory");
+#define SM100_MMA(COLLECTOR)                                                            \
+  asm volatile(                                                                         \
+      "{\n .reg .pred p;\n setp.ne.u32 p, %4, 0;\n"                                     \
+      " tcgen05.mma.cta_group::1.kind::f16" COLLECTOR " [%0], %1, %2, %3, p;\n}\n" ::"r"( \
+          d_tmem),                                                                      \
+      "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)                               \
+      : "memory")
+  if constexpr (C == FILL) SM100_MMA(".collector::a::fill");
+  else if constexpr (C == USE) SM100_MMA(".collector::a::use");
+  else if constexpr (C == LAST_USE) SM100_MMA(".collector::a::lastuse");
+  else SM100_MMA("");
+#undef SM100_MMA
 }
 
 // One lane of a converged warp.
@@ -159,12 +160,6 @@ __device__ __forceinline__ bool elect_one() {
       "{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.b32 %0, 1, 0, p;\n}\n"
       : "=r"(r));
   return r != 0;
-}
-
-// Copy a 128-row x 256-bit tile (128 x 16 BF16) from shared memory (matrix descriptor) into 8
-// TMEM columns starting at taddr.
-__device__ __forceinline__ void tmem_cp_128x256b(uint32_t taddr, uint64_t sdesc) {
-  asm volatile("tcgen05.cp.cta_group::1.128x256b [%0], %1;" ::"r"(taddr), "l"(sdesc) : "memory");
 }
 
 // Arrive on `bar` once every previously issued tcgen05.mma of this thread has completed.
@@ -183,16 +178,6 @@ __device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t (&r)[8]) {
                : "r"(taddr));
 }
 
-// 32 lanes x 32 bits, 16 consecutive columns per thread.
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,"
-      "%14,%15}, [%16];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
-        "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]),
-        "=r"(r[14]), "=r"(r[15])
-      : "r"(taddr));
-}
 __device__ __forceinline__ void tmem_wait_ld() {
   asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }

@@ -41,6 +41,21 @@ def test_split_gemm_widths(N, K):
         assert np.array_equal(split_gemm(dev(Ai), dev(Bi)).cpu().numpy(), Ai @ Bi), (M, N, K)
 
 
+# numbers of K blocks around the ends of a chunk's first turn and of a chunk (1, 4, 5, 6, 8, 15, 16, 17,
+# 20, 21, 33 blocks of 16), with up to three tiles in a row on one SM
+@pytest.mark.parametrize("kb", [1, 4, 5, 6, 8, 15, 16, 17, 20, 21, 33])
+@pytest.mark.parametrize("N", [48, 64, 128])
+def test_split_gemm_issuer_turns(N, kb):
+    from paper_2505_03755_gb300 import split_gemm
+    K = 16 * kb - 3
+    rng = np.random.default_rng(100 * N + kb)
+    A, B = rng.standard_normal((40000, K)), rng.standard_normal((K, N))
+    C = split_gemm(dev(A), dev(B)).cpu().numpy()
+    assert np.all(np.abs(C - A @ B) <= _bound(A, B))
+    Ai, Bi = np.rint(50 * A[:20000]), np.rint(50 * B)
+    assert np.array_equal(split_gemm(dev(Ai), dev(Bi)).cpu().numpy(), Ai @ Bi)
+
+
 # the longest row that fits a block's shared memory, one value more (the warp-per-row slicer), and
 # rows of odd length (8-byte loads); zero rows; rows of very different scale
 @pytest.mark.parametrize("K", [6127, 6128, 6129, 7001])
