@@ -414,8 +414,8 @@ SPLIT_MODES = ("split", "split_packed")
 # evaluation by the rows processed (the traffic is proportional to the rows: digits of B read
 # once, H written once).  "split_packed" sums the two launches of that layout (the whole 128-row
 # blocks and the ragged rows).
-S1_TRAFFIC_PER_ROW = {"split": (3527966208 + 378804224) / (200 * 1200),
-                      "split_packed": (2052677120 + 355101952 + 141710848 + 1297664) / (200 * 1200)}
+S1_TRAFFIC_PER_ROW = {"split": (3550457856 + 390161920) / (200 * 1200),
+                      "split_packed": (2057078528 + 364888576 + 142021120 + 1876736) / (200 * 1200)}
 
 
 def roofline_for(prec, r, work, peaks, s):

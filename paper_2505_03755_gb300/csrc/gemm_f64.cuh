@@ -9,7 +9,7 @@
 // product (f64_nj), four warps of 16 rows, and every 16 x 8 block beyond M or N, or above the
 // diagonal of a symmetric result, is left out; K steps of 16 are double-buffered so that one CTA per
 // SM keeps the pipe busy.  Against a fixed 64 x 64 tile (half transform of 237 x 237 blocks and 48
-// columns, 948 auxiliary rows: 6.86 ms) a quarter of the DMMAs were padding columns.
+// columns, 948 auxiliary rows: 6.86 ms, now 4.97) a quarter of the DMMAs were padding columns.
 #pragma once
 #include "las_common.cuh"
 
