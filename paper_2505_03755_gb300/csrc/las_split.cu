@@ -1378,6 +1378,18 @@ static cudaError_t ozaki_attr() {
   return e != cudaSuccess ? e : set(k_ozaki<OZ_BN, GROUPED, FIXBN, true>);
 }
 
+// Dynamic shared memory that a row-slicing launch may ask for: one row of 383 K blocks.  Beside it
+// stands the kernels' static part of 1 and 2 KB (the launch would be refused at the default limit,
+// which counts both), so ozaki_prepare raises the limit.
+constexpr int SLICE_SMEM = 48 * 1024;
+static cudaError_t slice_attr() {
+  auto set = [](auto kern) {
+    return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, SLICE_SMEM);
+  };
+  const cudaError_t e = set(k_slice_kmajor);
+  return e != cudaSuccess ? e : set(k_slice_operands);
+}
+
 // Does the product need the instantiation with the packed-triangle logic (its A is the packed
 // form, or its rows are the ragged rows of that form, with one exponent per auxiliary index)?
 static inline bool needs_pack(const OzParams& p) { return p.a_pack || p.ea_perL; }
@@ -1394,8 +1406,9 @@ static las_status ozaki_prepare() {
   if (e == cudaSuccess) e = ozaki_attr<true, 96>();
   if (e == cudaSuccess) e = ozaki_attr<true, 64>();
   if (e == cudaSuccess) e = ozaki_attr<true, 0>();
+  if (e == cudaSuccess) e = slice_attr();
   if (e != cudaSuccess) {
-    las_record_cuda_error(e, "cudaFuncSetAttribute(k_ozaki)", __FILE__, __LINE__);
+    las_record_cuda_error(e, "cudaFuncSetAttribute(split products)", __FILE__, __LINE__);
     return LAS_ERR_CUDA;
   }
   done[dev] = 1;
@@ -1708,7 +1721,7 @@ static las_status slice_rows(Acc acc, const Planes& P, int* ex, cudaStream_t st,
   return slice_done("k_slice_rows launch");
 }
 
-static bool slice_fits(long kb) { return (kb * BK + 2) * 8 <= 48 * 1024 - 512; }
+static bool slice_fits(long kb) { return (kb * BK + 2) * 8 <= SLICE_SMEM; }
 static int slice_lg(long S, long rows) {
   int lg = 0;
   while (lg < 5 && (S * 8 << (lg + 1)) <= 40 * 1024 && (rows >> (lg + 1)) >= 2 * num_sms()) ++lg;
@@ -2304,9 +2317,10 @@ extern "C" las_status las_split_gemm(long M, long N, long K, const double* A, lo
   w += rup(N * 4, 256);
   int* status = (int*)w;
   w += 256;
+  las_status rc = ozaki_prepare();
+  if (rc != LAS_OK) return rc;
   ChainScope chain(st);
   // the planes' padding rows stay unwritten: they only feed rows and columns that are not stored
-  las_status rc = LAS_OK;
   const RowsContig ra{A, lda};
   const RowsStrided rb{B, 1, ldb};
   if (slice_fits(Ad.nkb)) {

@@ -1,0 +1,44 @@
+"""Limits of buffers and launches: the longest rows that the slicers take through shared memory."""
+import numpy as np
+import pytest
+
+from gpu_common import built, dev, gpu_energy_grad, torch_cuda
+from las_inputs import make_system
+from oracle import las_oracle as O
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _gpu():
+    torch_cuda()
+    built()
+
+
+# The row buffer of the K-major slicers ends at 383 K blocks (6128 values); with their static shared
+# memory of 1 and 2 KB that is more than the 48 KB a kernel has without asking for more, from 368 and
+# 376 blocks on (5873 and 6001 values).
+@pytest.mark.parametrize("K", [5856, 5872, 5873, 5984, 6000, 6001, 6064, 6065, 6112, 6113, 6128, 6129])
+def test_split_gemm_longest_rows_in_shared_memory(K):
+    from paper_2505_03755_gb300 import split_gemm
+    rng = np.random.default_rng(K)
+    for M in (1, 40):
+        A, B = rng.standard_normal((M, K)), rng.standard_normal((K, 30))
+        # operand rounding, dropped digit pairs and FP32 tails: below 2^-43 K rowmax colmax
+        bound = 2.0 ** -43 * K * np.abs(A).max(1)[:, None] * np.abs(B).max(0)[None, :]
+        C = split_gemm(dev(A), dev(B)).cpu().numpy()
+        assert np.all(np.abs(C - A @ B) <= bound)
+
+
+# (auxiliary rows) x (padded occupied columns) of a chunk is the length of the projection's W rows:
+# 5984 to 6144 in steps of 16, and two lengths at the widest tile and at several tiles
+@pytest.mark.parametrize("n,c,X", [(20, 4, X) for X in range(374, 385)] +
+                         [(100, 88, 63), (150, 139, 42)])
+def test_energy_grad_longest_projection_rows(n, c, X):
+    s = make_system(n, X, c, [(2, 2), (2, 3)], seed=X)
+    ref = O.system_energy_grad(s)
+    for precision in ("split", "split_packed"):
+        E, G, g = gpu_energy_grad(s, precision)
+        assert abs(E - ref["E"]) <= 1e-8
+        assert np.abs(G - ref["G"]).max() <= 1e-8
+        assert np.abs(g - ref["gorb"]).max() <= 1e-7
