@@ -202,8 +202,10 @@ extern "C" las_status las_create(las_ctx** out, const las_dims* d, const double*
   const size_t fixed = sizeof(double) * ((size_t)x->n * x->op * 4 + E1_BLOCKS +
                                          (size_t)x->nmo * x->op + 3 * (size_t)x->X + x->npair);
   size_t cap = max_ws ? max_ws : (size_t)64 << 30;
+  const size_t part = sizeof(double) * (prec == LAS_SPLIT_BF16 ? split_part_elems(x->n, x->op)
+                                                               : (size_t)64 * x->n * x->op);
   int Lc = x->X;
-  while (Lc > 1 && fixed + chunk_bytes(x, Lc) + (size_t)64 * x->n * x->op * 8 > cap) Lc = (Lc + 1) / 2;
+  while (Lc > 1 && fixed + chunk_bytes(x, Lc) + part > cap) Lc = (Lc + 1) / 2;
   if (fixed + chunk_bytes(x, Lc) > cap) {
     free(x);
     return LAS_ERR_WORKSPACE;

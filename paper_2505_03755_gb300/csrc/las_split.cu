@@ -1800,14 +1800,14 @@ struct SplitState {
   Planes HdigT;          // rows mu, K = (L, p)
   Planes Wdig;           // rows q, K = (L, p)
   int* Wexp;             // [op]
-  double* part;          // [ksplit][n][op]
+  double* part;          // split_part_elems(n, op): [ks][n][op], or [ks][n][n] of the exchange
   unsigned long long* mx;  // [op + n] row maxima for long-row slicing
   Planes Mpd;            // rows p of C[:, p0:p1]^T (K = mu) for the (L|pu) transform (lazy)
   int* Mpexp;
   void* Mpblob;
   Planes hdig;           // rows mu of h, K = nu
   int* hexp;             // [n]
-  int ksplit6;           // partial buffers allocated for this many K splits
+  int ksplit6;           // the projection's partials fit `part` for this many K splits
   int ks;                // split-K factor of the projection GEMM (autotunable)
   int bn[SPLIT_NKIND];   // tile width of each product kind (64 or 96) as chosen by the caller or the
                          // autotuner, or 0: by the rule of its columns
@@ -1837,6 +1837,13 @@ size_t split_bytes_per_aux(int n, int op) {
   return (size_t)NDIG * op * rup(n, BK) * 2 * 2 + (size_t)NDIG * ROWPAD * op * 2 + (size_t)op * 4;
 }
 
+// Doubles of the partial buffer: 64 K splits of an n x op projection, and at least one n x n partial
+// of the exchange product (more when n > 64 op: few occupied orbitals in a large basis).
+constexpr int PART_KSPLIT = 64;
+size_t split_part_elems(int n, int op) {
+  return (size_t)n * std::max((long)PART_KSPLIT * op, (long)n);
+}
+
 las_status split_create(SplitState** out, int n, int X, int op, int Lc, const double* Bp,
                         int packed, int* status, cudaStream_t st, size_t* bytes) {
   *out = nullptr;
@@ -1848,7 +1855,7 @@ las_status split_create(SplitState** out, int n, int X, int op, int Lc, const do
   s->op = op;
   s->Lc = Lc;
   s->status = status;
-  s->ksplit6 = 64;
+  s->ksplit6 = PART_KSPLIT;
   // one-time launch attributes, so that later calls can be captured into CUDA graphs
   if (ozaki_prepare() != LAS_OK || num_sms() <= 0) {
     free(s);
@@ -1903,7 +1910,7 @@ las_status split_create(SplitState** out, int n, int X, int op, int Lc, const do
   A(&q, planes_bytes(n, R));         s->HdigT = make_planes(q, n, R);   q = nullptr;
   A(&q, planes_bytes(op, R));        s->Wdig = make_planes(q, op, R);   q = nullptr;
   A((void**)&s->Wexp, (size_t)op * 4);
-  A((void**)&s->part, (size_t)s->ksplit6 * n * op * 8);
+  A((void**)&s->part, split_part_elems(n, op) * 8);
   A((void**)&s->mx, (size_t)(op + n) * 8);
   A(&q, planes_bytes(n, n));         s->hdig = make_planes(q, n, n);    q = nullptr;
   A((void**)&s->hexp, (size_t)n * 4);
@@ -2208,12 +2215,13 @@ las_status split_exchange(SplitState* s, int nL, int oc, const double* Ht, doubl
   HT.K = R;
   las_status rc = slice_transposed(Ht, HT, s->hexp, s->mx, true, st);
   if (rc != LAS_OK) return rc;
-  // Partials live in the projection's partial buffer (64 * n * op doubles).  Only tiles that touch
+  // Partials live in the projection's partial buffer (room rows of n doubles).  Only tiles that touch
   // the lower triangle are computed; the caller mirrors the result.  When the rows past the last
   // whole 128-row tile are few, their row tile is mostly padding: they then go as the columns of a
   // second product instead, stored transposed, if that ends sooner (800 orbitals: 30 row-column
   // tiles and 7 narrow ones instead of 39).
-  const long kb = (R + BK - 1) / BK, n1 = n / BM * BM, r = n - n1, room = 64L * s->op;
+  const long kb = (R + BK - 1) / BK, n1 = n / BM * BM, r = n - n1,
+             room = (long)(split_part_elems(s->n, s->op) / n);
   auto rounds = [&](long tiles, long ks) {
     return (tiles * ks + num_sms() - 1) / num_sms() * ((kb + ks - 1) / ks + CHUNK);
   };
@@ -2235,6 +2243,7 @@ las_status split_exchange(SplitState* s, int nL, int oc, const double* Ht, doubl
       ksr = k2;
     }
   }
+  if (ks * n0 + ksr * r > room) return LAS_ERR_INTERNAL;
   rc = ozaki_gemm(HT, 0, s->hexp, n0, HT, 0, s->hexp, n0, R, ks, 0, s->part, n, n0 * n, 0, 0,
                   s->status, st, 1, OZ_BN);
   if (rc != LAS_OK) return rc;

@@ -12,6 +12,8 @@ las_status split_create(SplitState** s, int n, int X, int op, int Lc, const doub
                         int packed, int* status, cudaStream_t st, size_t* bytes);
 // Device bytes per auxiliary index of the per-evaluation digit workspace.
 size_t split_bytes_per_aux(int n, int op);
+// doubles of the buffer of K-split partials
+size_t split_part_elems(int n, int op);
 // Row exponents of the current chunk's half-transformed rows (L, p): the per-aux kernel scales
 // the projection matrix by 2^exp so that the exponents can be moved out of the left operand.
 const int* split_hexp(SplitState* s);

@@ -1,8 +1,9 @@
-"""Limits of buffers and launches: the longest rows that the slicers take through shared memory."""
+"""Limits of buffers and launches: the longest rows that the slicers take through shared memory, and
+exchange partials of a basis with few occupied orbitals."""
 import numpy as np
 import pytest
 
-from gpu_common import built, dev, gpu_energy_grad, torch_cuda
+from gpu_common import built, dev, gpu_energy_grad, make_las, torch_cuda
 from las_inputs import make_system
 from oracle import las_oracle as O
 
@@ -42,3 +43,27 @@ def test_energy_grad_longest_projection_rows(n, c, X):
         assert abs(E - ref["E"]) <= 1e-8
         assert np.abs(G - ref["G"]).max() <= 1e-8
         assert np.abs(g - ref["gorb"]).max() <= 1e-7
+
+
+# More than 64 basis functions per padded occupied column: one n x n partial of the exchange is larger
+# than the projection's partials.  1030 orbitals also leave 6 rows past the last row tile, and 1024
+# (no more than 64 per column) is the other side of the edge.
+@pytest.mark.parametrize("n", [1024, 1030, 1152])
+@pytest.mark.parametrize("precision", ["split", "split_packed"])
+def test_exchange_with_few_occupied_orbitals(n, precision):
+    s = make_system(n, 5, 8, [(2, 2), (2, 3)], seed=n)
+    las = make_las(s, precision)
+    (Jr,), (Kr,) = O.df_jk(s.Bp, n, [2.0 * s.C[:, :8] @ s.C[:, :8].T])
+    J, K = las.df_jk(dev(s.C))
+    las.sync()
+    assert np.abs(J.cpu().numpy() - Jr).max() <= 1e-11 * np.abs(Jr).max()
+    assert np.abs(K.cpu().numpy() - Kr).max() <= 1e-11 * np.abs(Kr).max()
+    # densities of both spins, one with a weight of the other sign
+    Cx, w = np.ascontiguousarray(s.C[:, :13]), np.linspace(1.0, 0.4, 13)
+    wb = np.where(np.arange(13) < 9, w, -w)
+    va_r, vb_r = O.embedding_potentials(s.Bp, n, Cx * w @ Cx.T, Cx * wb @ Cx.T)
+    va, vb = las.veff(dev(Cx), dev(w), dev(Cx), dev(wb))
+    las.sync()
+    for v, ref in ((va, va_r), (vb, vb_r)):
+        assert np.abs(v.cpu().numpy() - ref).max() <= 1e-11 * np.abs(ref).max()
+    las.close()
