@@ -198,14 +198,19 @@ extern "C" las_status las_create(las_ctx** out, const las_dims* d, const double*
   memset(&x->fi_c, 0, sizeof(x->fi_c));
   x->fi_c.ncore = d->ncore;
 
-  // Workspace plan: the largest auxiliary chunk that fits the cap.
+  // Workspace plan: the largest auxiliary chunk that fits the cap, beside one part of the Coulomb sum
+  // and the pair-transposed 2-RDMs; then as many more parts as are wanted and still fit.  (A chunk of
+  // one row is accepted without room for the transposed 2-RDMs, which then come on top of the cap,
+  // as the staging buffers of the host-buffer call always do.)
   const size_t fixed = sizeof(double) * ((size_t)x->n * x->op * 4 + E1_BLOCKS +
                                          (size_t)x->nmo * x->op + 3 * (size_t)x->X + x->npair);
   size_t cap = max_ws ? max_ws : (size_t)64 << 30;
   const size_t part = sizeof(double) * (prec == LAS_SPLIT_BF16 ? split_part_elems(x->n, x->op)
                                                                : (size_t)64 * x->n * x->op);
+  const size_t dm2t = sizeof(double) * (size_t)x->ndm2;
+  auto planned = [&](int rows) { return fixed + dm2t + chunk_bytes(x, rows) + part; };
   int Lc = x->X;
-  while (Lc > 1 && fixed + chunk_bytes(x, Lc) + part > cap) Lc = (Lc + 1) / 2;
+  while (Lc > 1 && planned(Lc) > cap) Lc = (Lc + 1) / 2;
   if (fixed + chunk_bytes(x, Lc) > cap) {
     free(x);
     return LAS_ERR_WORKSPACE;
@@ -218,6 +223,10 @@ extern "C" las_status las_create(las_ctx** out, const las_dims* d, const double*
         cudaDeviceGetAttribute(&x->sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
         x->sms <= 0)
       x->sms = 152;
+  }
+  {
+    const size_t used = planned(Lc), left = cap > used ? (cap - used) / (sizeof(double) * x->npair) : 0;
+    x->jparts = (int)std::min<size_t>(coulomb_parts(x->npair, x->X, x->sms), 1 + left);
   }
   {
     int tiles = ((x->n + 63) / 64) * ((x->op + 63) / 64);
@@ -240,7 +249,6 @@ extern "C" las_status las_create(las_ctx** out, const las_dims* d, const double*
   ALLOC(eps, x->X);
   ALLOC(vc, x->X);
   ALLOC(va, x->X);
-  x->jparts = coulomb_parts(x->npair, x->X, x->sms);
   ALLOC(Jp, (size_t)x->jparts * x->npair);
   ALLOC(widx, 4 * (size_t)x->o + 4);
   ALLOC(status, 4);

@@ -1,5 +1,5 @@
-"""Limits of buffers and launches: the longest rows that the slicers take through shared memory, and
-exchange partials of a basis with few occupied orbitals."""
+"""Limits of buffers and launches: the longest rows that the slicers take through shared memory,
+exchange partials of a basis with few occupied orbitals, and the workspace cap."""
 import numpy as np
 import pytest
 
@@ -67,3 +67,33 @@ def test_exchange_with_few_occupied_orbitals(n, precision):
     for v, ref in ((va, va_r), (vb, vb_r)):
         assert np.abs(v.cpu().numpy() - ref).max() <= 1e-11 * np.abs(ref).max()
     las.close()
+
+
+# n = 200, X = 1600, one fragment of 24 orbitals: the partial sums of the Coulomb matrix and the
+# transposed 2-RDM are each larger than what the plan leaves unused of the K-split partials
+@pytest.mark.parametrize("rows", [1600, 800, 200, 25])
+def test_workspace_cap_holds_every_buffer(rows):
+    torch = torch_cuda()
+    from paper_2505_03755_gb300 import LasDF
+    n, X, c, m, op = 200, 1600, 4, 24, 32
+    npair, ndm1, ndm2 = n * (n + 1) // 2, 2 * m * m, m ** 4
+    g = torch.Generator(device="cuda")
+    g.manual_seed(rows)
+    B = torch.randn(X, npair, generator=g, device="cuda", dtype=torch.float64)
+    C = torch.linalg.qr(torch.randn(n, n, generator=g, device="cuda", dtype=torch.float64))[0].contiguous()
+    # what the plan counts, with the chunk of `rows` auxiliary rows that it then chooses
+    cap = 8 * (4 * n * op + 256 + n * op + 3 * X + npair + ndm2 + 64 * n * op
+               + rows * op * (n + 2 * op))
+    out = []
+    for limit in (0, cap):
+        las = LasDF(B, n, X, n, c, [m], precision="fp64", max_workspace_bytes=limit)
+        # beside the workspace: the staging buffers of the host-buffer call
+        staging = 8 * (2 * n * n + n * n + ndm1 + ndm2)
+        if limit:
+            assert las.device_bytes() - staging <= limit
+        J, K = las.df_jk(C)
+        las.sync()
+        out.append((J.cpu().numpy(), K.cpu().numpy()))
+        las.close()
+    for x, y in zip(*out):
+        assert np.abs(x - y).max() <= 1e-12 * np.abs(x).max()
