@@ -224,18 +224,19 @@ las_status las_energy_grad_batched(int nsys, las_ctx* const* ctxs, const las_bat
                                    void* stream);
 
 /* Autotuner (split mode; no-op in FP64 mode): by timing whole evaluations with per-stage CUDA
- * events, chooses for this context the tile width (64 or 96 output columns) of each product kind
- * -- the half transform S1, the full transform S2, the projection S5/S6 and the one-electron
- * products -- and then the split-K factor of the projection, keeping the fastest of each.  The
- * choices apply to every later call of the context, batched evaluations included.  Writes E and
+ * events, chooses for this context the tile width (64 or 96 output columns, or the library's rule:
+ * las_get_tiles) of each product kind -- the half transform S1, the full transform S2, the
+ * projection S5/S6 and the one-electron products -- and then the split-K factor of the projection,
+ * keeping the fastest of each.  The choices apply to every later call of the context, batched evaluations included.  Writes E and
  * dEdC as a side effect.  Synchronous. */
 las_status las_autotune(las_ctx* ctx, const double* C, const double* h, const double* dm1s,
                         const double* dm2, double* E, double* dEdC);
 
 /* Tile widths of the split products of a context (bn4: host int[4], for S1, S2, projection and
- * one-electron products; each 64 or 96), as chosen by las_autotune or set by hand; products left to
- * the library may run narrower tiles (results do not depend on the width).  Split mode only
- * (LAS_ERR_UNSUPPORTED otherwise). */
+ * one-electron products; each 64, 96 or 0), as chosen by las_autotune or set by hand.  0, the
+ * default, leaves the product to the library's rule, by which it may run tiles of 48 and 80 columns
+ * too.  Setting what las_get_tiles returned restores that choice.  Results do not depend on the
+ * width.  Split mode only (LAS_ERR_UNSUPPORTED otherwise). */
 las_status las_get_tiles(const las_ctx* ctx, int* bn4);
 las_status las_set_tiles(las_ctx* ctx, const int* bn4);
 

@@ -1340,7 +1340,7 @@ extern "C" las_status las_autotune(las_ctx* x, const double* C, const double* h,
 }
 
 // Tile widths chosen for a split context (or set by hand): product kinds S1, S2, projection,
-// one-electron.
+// one-electron; 0 where the rule of the columns is in force.
 extern "C" las_status las_get_tiles(const las_ctx* x, int* bn4) {
   if (!x || !bn4) return LAS_ERR_ARG;
   if (x->prec != LAS_SPLIT_BF16) return LAS_ERR_UNSUPPORTED;
@@ -1352,7 +1352,7 @@ extern "C" las_status las_set_tiles(las_ctx* x, const int* bn4) {
   if (!x || !bn4) return LAS_ERR_ARG;
   if (x->prec != LAS_SPLIT_BF16) return LAS_ERR_UNSUPPORTED;
   for (int k = 0; k < SPLIT_NKIND; ++k)
-    if (bn4[k] != 64 && bn4[k] != 96) return LAS_ERR_ARG;
+    if (bn4[k] != 0 && bn4[k] != 64 && bn4[k] != 96) return LAS_ERR_ARG;
   for (int k = 0; k < SPLIT_NKIND; ++k) {
     las_status st = split_set_tile(x->split, k, bn4[k]);
     if (st != LAS_OK) return st;

@@ -1991,10 +1991,7 @@ static int project_ksplit(const SplitState* s, long R) {
   const long per = (kb + ks - 1) / ks;
   return (int)((kb + per - 1) / per);
 }
-int split_get_tile(SplitState* s, int kind) {
-  if (s->bn[kind]) return s->bn[kind];
-  return kind == SPLIT_ONE_ELECTRON || cols_time(s->op, 64) < cols_time(s->op, 96) ? 64 : 96;
-}
+int split_get_tile(SplitState* s, int kind) { return s->bn[kind]; }
 las_status split_set_tile(SplitState* s, int kind, int bn) {
   if (kind < 0 || kind >= SPLIT_NKIND || (bn != 0 && bn != 64 && bn != 96)) return LAS_ERR_ARG;
   s->bn[kind] = bn;

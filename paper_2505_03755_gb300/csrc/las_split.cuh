@@ -31,7 +31,7 @@ las_status split_exchange_max(SplitState* s, unsigned long long** mx, cudaStream
 las_status split_exchange(SplitState* s, int nL, int oc, const double* Ht, double* K, int accumulate,
                           double sgn, cudaStream_t st);
 // Product kinds of an evaluation, each with its own tile width (64 or 96 columns as set, or 0, the
-// default: 48 to 96 by a rule of its columns; split_get_tile then gives the nearer of 64 and 96):
+// default: 48 to 96 by a rule of its columns):
 // S1, S2 (with its H slicer), the projection and the one-electron product.
 enum { SPLIT_HALF = 0, SPLIT_FULL = 1, SPLIT_PROJECT = 2, SPLIT_ONE_ELECTRON = 3, SPLIT_NKIND = 4 };
 int split_get_tile(SplitState* s, int kind);

@@ -291,12 +291,15 @@ class LasDF:
                                       _ptr(G)), "las_autotune")
 
     def tiles(self) -> list[int]:
-        """Tile widths (64 or 96) of the split products: S1, S2, projection, one-electron."""
+        """Tile widths of the split products S1, S2, projection and one-electron: 64 or 96 where set
+        or chosen by autotune, 0 (the default) where the library's rule of the columns is in force."""
         buf = (ctypes.c_int * 4)()
         _check(self._lib.las_get_tiles(self._h, buf), "las_get_tiles")
         return list(buf)
 
     def set_tiles(self, widths) -> None:
+        """Set the four widths (64, 96 or 0), e.g. to what tiles() returned; results do not depend on
+        them."""
         buf = (ctypes.c_int * 4)(*[int(w) for w in widths])
         _check(self._lib.las_set_tiles(self._h, buf), "las_set_tiles")
 

@@ -1,5 +1,6 @@
 """Limits of buffers and launches: the longest rows that the slicers take through shared memory,
-exchange partials of a basis with few occupied orbitals, and the workspace cap."""
+exchange partials of a basis with few occupied orbitals, the workspace cap, and the choice of
+tile widths set and read back."""
 import numpy as np
 import pytest
 
@@ -97,3 +98,35 @@ def test_workspace_cap_holds_every_buffer(rows):
         las.close()
     for x, y in zip(*out):
         assert np.abs(x - y).max() <= 1e-12 * np.abs(x).max()
+
+
+@pytest.mark.parametrize("precision", ["split", "split_packed"])
+def test_tile_widths_round_trip(precision):
+    """What tiles() returns can be set again and restores the same choice: 0 stands for the library's
+    rule, in force until a width is set."""
+    s = make_system(60, 80, 30, [(2, 2), (2, 3)], seed=60)
+    las = make_las(s, precision)
+    args = (dev(s.C), dev(s.h), dev(s.dm1s_flat()), dev(s.dm2_flat()))
+
+    def evaluate():
+        E, G = las.energy_grad(*args)
+        las.sync()
+        return float(E), G.cpu().numpy()
+
+    first = las.tiles()
+    assert first == [0, 0, 0, 0]
+    e0, g0 = evaluate()
+    for widths in ([96, 64, 96, 64], [0, 96, 0, 64], first):
+        las.set_tiles(widths)
+        assert las.tiles() == widths
+        e, g = evaluate()
+        assert e == e0 and np.array_equal(g, g0)
+    las.autotune(*args)
+    chosen = las.tiles()
+    las.set_tiles(chosen)
+    assert las.tiles() == chosen
+    for bad in (48, 80, -64, 1):
+        with pytest.raises(Exception):
+            las.set_tiles([bad, 96, 96, 96])
+    assert las.tiles() == chosen
+    las.close()
