@@ -422,7 +422,9 @@ __global__ void k_reduce_partials(const double* __restrict__ part, int nsplit, l
 }
 
 // One-electron energy sum_mu ( 2 sum_i C(mu,i) hC(mu,i) + sum_u C(mu,u) sum_v D_uv hC(mu,v) ): one
-// warp per row mu, one partial per block.  (Only these elements of C_occ^T h C_occ enter the
+// warp per row mu, one partial per block.  The terms have either sign and n o of them cancel to the
+// energy, so each thread carries the rounding errors of its products and sums along (1 to 6 terms of
+// 9 FP64 instructions; 98.2 us for 97.9 at 48 orbitals).  (Only these elements of C_occ^T h C_occ enter the
 // energy; forming the whole matrix took a slicing pass and a product of its own, 45 us at 400
 // orbitals against 4.)
 __global__ void __launch_bounds__(256)
@@ -431,23 +433,29 @@ k_energy_one(const double* __restrict__ Cocc, const double* __restrict__ hC, int
   pdl_begin();
   __shared__ double red[256];
   const int lane = threadIdx.x & 31, c = fi.ncore, o = c + fi.nact;
-  double s = 0.0;
+  double s = 0.0, comp = 0.0;
+  auto add = [&](double a, double b) {   // s + comp += a b
+    const double x = __dmul_rn(a, b), t = s + x, d = t - s;   // (no contraction into s + x)
+    comp += fma(a, b, -x);
+    comp += (s - (t - d)) + (x - d);
+    s = t;
+  };
   for (long mu = blockIdx.x * 8L + (threadIdx.x >> 5); mu < n; mu += gridDim.x * 8L) {
     const double* Cr = Cocc + mu * op;
     const double* hr = hC + mu * op;
     for (int p = lane; p < o; p += 32) {
       if (p < c) {
-        s += 2.0 * Cr[p] * hr[p];
+        add(2.0 * Cr[p], hr[p]);
       } else {
         const int u = p - c, K = frag_of(fi, u), oK = fi.off[K], m = fi.off[K + 1] - oK;
         const double* g = dm1s + fi.dm1_off[K] + (u - oK) * m;
         double t = 0.0;
         for (int v = 0; v < m; ++v) t += (g[v] + g[m * m + v]) * hr[c + oK + v];
-        s += Cr[p] * t;
+        add(Cr[p], t);
       }
     }
   }
-  const double t = block_sum0<256>(s, red);
+  const double t = block_sum0<256>(s + comp, red);
   if (threadIdx.x == 0) e1[blockIdx.x] = t;
 }
 

@@ -1,6 +1,6 @@
 """Limits of buffers and launches: the longest rows that the slicers take through shared memory,
-exchange partials of a basis with few occupied orbitals, the workspace cap, and the choice of
-tile widths set and read back."""
+exchange partials of a basis with few occupied orbitals, the workspace cap, the choice of tile
+widths set and read back, and the rounding of the one-electron energy."""
 import numpy as np
 import pytest
 
@@ -129,4 +129,20 @@ def test_tile_widths_round_trip(precision):
         with pytest.raises(Exception):
             las.set_tiles([bad, 96, 96, 96])
     assert las.tiles() == chosen
+    las.close()
+
+
+def test_one_electron_energy_is_compensated():
+    """Row 0 holds 2^60, 1 and -2^60 in columns 0, 32 and 64, and row 1 again: a sum that does not
+    carry its rounding errors loses the ones.  All values and their products are exact; E = 4."""
+    from paper_2505_03755_gb300 import LasDF
+    n, c, X = 70, 67, 2
+    B, h, C = np.zeros((X, n * (n + 1) // 2)), np.zeros((n, n)), np.zeros((n, n))
+    h[0, 1] = h[1, 0] = 2.0 ** 60
+    C[0, [0, 32, 64]] = 1.0
+    C[1, [0, 32, 64]] = 1.0, 2.0 ** -60, -1.0
+    las = LasDF(dev(B), n, X, n, c, [], precision="fp64")
+    E = las.energy(dev(C), dev(h), dev(np.zeros(0)), dev(np.zeros(0)))
+    las.sync()
+    assert float(E) == 4.0
     las.close()
