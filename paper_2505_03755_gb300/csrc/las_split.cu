@@ -2606,8 +2606,9 @@ extern "C" las_status las_split_gemm_noalloc(long M, long N, long K, const doubl
     }
     scratch = g_noalloc_addr[dev];
   }
-  // The shared array keeps whatever the previous call left; las_split_gemm clears the status
-  // word it keeps there before use and overwrites every digit plane it reads.
+  // The shared array keeps whatever the previous call left: las_split_gemm clears the status word it
+  // keeps there, and writes every digit of the M rows and N columns.  The planes' padding rows stay
+  // as they are; tiles read them, but only for rows and columns of the product that are not stored.
   return las_split_gemm(M, N, K, A, lda, B, ldb, C, ldc, scratch, LAS_NOALLOC_SCRATCH_BYTES,
                         stream);
 }

@@ -48,19 +48,6 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
   return ok != 0;
 }
 
-// Non-blocking test of phase `parity` (try_wait may suspend the thread for a while before it
-// returns false; test_wait returns at once).
-__device__ __forceinline__ bool mbar_test_wait(uint64_t* bar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n .reg .pred p;\n mbarrier.test_wait.parity.acquire.cta.shared::cta.b64 p, [%1], %2;\n"
-      " selp.u32 %0, 1, 0, p;\n}\n"
-      : "=r"(ok)
-      : "r"(smem_u32(bar)), "r"(parity)
-      : "memory");
-  return ok != 0;
-}
-
 // Bounded wait on phase `parity`.  Returns false (and raises the abort flag) on timeout or when
 // another role already aborted.  sleep_ns > 0 backs off between polls (for waiters whose latency
 // does not matter, so that they leave issue slots to the latency-critical warps).
@@ -182,19 +169,8 @@ __device__ __forceinline__ void tmem_wait_ld() {
   asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
 
-// Shared-memory matrix descriptor (tcgen05 format): K-major operand tile whose rows are 64 bytes
-// (32 BF16) in the 64-byte swizzle mode; 8-row core groups are 512 bytes apart.
-__device__ __forceinline__ uint64_t smem_desc_sw64(uint32_t saddr) {
-  uint64_t d = 0;
-  d |= (uint64_t)((saddr >> 4) & 0x3FFF);          // start address
-  d |= (uint64_t)1 << 16;                          // leading byte offset (unused here)
-  d |= (uint64_t)(512 >> 4) << 32;                 // stride byte offset: 8 rows x 64 B
-  d |= (uint64_t)1 << 46;                          // descriptor version
-  d |= (uint64_t)4 << 61;                          // swizzle: 64-byte
-  return d;
-}
-
-// The same for 32-byte rows (16 BF16) in the 32-byte swizzle mode; 8-row groups 256 bytes apart.
+// Shared-memory matrix descriptor (tcgen05 format): K-major operand tile whose rows are 32 bytes
+// (16 BF16) in the 32-byte swizzle mode; 8-row core groups are 256 bytes apart.
 __device__ __forceinline__ uint64_t smem_desc_sw32(uint32_t saddr) {
   uint64_t d = 0;
   d |= (uint64_t)((saddr >> 4) & 0x3FFF);          // start address
