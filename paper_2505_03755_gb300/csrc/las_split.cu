@@ -26,14 +26,12 @@
 #include <type_traits>
 #include <vector>
 
+#include "digit_planes.h"
 #include "las_split.cuh"
 #include "sm100_ptx.cuh"
 
 namespace lasdf_split {
 
-constexpr int NDIG = 6;
-constexpr int BM = 128;          // rows per CTA tile (tcgen05 M)
-constexpr int BK = 16;           // K per pipeline stage (one 32-byte swizzle row of BF16)
 constexpr int NEXACT = 4;        // exact weight groups q = 0..3
 constexpr int NGROUP = 6;        // weight groups q = s + t = 0..5 kept (21 digit pairs)
 
@@ -70,85 +68,6 @@ struct OzTile {
   static constexpr int SMEM_BYTES = NSTAGE * STAGE_BYTES + 1024 + 256;
   static_assert(STAGE_BYTES % 1024 == 0, "stages stay 1024-byte aligned");
 };
-
-// Digit planes are stored K-blocked: the 16 values of K block k / BK of row r of plane s lie at
-//   s*plane + (k / BK) * (Rpad * BK) + r * BK,   Rpad = R rounded up to ROWPAD,
-// so that every pipeline stage of every tile is one contiguous block per plane, and the two
-// 8-value halves of such a 32-byte row are swapped when bit 2 of r is set.  That is the image the
-// MMA's 32-byte-swizzle operand has in shared memory (16-byte chunk index ^= address bit 7), so a
-// stage is a plain copy: the tensor maps see rows of 256 elements (16 stored rows, 512 bytes) and
-// do not swizzle.  The TMA unit works through a box row by row, about 1.4 clocks per row however
-// short it is: loads of 32-byte rows with the swizzle done by the TMA took 1810 clocks per 42 KB
-// stage on every SM, as long as the MMAs, and 512-byte rows take 760 (18 TB/s over the chip).  Row
-// coordinates of a box are therefore multiples of ROWGRAN (OzParams::row_skip).
-// A tile box that reaches past Rpad reads the next K block's rows (finite digits) or, at the end
-// of a plane, the TMA's zero fill: those rows only feed output rows or columns beyond M or N,
-// which are never stored.
-constexpr long ROWPAD = 384;
-constexpr int ROWGRAN = 16;      // stored rows per 512-byte row of the tensor maps
-
-struct Planes {
-  __nv_bfloat16* p;
-  long R, Rpad, K, nkb, plane;   // rows, padded rows, K, K blocks, elements per plane
-  __host__ __device__ __forceinline__ long idx(int s, long r, long k) const {
-    return s * plane + (k / BK) * (Rpad * BK) + swz(r, (int)(k % BK));
-  }
-  // Position of value c (0..15) of row r inside a K block: the 8-value halves swap with bit 2 of r.
-  static __host__ __device__ __forceinline__ long swz(long r, int c) {
-    return r * BK + (c ^ ((int)(r & 4) << 1));
-  }
-};
-
-static inline long planes_rpad(long R) { return (R + ROWPAD - 1) / ROWPAD * ROWPAD; }
-static inline long planes_nkb(long K) { return (K + BK - 1) / BK; }
-static inline size_t planes_bytes(long R, long K) {
-  return (size_t)NDIG * planes_rpad(R) * planes_nkb(K) * BK * 2;
-}
-static inline Planes make_planes(void* p, long R, long K) {
-  Planes P;
-  P.p = (__nv_bfloat16*)p;
-  P.R = R;
-  P.Rpad = planes_rpad(R);
-  P.K = K;
-  P.nkb = planes_nkb(K);
-  P.plane = P.nkb * P.Rpad * BK;
-  return P;
-}
-
-// The Cholesky vectors as digit planes in packed-triangle form.  The first n1 = 128 nb1 rows of
-// every b^L lie in full 128-row blocks, of which only the lower tiles (I >= J) are stored (the
-// diagonal tiles whole): T = nb1 (nb1 + 1) / 2 tiles per L, tile (I, J) of L at index
-// L T + I (I + 1) / 2 + J, each as 8 K blocks of 128 rows x 16 (the Planes layout with 128 rows
-// and 8 X T K blocks).  The half transform reads a tile as it is stored for the rows of block I
-// and MN-major (transposed) for the rows of block J.  The r = n - n1 ragged rows mu >= n1 of each
-// b^L are stored whole (rows (L, mu - n1), K = nu; when there are full blocks each L's rows are
-// padded with zero rows to rp, a multiple of ROWGRAN, so that every L starts at a box coordinate);
-// they are read as they are for their own rows and MN-major for the columns nu >= n1 of the full
-// blocks.  One exponent per L (max |b^L| < 2^e(L)), so that a stored element has the same scale for
-// both rows that use it.
-struct BPacked {
-  int n, X, nb1, T, r, rp, n1;
-  Planes tiles;       // R = Rpad = 128, nkb = 8 X T
-  Planes rag;         // rows (L, j), j < rp, of all X rp; K = n
-  int* exp;           // [X]
-  unsigned long long* mx;   // [X] max |b^L| as ordered bit patterns (set-up scratch)
-};
-
-static inline BPacked bpacked_geometry(int n, int X) {
-  BPacked b;
-  memset(&b, 0, sizeof(b));
-  b.n = n;
-  b.X = X;
-  b.nb1 = n / 128;
-  b.T = b.nb1 * (b.nb1 + 1) / 2;
-  b.n1 = 128 * b.nb1;
-  b.r = n - b.n1;
-  b.rp = b.nb1 > 0 ? (b.r + ROWGRAN - 1) / ROWGRAN * ROWGRAN : b.r;
-  return b;
-}
-static inline size_t bpacked_tile_bytes(const BPacked& b) {
-  return (size_t)NDIG * 8 * (size_t)b.X * b.T * 128 * BK * 2;
-}
 
 struct OzParams {
   int M, N;                // output rows / columns
@@ -665,19 +584,8 @@ k_ozaki(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtenso
         }
       }
       const OzParams& p = *cur.P;
-      // packed-triangle A, per tile: its row block R of b^L (tile (L, R) of the chunk), the K
-      // block of stored tile (R, 0), the index of stored tile (R, R) less R (R + 1) / 2, and the
-      // ragged row of K block 0, so that each stage adds its K block kb = 8 J + kk only
-      int pk_R = 0;
-      long pk_row = 0, pk_col = 0, pk_rag = 0;
-      if (PACK && p.a_pack) {
-        const int mt = cur.m0 / BM, Lr = mt / p.pk_nb1;
-        pk_R = mt - Lr * p.pk_nb1;
-        const long Lg = (long)p.pk_L0 + Lr;
-        pk_row = (Lg * p.pk_T + pk_R * (pk_R + 1) / 2) * 8;
-        pk_col = Lg * p.pk_T + pk_R;
-        pk_rag = Lg * p.pk_rp - 8L * p.pk_nb1 * BK;
-      }
+      PackedBoxes pk = {};
+      if (PACK && p.a_pack) pk = packed_boxes(p.pk_L0, cur.m0 / BM, p.pk_nb1, p.pk_T, p.pk_rp);
       for (int i = 0; i < cur.nkb; ++i) {
         if (filled == NSTAGE && !sm100::mbar_wait(&empty[st], phase ^ 1, abort_flag, p.status,
                                                   LAS_ERR_TIMEOUT)) {
@@ -689,22 +597,19 @@ k_ozaki(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtenso
         const int kb = cur.kb0 + i;
         if (PACK && p.a_pack) {   // K block kb = 8 J + kk lies in column block J of b^L
           const int J = kb >> 3;
-          if (J <= pk_R)           // stored lower tile (R, J): rows mu, K = nu
-            sm100::tma_load_3d(sa, cur.ma, &full[st], 0, (int)((pk_row + kb) * (BM / ROWGRAN)), 0);
+          if (J <= pk.R)           // stored lower tile (R, J): rows mu, K = nu
+            sm100::tma_load_3d(sa, cur.ma, &full[st], 0, pk.lower(kb), 0);
           else if (J < p.pk_nb1)   // stored tile (J, R) read MN-major: its rows are this K
-            sm100::tma_load_4d(sa, cur.ma2, &full[st], 0, kb & 7,
-                               (int)((pk_col + J * (J + 1) / 2) * 8), 0);
+            sm100::tma_load_4d(sa, cur.ma2, &full[st], 0, kb & 7, pk.mirror(J), 0);
           else                     // ragged rows nu >= n1 of b^L, MN-major
-            sm100::tma_load_4d(sa, cur.ma3, &full[st], 0, (int)((pk_rag + (long)kb * BK) / ROWGRAN),
-                               pk_R * (BM / BK), 0);
+            sm100::tma_load_4d(sa, cur.ma3, &full[st], 0, pk.ragged(kb), pk.R * (BM / BK), 0);
         } else if (p.a_mn) {   // rows of the stored planes are this product's K, their K blocks its M
           sm100::tma_load_4d(sa, cur.ma, &full[st], 0, p.a_row0 / ROWGRAN + kb, cur.m0 / BK, 0);
         } else {
-          sm100::tma_load_3d(sa, cur.ma, &full[st], 0,
-                             (int)(((long)kb * p.a_rpad + p.a_row0 + cur.m0) / ROWGRAN), 0);
+          sm100::tma_load_3d(sa, cur.ma, &full[st], 0, box_row(kb, p.a_rpad, p.a_row0, cur.m0), 0);
         }
         sm100::tma_load_3d(sa + A_BYTES, cur.mb, &full[st], 0,
-                           (int)(((long)kb * p.b_rpad + p.b_row0 + cur.n0) / ROWGRAN), 0);
+                           box_row(kb, p.b_rpad, p.b_row0, cur.n0), 0);
         if (filled < NSTAGE) ++filled;
         if (++st == NSTAGE) {
           st = 0;
@@ -1573,7 +1478,7 @@ static las_status ozaki_setup(OzProblem& pr, const Planes& A, long a_row0, const
     return LAS_ERR_INTERNAL;
   // box coordinates are multiples of ROWGRAN rows: the product starts up to 15 rows early and
   // drops what it computes there
-  const int skip = (int)(a_row0 % ROWGRAN);
+  const int skip = box_skip(a_row0);
   if (b_row0 % ROWGRAN || (skip && (a_mn || lower)) || M + skip > 0x7FFFFFFFL)
     return LAS_ERR_INTERNAL;
   las_status s = ozaki_prepare();
