@@ -153,7 +153,7 @@ void launch_pack_weighted(const double* Cx, const double* w, const int* idx, int
 // out (+)= scale sum_k part[k*count ...] in order of k; with cols < ld the values are rows of
 // `cols` that land `ld` apart in out
 void launch_reduce_partials(const double* part, int nsplit, long count, double* out,
-                            int accumulate, cudaStream_t s, int cols = 0, int ld = 0,
+                            int accumulate, cudaStream_t s, long cols = 0, long ld = 0,
                             double scale = 1.0);
 void launch_assemble_grad(const double* Out, const double* hC, const double* dm1s,
                           const FragInfo& fi, int n, int nmo, int op, double* G,

@@ -409,7 +409,7 @@ __global__ void k_sym_add(const double* __restrict__ X, long nL, int op, double*
 
 // Partials of rows of `cols` values, summed in order into rows `ld` apart.
 __global__ void k_reduce_partials(const double* __restrict__ part, int nsplit, long count,
-                                  double* __restrict__ out, int accumulate, int cols, int ld,
+                                  double* __restrict__ out, int accumulate, long cols, long ld,
                                   double scale) {
   pdl_begin();
   long i = blockIdx.x * (long)blockDim.x + threadIdx.x;
@@ -761,7 +761,7 @@ void launch_trace_ht(const double* Ht, const double* CT, int nL, int r, int n, d
 }
 
 void launch_reduce_partials(const double* part, int nsplit, long count, double* out,
-                            int accumulate, cudaStream_t s, int cols, int ld, double scale) {
+                            int accumulate, cudaStream_t s, long cols, long ld, double scale) {
   launch_chained(k_reduce_partials, nblk(count, 256), 256, 0, s, part, nsplit, count, out, accumulate, cols,
                                                      ld, scale);
   las_count_launch();

@@ -2253,7 +2253,7 @@ extern "C" las_status las_split_gemm(long M, long N, long K, const double* A, lo
     rc = ozaki_gemm(Ad, 0, ea, M, Bd, 0, eb, N, K, 1, 0, C, ldc, 0, 0, 0, status, st);
   } else {
     rc = ozaki_gemm(Ad, 0, ea, M, Bd, 0, eb, N, K, ks, 0, part, N, M * N, 0, 0, status, st);
-    if (rc == LAS_OK) launch_reduce_partials(part, ks, M * N, C, 0, st, (int)N, (int)ldc);
+    if (rc == LAS_OK) launch_reduce_partials(part, ks, M * N, C, 0, st, N, ldc);
   }
   if (rc != LAS_OK) return rc;
   int h = 0;

@@ -1,6 +1,7 @@
 """Limits of buffers and launches: the longest rows that the slicers take through shared memory,
 exchange partials of a basis with few occupied orbitals, the workspace cap, the choice of tile
-widths set and read back, and the rounding of the one-electron energy."""
+widths set and read back, the rounding of the one-electron energy, and results whose rows are far
+apart."""
 import numpy as np
 import pytest
 
@@ -146,3 +147,28 @@ def test_one_electron_energy_is_compensated():
     las.sync()
     assert float(E) == 4.0
     las.close()
+
+
+@pytest.mark.parametrize("K", [1041, 40])
+def test_split_gemm_rows_of_the_result_far_apart(K):
+    """A leading dimension of C beyond 2^31 values (a product that is split over K, and one that is
+    not): the two rows land where they belong."""
+    torch = torch_cuda()
+    from paper_2505_03755_gb300 import load_library
+    lib = load_library()
+    M, N, ldc = 2, 5, 2 ** 31 + 8
+    if torch.cuda.mem_get_info()[0] < 40 << 30:
+        pytest.skip("needs 18 GB")
+    rng = np.random.default_rng(K)
+    A, B = np.rint(50 * rng.standard_normal((M, K))), np.rint(50 * rng.standard_normal((K, N)))
+    a, b = dev(A), dev(B)
+    c = torch.empty((M - 1) * ldc + N, dtype=torch.float64, device="cuda")
+    need = lib.las_split_gemm_workspace(M, N, K)
+    ws = torch.empty(need, dtype=torch.uint8, device="cuda")
+    st = torch.cuda.current_stream().cuda_stream
+    assert lib.las_split_gemm(M, N, K, a.data_ptr(), K, b.data_ptr(), N, c.data_ptr(), ldc,
+                              ws.data_ptr(), need, st) == 0
+    got = torch.stack([c[:N], c[ldc:ldc + N]]).cpu().numpy()
+    del c
+    torch.cuda.empty_cache()
+    assert np.array_equal(got, A @ B)
