@@ -261,7 +261,11 @@ int las_stage_times(las_ctx* ctx, float* ms, int cap);
  * only as an outlook, section "Outlook"); it implements that outlook for this hardware.
  * workspace: device buffer of at least las_split_gemm_workspace(M, N, K) bytes, 256-byte
  * aligned, owned by the caller: the digit planes, and where few tiles would leave SMs idle the
- * partial sums of a K split (a buffer that holds only the planes is accepted too).  Synchronous: returns after C is written (or an error). */
+ * partial sums of a K split.  A buffer that holds only the planes, or fewer partial sums, is
+ * accepted too: K is then split into as many parts as fit.  The number of parts decides the order of
+ * the FP32 and FP64 additions, so C is the same to the last bit for the same sizes and the same
+ * workspace_bytes, and agrees within the error above between different ones.  Synchronous: returns
+ * after C is written (or an error). */
 size_t las_split_gemm_workspace(long M, long N, long K);
 las_status las_split_gemm(long M, long N, long K, const double* A, long lda, const double* B,
                           long ldb, double* C, long ldc, void* workspace,
@@ -276,7 +280,8 @@ las_status las_split_gemm(long M, long N, long K, const double* A, long lda, con
  * every GPU that loads the library until the process exits); nothing is allocated or freed.
  * Sizes whose digit planes do not fit the array are rejected with LAS_ERR_WORKSPACE before any
  * GPU work.  (las_split_gemm_workspace may ask for more: it counts the partial sums of a K split,
- * which is shortened to what is left of the array.)
+ * which is shortened to what is left of the array; las_split_gemm with more workspace than that
+ * may then differ in the last bits.)
  * The first call on each device looks up the array's device address (with that device
  * current) and keeps it for later calls; make that first call before any stream capture
  * begins.  A reset of the device's primary context (cudaDeviceReset) invalidates the kept
