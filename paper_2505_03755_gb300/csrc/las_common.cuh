@@ -127,13 +127,14 @@ void launch_pack_cocc(const double* C, int n, int nmo, int o, int op, double* Co
                       cudaStream_t s, const double* dm2 = nullptr, const FragInfo* fi = nullptr,
                       double* dm2t = nullptr);
 las_status per_aux_prepare();
-// gexp == nullptr: W[L][p][q];  otherwise W is written as Wt[q][L*op + p] * 2^gexp[L*op + p]
 // CT[k][mu] = Cocc[mu][k] for k < r (Cocc is n x op)
 void launch_transpose_cols(const double* Cocc, int n, int op, int r, double* CT, cudaStream_t s);
 // vc[b] (+)= sgn sum_{k<r} sum_mu Ht[(b*r + k)*n + mu] * CT[k*n + mu], b < nL (fixed summation
 // order); and mx[mu] = max(mx[mu], max_{b,k} |Ht|) as bit patterns.  Either of vc, mx may be null.
 void launch_trace_ht(const double* Ht, const double* CT, int nL, int r, int n, double* vc,
                      double sgn, int accumulate, unsigned long long* mx, cudaStream_t s);
+// W_L of every aux row, and eps, vc, va.  gexp == nullptr: W[L][p][q]; otherwise W is written as
+// Wt[q][L*op + p] * 2^gexp[L*op + p]
 void launch_per_aux(const double* T, int nL, int op, const double* dm1s, const double* dm2t,
                     const FragInfo& fi, double* W, double* eps, double* vc, double* va,
                     int with_grad, const int* gexp, cudaStream_t s);

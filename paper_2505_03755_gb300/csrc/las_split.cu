@@ -1252,10 +1252,14 @@ static las_status make_plane_map_mn(CUtensorMap* m, const Planes& P) {
 // tail take 480 of the 512 TMEM columns.  A product runs with tiles of 48, 64, 80 or 96 columns.
 constexpr int OZ_BN = 96;
 constexpr int TILE_WIDTHS[] = {48, 64, 80, 96};
-// Measured time of a stage of each width (clocks per 16 values of K, 50 to 75 stages a tile): what a
-// narrow one saves is its B planes and, at 48 and 64 columns, the issue in turn, so the width that
-// wins is mostly the one that fits.  op = 128 (800 orbitals): 2 x 64 columns 2040, 96 + 64 2450 and B
-// read twice.
+// Time of a stage (16 values of K) of each width in launches of 50 to 75 stages a tile, in clocks of
+// 2070 MHz; only the ratios are used.  (The SMs run this kernel at 1.95 to 2.0 GHz: 503 ns at 64
+// columns, 679 in the half transform and 699 in the full transform at 96, the half transform's being
+// 1340 clocks by the SM's own counter.)  What a narrow tile saves is its B planes and, at 48 and 64
+// columns, the issue in turn, so the width that wins is mostly the one that fits.  op = 128 (800
+// orbitals): 2 x 64 columns 2040, 96 + 64 2450 and B read twice.  Grouped launches, which issue by
+// group, take 1130 to 1170 at 64 columns; the rule is the same there, and for 241 to 256 columns takes
+// 4 x 64 although 3 x 96 would end about 7 % sooner.
 constexpr int STAGE_TIME[] = {1000, 1020, 1310, 1430};
 static bool valid_bn(int bn) { return bn == 48 || bn == 64 || bn == 80 || bn == 96; }
 static int stage_time(int bn) { return STAGE_TIME[(bn - 48) / 16]; }
@@ -1819,7 +1823,8 @@ las_status split_create(SplitState** out, int n, int X, int op, int Lc, const do
   A((void**)&s->mx, (size_t)(op + n) * 8);
   A(&q, planes_bytes(n, n));         s->hdig = make_planes(q, n, n);    q = nullptr;
   A((void**)&s->hexp, (size_t)n * 4);
-  // rows mu >= n of the transposed planes and the padding rows of C, W and h are never written by the per-evaluation slicers: make them zero once
+  // rows mu >= n of the transposed planes and the padding rows of C, W and h are never written by the
+  // per-evaluation slicers: make them zero once
   const struct { void* p; size_t b; } zero[] = {
       {s->HdigT.p, planes_bytes(n, R)}, {s->Wdig.p, planes_bytes(op, R)},
       {s->Cdig.p, planes_bytes(op, n)}, {s->hdig.p, planes_bytes(n, n)}};
@@ -2178,8 +2183,10 @@ static size_t sgemm_ws(long M, long N, long K) {
          rup(N * 4, 256) + 256;
 }
 
-// K splits of the product: few tiles leave SMs idle, and a split costs the sum of its partials (about
-// 6 K blocks' time).  2999 x 1201 x 187: 48 tiles in 3 parts.
+// K splits of the product: few tiles leave SMs idle, and a split costs the sum of its partials: 6 K
+// blocks' time at 2999 x 1201 x 187 (48 tiles in 3 parts), taken for all sizes, although the sum grows
+// with M N ks.  (us without and with the split: 116 and 81 at 3000 x 1500 x 96, 127 and 56 at 40 x 2000
+// x 96, 104 and 84 at 2999 x 1201 x 187, 177 and 107 at 2000 x 3000 x 64.)
 static int sgemm_ksplit(long M, long N, long K, size_t room) {
   const long tiles = ozaki_tiles(M, N, 0, pick_bn(N)), kb = planes_nkb(K), sms = num_sms();
   const long cap = std::min<long>({16, kb / 4, (long)(room / ((size_t)M * N * 8))});
