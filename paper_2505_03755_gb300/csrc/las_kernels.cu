@@ -424,14 +424,16 @@ __global__ void k_reduce_partials(const double* __restrict__ part, int nsplit, l
 // One-electron energy sum_mu ( 2 sum_i C(mu,i) hC(mu,i) + sum_u C(mu,u) sum_v D_uv hC(mu,v) ): one
 // warp per row mu, one partial per block.  The terms have either sign and n o of them cancel to the
 // energy, so each thread carries the rounding errors of its products and sums along (1 to 6 terms of
-// 9 FP64 instructions; 98.2 us for 97.9 at 48 orbitals).  (Only these elements of C_occ^T h C_occ enter the
-// energy; forming the whole matrix took a slicing pass and a product of its own, 45 us at 400
-// orbitals against 4.)
-__global__ void __launch_bounds__(256)
+// 9 FP64 instructions).  Two rows to a block, so that these are shared out over the SMs (48 orbitals:
+// 96.7 us; 98.2 with eight rows to a block, 97.7 with eight rows and plain sums).  (Only these elements
+// of C_occ^T h C_occ enter the energy; forming the whole matrix took a slicing pass and a product of
+// its own, 45 us at 400 orbitals against 4.)
+constexpr int E1_WARPS = 2;
+__global__ void __launch_bounds__(32 * E1_WARPS)
 k_energy_one(const double* __restrict__ Cocc, const double* __restrict__ hC, int n, int op,
              const double* __restrict__ dm1s, FragInfo fi, double* __restrict__ e1) {
   pdl_begin();
-  __shared__ double red[256];
+  __shared__ double red[32 * E1_WARPS];
   const int lane = threadIdx.x & 31, c = fi.ncore, o = c + fi.nact;
   double s = 0.0, comp = 0.0;
   auto add = [&](double a, double b) {   // s + comp += a b
@@ -440,7 +442,8 @@ k_energy_one(const double* __restrict__ Cocc, const double* __restrict__ hC, int
     comp += (s - (t - d)) + (x - d);
     s = t;
   };
-  for (long mu = blockIdx.x * 8L + (threadIdx.x >> 5); mu < n; mu += gridDim.x * 8L) {
+  for (long mu = blockIdx.x * (long)E1_WARPS + (threadIdx.x >> 5); mu < n;
+       mu += gridDim.x * (long)E1_WARPS) {
     const double* Cr = Cocc + mu * op;
     const double* hr = hC + mu * op;
     for (int p = lane; p < o; p += 32) {
@@ -455,7 +458,7 @@ k_energy_one(const double* __restrict__ Cocc, const double* __restrict__ hC, int
       }
     }
   }
-  const double t = block_sum0<256>(s + comp, red);
+  const double t = block_sum0<32 * E1_WARPS>(s + comp, red);
   if (threadIdx.x == 0) e1[blockIdx.x] = t;
 }
 
@@ -778,8 +781,8 @@ void launch_assemble_grad(const double* Out, const double* hC, const double* dm1
 void launch_energy(const double* eps, int X, const double* Cocc, const double* hC, int n, int op,
                    const double* dm1s, const FragInfo& fi, double* e1, double* E,
                    cudaStream_t s, const double* Out, int nmo, double* G) {
-  const int nb = (int)std::min<long>(nblk(n, 8), E1_BLOCKS);
-  launch_chained(k_energy_one, nb, 256, 0, s, Cocc, hC, n, op, dm1s, fi, e1);
+  const int nb = (int)std::min<long>(nblk(n, E1_WARPS), E1_BLOCKS);
+  launch_chained(k_energy_one, nb, 32 * E1_WARPS, 0, s, Cocc, hC, n, op, dm1s, fi, e1);
   const EnergySum es{eps, X, e1, nb, E};
   if (G)
     launch_chained(k_assemble_grad, nblk((long)n * nmo, 256) + 1, 256, 0, s, Out, hC, dm1s, fi, n,
